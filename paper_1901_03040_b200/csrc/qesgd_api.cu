@@ -68,15 +68,19 @@ int qesgd_create(qesgd_ctx **out, int device, void *cuda_stream)
     ctx->last_cuda_error = 0;
     ctx->d_status = nullptr;
     ctx->d_lr_work = nullptr;
+    ctx->d_lr_epoch = nullptr;
     ctx->lr_work_floats = QESGD_LR_WORK_FLOATS;
     ctx->wait_ns = QESGD_DEFAULT_WAIT_NS;
     ctx->drop_cta = 0xFFFFFFFFu;
     DeviceGuard guard(device);
     if (!guard.ok) { delete ctx; return QESGD_ECUDA; }
     cudaError_t e = cudaMalloc((void **)&ctx->d_status, 256);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&ctx->d_lr_work, ctx->lr_work_floats * sizeof(float));
-    // the head of the workspace holds arrival counters that the kernels leave at zero
+    if (e == cudaSuccess) e = cudaMalloc((void **)&ctx->d_lr_work, (ctx->lr_work_floats + QESGD_LR_EPOCH_FLOATS) * sizeof(float));
+    if (e == cudaSuccess) ctx->d_lr_epoch = ctx->d_lr_work + ctx->lr_work_floats;
+    // the head of the workspace holds arrival counters, its end the accumulators of the persistent
+    // kernel: both are left at zero by the kernels that use them
     if (e == cudaSuccess) e = cudaMemset(ctx->d_lr_work, 0, 256);
+    if (e == cudaSuccess) e = cudaMemset(ctx->d_lr_epoch, 0, QESGD_LR_EPOCH_FLOATS * sizeof(float));
     if (e == cudaSuccess) e = cudaMemset(ctx->d_status, 0, 256);
     if (e == cudaSuccess)
         e = cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, device);
@@ -386,9 +390,8 @@ int qesgd_lr_local_epoch_batch(qesgd_ctx *ctx, const float *X, const float *y, u
     {   // the whole epoch in one persistent kernel where its shape allows
         int launched = 0;
         const int e = qesgd_launch_lr_epoch_fused(X, y, n_local, d, K, batch, lr, u, K > 1 ? u_stride : 0,
-                                                  ctx->d_lr_work, ctx->lr_work_floats, ctx->d_status,
-                                                  ctx->device, ctx->sm_count, ctx->wait_ns, ctx->drop_cta,
-                                                  ctx->stream, &launched);
+                                                  ctx->d_lr_epoch, ctx->d_status, ctx->device, ctx->sm_count,
+                                                  ctx->wait_ns, ctx->drop_cta, ctx->stream, &launched);
         ctx->launches += (uint64_t)launched;
         if (e > 0) return cuda_fail(ctx, e);
         if (e == 0) return QESGD_OK;

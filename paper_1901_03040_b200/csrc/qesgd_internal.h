@@ -21,6 +21,7 @@ struct qesgd_ctx {
     uint32_t *d_status;     // device status word (bit set by kernels)
     float *d_lr_work;       // logistic-regression partial margins
     uint64_t lr_work_floats;
+    float *d_lr_epoch;      // inter-CTA accumulators of the persistent kernel, behind d_lr_work
     uint64_t launches;
     int last_cuda_error;
     int sm_count;
@@ -30,8 +31,12 @@ struct qesgd_ctx {
 static const uint64_t QESGD_DEFAULT_WAIT_NS = 1000000000ull;
 static const uint64_t QESGD_MAX_WAIT_NS = 10000000000ull;
 
-// Workspace for partial margins: K * P * m floats must fit.
-static const uint64_t QESGD_LR_WORK_FLOATS = 1ull << 20;
+// Workspace (4 MiB): partial margins of the two-pass steps, K * P * m floats, and behind them what the
+// persistent kernel's CTAs exchange: a header of 16 words per group of CTAs, then for each of 8 ring
+// slots the accumulators (four 64-bit words) of up to QESGD_LR_EPOCH_ROWS rows of all groups.
+static const uint32_t QESGD_LR_EPOCH_ROWS = 2048;
+static const uint64_t QESGD_LR_EPOCH_FLOATS = QESGD_MAX_WORKERS * 16ull + 8ull * QESGD_LR_EPOCH_ROWS * 8ull;
+static const uint64_t QESGD_LR_WORK_FLOATS = (1ull << 20) - QESGD_LR_EPOCH_FLOATS;
 
 struct EncodeArgs {
     const float *local;
@@ -135,12 +140,11 @@ int qesgd_launch_lr_margins(const float *Xb, const float *yb, uint32_t m, uint64
 int qesgd_launch_lr_gradient(const float *Xb, const float *yb, uint32_t m, uint64_t d,
                              const float *w, float *g, float *work, uint64_t work_floats,
                              cudaStream_t stream, int *launched);
-// A whole local epoch of K workers as one persistent kernel that keeps each minibatch in
-// shared memory between its two uses.  Returns 0 = launched (one memset + one kernel),
-// -1 = shape not covered (the caller falls back to qesgd_launch_lr_step per minibatch),
-// > 0 = cudaError_t.  `work` is zeroed and used for the inter-CTA counters and partial margins.
+// A whole local epoch of K workers as one persistent kernel that reads X once.  Returns 0 =
+// launched (one kernel), -1 = shape not covered (the caller falls back to qesgd_launch_lr_step per
+// minibatch), > 0 = cudaError_t.  `work` (QESGD_LR_EPOCH_FLOATS floats) holds the inter-CTA
+// accumulators: zero before the first launch, and every launch leaves it at zero.
 int qesgd_launch_lr_epoch_fused(const float *X, const float *y, uint64_t n_local, uint64_t d,
                                 uint32_t K, uint32_t batch, float lr, float *u, uint64_t u_stride,
-                                float *work, uint64_t work_floats, uint32_t *status, int device,
-                                int sm_count, uint64_t wait_ns, uint32_t drop_cta, cudaStream_t stream,
-                                int *launched);
+                                float *work, uint32_t *status, int device, int sm_count, uint64_t wait_ns,
+                                uint32_t drop_cta, cudaStream_t stream, int *launched);

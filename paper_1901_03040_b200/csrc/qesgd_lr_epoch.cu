@@ -3,57 +3,59 @@
 // worker task of Algorithm 3: consecutive minibatches of the worker's shard).
 //
 // A step needs the minibatch twice -- once for the margins x_j . u, once for the update
-// sum_j c_j x_j -- with a reduction over all columns in between.  Here every CTA owns a
-// slice of `cols` columns for the whole epoch and keeps its slice of each minibatch in
-// shared memory between the two uses, so X is read from HBM exactly once:
+// sum_j c_j x_j -- with a reduction over all columns in between.  The K workers are dealt out to
+// G groups of P CTAs; a group runs the epochs of its workers, and each of its CTAs owns a slice
+// of `cols` columns for the whole epoch.  The slice of a minibatch (a "tile") passes through the
+// SM once, so X is read from HBM exactly once:
 //
-//   tile (t, k)  = minibatch t of worker k; tiles are processed t-major, k-minor, and
-//                  alternate between two shared-memory buffers
-//   sub-tile     = SUB rows of a tile's column slice, fetched by TMA (one or two 2-D boxes,
-//                  cp.async.bulk.tensor global -> shared, completion on an mbarrier per
-//                  sub-tile); a producer warp issues the copies of tile i+2 as soon as the
-//                  consumer warps have released the buffer of tile i
-//   M(i)  margins of tile i over the CTA's columns; each row's partial margin is added, as a
-//         fixed-point integer, to the row's accumulator acc[i % RING][row] by one 64-bit
-//         reduction that also counts the contribution in the word's top bits
-//   W(i)  wait until every row's count equals the number of CTAs, margins from the sums,
-//         coefficients (lr/m) y_j / (1 + exp(y_j m_j)) into shared memory
-//   U(i)  u[cols] += sum_j coef_j x_j from the tile
+//   producer warp   fetches sub-tiles (8 rows of the slice) by TMA (2-D boxes of at most 256
+//                   columns, cp.async.bulk.tensor global -> shared, completion on an mbarrier
+//                   per slot) into a ring of slots, as far ahead as the ring reaches
+//   consumer chain  eight warps; tile i = minibatch i / Kg of the group's worker i % Kg:
+//     M(i)  warp w takes the sub-tiles w, w + 8, ...: partial margins of the rows over the slice;
+//           the values it reads go to tensor memory on the way (tcgen05.st), so the slot returns
+//           to the producer at once; the partial margins go out to the group's other CTAs
+//     W(i)  wait for the partial margins of all P CTAs; coefficients (lr/m) y_j / (1 + exp(y_j m_j))
+//     U(i)  every warp reads back what it stored (tcgen05.ld), forms coef_j x_j summed over its
+//           rows, the eight warps' sums meet in shared memory and are added to the slice of u,
+//           which stays in shared memory from the first minibatch to the last
 //
-// The exchange of the margins is what the epoch waits for, so it is one step: integer addition
-// is exact and commutes, so the sum over the CTAs needs no order, no second pass over 148
-// partials and -- the count travelling in the same word as the sum -- no fence between data and
-// signal; the result is the same in every run.  A word is count << 55 | sum, every contribution
-// adds 1 << 55 plus 2^45 + round(partial * 2^28) (the 2^45 keeps it positive; |partial| < 2^17;
-// up to 511 CTAs fit below the count).  A larger finite partial goes, in units of 2^-6 (the
-// spacing of fp32 at 2^17), into the second word of the row; a NaN is counted in the third word
-// and makes the margin NaN; an infinite partial, or one of 2^49 or more, is counted by sign in
-// the fourth and makes the margin that infinity (NaN if both signs occur), which the step
-// coefficient saturates on as it would on the number itself.  These rare kinds fence before they
-// count themselves in the first word.  The slot that tile i + RING/2 will use is cleared by one CTA
-// during M(i): every CTA has read it by then (it has taken part in tile i-2, hence finished
-// tile i-4) and none adds to it before it has seen that CTA's contributions to tile i+2.
+// What bounds it.  X is read once, so HBM bounds large minibatches; below, every step is a chain
+// M - exchange - U - M of dependent latencies (2 to 3 us through global memory).  Workers are
+// independent, so groups run side by side (G > 1 divides the number of chained tiles by G), and
+// where one group holds several workers two chains (NC = 2) alternate over its tiles, one
+// computing while the other waits.  The tensor memory (256 KB) holds what waits for its
+// coefficients: 64 rows x 512 columns for each of two chains or x 1024 columns for one.
+// Measured against the kernel this one replaces (one group, u in global memory, tiles kept in two
+// shared-memory buffers, at most 512 columns per SM): K = 8, n = 1010, d = 10000, batch 50:
+// 429 -> 126 us; K = 4, n = 128, d = 4096, batch 32: 38 -> 17; K = 4, n = 512, d = 131072 (two
+// passes before): 426 -> 275; K = 4, n = 2048, d = 65536: 461 -> 421.
 //
-// Where the minibatch has at most 64 rows the tile does not wait in shared memory between M
-// and U: right after M every thread moves its share of it into tensor memory (tcgen05.st;
-// the SM's 256 KB of it hold one tile per consumer group and are otherwise unused here) and
-// the shared-memory slots go back to the producer, so the next tile's copies run while this
-// one waits for the other CTAs; U reads the tile back with tcgen05.ld.  Larger minibatches
-// stay in shared memory and release their slots during U.
-//
-// Each tile's M, W, U is a chain of dependent round trips to global memory (reductions out,
-// sums back) that lasts longer than the tile's own transfer from HBM.  The eight
-// consumer warps therefore form two groups of four; group g owns buffer g and the tiles
-// g, g+2, g+4, ... and runs M(i), W(i), U(i) for them, so one group computes while the other
-// waits, and the copies of the tile after next are in flight meanwhile.  A worker's
-// consecutive minibatches are K tiles apart: with an even K they stay in one group, with an
-// odd K a group waits for the other group's update before it takes the margins.
+// Exchange through global memory: each row's partial margin is added, as a fixed-point integer,
+// to the row's accumulator acc[i % RING][row] by one 64-bit reduction that also counts the
+// contribution in the word's top bits.  Integer addition is exact and commutes, so the sum over
+// the CTAs needs no order, no second pass over the partials and -- the count travelling in the
+// same word as the sum -- no fence between data and signal; the result is the same in every run.
+// A word is count << 55 | special << 54 | sum, every contribution adds 1 << 55 plus 2^45 +
+// round(partial * 2^28) (the 2^45 keeps it positive; |partial| < 2^17; up to 256 CTAs fit below
+// bit 54).  A larger finite partial goes, in units of 2^-6 (the spacing of fp32 at 2^17), into a
+// second word of the row; a NaN is counted in the third word and makes the margin NaN; an infinite
+// partial, or one of 2^49 or more, is counted by sign in the fourth and makes the margin that
+// infinity (NaN if both signs occur), which the step coefficient saturates on as it would on the
+// number itself.  These rare kinds set the special bit, and fence before they count themselves in
+// the first word, so a reader looks at the other words only where the bit is set: one round trip
+// to L2 in place of two.  Every thread that owns a row polls that row's word itself, eight rows
+// to 64 bytes, so a warp's poll and a warp's reduction touch two sectors per sub-tile.
+// The slot that tile i + RING/2 will use is cleared by one CTA after M(i), while it waits: every
+// CTA has read it by then (it has taken part in tile i-2, hence finished tile i-4) and none adds
+// to it before it has seen that CTA's contributions to tile i+2.  The CTA of a group that leaves
+// last clears what is left, so every launch finds the accumulators at zero.
 //
 // The CTAs wait on one another, so the kernel is launched cooperatively (all CTAs are
 // resident by construction: at most one per SM).  Every wait the kernel itself loops on is
 // bounded by the context's wait limit: a wait that runs out sets QESGD_STATUS_TIMEOUT and an
-// abort word that the other CTAs poll, and the CTA's consumer warps leave.  The producer warp
-// is the last to go on every path: it waits (on a bound of its own) for each copy it has
+// abort word that the group's other CTAs poll, and the CTA's consumer warps leave.  The producer
+// warp is the last to go on every path: it waits (on a bound of its own) for each copy it has
 // requested and nobody has consumed, so no CTA ends with a copy still writing its shared
 // memory.  The one wait without a bound is the tensor-memory allocation at the start, which
 // blocks while another kernel resident on the same SM holds tensor memory (until that kernel
@@ -66,42 +68,46 @@
 
 namespace {
 
-constexpr int EP_CONSUMERS = 256;                 // 8 consumer warps
-constexpr int EP_GROUP = EP_CONSUMERS / 2;        // two groups of 4 warps, one per tile buffer
-constexpr int EP_THREADS = EP_CONSUMERS + 32;     // + 1 producer warp
+constexpr int EP_WARPS = 8;                       // consumer warps of a chain
+constexpr int EP_CHAIN = EP_WARPS * 32;
 constexpr int SUB = 8;               // rows per sub-tile
 constexpr int EP_RING = 8;           // accumulator slots; a slot is cleared RING/2 tiles before its use
-constexpr int EP_MAX_COLS = 512;     // columns per CTA: 128 groups of 4
 constexpr int EP_BOX_COLS = 256;     // widest TMA box
-constexpr int EP_MAX_M = 256;        // rows per minibatch the fused path takes
-constexpr int EP_MAX_NSUB = EP_MAX_M / SUB;
+constexpr int EP_MAX_M = EP_CHAIN;   // rows per minibatch: a thread of the chain per row
+constexpr int EP_MAX_SLOTS = 64;     // ring slots
+constexpr int EP_UNITS = 8;          // 8 x 128 blocks of a tile that the tensor memory holds per warp
+constexpr float EP_CHAIN_US = 2.5f, EP_UNIT_US = 0.25f;   // a tile's latency: exchange, and per block of a warp
 constexpr uint64_t DRAIN_LIMIT_NS = 2000000000ull;   // the producer's last wait for its own copies
 constexpr uint64_t COARSE_TIMER_NS = 1024ull;        // limits below this mean "one look, then give up"
-constexpr uint32_t EP_HEADER_WORDS = 64;             // word 0 = abort flag
-constexpr uint32_t EP_ROW_WORDS = 4;                 // 64-bit words per accumulator row (one 32-byte sector)
+constexpr uint32_t EP_HEADER_WORDS = 16;             // per group: [0] abort flag, [1] CTAs that have left
+constexpr uint32_t EP_WIDE_WORDS = 3;                // rarely used 64-bit words per accumulator row
 constexpr float FX_SCALE = 268435456.0f;             // 2^28: unit of the first word
 constexpr float FX_LIMIT = 131072.0f;                // 2^17: partials below go to the first word
 constexpr float FX_WIDE_SCALE = 64.0f;               // 2^6: unit of the second word
 constexpr float FX_WIDE_LIMIT = 562949953421312.0f;  // 2^49: partials below go to the second word
 constexpr unsigned long long FX_BIAS = 1ull << 45;   // makes every contribution to the first word positive
 constexpr unsigned long long FX_ONE = 1ull << 55;    // one contribution counted
+constexpr unsigned long long FX_SPECIAL = 1ull << 54;   // one of the row's other words is in use
 
 struct EpochArgs {
     const float *y;
-    uint64_t y_stride;
     uint64_t n_local;       // rows per worker
     uint64_t d;
-    uint32_t K, batch, nsteps;
+    uint32_t K, G, P;       // workers, groups, CTAs per group
+    uint32_t batch, nsteps;
     uint32_t m_last;        // rows of the last minibatch
     uint32_t nsub_max, nsub_last;
-    uint32_t cols;          // columns per CTA, multiple of 4
+    uint32_t cols, nit;     // columns per CTA (a multiple of 4), blocks of 128 columns
+    uint32_t nslots;        // sub-tiles the ring holds
+    uint32_t off_u, off_part, off_coef, off_bars, off_flags;   // shared-memory layout, bytes
     float lr;
     float *u;
     uint64_t u_stride;
-    uint32_t *header;       // [0] abort flag
-    unsigned long long *acc;   // [EP_RING][batch][EP_ROW_WORDS] margin accumulators, zero at launch
+    uint32_t *header;       // [G][EP_HEADER_WORDS]
+    unsigned long long *acc;    // [G][EP_RING][8 * nsub_max] margin accumulators, zero between launches
+    unsigned long long *wide;   // [G][EP_RING][8 * nsub_max][EP_WIDE_WORDS]
     uint32_t *status;
-    uint64_t wait_ns;       // limit of every wait on another CTA, warp group or copy
+    uint64_t wait_ns;       // limit of every wait on another CTA, chain or copy
     uint32_t poll_mask;     // the clock is read every (poll_mask + 1) looks at a counter
     uint32_t drop_cta;      // test hook: this CTA does not count itself for tile 0 (none: ~0)
 };
@@ -163,6 +169,18 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, const 
         if (*stop != 0u || expired(t0, limit)) return false;
     }
 }
+// Bounded wait until the counter *flag, which another warp of this CTA advances, exceeds `value`.
+__device__ __forceinline__ bool flag_above(const volatile uint32_t *flag, uint32_t value,
+                                           const volatile uint32_t *stop, uint64_t limit)
+{
+    if (*flag > value) return true;
+    const uint64_t t0 = now_ns();
+    for (;;) {
+        for (int n = 0; n < 32; ++n)
+            if (*flag > value) return true;
+        if (*stop != 0u || expired(t0, limit)) return false;
+    }
+}
 // One 2-D box of the row-major matrix X: columns [x, x + box width), rows [y, y + SUB).
 // x * 4 bytes is a multiple of 16; dst is 128-byte aligned.  The copy goes to this CTA alone.
 __device__ __forceinline__ void tma_load_box(float *dst, const CUtensorMap *map, uint32_t x, uint32_t y,
@@ -181,10 +199,10 @@ __device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p)
     return v;
 }
 
-__device__ __forceinline__ ulonglong2 ld_relaxed_v2(const unsigned long long *p)
+__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long *p)
 {
-    ulonglong2 v;
-    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
 
@@ -210,10 +228,10 @@ __device__ __forceinline__ bool sync_any(uint32_t id, uint32_t count, uint32_t f
 
 // ---- tensor memory as a stash for a tile between its two uses --------------------------
 // The SM's 256 KB of tensor memory (128 lanes x 512 columns of 32 bits) is not needed for
-// any matrix product here, so it holds a consumer group's tile while the group waits for the
+// any matrix product here, so it holds a chain's tile while the chain waits for the
 // other CTAs: thread t of a warp owns lane 32 * (warp % 4) + t and reads back exactly what it
 // stored, so no ordering between threads is involved.  One access moves 32 registers of
-// every thread of the warp (the 8 rows x 4 columns a thread takes of a sub-tile).
+// every thread of the warp (the 8 rows x 4 columns a thread takes of an 8 x 128 block).
 __device__ __forceinline__ void tmem_alloc_all(uint32_t *smem_result)   // one whole warp
 {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(smem_result))
@@ -280,374 +298,338 @@ __device__ __forceinline__ uint32_t reduce8_row(uint32_t lane)
 }
 
 struct Tile {
-    uint32_t t, k, m, nsub;
+    uint32_t t, kk, k, m, nsub, first;   // step, worker within the group, worker, rows, sub-tiles, number of the first
 };
-__device__ __forceinline__ Tile tile_of(const EpochArgs &a, uint32_t i)
+__device__ __forceinline__ Tile tile_of(const EpochArgs &a, uint32_t grp, uint32_t kg, uint32_t i)
 {
     Tile r;
-    r.t = i / a.K;
-    r.k = i - r.t * a.K;
+    r.t = i / kg;
+    r.kk = i - r.t * kg;
+    r.k = grp + r.kk * a.G;
     const bool last = r.t == a.nsteps - 1u;
     r.m = last ? a.m_last : a.batch;
     r.nsub = last ? a.nsub_last : a.nsub_max;
+    const uint32_t full = (a.nsteps - 1u) * kg;     // tiles of the steps before the last
+    r.first = last ? full * a.nsub_max + (i - full) * a.nsub_last : i * a.nsub_max;
     return r;
 }
 
 extern __shared__ __align__(1024) unsigned char ep_smem[];
 
-// Shared memory: two tile buffers of nsub_max slots of SUB x cols floats (a slot holds
-// the box of the first 256 columns, then the box of the rest), the step coefficients of
-// the two consumer groups, the barriers, a few flag words.
-__global__ void __launch_bounds__(EP_THREADS, 1)
-    qesgd_lr_epoch_kernel(const EpochArgs a, const __grid_constant__ CUtensorMap map_a,
-                          const __grid_constant__ CUtensorMap map_b)
+// Shared memory: the ring of slots of SUB x cols floats (a slot holds its boxes of 256 columns one
+// after the other, the last one narrower), the slices of u of the group's workers, the warps'
+// partial updates, the step coefficients, the barriers, a few flag words.
+template <int NC>
+__global__ void __launch_bounds__(NC * EP_CHAIN + 32, 1)
+    qesgd_lr_epoch_kernel(const EpochArgs a, const __grid_constant__ CUtensorMap map_full,
+                          const __grid_constant__ CUtensorMap map_rest)
 {
-    const uint32_t slot_floats = SUB * a.cols;
-    float *const tile = reinterpret_cast<float *>(ep_smem);
-    float *const s_coef = tile + (size_t)2u * a.nsub_max * slot_floats;
-    uint64_t *const full = reinterpret_cast<uint64_t *>(s_coef + 2 * EP_MAX_M);
-    uint64_t *const consumed = full + 2 * EP_MAX_NSUB;
-    // [0] a wait ran out in this CTA, [3] always zero, [4], [5] tiles completed by consumer
-    // group 0, 1, [8] base address of the tensor memory
-    volatile uint32_t *const s_flag = reinterpret_cast<volatile uint32_t *>(consumed + 2 * EP_MAX_NSUB);
+    const uint32_t slot_floats = SUB * a.cols, ucols = a.nit * 128u;
+    float *const ring = reinterpret_cast<float *>(ep_smem);
+    float *const s_u = reinterpret_cast<float *>(ep_smem + a.off_u);
+    float *const s_part = reinterpret_cast<float *>(ep_smem + a.off_part);
+    float *const s_coef = reinterpret_cast<float *>(ep_smem + a.off_coef);
+    uint64_t *const full = reinterpret_cast<uint64_t *>(ep_smem + a.off_bars);
+    uint64_t *const empty = full + a.nslots;
+    // [0] a wait ran out in this CTA, [3] always zero, [4], [5] tiles completed by chain 0, 1,
+    // [6] sub-tiles requested by the producer, [8] base address of the tensor memory, [9] last CTA
+    // of the group to leave
+    volatile uint32_t *const s_flag = reinterpret_cast<volatile uint32_t *>(ep_smem + a.off_flags);
 
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-    const uint32_t cta = blockIdx.x, ncta = gridDim.x;
-    const uint32_t c0 = cta * a.cols;
-    const uint32_t cols_a = min(a.cols, (uint32_t)EP_BOX_COLS), cols_b = a.cols - cols_a;
-    const uint32_t ntiles = a.nsteps * a.K;
+    const uint32_t grp = blockIdx.x / a.P, rank = blockIdx.x - grp * a.P;
+    const uint32_t kg = (a.K - grp + a.G - 1u) / a.G;      // workers of this group
+    const uint32_t c0 = rank * a.cols;
+    const uint32_t ntiles = a.nsteps * kg;
 
     if (tid == 0) {
-        for (uint32_t s = 0; s < 2u * a.nsub_max; ++s) mbar_init(&full[s], 1u);
-        for (uint32_t s = 0; s < 2u * a.nsub_max; ++s) mbar_init(&consumed[s], EP_GROUP / 32);
+        for (uint32_t s = 0; s < 2u * a.nslots; ++s) mbar_init(&full[s], 1u);
         for (int f = 0; f < 16; ++f) s_flag[f] = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    // Minibatches of at most 64 rows (8 sub-tiles x 32 registers x 2 groups = all 512 columns)
-    // are stashed in tensor memory between their two uses; larger ones stay in shared memory.
-    const bool stash = a.nsub_max <= 8u;
-    if (stash && warp == 0) tmem_alloc_all(const_cast<uint32_t *>(&s_flag[8]));
+    if (warp == 0) tmem_alloc_all(const_cast<uint32_t *>(&s_flag[8]));
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = s_flag[8];
 
     // ------------------------------------------------------------ producer ----
-    if (warp == EP_CONSUMERS / 32) {
-        // Lane L remembers, for slots L and L + 32 of the 2 * nsub_max slots, the tile whose copy
-        // was requested into the slot last (none: ~0).
-        uint32_t last_tile[2] = {0xFFFFFFFFu, 0xFFFFFFFFu};
-        for (uint32_t i = 0; i < ntiles; ++i) {
-            const uint32_t b = i & 1u;
-            const Tile T = tile_of(a, i);
+    if (warp == NC * EP_WARPS) {
+        // the sub-tiles in the order in which the chains take them, round the ring
+        uint32_t slot = 0u, turn = 0u, issued = 0u;
+        bool ok = true;
+        for (uint32_t i = 0; i < ntiles && ok; ++i) {
+            const Tile T = tile_of(a, grp, kg, i);
             const uint32_t row0 = (uint32_t)((uint64_t)T.k * a.n_local + (uint64_t)T.t * a.batch);
-            bool ok = true;
-            for (uint32_t s = 0; s < T.nsub && ok; ++s) {
-                // a slot is free once the update of tile i-2 has read sub-tile s
-                if (i >= 2u)
-                    ok = __all_sync(0xFFFFFFFFu, mbar_wait(&consumed[b * a.nsub_max + s], ((i - 2u) >> 1) & 1u,
-                                                           &s_flag[0], a.wait_ns)) != 0;
-                if (ok) {
-                    const uint32_t q = b * a.nsub_max + s;
-                    if (q == lane) last_tile[0] = i;
-                    if (q == lane + 32u) last_tile[1] = i;
-                }
-                if (ok && lane == 0) {
-                    uint64_t *const bar = &full[b * a.nsub_max + s];
-                    float *const dst = tile + (size_t)(b * a.nsub_max + s) * slot_floats;
-                    mbar_arrive_expect_tx(bar, slot_floats * 4u);
-                    tma_load_box(dst, &map_a, c0, row0 + s * SUB, bar);
-                    if (cols_b) tma_load_box(dst + SUB * cols_a, &map_b, c0 + cols_a, row0 + s * SUB, bar);
-                }
-            }
-            if (!ok) {
+            for (uint32_t s = 0; s < T.nsub; ++s) {
+                if (turn != 0u)   // the slot's previous sub-tile has been taken
+                    ok = __all_sync(0xFFFFFFFFu,
+                                    mbar_wait(&empty[slot], (turn - 1u) & 1u, &s_flag[0], a.wait_ns)) != 0;
+                if (!ok) break;
                 if (lane == 0) {
-                    s_flag[0] = 1u;
-                    atomicOr(a.status, QESGD_STATUS_TIMEOUT);
-                    atomicExch(a.header, 1u);
+                    float *dst = ring + (size_t)slot * slot_floats;
+                    mbar_arrive_expect_tx(&full[slot], slot_floats * 4u);
+                    uint32_t c = 0u;
+                    for (; c + EP_BOX_COLS <= a.cols; c += EP_BOX_COLS, dst += SUB * EP_BOX_COLS)
+                        tma_load_box(dst, &map_full, c0 + c, row0 + s * SUB, &full[slot]);
+                    if (c < a.cols) tma_load_box(dst, &map_rest, c0 + c, row0 + s * SUB, &full[slot]);
+                    s_flag[6] = issued + 1u;
                 }
-                break;
+                ++issued;
+                if (++slot == a.nslots) { slot = 0u; ++turn; }
             }
+        }
+        if (!ok && lane == 0) {
+            s_flag[0] = 1u;
+            atomicOr(a.status, QESGD_STATUS_TIMEOUT);
         }
         // Last out, on every path: each slot's latest copy has been consumed (then it has
         // landed) or is waited for here, so that the CTA does not end -- and its shared memory
         // is not handed to another CTA -- while a copy is still writing it.  After a normal
         // epoch these waits end with the consumers' last tiles.
         __syncwarp();
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-            if (last_tile[h] != 0xFFFFFFFFu)
-                mbar_wait(&full[lane + 32u * h], (last_tile[h] >> 1) & 1u, &s_flag[3], DRAIN_LIMIT_NS);
+        for (uint32_t q = lane; q < a.nslots && q < issued; q += 32u) {
+            const uint32_t turns = (issued - 1u - q) / a.nslots;    // the slot's latest copy is its turn number `turns`
+            mbar_wait(&full[q], turns & 1u, &s_flag[3], DRAIN_LIMIT_NS);
+        }
         return;
     }
 
     // ----------------------------------------------------------- consumers ----
-    // Two groups of four warps; group g owns buffer g and the tiles i = g, g+2, g+4, ...
-    // Each runs M(i), W(i), U(i) for its own tiles, so that one group computes while the
-    // other waits for the other CTAs.
-    const uint32_t g = warp >> 2, wg = warp & 3u, tg = tid & (EP_GROUP - 1u);
+    const uint32_t g = NC == 2 ? warp / EP_WARPS : 0u, wg = warp % EP_WARPS, tg = tid % EP_CHAIN;
     float *const coef = s_coef + g * EP_MAX_M;
-    auto group_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1u + g), "n"(EP_GROUP) : "memory"); };
+    float *const part = s_part + (size_t)g * EP_WARPS * ucols;
+    auto chain_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1u + g), "n"(EP_CHAIN) : "memory"); };
+    // this thread's lane of the tensor memory, this warp's columns
+    const uint32_t taddr = tmem_base + ((32u * (wg & 3u)) << 16) +
+                           (NC == 2 ? 256u * g + 128u * (wg >> 2) : 256u * (wg >> 2));
+    const uint32_t mpad = SUB * a.nsub_max;
+    unsigned long long *const acc_g = a.acc + (size_t)grp * EP_RING * mpad;
+    unsigned long long *const wide_g = a.wide + (size_t)grp * EP_RING * mpad * EP_WIDE_WORDS;
+    uint32_t *const header = a.header + grp * EP_HEADER_WORDS;
 
-    // this lane's columns of worker k's u (columns lane*4 + 128*it), zeros past the slice
-    auto load_u = [&](uint32_t k, float4 (&uu)[EP_MAX_COLS / 128]) {
-        const float *__restrict__ ug = a.u + (uint64_t)k * a.u_stride + c0;
-#pragma unroll
-        for (int it = 0; it < EP_MAX_COLS / 128; ++it) {
-            const uint32_t c = lane * 4u + it * 128u;
-            uu[it] = (c < a.cols && (uint64_t)c0 + c < a.d) ? *reinterpret_cast<const float4 *>(ug + c)
-                                                           : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-    };
-    // With an even K >= 4 the group's next tile belongs to a worker whose previous minibatch
-    // this group finished an iteration ago: its slice of u is requested a tile early.
-    const bool early_u = (a.K & 1u) == 0u && a.K >= 4u;
-    float4 un[EP_MAX_COLS / 128];
-    if (early_u && g < ntiles) load_u(g % a.K, un);
+    // the slices of u of the group's workers, zeros past the slice
+    for (uint32_t q = tid; q < kg * (ucols / 4u); q += NC * EP_CHAIN) {
+        const uint32_t kk = q / (ucols / 4u), c = (q - kk * (ucols / 4u)) * 4u;
+        const bool in = c < a.cols && (uint64_t)c0 + c < a.d;
+        reinterpret_cast<float4 *>(s_u)[q] =
+            in ? *reinterpret_cast<const float4 *>(a.u + (uint64_t)(grp + kk * a.G) * a.u_stride + c0 + c)
+               : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    asm volatile("bar.sync 3, %0;" ::"n"(NC * EP_CHAIN) : "memory");
 
-    // the update's (and the stash's) share of a tile: four columns, all rows
-    const uint32_t col = tg * 4u;
-    const bool colok = col < a.cols && (uint64_t)c0 + col < a.d;
-    const bool first = col < (uint32_t)EP_BOX_COLS;
-    const uint32_t off = first ? col : SUB * cols_a + (col - EP_BOX_COLS);
-    const uint32_t pitch = first ? cols_a : cols_b;
-    const uint32_t taddr = tmem_base + ((32u * wg) << 16) + 256u * g;   // this thread's lane, this group's columns
+    for (uint32_t i = g; i < ntiles; i += NC) {
+        const Tile T = tile_of(a, grp, kg, i);
+        float *const us = s_u + (size_t)T.kk * ucols;
 
-    for (uint32_t i = g; i < ntiles; i += 2u) {
-        const Tile T = tile_of(a, i);
-        const uint32_t parity = (i >> 1) & 1u;
-        uint64_t *const bars = full + g * a.nsub_max;
-        const float *const buf = tile + (size_t)g * a.nsub_max * slot_floats;
-
-        // The worker's previous minibatch is tile i-K.  With an odd K it belonged to the other
-        // group: wait until that group has stored its update.
-        if (i >= a.K && ((i - a.K) & 1u) != g) {
-            const uint32_t need = ((i - a.K) >> 1) + 1u;
+        // The worker's previous minibatch is tile i-kg.  With two chains and an odd kg it belonged
+        // to the other chain: wait until that chain has stored its update.
+        if (NC == 2 && i >= kg && ((i - kg) & 1u) != g) {
+            const uint32_t need = ((i - kg) >> 1) + 1u;
             if (tg == 0) {
-                const uint64_t t0 = now_ns();
-                while (s_flag[4u + (g ^ 1u)] < need) {
-                    if (s_flag[0] != 0u || expired(t0, a.wait_ns)) {
-                        s_flag[0] = 1u;
-                        break;
-                    }
-                }
+                if (!flag_above(&s_flag[4u + (g ^ 1u)], need - 1u, &s_flag[0], a.wait_ns)) s_flag[0] = 1u;
                 __threadfence_block();
             }
-            if (sync_any(1u + g, EP_GROUP, s_flag[0])) break;
+            if (sync_any(1u + g, EP_CHAIN, s_flag[0])) break;
         }
 
-        // ---- M(i): margins over this CTA's columns, then the signal to the other CTAs ----
-        {
-            float4 uu[EP_MAX_COLS / 128];
-            if (early_u) {
-#pragma unroll
-                for (int it = 0; it < EP_MAX_COLS / 128; ++it) uu[it] = un[it];
-                if (i + 2u < ntiles) load_u((i + 2u) % a.K, un);
-            } else {
-                load_u(T.k, uu);
-            }
-            unsigned long long *const arow = a.acc + (uint64_t)(i % EP_RING) * a.batch * EP_ROW_WORDS;
-            if (cta == i % ncta) {   // this CTA clears the slot that tile i + RING/2 will add into
-                ulonglong2 *z = reinterpret_cast<ulonglong2 *>(
-                    a.acc + (uint64_t)((i + EP_RING / 2) % EP_RING) * a.batch * EP_ROW_WORDS);
-                for (uint32_t j = tg; j < 2u * a.batch; j += EP_GROUP) z[j] = make_ulonglong2(0ull, 0ull);
-                __threadfence();     // cleared for every CTA before this thread goes on
-            }
-            const bool signal = i != 0u || cta != a.drop_cta;
-            bool ok = true;
-            for (uint32_t s = wg; s < T.nsub; s += EP_GROUP / 32) {   // a warp per sub-tile
-                ok = __all_sync(0xFFFFFFFFu, mbar_wait(&bars[s], parity, &s_flag[0], a.wait_ns)) != 0;
-                if (!ok) break;
-                const float *__restrict__ xs = buf + (size_t)s * slot_floats;
-                float acc[SUB];
-#pragma unroll
-                for (int r = 0; r < SUB; ++r) acc[r] = 0.0f;
-#pragma unroll
-                for (int it = 0; it < EP_MAX_COLS / 128; ++it) {
-                    const uint32_t c = lane * 4u + it * 128u;
-                    if (c < a.cols) {
-                        const bool first = it < EP_BOX_COLS / 128;
-                        const float *__restrict__ base = first ? xs + c : xs + SUB * cols_a + (c - EP_BOX_COLS);
-                        const uint32_t pitch = first ? cols_a : cols_b;
-#pragma unroll
-                        for (int r = 0; r < SUB; ++r) {
-                            const float4 x = *reinterpret_cast<const float4 *>(base + r * pitch);
-                            acc[r] = fmaf(x.x, uu[it].x, acc[r]);
-                            acc[r] = fmaf(x.y, uu[it].y, acc[r]);
-                            acc[r] = fmaf(x.z, uu[it].z, acc[r]);
-                            acc[r] = fmaf(x.w, uu[it].w, acc[r]);
-                        }
-                    }
-                }
-                const float tot = reduce8(acc, lane);
-                const uint32_t jj = s * SUB + reduce8_row(lane);
-                if ((lane & 3u) == 0u && jj < T.m && signal) {
-                    unsigned long long *const r = arow + (uint64_t)jj * EP_ROW_WORDS;
-                    if (fabsf(tot) < FX_LIMIT) {
-                        atomicAdd(r, FX_ONE + FX_BIAS + (unsigned long long)__float2ll_rn(tot * FX_SCALE));
-                    } else {
-                        // rare: the wide word or the not-a-number count first, visible before the count
-                        if (fabsf(tot) < FX_WIDE_LIMIT)
-                            atomicAdd(r + 1, (unsigned long long)__float2ll_rn(tot * FX_WIDE_SCALE));
-                        else if (tot != tot)
-                            atomicAdd(r + 2, 1ull);                               // NaN
-                        else
-                            atomicAdd(r + 3, tot > 0.0f ? (1ull << 32) : 1ull);   // +-Inf, or beyond the wide word
-                        __threadfence();
-                        atomicAdd(r, FX_ONE + FX_BIAS);
-                    }
-                }
-            }
-            if (!ok) s_flag[0] = 1u;
-            if (sync_any(1u + g, EP_GROUP, s_flag[0])) break;
-        }
+        // the label of the row this thread will finish, requested before it is needed
+        const float yj = tg < T.m ? __ldg(a.y + (uint64_t)T.k * a.n_local + (uint64_t)T.t * a.batch + tg) : 0.0f;
 
-        // ---- stash: the tile moves from shared to tensor memory and its slots go back to the
-        // producer now, so that the copies of the group's next tile run during the exchange ----
-        if (stash) {
-            // every warp observes the arrival of every sub-tile itself (lane s looks at sub-tile s)
-            for (uint32_t s = lane; s < T.nsub; s += 32u) mbar_wait(&bars[s], parity, &s_flag[0], a.wait_ns);
-            __syncwarp();
-            for (uint32_t s = 0; s < T.nsub; ++s) {
-                const float *__restrict__ base = buf + (size_t)s * slot_floats + off;
+        // ---- M(i): margins over this CTA's columns, the values to tensor memory ----
+        unsigned long long *const acc_t = acc_g + (size_t)(i % EP_RING) * mpad;
+        unsigned long long *const wide_t = wide_g + (size_t)(i % EP_RING) * mpad * EP_WIDE_WORDS;
+        const bool signal = i != 0u || blockIdx.x != a.drop_cta;
+        uint32_t unit = 0u;      // 8 x 128 blocks stored so far
+        for (uint32_t s = wg; s < T.nsub; s += EP_WARPS) {
+            const uint32_t n = T.first + s, turn = n / a.nslots, slot = n - turn * a.nslots;
+            // a barrier's parity tells neighbouring turns apart and no more, so see this turn begin first
+            if (__all_sync(0xFFFFFFFFu, flag_above(&s_flag[6], n, &s_flag[0], a.wait_ns) &&
+                                            mbar_wait(&full[slot], turn & 1u, &s_flag[0], a.wait_ns)) == 0) {
+                s_flag[0] = 1u;
+                break;
+            }
+            const float *const xs = ring + (size_t)slot * slot_floats;
+            const uint32_t rows = T.m - s * SUB;     // rows of the minibatch in this sub-tile, if below 8
+            float acc[SUB];
+#pragma unroll
+            for (int r = 0; r < SUB; ++r) acc[r] = 0.0f;
+#pragma unroll 1
+            for (uint32_t it = 0; it < a.nit; ++it) {
+                const uint32_t b0 = (it >> 1) * EP_BOX_COLS, c = it * 128u + lane * 4u;
+                const uint32_t pitch = min(a.cols - b0, (uint32_t)EP_BOX_COLS);
+                const float *const base = xs + SUB * b0 + (c - b0);
+                const float4 uu = *reinterpret_cast<const float4 *>(us + c);
                 float4 x[SUB];
 #pragma unroll
                 for (uint32_t r = 0; r < (uint32_t)SUB; ++r)
-                    x[r] = colok ? *reinterpret_cast<const float4 *>(base + (size_t)r * pitch)
-                                 : make_float4(0.f, 0.f, 0.f, 0.f);
-                tmem_st32(taddr + 32u * s, x);
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&consumed[g * a.nsub_max + s]);
+                    x[r] = (c < a.cols && r < rows) ? *reinterpret_cast<const float4 *>(base + r * pitch)
+                                                    : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int r = 0; r < SUB; ++r) {
+                    acc[r] = fmaf(x[r].x, uu.x, acc[r]);
+                    acc[r] = fmaf(x[r].y, uu.y, acc[r]);
+                    acc[r] = fmaf(x[r].z, uu.z, acc[r]);
+                    acc[r] = fmaf(x[r].w, uu.w, acc[r]);
+                }
+                tmem_st32(taddr + 32u * unit, x);
+                ++unit;
             }
-            tmem_wait_st();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&empty[slot]);
+            const float tot = reduce8(acc, lane);
+            const uint32_t jj = s * SUB + reduce8_row(lane);
+            if ((lane & 3u) == 0u && jj < T.m && signal) {
+                unsigned long long *const r = acc_t + jj;
+                if (fabsf(tot) < FX_LIMIT) {
+                    atomicAdd(r, FX_ONE + FX_BIAS + (unsigned long long)__float2ll_rn(tot * FX_SCALE));
+                } else {
+                    // rare: the special bit and the row's other words first, visible before the count
+                    unsigned long long *const w = wide_t + (size_t)jj * EP_WIDE_WORDS;
+                    atomicOr(r, FX_SPECIAL);
+                    if (fabsf(tot) < FX_WIDE_LIMIT)
+                        atomicAdd(w, (unsigned long long)__float2ll_rn(tot * FX_WIDE_SCALE));
+                    else if (tot != tot)
+                        atomicAdd(w + 1, 1ull);                               // NaN
+                    else
+                        atomicAdd(w + 2, tot > 0.0f ? (1ull << 32) : 1ull);   // +-Inf, or beyond the wide word
+                    __threadfence();
+                    atomicAdd(r, FX_ONE + FX_BIAS);
+                }
+            }
         }
+        tmem_wait_st();
 
         // ---- W(i): all CTAs' partial margins -> step coefficients in shared memory ----
-        {
-            // the labels of the rows this lane will finish, requested before the wait
-            const float *__restrict__ yt = a.y + (uint64_t)T.k * a.y_stride + (uint64_t)T.t * a.batch;
-            const unsigned long long *const ain = a.acc + (uint64_t)(i % EP_RING) * a.batch * EP_ROW_WORDS;
-            if (tg == 0) {   // one thread waits for the row that every CTA adds to last
-                const unsigned long long *const last = ain + (uint64_t)(T.m - 1u) * EP_ROW_WORDS;
-                const uint64_t t0 = now_ns();
-                uint32_t n = 0u;
-                while ((ld_relaxed_v2(last).x >> 55) < ncta) {
-                    if ((++n & a.poll_mask) == 0u) {
-                        if (s_flag[0] != 0u || ld_acquire(a.header) != 0u || expired(t0, a.wait_ns)) {
-                            s_flag[0] = 1u;
-                            break;
-                        }
-                        __nanosleep(64);
-                    }
-                }
+        if (rank == i % a.P) {   // this CTA clears the slot that tile i + RING/2 will add into
+            const size_t z = (size_t)((i + EP_RING / 2) % EP_RING) * mpad;
+            for (uint32_t j = EP_CHAIN - 1u - tg; j < mpad; j += EP_CHAIN) {
+                acc_g[z + j] = 0ull;
+#pragma unroll
+                for (uint32_t w = 0; w < EP_WIDE_WORDS; ++w) wide_g[(z + j) * EP_WIDE_WORDS + w] = 0ull;
+                __threadfence();     // cleared for every CTA before this thread goes on
             }
-            if (sync_any(1u + g, EP_GROUP, s_flag[0])) break;
-            // a thread per row: the other rows are complete by now or within a few looks
-            for (uint32_t j = tg; j < T.m; j += EP_GROUP) {
-                const unsigned long long *const r = ain + (uint64_t)j * EP_ROW_WORDS;
-                const float yj = __ldg(yt + j);
-                ulonglong2 v = ld_relaxed_v2(r);
-                if ((v.x >> 55) < ncta) {
+        }
+        if (tg < SUB * T.nsub) {
+            float cj = 0.0f;
+            if (tg < T.m) {
+                const unsigned long long *const r = acc_t + tg;
+                unsigned long long v = ld_relaxed(r);
+                if ((v >> 55) < a.P) {
                     const uint64_t t0 = now_ns();
                     uint32_t n = 0u;
-                    while (((v = ld_relaxed_v2(r)).x >> 55) < ncta) {
+                    while (((v = ld_relaxed(r)) >> 55) < a.P) {
                         if ((++n & a.poll_mask) == 0u &&
-                            (s_flag[0] != 0u || ld_acquire(a.header) != 0u || expired(t0, a.wait_ns))) {
+                            (s_flag[0] != 0u || ld_acquire(header) != 0u || expired(t0, a.wait_ns))) {
                             s_flag[0] = 1u;
                             break;
                         }
                     }
                 }
-                const ulonglong2 special = ld_relaxed_v2(r + 2);   // NaN count | +Inf count << 32 + -Inf count
-                const long long fine = (long long)((v.x & (FX_ONE - 1ull)) - (unsigned long long)ncta * FX_BIAS);
-                float margin = (float)((double)fine * (1.0 / (double)FX_SCALE) +
-                                       (double)(long long)v.y * (1.0 / (double)FX_WIDE_SCALE));
-                if (special.y != 0ull) {
-                    const bool pos = (special.y >> 32) != 0ull, neg = (special.y & 0xFFFFFFFFull) != 0ull;
-                    margin = pos && neg ? __int_as_float(0x7FC00000)
-                                        : __int_as_float(pos ? 0x7F800000 : (int)0xFF800000);
-                }
-                if (special.x != 0ull) margin = __int_as_float(0x7FC00000);
-                // -(lr/m) * c_j with c_j = -y_j / (1 + exp(y_j m_j))
-                coef[j] = (a.lr / (float)T.m) * yj / (1.0f + expf(yj * margin));
-            }
-            if (sync_any(1u + g, EP_GROUP, s_flag[0])) break;
-        }
-
-        // ---- U(i): update this CTA's columns of u from the buffer, release the buffer ----
-        {
-            float4 *const up = reinterpret_cast<float4 *>(a.u + (uint64_t)T.k * a.u_stride + c0 + col);
-            float4 uold = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (colok) uold = *up;                       // requested now, needed after the loop
-            // Every warp observes the arrival of every sub-tile itself before it reads what TMA
-            // wrote: lane s looks at sub-tile s (a look costs about 0.1 us, so the lanes look in
-            // parallel), and the warp follows its lanes through __syncwarp.  All of them have
-            // landed: the warps that took the margins waited for them.
-            if (!stash)
-                for (uint32_t s = lane; s < T.nsub; s += 32u) mbar_wait(&bars[s], parity, &s_flag[0], a.wait_ns);
-            __syncwarp();
-            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (uint32_t s = 0; stash && s < T.nsub; ++s) {
-                float4 x[SUB];
-                tmem_ld32(taddr + 32u * s, x);
-                tmem_wait_ld();
-#pragma unroll
-                for (uint32_t r = 0; r < (uint32_t)SUB; ++r) {
-                    const uint32_t jj = s * SUB + r;
-                    if (colok && jj < T.m) {
-                        const float cj = coef[jj];
-                        acc.x = fmaf(cj, x[r].x, acc.x);
-                        acc.y = fmaf(cj, x[r].y, acc.y);
-                        acc.z = fmaf(cj, x[r].z, acc.z);
-                        acc.w = fmaf(cj, x[r].w, acc.w);
+                const long long fine = (long long)((v & (FX_SPECIAL - 1ull)) - (unsigned long long)a.P * FX_BIAS);
+                float margin = (float)((double)fine * (1.0 / (double)FX_SCALE));
+                if ((v & FX_SPECIAL) != 0ull) {
+                    const unsigned long long *const w = wide_t + (size_t)tg * EP_WIDE_WORDS;
+                    __threadfence();
+                    const unsigned long long w0 = ld_relaxed(w), w1 = ld_relaxed(w + 1), w2 = ld_relaxed(w + 2);
+                    margin = (float)((double)fine * (1.0 / (double)FX_SCALE) +
+                                     (double)(long long)w0 * (1.0 / (double)FX_WIDE_SCALE));
+                    if (w2 != 0ull) {   // +Inf count << 32 + -Inf count
+                        const bool pos = (w2 >> 32) != 0ull, neg = (w2 & 0xFFFFFFFFull) != 0ull;
+                        margin = pos && neg ? __int_as_float(0x7FC00000)
+                                            : __int_as_float(pos ? 0x7F800000 : (int)0xFF800000);
                     }
+                    if (w1 != 0ull) margin = __int_as_float(0x7FC00000);
                 }
+                // -(lr/m) * c_j with c_j = -y_j / (1 + exp(y_j m_j))
+                cj = (a.lr / (float)T.m) * yj / (1.0f + expf(yj * margin));
             }
-            for (uint32_t s = 0; !stash && s < T.nsub; ++s) {
-                if (colok) {
-                    const float *__restrict__ base = buf + (size_t)s * slot_floats + off;
+            coef[tg] = cj;
+        }
+        if (sync_any(1u + g, EP_CHAIN, s_flag[0])) break;
+
+        // ---- U(i): coef_j x_j summed over the warp's rows, then over the warps, onto u ----
+        if (wg < T.nsub) {
+            // one chain has the registers for two blocks at a time
+            for (uint32_t it = 0; it < a.nit; it += 3u - NC) {
+                const bool two = NC == 1 && it + 1u < a.nit;
+                float4 s0 = make_float4(0.f, 0.f, 0.f, 0.f), s1 = s0;
+                uint32_t q = it;
+                for (uint32_t s = wg; s < T.nsub; s += EP_WARPS, q += a.nit) {
+                    float4 x0[SUB], x1[SUB];
+                    tmem_ld32(taddr + 32u * q, x0);
+                    if (NC == 1 && two) tmem_ld32(taddr + 32u * (q + 1u), x1);
+                    const float4 ca = *reinterpret_cast<const float4 *>(coef + s * SUB);
+                    const float4 cb = *reinterpret_cast<const float4 *>(coef + s * SUB + 4u);
+                    const float cs[SUB] = {ca.x, ca.y, ca.z, ca.w, cb.x, cb.y, cb.z, cb.w};
+                    tmem_wait_ld();
 #pragma unroll
-                    for (uint32_t r = 0; r < (uint32_t)SUB; ++r) {
-                        const uint32_t jj = s * SUB + r;
-                        if (jj < T.m) {
-                            const float4 x = *reinterpret_cast<const float4 *>(base + (size_t)r * pitch);
-                            const float cj = coef[jj];
-                            acc.x = fmaf(cj, x.x, acc.x);
-                            acc.y = fmaf(cj, x.y, acc.y);
-                            acc.z = fmaf(cj, x.z, acc.z);
-                            acc.w = fmaf(cj, x.w, acc.w);
+                    for (int r = 0; r < SUB; ++r) {
+                        s0.x = fmaf(cs[r], x0[r].x, s0.x);
+                        s0.y = fmaf(cs[r], x0[r].y, s0.y);
+                        s0.z = fmaf(cs[r], x0[r].z, s0.z);
+                        s0.w = fmaf(cs[r], x0[r].w, s0.w);
+                    }
+                    if (NC == 1 && two) {
+#pragma unroll
+                        for (int r = 0; r < SUB; ++r) {
+                            s1.x = fmaf(cs[r], x1[r].x, s1.x);
+                            s1.y = fmaf(cs[r], x1[r].y, s1.y);
+                            s1.z = fmaf(cs[r], x1[r].z, s1.z);
+                            s1.w = fmaf(cs[r], x1[r].w, s1.w);
                         }
                     }
                 }
-                // the warp is through with this slot: one arrival per warp hands it back to the
-                // producer, which refills it while the update goes on
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&consumed[g * a.nsub_max + s]);
+                float *const pw = part + (size_t)wg * ucols + it * 128u + lane * 4u;
+                *reinterpret_cast<float4 *>(pw) = s0;
+                if (NC == 1 && two) *reinterpret_cast<float4 *>(pw + 128) = s1;
             }
-            if (colok) {
-                uold.x += acc.x;
-                uold.y += acc.y;
-                uold.z += acc.z;
-                uold.w += acc.w;
-                *up = uold;
+        }
+        chain_sync();
+        if (tg < ucols / 4u) {
+            const uint32_t c = tg * 4u;
+            float4 t = *reinterpret_cast<const float4 *>(part + c);
+            const uint32_t nw = min(T.nsub, (uint32_t)EP_WARPS);
+            for (uint32_t w = 1; w < nw; ++w) {
+                const float4 v = *reinterpret_cast<const float4 *>(part + (size_t)w * ucols + c);
+                t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
             }
-            group_sync();                                 // u stored by the whole group
-            if (tg == 0) {
-                __threadfence_block();
-                s_flag[4u + g] = (i >> 1) + 1u;           // this group's tiles completed
-            }
+            const float4 o = *reinterpret_cast<const float4 *>(us + c);
+            t.x += o.x; t.y += o.y; t.z += o.z; t.w += o.w;
+            *reinterpret_cast<float4 *>(us + c) = t;
+            if (T.t == a.nsteps - 1u && c < a.cols && (uint64_t)c0 + c < a.d)   // the worker's last minibatch
+                *reinterpret_cast<float4 *>(a.u + (uint64_t)T.k * a.u_stride + c0 + c) = t;
+        }
+        chain_sync();                                     // u complete for the next minibatch
+        if (NC == 2 && tg == 0) {
+            __threadfence_block();
+            s_flag[4u + g] = (i >> 1) + 1u;               // this chain's tiles completed
         }
     }
 
-    // Both groups meet here, whether they finished or gave up.
-    asm volatile("bar.sync 3, %0;" ::"n"(EP_CONSUMERS) : "memory");
-    if (stash && warp == 0) tmem_free_all(tmem_base);   // on every path out of the kernel
-    // A wait ran out: tell the host and the other CTAs.  The copies still in flight are the
+    // All chains meet here, whether they finished or gave up.
+    asm volatile("bar.sync 3, %0;" ::"n"(NC * EP_CHAIN) : "memory");
+    if (warp == 0) tmem_free_all(tmem_base);              // on every path out of the kernel
+    // A wait ran out: tell the host and the group's other CTAs.  The copies still in flight are the
     // producer warp's to wait for.
-    if (s_flag[0] != 0u && tid == 0) {
-        atomicOr(a.status, QESGD_STATUS_TIMEOUT);
-        atomicExch(a.header, 1u);
+    if (tid == 0) {
+        if (s_flag[0] != 0u) {
+            atomicOr(a.status, QESGD_STATUS_TIMEOUT);
+            atomicExch(header, 1u);
+        }
+        __threadfence();
+        s_flag[9] = atomicAdd(header + 1, 1u) == a.P - 1u ? 1u : 0u;
+    }
+    asm volatile("bar.sync 3, %0;" ::"n"(NC * EP_CHAIN) : "memory");
+    if (s_flag[9] != 0u) {   // last of the group to leave: nobody adds or reads any more
+        __threadfence();
+        for (uint32_t j = tid; j < EP_RING * mpad; j += NC * EP_CHAIN) {
+            acc_g[j] = 0ull;
+#pragma unroll
+            for (uint32_t w = 0; w < EP_WIDE_WORDS; ++w) wide_g[(size_t)j * EP_WIDE_WORDS + w] = 0ull;
+        }
+        if (tid < 2u) header[tid] = 0u;
     }
 }
 
@@ -657,7 +639,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
                                   CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
                                   CUtensorMapFloatOOBfill);
 
-// Per-device set-up: shared-memory limit of the kernel, the driver's tensor-map encoder.
+// Per-device set-up: shared-memory limit of the kernels, the driver's tensor-map encoder.
 constexpr int MAX_DEVICES = 64;
 std::mutex g_epoch_mutex;
 int g_epoch_smem_limit[MAX_DEVICES] = {0};   // 0 = not queried, -1 = unsupported
@@ -673,8 +655,9 @@ int epoch_smem_limit(int device)
         if (e == cudaSuccess)
             e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
         if (e == cudaSuccess && coop && optin > 0)
-            e = cudaFuncSetAttribute(qesgd_lr_epoch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     optin);
+            e = cudaFuncSetAttribute(qesgd_lr_epoch_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+        if (e == cudaSuccess && coop && optin > 0)
+            e = cudaFuncSetAttribute(qesgd_lr_epoch_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
         if (e == cudaSuccess && !g_encode_tiled) {
             void *fn = nullptr;
             cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
@@ -702,15 +685,70 @@ bool make_map(CUtensorMap *map, const float *X, uint64_t rows, uint64_t d, uint3
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// One way to deal the epoch out: G groups of P CTAs, NC chains per CTA.
+struct Split {
+    uint32_t G, P, NC, cols, nit, nslots;
+    uint32_t off_u, off_part, off_coef, off_bars, off_flags, bytes;
+    float us;            // modelled time of a step of all workers
+};
+
+// Fills in the rest of a split with G groups and P CTAs each; false where it does not fit.
+bool complete_split(Split &s, uint64_t d, uint32_t K, uint32_t m, uint32_t nsub, uint32_t limit)
+{
+    const uint64_t cols = ((d + s.P - 1) / s.P + 3) / 4 * 4;
+    if (cols > 1024) return false;
+    s.cols = (uint32_t)cols;
+    s.P = (uint32_t)((d + cols - 1) / cols);
+    s.nit = (s.cols + 127u) / 128u;
+    const uint32_t kg = (K + s.G - 1u) / s.G;
+    const uint32_t units = (nsub + EP_WARPS - 1u) / EP_WARPS * s.nit;    // tensor-memory blocks per warp
+    if (units > (uint32_t)EP_UNITS) return false;
+    s.NC = kg >= 2u && units <= (uint32_t)EP_UNITS / 2u ? 2u : 1u;
+    const uint32_t slot = SUB * s.cols * 4u, ubytes = s.nit * 512u;
+    const uint32_t fixed = kg * ubytes + s.NC * EP_WARPS * ubytes + s.NC * EP_MAX_M * 4u + 2u * EP_MAX_SLOTS * 8u + 64u;
+    if (fixed + 2u * slot > limit) return false;
+    s.nslots = (limit - fixed) / slot;
+    if (s.nslots > (uint32_t)EP_MAX_SLOTS) s.nslots = EP_MAX_SLOTS;
+    s.off_u = s.nslots * slot;                   // slots are multiples of 128 bytes
+    s.off_part = s.off_u + kg * ubytes;
+    s.off_coef = s.off_part + s.NC * EP_WARPS * ubytes;
+    s.off_bars = s.off_coef + s.NC * EP_MAX_M * 4u;
+    s.off_flags = s.off_bars + 2u * EP_MAX_SLOTS * 8u;
+    s.bytes = s.off_flags + 64u;
+    const float hbm = (float)((double)K * m * d * 4.0 / 6.5e6);          // us at 6.5 TB/s
+    const float chain = EP_CHAIN_US + EP_UNIT_US * (float)units;
+    const float chained = chain * (float)kg / (float)s.NC;
+    s.us = hbm > chained ? hbm : chained;
+    return true;
+}
+
+// The modelled time picks the split; ties go to fewer groups.
+bool choose_split(Split &best, uint64_t d, uint32_t K, uint32_t m, uint32_t nsub, uint32_t sm_count, uint32_t limit)
+{
+    bool any = false;
+    for (uint32_t G = 1; G <= K && G <= sm_count; ++G) {
+        if (G * nsub * SUB > QESGD_LR_EPOCH_ROWS) break;     // accumulators of all groups
+        if (G > 1u && (K + G - 1u) / G == (K + G - 2u) / (G - 1u)) continue;   // no fewer workers per group than before
+        Split s;
+        s.G = G;
+        s.P = sm_count / G;
+        const uint64_t most = (d + 127u) / 128u;              // a warp takes 128 columns at a time
+        if (s.P > most) s.P = (uint32_t)most;
+        if (!complete_split(s, d, K, m, nsub, limit)) continue;
+        if (!any || s.us < 0.99f * best.us) best = s;
+        any = true;
+    }
+    return any;
+}
+
 }  // namespace
 
 // Returns 0 = launched, -1 = shape not covered by the fused kernel (caller uses the
 // two-pass steps), > 0 = cudaError_t.
 int qesgd_launch_lr_epoch_fused(const float *X, const float *y, uint64_t n_local, uint64_t d,
                                 uint32_t K, uint32_t batch, float lr, float *u, uint64_t u_stride,
-                                float *work, uint64_t work_floats, uint32_t *status, int device,
-                                int sm_count, uint64_t wait_ns, uint32_t drop_cta, cudaStream_t stream,
-                                int *launched)
+                                float *work, uint32_t *status, int device, int sm_count, uint64_t wait_ns,
+                                uint32_t drop_cta, cudaStream_t stream, int *launched)
 {
     *launched = 0;
     const uint32_t m_full = (uint32_t)(n_local < batch ? n_local : batch);
@@ -719,51 +757,44 @@ int qesgd_launch_lr_epoch_fused(const float *X, const float *y, uint64_t n_local
     if (nsteps64 * K > (1u << 20)) return -1;
     if ((uint64_t)K * n_local + EP_MAX_M >= (1ull << 31)) return -1;   // TMA row coordinates
     if (d % 4 != 0 || u_stride % 4 != 0 || ((uintptr_t)X | (uintptr_t)u) % 16 != 0) return -1;
-    if (sm_count < 1) return -1;
-    uint64_t cols = (d + (uint64_t)sm_count - 1) / (uint64_t)sm_count;
-    cols = (cols + 3) / 4 * 4;
-    if (cols > (uint64_t)EP_MAX_COLS) return -1;
-    const uint32_t ncta = (uint32_t)((d + cols - 1) / cols);
-    if (ncta > 256u) return -1;   // the accumulator word counts up to 511 contributions
+    if (sm_count < 1 || d > 1024ull * (uint64_t)sm_count) return -1;
     const int limit = epoch_smem_limit(device);
     if (limit <= 0) return -1;
+    const uint32_t nsub = (m_full + SUB - 1) / SUB;
+    Split s;
+    // the accumulator word counts up to 256 contributions
+    if (!choose_split(s, d, K, m_full, nsub, (uint32_t)(sm_count < 256 ? sm_count : 256), (uint32_t)limit)) return -1;
 
     EpochArgs a;
-    a.y = y; a.y_stride = n_local; a.n_local = n_local;
-    a.d = d; a.K = K; a.batch = m_full; a.nsteps = (uint32_t)nsteps64;
+    a.y = y; a.n_local = n_local;
+    a.d = d; a.K = K; a.G = s.G; a.P = s.P;
+    a.batch = m_full; a.nsteps = (uint32_t)nsteps64;
     a.m_last = (uint32_t)(n_local - (nsteps64 - 1) * m_full);
-    a.nsub_max = (m_full + SUB - 1) / SUB;
+    a.nsub_max = nsub;
     a.nsub_last = (a.m_last + SUB - 1) / SUB;
-    a.cols = (uint32_t)cols;
+    a.cols = s.cols; a.nit = s.nit; a.nslots = s.nslots;
+    a.off_u = s.off_u; a.off_part = s.off_part; a.off_coef = s.off_coef; a.off_bars = s.off_bars; a.off_flags = s.off_flags;
     a.lr = lr;
     a.u = u; a.u_stride = u_stride;
     a.status = status;
     a.wait_ns = wait_ns;
     a.poll_mask = wait_ns < COARSE_TIMER_NS ? 0u : 31u;
     a.drop_cta = drop_cta;
-
-    // shared memory: two tile buffers | coefficients of both groups | barriers | flags
-    const size_t smem = (size_t)2 * a.nsub_max * SUB * cols * sizeof(float) + 2 * EP_MAX_M * sizeof(float) +
-                        (4 * EP_MAX_NSUB) * sizeof(uint64_t) + 64;
-    if (smem > (size_t)limit) return -1;
-
-    // workspace: header | margin accumulators (the workspace is 256-byte aligned)
-    const uint64_t words = EP_HEADER_WORDS + (uint64_t)EP_RING * m_full * EP_ROW_WORDS * 2u;
-    if (words > work_floats) return -1;
+    // workspace, all zero between launches: headers | accumulators | their rarely used words
     a.header = reinterpret_cast<uint32_t *>(work);
-    a.acc = reinterpret_cast<unsigned long long *>(work + EP_HEADER_WORDS);
+    a.acc = reinterpret_cast<unsigned long long *>(work + QESGD_MAX_WORKERS * EP_HEADER_WORDS);
+    a.wide = a.acc + (size_t)EP_RING * QESGD_LR_EPOCH_ROWS;
 
-    CUtensorMap map_a, map_b;
-    const uint32_t cols_a = cols < (uint64_t)EP_BOX_COLS ? (uint32_t)cols : (uint32_t)EP_BOX_COLS;
-    const uint32_t cols_b = (uint32_t)cols - cols_a;
-    if (!make_map(&map_a, X, (uint64_t)K * n_local, d, cols_a)) return -1;
-    if (!make_map(&map_b, X, (uint64_t)K * n_local, d, cols_b ? cols_b : cols_a)) return -1;
+    CUtensorMap map_full, map_rest;
+    const uint32_t wide_box = s.cols < (uint32_t)EP_BOX_COLS ? s.cols : (uint32_t)EP_BOX_COLS;
+    const uint32_t rest = s.cols % EP_BOX_COLS;
+    if (!make_map(&map_full, X, (uint64_t)K * n_local, d, wide_box)) return -1;
+    if (!make_map(&map_rest, X, (uint64_t)K * n_local, d, rest ? rest : wide_box)) return -1;
 
-    cudaError_t e = cudaMemsetAsync(work, 0, words * sizeof(float), stream);
-    if (e != cudaSuccess) return (int)e;
-    void *params[] = {(void *)&a, (void *)&map_a, (void *)&map_b};
-    e = cudaLaunchCooperativeKernel((const void *)qesgd_lr_epoch_kernel, dim3(ncta), dim3(EP_THREADS), params,
-                                    smem, stream);
+    void *params[] = {(void *)&a, (void *)&map_full, (void *)&map_rest};
+    const void *kernel = s.NC == 2u ? (const void *)qesgd_lr_epoch_kernel<2> : (const void *)qesgd_lr_epoch_kernel<1>;
+    const cudaError_t e = cudaLaunchCooperativeKernel(kernel, dim3(s.G * s.P), dim3(s.NC * EP_CHAIN + 32), params,
+                                                      s.bytes, stream);
     if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources ||
         e == cudaErrorInvalidConfiguration || e == cudaErrorNotSupported) {
         cudaGetLastError();   // the device cannot hold all CTAs at once as configured: two-pass steps

@@ -360,6 +360,41 @@ def test_lr_local_epoch_shapes_match_oracle(K, n_local, d, batch):
     assert torch.equal(tu, tu2)
 
 
+@pytest.mark.parametrize("K,n_local,d,batch", [
+    (1, 1, 20, 1),           # one row, one slice of 20 columns
+    (1, 20, 4, 8),           # one column group, ragged last minibatch
+    (7, 90, 50000, 32),      # uneven groups: some hold one worker more than others
+    (64, 20, 2000, 16),      # the largest worker count
+    (3, 100, 1000, 33),      # a last sub-tile of one row
+    (1, 300, 140000, 64),    # 948 columns per CTA: fewer slots in the ring than sub-tiles in a minibatch
+    (4, 130, 131072, 64),    # wide slices, one chain, last minibatch of two rows
+    (4, 200, 65536, 64),     # two chains, last minibatch of eight rows
+    (3, 130, 65536, 64),     # two chains over an odd number of workers
+    (2, 150, 30000, 100),    # more rows than the warps of a chain take in one go
+    (1, 2000, 784, 16),      # many short steps of one group: the accumulator ring goes round 15 times
+    (2, 40, 160000, 16),     # above 1024 columns per SM: two-pass steps
+])
+def test_lr_local_epoch_splits_match_oracle(K, n_local, d, batch):
+    """The ways the persistent kernel deals an epoch out (groups of CTAs, one or two chains, slices
+    of up to 1024 columns, rings shorter than a minibatch) at the edges of their ranges, twice: the
+    second call finds the workspace as the first one left it.  Bound: fp32 dot products of d terms
+    against fp64, as for the other logistic steps (1e-5)."""
+    X, y, _ = synthetic.logistic_problem(K * n_local, d, seed=K + n_local + d)
+    u0 = (0.1 * synthetic.normal_f32(d, 1.0, 22)).astype(np.float32)
+    c, tX, ty = G.ctx(), G.dev(X), G.dev(y)
+    runs = []
+    for _ in range(2):
+        tu = G.dev(u0).repeat(K, 1)
+        c.qesgd_lr_local_epoch_batch(tX, ty, n_local, d, K, batch, 0.5, tu, d)
+        assert c.qesgd_status() == 0
+        runs.append(tu)
+    assert torch.equal(runs[0], runs[1])
+    got = runs[0].cpu().numpy()
+    for k in sorted({0, K // 2, K - 1}):
+        rows = slice(k * n_local, (k + 1) * n_local)
+        _lr_close(got[k], ref.lr_local_epoch(X[rows], y[rows], batch, 0.5, u0))
+
+
 @pytest.mark.parametrize("gain", [2e7, 1e9])
 def test_local_epoch_partial_margins_beyond_the_fine_fixed_point_range(gain):
     """The CTAs of the persistent kernel add their partial margins as fixed-point integers: units
