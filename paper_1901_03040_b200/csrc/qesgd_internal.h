@@ -33,9 +33,10 @@ static const uint64_t QESGD_MAX_WAIT_NS = 10000000000ull;
 
 // Workspace (4 MiB): partial margins of the two-pass steps, K * P * m floats, and behind them what the
 // persistent kernel's CTAs exchange: a header of 16 words per group of CTAs, then for each of 8 ring
-// slots the accumulators (four 64-bit words) of up to QESGD_LR_EPOCH_ROWS rows of all groups.
+// slots the accumulators (four 64-bit words and three of space per row) of up to
+// QESGD_LR_EPOCH_ROWS rows of all groups.
 static const uint32_t QESGD_LR_EPOCH_ROWS = 2048;
-static const uint64_t QESGD_LR_EPOCH_FLOATS = QESGD_MAX_WORKERS * 16ull + 8ull * QESGD_LR_EPOCH_ROWS * 8ull;
+static const uint64_t QESGD_LR_EPOCH_FLOATS = QESGD_MAX_WORKERS * 16ull + 8ull * QESGD_LR_EPOCH_ROWS * 14ull;
 static const uint64_t QESGD_LR_WORK_FLOATS = (1ull << 20) - QESGD_LR_EPOCH_FLOATS;
 
 struct EncodeArgs {

@@ -44,8 +44,12 @@
 // infinity (NaN if both signs occur), which the step coefficient saturates on as it would on the
 // number itself.  These rare kinds set the special bit, and fence before they count themselves in
 // the first word, so a reader looks at the other words only where the bit is set: one round trip
-// to L2 in place of two.  Every thread that owns a row polls that row's word itself, eight rows
-// to 64 bytes, so a warp's poll and a warp's reduction touch two sectors per sub-tile.
+// to L2 in place of two.  Every thread that owns a row polls that row's word itself; the eight
+// rows of a sub-tile lie in 64 bytes, so a warp's reduction touches two sectors, and the sub-tiles
+// 256 bytes apart: they then fall into different parts of L2, whose atomic units and read ports
+// 148 CTAs otherwise queue at (an exchange of 64 rows, nothing else running: all rows in 512 bytes
+// 3590 clocks at 148 CTAs and 2250 at 74; 256 bytes apart 2375 and 1570; every row 256 bytes from
+// the next 2470 and 1970; one reader per row that hands the margin on 3640 and 3020).
 // The slot that tile i + RING/2 will use is cleared by one CTA after M(i), while it waits: every
 // CTA has read it by then (it has taken part in tile i-2, hence finished tile i-4) and none adds
 // to it before it has seen that CTA's contributions to tile i+2.  The CTA of a group that leaves
@@ -80,6 +84,7 @@ constexpr float EP_CHAIN_US = 2.5f, EP_UNIT_US = 0.25f;   // a tile's latency: e
 constexpr uint64_t DRAIN_LIMIT_NS = 2000000000ull;   // the producer's last wait for its own copies
 constexpr uint64_t COARSE_TIMER_NS = 1024ull;        // limits below this mean "one look, then give up"
 constexpr uint32_t EP_HEADER_WORDS = 16;             // per group: [0] abort flag, [1] CTAs that have left
+constexpr uint32_t EP_ACC_PITCH = 32;                // 64-bit words from one 8-row group of accumulators to the next
 constexpr uint32_t EP_WIDE_WORDS = 3;                // rarely used 64-bit words per accumulator row
 constexpr float FX_SCALE = 268435456.0f;             // 2^28: unit of the first word
 constexpr float FX_LIMIT = 131072.0f;                // 2^17: partials below go to the first word
@@ -104,7 +109,7 @@ struct EpochArgs {
     float *u;
     uint64_t u_stride;
     uint32_t *header;       // [G][EP_HEADER_WORDS]
-    unsigned long long *acc;    // [G][EP_RING][8 * nsub_max] margin accumulators, zero between launches
+    unsigned long long *acc;    // [G][EP_RING][nsub_max][EP_ACC_PITCH] margin accumulators, zero between launches
     unsigned long long *wide;   // [G][EP_RING][8 * nsub_max][EP_WIDE_WORDS]
     uint32_t *status;
     uint64_t wait_ns;       // limit of every wait on another CTA, chain or copy
@@ -297,6 +302,9 @@ __device__ __forceinline__ uint32_t reduce8_row(uint32_t lane)
     return ((lane >> 4) & 1u) * 4u + ((lane >> 3) & 1u) * 2u + ((lane >> 2) & 1u);
 }
 
+// Where row j's accumulator lies within its ring slot: eight rows in a row, the eights 256 bytes apart.
+__device__ __forceinline__ uint32_t acc_index(uint32_t j) { return (j / SUB) * EP_ACC_PITCH + j % SUB; }
+
 struct Tile {
     uint32_t t, kk, k, m, nsub, first;   // step, worker within the group, worker, rows, sub-tiles, number of the first
 };
@@ -405,7 +413,7 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + 32, 1)
     const uint32_t taddr = tmem_base + ((32u * (wg & 3u)) << 16) +
                            (NC == 2 ? 256u * g + 128u * (wg >> 2) : 256u * (wg >> 2));
     const uint32_t mpad = SUB * a.nsub_max;
-    unsigned long long *const acc_g = a.acc + (size_t)grp * EP_RING * mpad;
+    unsigned long long *const acc_g = a.acc + (size_t)grp * EP_RING * a.nsub_max * EP_ACC_PITCH;
     unsigned long long *const wide_g = a.wide + (size_t)grp * EP_RING * mpad * EP_WIDE_WORDS;
     uint32_t *const header = a.header + grp * EP_HEADER_WORDS;
 
@@ -438,7 +446,7 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + 32, 1)
         const float yj = tg < T.m ? __ldg(a.y + (uint64_t)T.k * a.n_local + (uint64_t)T.t * a.batch + tg) : 0.0f;
 
         // ---- M(i): margins over this CTA's columns, the values to tensor memory ----
-        unsigned long long *const acc_t = acc_g + (size_t)(i % EP_RING) * mpad;
+        unsigned long long *const acc_t = acc_g + (size_t)(i % EP_RING) * a.nsub_max * EP_ACC_PITCH;
         unsigned long long *const wide_t = wide_g + (size_t)(i % EP_RING) * mpad * EP_WIDE_WORDS;
         const bool signal = i != 0u || blockIdx.x != a.drop_cta;
         uint32_t unit = 0u;      // 8 x 128 blocks stored so far
@@ -481,7 +489,7 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + 32, 1)
             const float tot = reduce8(acc, lane);
             const uint32_t jj = s * SUB + reduce8_row(lane);
             if ((lane & 3u) == 0u && jj < T.m && signal) {
-                unsigned long long *const r = acc_t + jj;
+                unsigned long long *const r = acc_t + acc_index(jj);
                 if (fabsf(tot) < FX_LIMIT) {
                     atomicAdd(r, FX_ONE + FX_BIAS + (unsigned long long)__float2ll_rn(tot * FX_SCALE));
                 } else {
@@ -503,18 +511,20 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + 32, 1)
 
         // ---- W(i): all CTAs' partial margins -> step coefficients in shared memory ----
         if (rank == i % a.P) {   // this CTA clears the slot that tile i + RING/2 will add into
-            const size_t z = (size_t)((i + EP_RING / 2) % EP_RING) * mpad;
+            const uint32_t zs = (i + EP_RING / 2) % EP_RING;
+            unsigned long long *const az = acc_g + (size_t)zs * a.nsub_max * EP_ACC_PITCH;
+            unsigned long long *const wz = wide_g + (size_t)zs * mpad * EP_WIDE_WORDS;
             for (uint32_t j = EP_CHAIN - 1u - tg; j < mpad; j += EP_CHAIN) {
-                acc_g[z + j] = 0ull;
+                az[acc_index(j)] = 0ull;
 #pragma unroll
-                for (uint32_t w = 0; w < EP_WIDE_WORDS; ++w) wide_g[(z + j) * EP_WIDE_WORDS + w] = 0ull;
+                for (uint32_t w = 0; w < EP_WIDE_WORDS; ++w) wz[(size_t)j * EP_WIDE_WORDS + w] = 0ull;
                 __threadfence();     // cleared for every CTA before this thread goes on
             }
         }
         if (tg < SUB * T.nsub) {
             float cj = 0.0f;
             if (tg < T.m) {
-                const unsigned long long *const r = acc_t + tg;
+                const unsigned long long *const r = acc_t + acc_index(tg);
                 unsigned long long v = ld_relaxed(r);
                 if ((v >> 55) < a.P) {
                     const uint64_t t0 = now_ns();
@@ -625,7 +635,7 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + 32, 1)
     if (s_flag[9] != 0u) {   // last of the group to leave: nobody adds or reads any more
         __threadfence();
         for (uint32_t j = tid; j < EP_RING * mpad; j += NC * EP_CHAIN) {
-            acc_g[j] = 0ull;
+            acc_g[acc_index(j)] = 0ull;   // slots follow one another at the same pitch
 #pragma unroll
             for (uint32_t w = 0; w < EP_WIDE_WORDS; ++w) wide_g[(size_t)j * EP_WIDE_WORDS + w] = 0ull;
         }
@@ -783,7 +793,7 @@ int qesgd_launch_lr_epoch_fused(const float *X, const float *y, uint64_t n_local
     // workspace, all zero between launches: headers | accumulators | their rarely used words
     a.header = reinterpret_cast<uint32_t *>(work);
     a.acc = reinterpret_cast<unsigned long long *>(work + QESGD_MAX_WORKERS * EP_HEADER_WORDS);
-    a.wide = a.acc + (size_t)EP_RING * QESGD_LR_EPOCH_ROWS;
+    a.wide = a.acc + (size_t)EP_RING * (QESGD_LR_EPOCH_ROWS / SUB) * EP_ACC_PITCH;
 
     CUtensorMap map_full, map_rest;
     const uint32_t wide_box = s.cols < (uint32_t)EP_BOX_COLS ? s.cols : (uint32_t)EP_BOX_COLS;
