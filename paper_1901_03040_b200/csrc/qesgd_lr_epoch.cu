@@ -8,9 +8,15 @@
 // of `cols` columns for the whole epoch.  The slice of a minibatch (a "tile") passes through the
 // SM once, so X is read from HBM exactly once:
 //
-//   producer warp   fetches sub-tiles (8 rows of the slice) by TMA (2-D boxes of at most 256
+//   producer warps  fetch sub-tiles (8 rows of the slice) by TMA (2-D boxes of at most 256
 //                   columns, cp.async.bulk.tensor global -> shared, completion on an mbarrier
-//                   per slot) into a ring of slots, as far ahead as the ring reaches
+//                   per slot) into a ring of slots, as far ahead as the ring reaches.  Several
+//                   warps, one thread of each, take the slots in turn: looking at the slot, arming
+//                   its barrier and issuing two to four boxes takes a thread about 650 clocks, which
+//                   with one producer bounded the whole kernel at 27 bytes per clock and SM.  Two are best:
+//                   K = 4, n = 2048, d = 65536: 409 us with one, 350, 348 and 349 with two, three and
+//                   four; K = 8, n = 1010, d = 10000: 121, 83, 89, 90; K = 4, n = 512, d = 131072:
+//                   270, 268, 279, 295 (more requests at once delay the exchange between the CTAs)
 //   consumer chain  eight warps; tile i = minibatch i / Kg of the group's worker i % Kg:
 //     M(i)  warp w takes the sub-tiles w, w + 8, ...: partial margins of the rows over the slice;
 //           the values it reads go to tensor memory on the way (tcgen05.st), so the slot returns
@@ -59,7 +65,7 @@
 // resident by construction: at most one per SM).  Every wait the kernel itself loops on is
 // bounded by the context's wait limit: a wait that runs out sets QESGD_STATUS_TIMEOUT and an
 // abort word that the group's other CTAs poll, and the CTA's consumer warps leave.  The producer
-// warp is the last to go on every path: it waits (on a bound of its own) for each copy it has
+// warps are the last to go on every path: they wait (on a bound of its own) for each copy they have
 // requested and nobody has consumed, so no CTA ends with a copy still writing its shared
 // memory.  The one wait without a bound is the tensor-memory allocation at the start, which
 // blocks while another kernel resident on the same SM holds tensor memory (until that kernel
@@ -79,9 +85,11 @@ constexpr int EP_RING = 8;           // accumulator slots; a slot is cleared RIN
 constexpr int EP_BOX_COLS = 256;     // widest TMA box
 constexpr int EP_MAX_M = EP_CHAIN;   // rows per minibatch: a thread of the chain per row
 constexpr int EP_MAX_SLOTS = 64;     // ring slots
+constexpr uint32_t EP_FLAG_BYTES = (16 + EP_MAX_SLOTS) * 4;
+constexpr int EP_PRODUCERS = 2;      // producer warps
 constexpr int EP_UNITS = 8;          // 8 x 128 blocks of a tile that the tensor memory holds per warp
 constexpr float EP_CHAIN_US = 2.5f, EP_UNIT_US = 0.25f;   // a tile's latency: exchange, and per block of a warp
-constexpr uint64_t DRAIN_LIMIT_NS = 2000000000ull;   // the producer's last wait for its own copies
+constexpr uint64_t DRAIN_LIMIT_NS = 2000000000ull;   // the producers' last wait for their own copies
 constexpr uint64_t COARSE_TIMER_NS = 1024ull;        // limits below this mean "one look, then give up"
 constexpr uint32_t EP_HEADER_WORDS = 16;             // per group: [0] abort flag, [1] CTAs that have left
 constexpr uint32_t EP_ACC_PITCH = 32;                // 64-bit words from one 8-row group of accumulators to the next
@@ -328,7 +336,7 @@ extern __shared__ __align__(1024) unsigned char ep_smem[];
 // after the other, the last one narrower), the slices of u of the group's workers, the warps'
 // partial updates, the step coefficients, the barriers, a few flag words.
 template <int NC>
-__global__ void __launch_bounds__(NC * EP_CHAIN + 32, 1)
+__global__ void __launch_bounds__(NC * EP_CHAIN + EP_PRODUCERS * 32, 1)
     qesgd_lr_epoch_kernel(const EpochArgs a, const __grid_constant__ CUtensorMap map_full,
                           const __grid_constant__ CUtensorMap map_rest)
 {
@@ -340,9 +348,9 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + 32, 1)
     uint64_t *const full = reinterpret_cast<uint64_t *>(ep_smem + a.off_bars);
     uint64_t *const empty = full + a.nslots;
     // [0] a wait ran out in this CTA, [3] always zero, [4], [5] tiles completed by chain 0, 1,
-    // [6] sub-tiles requested by the producer, [8] base address of the tensor memory, [9] last CTA
-    // of the group to leave
+    // [8] base address of the tensor memory, [9] last CTA of the group to leave
     volatile uint32_t *const s_flag = reinterpret_cast<volatile uint32_t *>(ep_smem + a.off_flags);
+    volatile uint32_t *const s_turn = s_flag + 16;         // copies requested into each slot so far
 
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const uint32_t grp = blockIdx.x / a.P, rank = blockIdx.x - grp * a.P;
@@ -350,11 +358,11 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + 32, 1)
     const uint32_t c0 = rank * a.cols;
     const uint32_t ntiles = a.nsteps * kg;
 
-    if (tid == 0) {
-        for (uint32_t s = 0; s < 2u * a.nslots; ++s) mbar_init(&full[s], 1u);
-        for (int f = 0; f < 16; ++f) s_flag[f] = 0u;
+    if (tid < 2u * a.nslots) {
+        mbar_init(&full[tid], 1u);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (tid < 16u + EP_MAX_SLOTS) s_flag[tid] = 0u;
     __syncthreads();
     if (warp == 0) tmem_alloc_all(const_cast<uint32_t *>(&s_flag[8]));
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -362,45 +370,52 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + 32, 1)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = s_flag[8];
 
-    // ------------------------------------------------------------ producer ----
-    if (warp == NC * EP_WARPS) {
-        // the sub-tiles in the order in which the chains take them, round the ring
-        uint32_t slot = 0u, turn = 0u, issued = 0u;
-        bool ok = true;
-        for (uint32_t i = 0; i < ntiles && ok; ++i) {
-            const Tile T = tile_of(a, grp, kg, i);
-            const uint32_t row0 = (uint32_t)((uint64_t)T.k * a.n_local + (uint64_t)T.t * a.batch);
-            for (uint32_t s = 0; s < T.nsub; ++s) {
-                if (turn != 0u)   // the slot's previous sub-tile has been taken
-                    ok = __all_sync(0xFFFFFFFFu,
-                                    mbar_wait(&empty[slot], (turn - 1u) & 1u, &s_flag[0], a.wait_ns)) != 0;
-                if (!ok) break;
-                if (lane == 0) {
-                    float *dst = ring + (size_t)slot * slot_floats;
-                    mbar_arrive_expect_tx(&full[slot], slot_floats * 4u);
-                    uint32_t c = 0u;
-                    for (; c + EP_BOX_COLS <= a.cols; c += EP_BOX_COLS, dst += SUB * EP_BOX_COLS)
-                        tma_load_box(dst, &map_full, c0 + c, row0 + s * SUB, &full[slot]);
-                    if (c < a.cols) tma_load_box(dst, &map_rest, c0 + c, row0 + s * SUB, &full[slot]);
-                    s_flag[6] = issued + 1u;
+    // ----------------------------------------------------------- producers ----
+    if (warp >= NC * EP_WARPS) {
+        // The sub-tiles go round the ring in the order in which the chains take them.  Warp p serves
+        // the slots p, p + EP_PRODUCERS, ... and each of them turn by turn: a slot that several warps
+        // refilled could be looked at two turns early, where a barrier's parity reads the same.
+        const uint32_t p = warp - NC * EP_WARPS;
+        if (lane == 0 && p < a.nslots) {
+            uint32_t i = 0u, s = p, slot = p, turn = 0u;
+            Tile T = tile_of(a, grp, kg, 0u);
+            for (;;) {
+                while (s >= T.nsub && i < ntiles) {
+                    s -= T.nsub;
+                    if (++i < ntiles) T = tile_of(a, grp, kg, i);
                 }
-                ++issued;
-                if (++slot == a.nslots) { slot = 0u; ++turn; }
+                if (i >= ntiles) break;
+                // the slot's previous sub-tile has been taken
+                if (turn != 0u && !mbar_wait(&empty[slot], (turn - 1u) & 1u, &s_flag[0], a.wait_ns)) {
+                    s_flag[0] = 1u;
+                    atomicOr(a.status, QESGD_STATUS_TIMEOUT);
+                    break;
+                }
+                const uint32_t row = (uint32_t)((uint64_t)T.k * a.n_local + (uint64_t)T.t * a.batch) + s * SUB;
+                float *dst = ring + (size_t)slot * slot_floats;
+                mbar_arrive_expect_tx(&full[slot], slot_floats * 4u);
+                uint32_t c = 0u;
+                for (; c + EP_BOX_COLS <= a.cols; c += EP_BOX_COLS, dst += SUB * EP_BOX_COLS)
+                    tma_load_box(dst, &map_full, c0 + c, row, &full[slot]);
+                if (c < a.cols) tma_load_box(dst, &map_rest, c0 + c, row, &full[slot]);
+                s_turn[slot] = turn + 1u;
+                if (slot + EP_PRODUCERS < a.nslots) {
+                    slot += EP_PRODUCERS;
+                    s += EP_PRODUCERS;
+                } else {
+                    s += a.nslots - slot + p;
+                    slot = p;
+                    ++turn;
+                }
             }
         }
-        if (!ok && lane == 0) {
-            s_flag[0] = 1u;
-            atomicOr(a.status, QESGD_STATUS_TIMEOUT);
-        }
+        __syncwarp();
         // Last out, on every path: each slot's latest copy has been consumed (then it has
         // landed) or is waited for here, so that the CTA does not end -- and its shared memory
         // is not handed to another CTA -- while a copy is still writing it.  After a normal
         // epoch these waits end with the consumers' last tiles.
-        __syncwarp();
-        for (uint32_t q = lane; q < a.nslots && q < issued; q += 32u) {
-            const uint32_t turns = (issued - 1u - q) / a.nslots;    // the slot's latest copy is its turn number `turns`
-            mbar_wait(&full[q], turns & 1u, &s_flag[3], DRAIN_LIMIT_NS);
-        }
+        for (uint32_t q = p + EP_PRODUCERS * lane; q < a.nslots; q += EP_PRODUCERS * 32u)
+            if (s_turn[q] != 0u) mbar_wait(&full[q], (s_turn[q] - 1u) & 1u, &s_flag[3], DRAIN_LIMIT_NS);
         return;
     }
 
@@ -453,7 +468,7 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + 32, 1)
         for (uint32_t s = wg; s < T.nsub; s += EP_WARPS) {
             const uint32_t n = T.first + s, turn = n / a.nslots, slot = n - turn * a.nslots;
             // a barrier's parity tells neighbouring turns apart and no more, so see this turn begin first
-            if (__all_sync(0xFFFFFFFFu, flag_above(&s_flag[6], n, &s_flag[0], a.wait_ns) &&
+            if (__all_sync(0xFFFFFFFFu, flag_above(&s_turn[slot], turn, &s_flag[0], a.wait_ns) &&
                                             mbar_wait(&full[slot], turn & 1u, &s_flag[0], a.wait_ns)) == 0) {
                 s_flag[0] = 1u;
                 break;
@@ -622,7 +637,7 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + 32, 1)
     asm volatile("bar.sync 3, %0;" ::"n"(NC * EP_CHAIN) : "memory");
     if (warp == 0) tmem_free_all(tmem_base);              // on every path out of the kernel
     // A wait ran out: tell the host and the group's other CTAs.  The copies still in flight are the
-    // producer warp's to wait for.
+    // producer warps' to wait for.
     if (tid == 0) {
         if (s_flag[0] != 0u) {
             atomicOr(a.status, QESGD_STATUS_TIMEOUT);
@@ -715,7 +730,7 @@ bool complete_split(Split &s, uint64_t d, uint32_t K, uint32_t m, uint32_t nsub,
     if (units > (uint32_t)EP_UNITS) return false;
     s.NC = kg >= 2u && units <= (uint32_t)EP_UNITS / 2u ? 2u : 1u;
     const uint32_t slot = SUB * s.cols * 4u, ubytes = s.nit * 512u;
-    const uint32_t fixed = kg * ubytes + s.NC * EP_WARPS * ubytes + s.NC * EP_MAX_M * 4u + 2u * EP_MAX_SLOTS * 8u + 64u;
+    const uint32_t fixed = kg * ubytes + s.NC * EP_WARPS * ubytes + s.NC * EP_MAX_M * 4u + 2u * EP_MAX_SLOTS * 8u + EP_FLAG_BYTES;
     if (fixed + 2u * slot > limit) return false;
     s.nslots = (limit - fixed) / slot;
     if (s.nslots > (uint32_t)EP_MAX_SLOTS) s.nslots = EP_MAX_SLOTS;
@@ -724,7 +739,7 @@ bool complete_split(Split &s, uint64_t d, uint32_t K, uint32_t m, uint32_t nsub,
     s.off_coef = s.off_part + s.NC * EP_WARPS * ubytes;
     s.off_bars = s.off_coef + s.NC * EP_MAX_M * 4u;
     s.off_flags = s.off_bars + 2u * EP_MAX_SLOTS * 8u;
-    s.bytes = s.off_flags + 64u;
+    s.bytes = s.off_flags + EP_FLAG_BYTES;
     const float hbm = (float)((double)K * m * d * 4.0 / 6.5e6);          // us at 6.5 TB/s
     const float chain = EP_CHAIN_US + EP_UNIT_US * (float)units;
     const float chained = chain * (float)kg / (float)s.NC;
@@ -803,7 +818,7 @@ int qesgd_launch_lr_epoch_fused(const float *X, const float *y, uint64_t n_local
 
     void *params[] = {(void *)&a, (void *)&map_full, (void *)&map_rest};
     const void *kernel = s.NC == 2u ? (const void *)qesgd_lr_epoch_kernel<2> : (const void *)qesgd_lr_epoch_kernel<1>;
-    const cudaError_t e = cudaLaunchCooperativeKernel(kernel, dim3(s.G * s.P), dim3(s.NC * EP_CHAIN + 32), params,
+    const cudaError_t e = cudaLaunchCooperativeKernel(kernel, dim3(s.G * s.P), dim3(s.NC * EP_CHAIN + EP_PRODUCERS * 32), params,
                                                       s.bytes, stream);
     if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources ||
         e == cudaErrorInvalidConfiguration || e == cudaErrorNotSupported) {
