@@ -203,8 +203,9 @@ int qesgd_lr_sgd_step(qesgd_ctx *ctx, const float *Xb, const float *yb, uint32_t
                       float lr, float *u);
 /* The summand of Eq. 2 alone: g_out = (1/m) * sum_j grad f_j(w) on the m rows of Xb, for
  * workers that push (quantised) gradients instead of parameters.  w and g_out are float[d]
- * and must not overlap.  One margin pass and one pass that writes the gradient; fp32
- * arithmetic and accumulation as for qesgd_lr_sgd_step. */
+ * and must not overlap.  One launch of the persistent local-epoch kernel where it takes the shape
+ * (see qesgd_lr_local_epoch_batch; its waits are bounded, QESGD_STATUS_TIMEOUT), else one margin pass
+ * and one pass that writes the gradient; fp32 arithmetic and accumulation as for qesgd_lr_sgd_step. */
 int qesgd_lr_gradient(qesgd_ctx *ctx, const float *Xb, const float *yb, uint32_t m, uint64_t d,
                       const float *w, float *g_out);
 /* Rows [0, n_local) of X in consecutive minibatches of `batch` rows, in row

@@ -389,7 +389,7 @@ int qesgd_lr_local_epoch_batch(qesgd_ctx *ctx, const float *X, const float *y, u
     if (!guard.ok) return cuda_fail(ctx, (int)cudaErrorInvalidDevice);
     {   // the whole epoch in one persistent kernel where its shape allows
         int launched = 0;
-        const int e = qesgd_launch_lr_epoch_fused(X, y, n_local, d, K, batch, lr, u, K > 1 ? u_stride : 0,
+        const int e = qesgd_launch_lr_epoch_fused(X, y, n_local, d, K, batch, lr, u, u, false, K > 1 ? u_stride : 0,
                                                   ctx->d_lr_epoch, ctx->d_status, ctx->device, ctx->sm_count,
                                                   ctx->wait_ns, ctx->drop_cta, ctx->stream, &launched);
         ctx->launches += (uint64_t)launched;
@@ -432,7 +432,12 @@ int qesgd_lr_gradient(qesgd_ctx *ctx, const float *Xb, const float *yb, uint32_t
     DeviceGuard guard(ctx->device);
     if (!guard.ok) return cuda_fail(ctx, (int)cudaErrorInvalidDevice);
     int launched = 0;
-    const int e = qesgd_launch_lr_gradient(Xb, yb, m, d, w, g_out, ctx->d_lr_work,
+    int e = qesgd_launch_lr_epoch_fused(Xb, yb, m, d, 1, m, -1.0f, w, g_out, true, 0, ctx->d_lr_epoch, ctx->d_status,
+                                        ctx->device, ctx->sm_count, ctx->wait_ns, ctx->drop_cta, ctx->stream, &launched);
+    ctx->launches += (uint64_t)launched;
+    if (e > 0) return cuda_fail(ctx, e);
+    if (e == 0) return QESGD_OK;
+    e = qesgd_launch_lr_gradient(Xb, yb, m, d, w, g_out, ctx->d_lr_work,
                                            ctx->lr_work_floats, ctx->stream, &launched);
     ctx->launches += (uint64_t)launched;
     if (e != 0) return cuda_fail(ctx, e);

@@ -141,11 +141,13 @@ int qesgd_launch_lr_margins(const float *Xb, const float *yb, uint32_t m, uint64
 int qesgd_launch_lr_gradient(const float *Xb, const float *yb, uint32_t m, uint64_t d,
                              const float *w, float *g, float *work, uint64_t work_floats,
                              cudaStream_t stream, int *launched);
-// A whole local epoch of K workers as one persistent kernel that reads X once.  Returns 0 =
-// launched (one kernel), -1 = shape not covered (the caller falls back to qesgd_launch_lr_step per
-// minibatch), > 0 = cudaError_t.  `work` (QESGD_LR_EPOCH_FLOATS floats) holds the inter-CTA
-// accumulators: zero before the first launch, and every launch leaves it at zero.
+// A whole local epoch of K workers (or, with K = 1, n_local = batch and lr = -1, the mean gradient of
+// one minibatch at u) as one persistent kernel that reads X once.  Returns 0 = launched (one kernel),
+// -1 = shape not covered (the caller falls back to the two-pass steps), > 0 = cudaError_t.  `work`
+// (QESGD_LR_EPOCH_FLOATS floats) holds the inter-CTA accumulators: zero before the first launch, and
+// every launch leaves it at zero.
 int qesgd_launch_lr_epoch_fused(const float *X, const float *y, uint64_t n_local, uint64_t d,
-                                uint32_t K, uint32_t batch, float lr, float *u, uint64_t u_stride,
-                                float *work, uint32_t *status, int device, int sm_count, uint64_t wait_ns,
-                                uint32_t drop_cta, cudaStream_t stream, int *launched);
+                                uint32_t K, uint32_t batch, float lr, const float *u, float *dst,
+                                bool gradient, uint64_t u_stride, float *work, uint32_t *status, int device,
+                                int sm_count, uint64_t wait_ns, uint32_t drop_cta, cudaStream_t stream,
+                                int *launched);
