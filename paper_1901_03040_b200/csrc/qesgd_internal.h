@@ -69,6 +69,8 @@ struct QstepArgs {
     uint32_t m;
     float rate;             // lr / m
     const float *margins;   // the m margins, as the margin pass left them
+    uint32_t reverse;       // tiles from the last to the first (see qesgd_second_pass_reversed)
+    uint32_t wide;          // X and its rows, u, anchor and running sum 32-byte aligned
 };
 
 struct DecodeArgs {
@@ -133,6 +135,11 @@ int qesgd_launch_lr_step(const float *Xb, uint64_t x_worker_stride, const float 
                          uint64_t y_worker_stride, uint32_t m, uint64_t d, uint32_t K, float lr,
                          float *u, uint64_t u_stride, float *work, uint64_t work_floats,
                          cudaStream_t stream, int *launched);
+// A minibatch that does not fit L2 is read a second time from its end: what the margin pass, which walks
+// the columns upwards, read last is still there.  Measured (second pass included): 64 x 2^22 sgd_step 324 ->
+// 318 us, qstep 343 -> 337; 64 x 2^19 54 -> 50; where the minibatch fits, the plain order is the better
+// one (16 x 2^20, 67 MB: 31.8 against 33.8).
+inline bool qesgd_second_pass_reversed(uint64_t m, uint64_t d) { return m * d * 4u > (96ull << 20); }
 // The margin pass alone (pass 1 of a step) for one worker; *parts_out receives the number of
 // partial margins per row that the pass leaves in `work` ([parts][m]).
 int qesgd_launch_lr_margins(const float *Xb, const float *yb, uint32_t m, uint64_t d, const float *u,

@@ -20,7 +20,10 @@ constexpr int SEG = 1024;        // columns per segment in pass 1 (32 lanes x 8 
 #define QESGD_LR_MAX_PARTS 296
 #endif
 constexpr int MAX_PARTS = QESGD_LR_MAX_PARTS;   // CTAs of the margin pass per worker: two per SM of a B200
+constexpr int ROW_CTAS = 148;    // rows are split over CTAs up to this many
 constexpr int DONE_WORDS = 64;   // one arrival counter per worker at the head of the workspace
+// pass 2: eight CTAs per SM with 32 registers, so no run-time choice of direction (36 registers, six CTAs:
+// 16 x 2^20 32.8 -> 34.9 us)
 constexpr int UPD_COLS = 256;      // pass 2: columns per CTA (64 groups of 4)
 constexpr int UPD_ROWGROUPS = 4;   // pass 2: row groups per CTA
 constexpr int UPD_THREADS = (UPD_COLS / 4) * UPD_ROWGROUPS;
@@ -42,6 +45,7 @@ struct LrArgs {
     uint32_t *done;      // arrival counters [K], zero between launches
     uint32_t parts;      // P
     uint32_t nseg;
+    uint32_t row_groups; // CTAs that share a part's rows: rows 16 g .. 16 g + 15, then + 16 row_groups, ...
 };
 
 template <bool VEC>
@@ -49,7 +53,7 @@ __global__ void __launch_bounds__(256) qesgd_lr_margin_kernel(const LrArgs a)
 {
     __shared__ float s_part[QESGD_MAX_LR_BATCH];
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    const uint32_t k = blockIdx.y, p = blockIdx.x;
+    const uint32_t k = blockIdx.y, p = blockIdx.x, rg = blockIdx.z;
     const float *__restrict__ X = a.X + (uint64_t)k * a.x_stride;
     const float *__restrict__ u = a.u + (uint64_t)k * a.u_stride;
     for (uint32_t j = threadIdx.x; j < a.m; j += blockDim.x) s_part[j] = 0.0f;
@@ -72,7 +76,7 @@ __global__ void __launch_bounds__(256) qesgd_lr_margin_kernel(const LrArgs a)
         }
         // each row belongs to one warp; two rows at a time so that 16 loads are in flight
         // per lane and the two shuffle reductions interleave
-        for (uint32_t j = warp; j < a.m; j += 16) {
+        for (uint32_t j = 16u * rg + warp; j < a.m; j += 16u * a.row_groups) {
             const uint32_t j2 = j + 8;
             const bool two = j2 < a.m;
             const float *__restrict__ row0 = X + (uint64_t)j * a.d;
@@ -120,14 +124,15 @@ __global__ void __launch_bounds__(256) qesgd_lr_margin_kernel(const LrArgs a)
     }
     __syncthreads();
     float *__restrict__ out = a.work + ((uint64_t)k * a.parts + p) * a.m;
-    for (uint32_t j = threadIdx.x; j < a.m; j += blockDim.x) out[j] = s_part[j];
+    for (uint32_t j = threadIdx.x; j < a.m; j += blockDim.x)
+        if (j / 16u % a.row_groups == rg) out[j] = s_part[j];
     // The CTA that arrives last sums the partial margins of its worker, once, in an order that
     // does not depend on which CTA that is: a row's P partials in four consecutive runs (one
     // thread each, in index order), the four run sums added in run order.
     __shared__ uint32_t s_last;
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(a.done + k, 1u) == a.parts - 1u ? 1u : 0u;
+    if (threadIdx.x == 0) s_last = atomicAdd(a.done + k, 1u) == a.parts * a.row_groups - 1u ? 1u : 0u;
     __syncthreads();
     if (s_last == 0u) return;
     __threadfence();
@@ -153,7 +158,8 @@ __global__ void __launch_bounds__(256) qesgd_lr_margin_kernel(const LrArgs a)
 // Pass 2.  A CTA updates UPD_COLS consecutive columns: 64 column groups of 4 columns
 // times UPD_ROWGROUPS row groups; row group g sums rows g, g + G, g + 2G, ... (coalesced
 // 1 KB per row), the G partial sums meet in shared memory in fixed order.
-template <bool VEC>
+// REV: from the last columns to the first (see qesgd_second_pass_reversed).
+template <bool VEC, bool REV>
 __global__ void __launch_bounds__(UPD_THREADS) qesgd_lr_update_kernel(const LrArgs a)
 {
     __shared__ float s_coef[QESGD_MAX_LR_BATCH];
@@ -173,7 +179,7 @@ __global__ void __launch_bounds__(UPD_THREADS) qesgd_lr_update_kernel(const LrAr
 
     const uint32_t cg = threadIdx.x % (UPD_COLS / 4);     // column group inside the CTA
     const uint32_t rg = threadIdx.x / (UPD_COLS / 4);     // row group
-    const uint64_t c = (uint64_t)blockIdx.x * UPD_COLS + cg * 4u;
+    const uint64_t c = (uint64_t)(REV ? gridDim.x - 1u - blockIdx.x : blockIdx.x) * UPD_COLS + cg * 4u;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
     if (VEC && c + 4 <= a.d) {
         const float *__restrict__ col = X + c;
@@ -237,6 +243,14 @@ uint64_t lay_out_work(LrArgs &a, float *work, uint64_t work_floats, uint32_t K, 
     a.margins = work + DONE_WORDS;
     a.work = work + head;
     a.parts = (uint32_t)parts;
+    // Too few column segments for the SMs: the rows are split as well, sixteen (two per warp, one trip of
+    // the row loop) to a CTA at the least.  A gradient of 200 x 5001 37 -> 22 us, a step of 64 x 30002
+    // 18.6 -> 16.6; with more CTAs than SMs the arrivals at the end cost more than the trips saved
+    // (64 x 131072, margins and fused second pass: 21.0, at 296 CTAs 24.7).
+    const uint32_t trips = (m + 15u) / 16u;
+    uint32_t groups = parts > 0 && K * parts < (uint64_t)ROW_CTAS ? ROW_CTAS / (uint32_t)(K * parts) : 1u;
+    a.row_groups = groups < trips ? groups : trips;
+    if (a.row_groups < 1u) a.row_groups = 1u;
     return parts;
 }
 
@@ -260,7 +274,7 @@ int launch_lr_passes(const float *Xb, uint64_t x_worker_stride, const float *yb,
     a.nseg = (uint32_t)nseg;
     const bool vec = (d % 4 == 0) && (x_worker_stride % 4 == 0) && (u_stride % 4 == 0) &&
                      (((uintptr_t)Xb | (uintptr_t)u | (uintptr_t)dst) % 16 == 0);
-    dim3 g1((unsigned)parts, K), b1(256);
+    dim3 g1((unsigned)parts, K, a.row_groups), b1(256);
     if (vec) qesgd_lr_margin_kernel<true><<<g1, b1, 0, stream>>>(a);
     else qesgd_lr_margin_kernel<false><<<g1, b1, 0, stream>>>(a);
     cudaError_t e = cudaGetLastError();
@@ -269,8 +283,13 @@ int launch_lr_passes(const float *Xb, uint64_t x_worker_stride, const float *yb,
     const uint64_t ublocks = (d + UPD_COLS - 1) / UPD_COLS;
     if (ublocks > 0x7FFFFFFFull) return (int)cudaErrorInvalidValue;
     dim3 g2((unsigned)ublocks, K), b2(UPD_THREADS);
-    if (vec) qesgd_lr_update_kernel<true><<<g2, b2, 0, stream>>>(a);
-    else qesgd_lr_update_kernel<false><<<g2, b2, 0, stream>>>(a);
+    if (qesgd_second_pass_reversed((uint64_t)K * m, d)) {
+        if (vec) qesgd_lr_update_kernel<true, true><<<g2, b2, 0, stream>>>(a);
+        else qesgd_lr_update_kernel<false, true><<<g2, b2, 0, stream>>>(a);
+    } else {
+        if (vec) qesgd_lr_update_kernel<true, false><<<g2, b2, 0, stream>>>(a);
+        else qesgd_lr_update_kernel<false, false><<<g2, b2, 0, stream>>>(a);
+    }
     e = cudaGetLastError();
     if (e == cudaSuccess) *launched = 2;
     return (int)e;
@@ -292,7 +311,7 @@ int qesgd_launch_lr_margins(const float *Xb, const float *yb, uint32_t m, uint64
     if (parts == 0 || nseg > 0xFFFFFFFFull) return (int)cudaErrorInvalidValue;
     a.nseg = (uint32_t)nseg;
     const bool vec = (d % 4 == 0) && (((uintptr_t)Xb | (uintptr_t)u) % 16 == 0);
-    dim3 g1((unsigned)parts, 1), b1(256);
+    dim3 g1((unsigned)parts, 1, a.row_groups), b1(256);
     if (vec) qesgd_lr_margin_kernel<true><<<g1, b1, 0, stream>>>(a);
     else qesgd_lr_margin_kernel<false><<<g1, b1, 0, stream>>>(a);
     *margins_out = a.margins;
