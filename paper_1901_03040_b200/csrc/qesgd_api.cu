@@ -278,6 +278,8 @@ int qesgd_lr_qesgd_step(qesgd_ctx *ctx, const float *Xb, const float *yb, uint32
     q.m = m;
     q.rate = lr / (float)m;
     q.margins = margins;
+    q.reverse = qesgd_second_pass_reversed(m, d) ? 1u : 0u;
+    q.wide = d % 8 == 0 && aligned(Xb, 32) && aligned(u, 32) && aligned(anchor, 32) && aligned(zsum, 32) ? 1u : 0u;
     switch (bits) {
         case 2: e = qesgd_launch_lr_qstep_2(q, scale_mode, ctx->stream); break;
         case 4: e = qesgd_launch_lr_qstep_4(q, scale_mode, ctx->stream); break;

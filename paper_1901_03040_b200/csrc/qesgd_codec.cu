@@ -88,16 +88,17 @@ __device__ __forceinline__ void load_octet(const float *p, uint64_t eb, uint64_t
 // Philox4x32 with 10 rounds (Salmon, Moraes, Dror, Shaw, SC'11), written from the
 // published round function: two 32x32->64 multiplies, the high halves xor'ed with
 // the other counter words and the round key; the key grows by the Weyl constants.
-// Two independent blocks advanced round by round: four multiply chains in flight instead
+// N independent blocks advanced round by round; with two, four multiply chains are in flight instead
 // of two (measured 2 % faster than one block at a time; four at a time costs registers).
 // rk[r] = key + r * (0x9E3779B9, 0xBB67AE85): the ten round keys, prepared on the host so
 // that they reach the xor as kernel-parameter operands instead of per-thread additions.
-__device__ __forceinline__ void philox4x32_10_x2(uint32_t (&c)[2][4], const uint32_t (&rk)[10][2])
+template <int N>
+__device__ __forceinline__ void philox4x32_10(uint32_t (&c)[N][4], const uint32_t (&rk)[10][2])
 {
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
 #pragma unroll
-        for (int n = 0; n < 2; ++n) {
+        for (int n = 0; n < N; ++n) {
             const uint64_t p0 = (uint64_t)0xD2511F53u * c[n][0];
             const uint64_t p1 = (uint64_t)0xCD9E8D57u * c[n][2];
             const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c[n][1] ^ rk[r][0];
@@ -298,12 +299,12 @@ struct MaxU32 {
 template <int V>
 __device__ __forceinline__ uint32_t chunk_of_lane(uint32_t lane)
 {
-    return V == 4 ? 2u * (lane & 1u) + ((lane >> 1) & 1u) : (lane & 1u);
+    return V == 4 ? 2u * (lane & 1u) + ((lane >> 1) & 1u) : (V == 2 ? (lane & 1u) : 0u);
 }
 template <int V>
 __device__ __forceinline__ uint32_t lane_of_chunk(uint32_t lane, int c)
 {
-    return V == 4 ? ((lane & 28u) | ((c >> 1) & 1) | ((c & 1) << 1)) : ((lane & 30u) | (c & 1));
+    return V == 4 ? ((lane & 28u) | ((c >> 1) & 1) | ((c & 1) << 1)) : (V == 2 ? ((lane & 30u) | (c & 1)) : lane);
 }
 
 template <typename R>
@@ -341,6 +342,20 @@ __device__ __forceinline__ typename R::T reduce_chunks(const typename R::T (&t)[
     if (lb >= 7) k = R::op(k, __shfl_xor_sync(FULL, k, 8));
     if (lb >= 8) k = R::op(k, __shfl_xor_sync(FULL, k, 16));
     if (lb >= 9) k = R::op(k, __shfl_xor_sync(FULL, k, 1));    // both chunks
+    return k;
+}
+
+// One chunk: the plain tree over the lanes, every lane of a bucket ends with its total.
+template <typename R>
+__device__ __forceinline__ typename R::T reduce_chunks(const typename R::T (&t)[1], uint32_t lane,
+                                                       uint32_t lb)
+{
+    typename R::T k = t[0];
+    k = R::op(k, __shfl_xor_sync(FULL, k, 1));
+    k = R::op(k, __shfl_xor_sync(FULL, k, 2));
+    k = R::op(k, __shfl_xor_sync(FULL, k, 4));
+    if (lb >= 7) k = R::op(k, __shfl_xor_sync(FULL, k, 8));
+    if (lb >= 8) k = R::op(k, __shfl_xor_sync(FULL, k, 16));
     return k;
 }
 
@@ -386,7 +401,8 @@ __device__ __forceinline__ void encode_warp_tile(const EncodeArgs &a, float (&z)
                                                  uint64_t warp_base, uint32_t k, uint32_t lane,
                                                  uint32_t warp, EncodeShared &sh, uint32_t iter)
 {
-    constexpr uint32_t LOG2_WARP_ELEMS = V == 4 ? 10 : 9;
+    constexpr uint32_t LOG2_WARP_ELEMS = V == 4 ? 10 : (V == 2 ? 9 : 8);
+    constexpr int DRAWS = V > 1 ? 2 : 1;                        // Philox blocks advanced together
     const uint32_t lb = a.log2_bucket;
     const float sf = (float)a.s;
     float my_scale, my_inv, my_delta = 0.0f;
@@ -405,18 +421,18 @@ __device__ __forceinline__ void encode_warp_tile(const EncodeArgs &a, float (&z)
     const bool wide = lb > LOG2_WARP_ELEMS;                     // bucket spans several warps
     const bool wide_first = ((uint32_t)warp_base & bucket_mask) == 0u;   // this warp starts it
     const uint32_t wid = a.worker0 + k;
-    uint32_t xx[2][4];
+    uint32_t xx[DRAWS][4];
 
     // The draws of the first two chunks are computed before the scale: they depend on nothing
     // loaded, so they fill the time the reduction's shuffles and the square root wait.
 #pragma unroll
-    for (int n = 0; n < 2; ++n) {
+    for (int n = 0; n < DRAWS; ++n) {
         xx[n][0] = blk_lo + 32u * n;
         xx[n][1] = blk_hi;
         xx[n][2] = wid;
         xx[n][3] = a.epoch;
     }
-    philox4x32_10_x2(xx, a.round_key);
+    philox4x32_10(xx, a.round_key);
 
     // ---- per-bucket scale: one value per lane, then handed back per chunk ------
     if (MODE == 0) {
@@ -470,7 +486,7 @@ __device__ __forceinline__ void encode_warp_tile(const EncodeArgs &a, float (&z)
         const uint32_t off = (uint32_t)c * CHUNK + loff;        // element offset inside the tile
         const bool inside = FULL || warp_base + off < a.padded;
         float scale = my_scale, inv = my_inv, delta = my_delta;
-        if (MODE != 2) {   // fetch chunk c's bucket scale from the neighbour lane that carried it
+        if (MODE != 2 && V > 1) {   // fetch chunk c's bucket scale from the neighbour lane that carried it
             const int src = (int)lane_of_chunk<V>(lane, c);
             scale = __shfl_sync(FULL, my_scale, src);
             inv = __shfl_sync(FULL, my_inv, src);
@@ -488,15 +504,15 @@ __device__ __forceinline__ void encode_warp_tile(const EncodeArgs &a, float (&z)
 
         if ((c & 1) == 0 && c > 0) {   // draws for this chunk and the next, interleaved
 #pragma unroll
-            for (int n = 0; n < 2; ++n) {
+            for (int n = 0; n < DRAWS; ++n) {
                 xx[n][0] = blk_lo + 32u * (c + n);
                 xx[n][1] = blk_hi;
                 xx[n][2] = wid;
                 xx[n][3] = a.epoch;
             }
-            philox4x32_10_x2(xx, a.round_key);
+            philox4x32_10(xx, a.round_key);
         }
-        const uint32_t (&x)[4] = xx[c & 1];
+        const uint32_t (&x)[4] = xx[c & (DRAWS - 1)];
 
         uint32_t X[8], Z[8];
         const uint64_t inv2 = pack2f(inv, inv);
@@ -618,26 +634,93 @@ __global__ void __launch_bounds__(WARPS * 32, QESGD_ENCODE_MIN_WARPS / WARPS)
 }
 
 // ---------------------------------- update + requantise (Algorithm 2 inner step) ----
-// One inner iteration of QESGD on logistic regression after the margin pass: a CTA owns a
-// tile of 1024 columns, forms u^ = u - (lr/m) sum_j c_j x_j for them in shared memory (the
-// arithmetic of the plain update pass, in its order: rows split over four groups, group sums
-// added in group order), and its first warp then quantises u^ - w_t, writes u = w_t + Q(z^),
-// the running sum and the stream exactly as qesgd_requantize would.  The updated parameter
-// never travels to global memory before it is quantised.  Buckets of at most 1024 elements,
-// d a multiple of 4, 16-byte aligned X and u.  The register budget is set for three CTAs per SM
-// (the requantising warp needs its 80 registers, the update loop needs the occupancy: with two
-// CTAs per SM the call was 13 % slower than the two separate calls, with three it equals them).
-constexpr int QS_COLS = 256;                   // columns per sub-tile: 64 groups of 4
+// One inner iteration of QESGD on logistic regression after the margin pass: a lane owns 8
+// consecutive columns (an octet), a warp 256, a CTA 1024.  A lane forms u^ = u - (lr/m) sum_j c_j x_j
+// for its columns in registers -- the arithmetic of the plain update pass, in its order: rows split
+// over four groups, group sums added in group order -- and its warp then quantises u^ - w_t from
+// there, writes u = w_t + Q(z^), the running sum and the stream exactly as qesgd_requantize would.
+// The updated parameter never travels anywhere before it is quantised.  Buckets of at most 1024
+// elements, d a multiple of 4, 16-byte aligned X and u.  Bound by the second read of the minibatch:
+// with 8 columns per lane a row is one 256-bit load per lane (1 KB per warp) and every warp quantises
+// what it summed.  Four row
+// groups of eight columns, two rows of each requested at a time, take 128 registers: four CTAs per SM,
+// 128 KB of loads in flight.  Against the kernel before (one warp of eight quantised a tile that all
+// had summed into shared memory), margin pass included: 64 x 2^22 369 -> 335 us, 128 x 2^20 193 -> 176,
+// 16 x 2^20 53 -> 33, 256 x 4096 33 -> 23.
+constexpr int QS_WARPS = 4;
+constexpr int QS_THREADS = QS_WARPS * 32;
+constexpr int QS_TILE = QS_WARPS * CHUNK;      // columns per CTA
 constexpr int QS_ROWGROUPS = 4;
-constexpr int QS_THREADS = (QS_COLS / 4) * QS_ROWGROUPS;
-constexpr int QS_TILE = 4 * CHUNK;             // columns per CTA
+#ifndef QESGD_QS_CTAS
+#define QESGD_QS_CTAS 4                        // resident CTAs per SM the register budget is set for
+#endif
+
+// 8 floats at p (16-byte aligned; WIDE = 32-byte aligned)
+template <bool WIDE>
+__device__ __forceinline__ void load_eight(const float *p, float (&v)[8])
+{
+    if (WIDE) {
+        ld256(p, v);
+    } else {
+        const float4 a = __ldg(reinterpret_cast<const float4 *>(p)), b = __ldg(reinterpret_cast<const float4 *>(p) + 1);
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+        v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    }
+}
+
+// sum_j coef_j x_j of a lane's 8 columns over all rows, as four row groups added in order
+template <bool WIDE>
+__device__ __forceinline__ void sum_rows(const float *__restrict__ col, uint64_t d, uint32_t m, const float *s_coef,
+                                         float (&t)[8])
+{
+    float acc[QS_ROWGROUPS][8];
+#pragma unroll
+    for (int g = 0; g < QS_ROWGROUPS; ++g)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[g][j] = 0.0f;
+    uint32_t r = 0;
+#pragma unroll 1
+    for (; WIDE && r + 2 * QS_ROWGROUPS <= m; r += 2 * QS_ROWGROUPS) {   // eight rows requested at a time
+        float x[2 * QS_ROWGROUPS][8];
+#pragma unroll
+        for (int g = 0; g < 2 * QS_ROWGROUPS; ++g) load_eight<WIDE>(col + (uint64_t)(r + g) * d, x[g]);
+#pragma unroll
+        for (int g = 0; g < 2 * QS_ROWGROUPS; ++g)
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                acc[g % QS_ROWGROUPS][j] = fmaf(s_coef[r + g], x[g][j], acc[g % QS_ROWGROUPS][j]);
+    }
+#pragma unroll 1
+    for (; r + QS_ROWGROUPS <= m; r += QS_ROWGROUPS) {
+        float x[QS_ROWGROUPS][8];
+#pragma unroll
+        for (int g = 0; g < QS_ROWGROUPS; ++g) load_eight<WIDE>(col + (uint64_t)(r + g) * d, x[g]);
+#pragma unroll
+        for (int g = 0; g < QS_ROWGROUPS; ++g)
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[g][j] = fmaf(s_coef[r + g], x[g][j], acc[g][j]);
+    }
+#pragma unroll
+    for (int g = 0; g < QS_ROWGROUPS - 1; ++g) {
+        if (r + g < m) {
+            float x[8];
+            load_eight<WIDE>(col + (uint64_t)(r + g) * d, x);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[g][j] = fmaf(s_coef[r + g], x[j], acc[g][j]);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        t[j] = acc[0][j];
+#pragma unroll
+        for (int g = 1; g < QS_ROWGROUPS; ++g) t[j] = __fadd_rn(t[j], acc[g][j]);
+    }
+}
 
 template <int BITS, int MODE>
-__global__ void __launch_bounds__(QS_THREADS, 3) qesgd_lr_qstep_kernel(const QstepArgs q)
+__global__ void __launch_bounds__(QS_THREADS, QESGD_QS_CTAS) qesgd_lr_qstep_kernel(const QstepArgs q)
 {
     __shared__ float s_coef[QESGD_MAX_LR_BATCH];
-    __shared__ float4 s_sum[QS_ROWGROUPS][QS_COLS / 4];
-    __shared__ __align__(32) float s_u[QS_TILE];
     __shared__ EncodeShared sh;
     const EncodeArgs &a = q.e;
     for (uint32_t j = threadIdx.x; j < q.m; j += blockDim.x) {
@@ -647,78 +730,51 @@ __global__ void __launch_bounds__(QS_THREADS, 3) qesgd_lr_qstep_kernel(const Qst
         s_coef[j] = q.rate * yj / (1.0f + expf(yj * margin));
     }
     __syncthreads();
-    const uint32_t cg = threadIdx.x % (QS_COLS / 4), rg = threadIdx.x / (QS_COLS / 4);
-    const uint64_t tile0 = (uint64_t)blockIdx.x * QS_TILE;
-#pragma unroll 1
-    for (int sub = 0; sub < QS_TILE / QS_COLS; ++sub) {
-        const uint64_t c = tile0 + (uint64_t)sub * QS_COLS + cg * 4u;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (c + 4 <= a.d) {
-            const float *__restrict__ col = q.X + c;
-#pragma unroll 8
-            for (uint32_t j = rg; j < q.m; j += QS_ROWGROUPS) {
-                const float4 x = __ldg(reinterpret_cast<const float4 *>(col + (uint64_t)j * a.d));
-                const float cj = s_coef[j];
-                acc.x = fmaf(cj, x.x, acc.x);
-                acc.y = fmaf(cj, x.y, acc.y);
-                acc.z = fmaf(cj, x.z, acc.z);
-                acc.w = fmaf(cj, x.w, acc.w);
-            }
-        }
-        s_sum[rg][cg] = acc;
-        __syncthreads();
-        if (rg == 0) {
-            float4 uu = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (c + 4 <= a.d) {
-                float4 t = s_sum[0][cg];
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    const uint64_t tile0 = (uint64_t)(q.reverse ? gridDim.x - 1u - blockIdx.x : blockIdx.x) * QS_TILE, warp0 = tile0 + warp * (uint32_t)CHUNK;
+    const uint64_t c = warp0 + lane * 8u;
+    float z[1][8];
+    if (tile0 + QS_TILE <= a.d && q.wide) {   // interior tile, everything 32-byte aligned
+        float t[8], u[8], w[8];
+        sum_rows<true>(q.X + c, a.d, q.m, s_coef, t);
+        ld256_rw(a.local + c, u);
+        ld256(a.anchor + c, w);
 #pragma unroll
-                for (int g = 1; g < QS_ROWGROUPS; ++g) {
-                    const float4 v = s_sum[g][cg];
-                    t.x = __fadd_rn(t.x, v.x); t.y = __fadd_rn(t.y, v.y);
-                    t.z = __fadd_rn(t.z, v.z); t.w = __fadd_rn(t.w, v.w);
-                }
-                uu = *reinterpret_cast<const float4 *>(a.local + c);
-                uu.x = __fadd_rn(uu.x, t.x); uu.y = __fadd_rn(uu.y, t.y);
-                uu.z = __fadd_rn(uu.z, t.z); uu.w = __fadd_rn(uu.w, t.w);
-            }
-            *reinterpret_cast<float4 *>(s_u + sub * QS_COLS + cg * 4u) = uu;
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x >= 32) return;
-    // the first warp requantises the tile: z = u^ - w_t, zeros past d
-    const uint32_t lane = threadIdx.x;
-    float z[4][8];
-    const bool full = tile0 + QS_TILE <= a.d &&
-                      ((reinterpret_cast<uintptr_t>(a.anchor) | reinterpret_cast<uintptr_t>(a.u_out) |
-                        reinterpret_cast<uintptr_t>(a.zsum)) & 31u) == 0u;
-    if (full) {   // interior tile, aligned vectors: 256-bit loads and stores throughout
-        float w[4][8];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) ld256(a.anchor + tile0 + (uint64_t)c * CHUNK + lane * 8u, w[c]);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            const float4 u0 = *reinterpret_cast<const float4 *>(s_u + c * CHUNK + lane * 8u);
-            const float4 u1 = *reinterpret_cast<const float4 *>(s_u + c * CHUNK + lane * 8u + 4u);
-            const float uj[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
-#pragma unroll
-            for (int j = 0; j < 8; ++j) z[c][j] = __fsub_rn(uj[j], w[c][j]);
-        }
-        encode_warp_tile<BITS, MODE, 4, true, true>(a, z, tile0, 0u, lane, 0u, sh, 0u);
+        for (int j = 0; j < 8; ++j) z[0][j] = __fsub_rn(__fadd_rn(u[j], t[j]), w[j]);
+        encode_warp_tile<BITS, MODE, 1, true, true>(a, z, warp0, 0u, lane, warp, sh, 0u);
         return;
     }
+    float t[8];
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const uint64_t e0 = tile0 + (uint64_t)c * CHUNK + lane * 8u;
-        float w[8];
-        load_octet<false>(a.anchor, e0, a.d, w);
+    for (int j = 0; j < 8; ++j) t[j] = 0.0f;
+    if (c + 8 <= a.d) {
+        sum_rows<false>(q.X + c, a.d, q.m, s_coef, t);
+    } else if (c < a.d) {                     // the last four columns (d is a multiple of 4)
+        float acc[QS_ROWGROUPS][4];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const float uj = s_u[c * CHUNK + lane * 8u + j];
-            z[c][j] = (e0 + j < a.d) ? __fsub_rn(uj, w[j]) : 0.0f;
+        for (int g = 0; g < QS_ROWGROUPS; ++g) acc[g][0] = acc[g][1] = acc[g][2] = acc[g][3] = 0.0f;
+        for (uint32_t r = 0; r < q.m; r += QS_ROWGROUPS) {
+#pragma unroll
+            for (int g = 0; g < QS_ROWGROUPS; ++g) {
+                if (r + g < q.m) {
+                    const float4 x = __ldg(reinterpret_cast<const float4 *>(q.X + c + (uint64_t)(r + g) * a.d));
+                    const float cj = s_coef[r + g];
+                    acc[g][0] = fmaf(cj, x.x, acc[g][0]);
+                    acc[g][1] = fmaf(cj, x.y, acc[g][1]);
+                    acc[g][2] = fmaf(cj, x.z, acc[g][2]);
+                    acc[g][3] = fmaf(cj, x.w, acc[g][3]);
+                }
+            }
         }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) t[j] = __fadd_rn(__fadd_rn(__fadd_rn(acc[0][j], acc[1][j]), acc[2][j]), acc[3][j]);
     }
-    encode_warp_tile<BITS, MODE, 4, false, true>(a, z, tile0, 0u, lane, 0u, sh, 0u);
+    float u[8], w[8];
+    load_octet<false, true>(a.local, c, a.d, u);
+    load_octet<false>(a.anchor, c, a.d, w);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) z[0][j] = c + j < a.d ? __fsub_rn(__fadd_rn(u[j], t[j]), w[j]) : 0.0f;
+    encode_warp_tile<BITS, MODE, 1, false, true>(a, z, warp0, 0u, lane, warp, sh, 0u);
 }
 
 // ------------------------------------------------------------- decode -------

@@ -639,6 +639,58 @@ def test_fused_inner_step_equals_step_then_requantize(m, d, bucket, bits, s, mod
     assert (got_zsum.view(np.uint32) == want_zsum.view(np.uint32)).all()
 
 
+@pytest.mark.parametrize("m,d,bucket,bits,s,mode,shift", [
+    (1, 4, 64, 8, 127, ref.SCALE_NORM, 0),         # one row, one group of four columns
+    (9, 1020, 512, 4, 7, ref.SCALE_NORM, 0),       # a tile that ends four columns early, eight rows and one
+    (12, 1028, 1024, 8, 127, ref.SCALE_MAX, 0),    # four columns into the second tile, bucket over four warps
+    (7, 2048, 256, 2, 1, ref.SCALE_NORM, 0),       # fewer rows than are requested at a time
+    (20, 3072, 128, 4, 7, ref.SCALE_FIXED, 4),     # X and u aligned to 16 bytes only
+    (35, 4352, 1024, 8, 100, ref.SCALE_NORM, 4),
+])
+def test_fused_inner_step_at_the_edges_of_its_tiles(m, d, bucket, bits, s, mode, shift):
+    """The second kernel of the inner iteration: a warp sums and quantises 256 columns.  From the
+    two-pass step's own result on everything equals the oracle's requantisation bit for bit."""
+    X, y, _ = synthetic.logistic_problem(m, d, seed=m + d)
+    w = synthetic.anchor_vector(d, seed=8)
+    u0 = (w + _delta(d, 9, sigma=2e-3)).astype(np.float32)
+    zsum0 = _delta(d, 10, sigma=1e-3)
+    c, ty, fixed = G.ctx(), G.dev(y), 4e-3 / s
+
+    def place(a):
+        buf = torch.full((a.size + shift + 8,), 55.0, dtype=torch.float32, device="cuda")
+        buf[shift:shift + a.size] = G.dev(a.reshape(-1))
+        return buf, buf[shift:shift + a.size]
+    bX, tX = place(X)
+    u1 = G.dev(u0)
+    qesgd.qesgd_lr_sgd_step_noalloc(None, tX, ty, m, d, 0.3, u1)
+    _lr_close(u1.cpu().numpy(), ref.lr_sgd_step(X, y, 0.3, u0))
+    want = ref.requantize(u1.cpu().numpy(), w, bucket, s, bits, mode, 21, 3, 7, zsum=zsum0, fixed_delta=fixed)
+    bu, tu = place(u0)
+    bz, tz = place(zsum0)
+    codes = torch.zeros(qesgd.code_bytes(d, bucket, bits), dtype=torch.uint8, device="cuda")
+    scales = torch.zeros(qesgd.num_buckets(d, bucket), dtype=torch.float32, device="cuda")
+    c.qesgd_lr_qesgd_step(tX, ty, m, d, 0.3, tu, G.dev(w), bucket, s, bits, mode, 21, 3, 7, tz, codes, scales,
+                          fixed_delta=fixed)
+    assert c.qesgd_status() == want[4]
+    assert (bu[shift + d:] == 55.0).all().item() and (bz[shift + d:] == 55.0).all().item()
+    for got, exp in ((tu, want[0]), (tz, want[1]), (scales, want[3])):
+        assert (got.cpu().numpy().view(np.uint32) == exp.view(np.uint32)).all()
+    assert (codes.cpu().numpy().view(np.uint32) == want[2]).all()
+
+
+@pytest.mark.parametrize("m,d", [(200, 5001), (33, 65541), (17, 150001),    # rows split over 13, 2 and 1 CTAs per segment
+                                 (64, 150000), (256, 30000), (1, 4), (64, 419432)])
+def test_lr_gradient_shapes_match_oracle(m, d):
+    """Both forms of the gradient: two passes with the rows split over CTAs where segments are few, and
+    the persistent kernel as an epoch of one step.  fp32 sums of d (margins) and m terms against fp64."""
+    X, y, _ = synthetic.logistic_problem(m, d, seed=m + d)
+    w = (0.3 * synthetic.normal_f32(d, 1.0, 8)).astype(np.float32)
+    tg = torch.full((d + 4,), 9.0, dtype=torch.float32, device="cuda")
+    G.ctx().qesgd_lr_gradient(G.dev(X), G.dev(y), m, d, G.dev(w), tg)
+    assert G.ctx().qesgd_status() == 0 and (tg[d:] == 9.0).all().item()
+    _lr_close(tg[:d].cpu().numpy(), ref.lr_gradient(X, y, w))
+
+
 @pytest.mark.parametrize("alpha", [-0.1, 1.0, -3.5])
 @pytest.mark.parametrize("K,bucket,bits,s", [(4, 128, 4, 7), (16, 256, 2, 1), (3, 1024, 8, 127)])
 def test_decode_average_axpy_matches_oracle(K, bucket, bits, s, alpha):
