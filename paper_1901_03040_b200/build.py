@@ -6,6 +6,7 @@ the rounding chain is contracted; the logistic-regression unit keeps FMAs.
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -13,6 +14,7 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libqesgd.so")
 LIB_DEBUG = os.path.join(HERE, "libqesgd_debug.so")
+PY_MODULE = os.path.join(HERE, "_qesgd_py.so")      # argument marshalling of the Python binding (g++)
 
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
 COMMON = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"),
@@ -42,10 +44,21 @@ def _stale(target, sources):
     return any(os.path.getmtime(s) > t for s in sources)
 
 
+def build_py_module(force: bool = False) -> str:
+    """Compiles csrc/qesgd_py.cpp into the CPython module next to the library (no CUDA, nothing linked)."""
+    src = os.path.join(CSRC, "qesgd_py.cpp")
+    if force or _stale(PY_MODULE, [src, os.path.join(ROOT, "include", "qesgd.h"), os.path.abspath(__file__)]):
+        subprocess.run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+                        "-I", os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"], src,
+                        "-o", PY_MODULE], check=True)
+    return PY_MODULE
+
+
 def build(force: bool = False, verbose: bool = False, debug: bool = False) -> str:
     """Builds libqesgd.so, or with debug=True libqesgd_debug.so: the same library compiled with
     -DQESGD_DEBUG (the codec kernels check their indices and set QESGD_STATUS_RANGE)."""
     os.makedirs(OBJ, exist_ok=True)
+    build_py_module(force)
     headers = [os.path.join(CSRC, "qesgd_internal.h"), os.path.join(ROOT, "include", "qesgd.h"),
                os.path.abspath(__file__)]
     nvcc = _nvcc()

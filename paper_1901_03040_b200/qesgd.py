@@ -1,8 +1,11 @@
-"""Thin ctypes binding of libqesgd.so (include/qesgd.h) on torch CUDA tensors.
+"""Thin binding of libqesgd.so (include/qesgd.h) on torch CUDA tensors.
 
 Argument marshalling only: every step of the path runs in the library's CUDA
 kernels.  torch supplies device memory and streams.  There is no CPU fallback:
-importing this module without the built library raises.
+importing this module without the built library raises.  The library is loaded
+with ctypes; the entry points that are called per round or step are marshalled by
+the native module _qesgd_py (csrc/qesgd_py.cpp), because through ctypes a call with
+sixteen arguments costs more time than the GPU needs for a short vector.
 """
 import ctypes as C
 import os
@@ -67,6 +70,10 @@ for _name, (_res, _args) in SIGNATURES.items():
     _fn.restype = _res
     _fn.argtypes = _args
 
+from paper_1901_03040_b200 import _qesgd_py as _native      # noqa: E402  (built with the library)
+
+_native.bind({_name: C.cast(getattr(lib, _name), C.c_void_p).value for _name in SIGNATURES})
+
 
 class QesgdError(RuntimeError):
     def __init__(self, code, cuda_error=0):
@@ -84,10 +91,6 @@ def code_bytes(d, bucket, bits):
     return int(lib.qesgd_code_bytes(d, bucket, bits))
 
 
-def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
-
-
 class Context:
     """One qesgd_ctx: a device, a stream, a status word."""
 
@@ -101,12 +104,14 @@ class Context:
         if rc != OK:
             raise QesgdError(rc)
         self._h = handle
+        self._address = handle.value
         self.stream = stream
 
     def close(self):
         if getattr(self, "_h", None):
             lib.qesgd_destroy(self._h)
             self._h = None
+            self._address = 0
 
     def __del__(self):
         try:
@@ -131,61 +136,83 @@ class Context:
     # -- worker side ---------------------------------------------------------
     def qesgd_encode(self, local, anchor, d, bucket, s, bits, scale_mode, seed, worker, epoch,
                      codes_out, scales_out, fixed_delta=0.0):
-        self._check(lib.qesgd_encode(self._h, _ptr(local), _ptr(anchor), d, bucket, s, bits,
-                                     scale_mode, fixed_delta, seed, worker, epoch,
-                                     _ptr(codes_out), _ptr(scales_out)))
+        rc = _native.qesgd_encode(self._address, local, anchor, d, bucket, s, bits,
+                                  scale_mode, fixed_delta, seed, worker, epoch,
+                                  codes_out, scales_out)
+        if rc:
+            self._check(rc)
 
     def qesgd_encode_batch(self, local, local_stride, anchor, d, K, bucket, s, bits, scale_mode,
                            seed, worker0, epoch, codes_out, code_stride, scales_out, scale_stride,
                            fixed_delta=0.0):
-        self._check(lib.qesgd_encode_batch(self._h, _ptr(local), local_stride, _ptr(anchor), d, K,
-                                           bucket, s, bits, scale_mode, fixed_delta, seed, worker0,
-                                           epoch, _ptr(codes_out), code_stride, _ptr(scales_out),
-                                           scale_stride))
+        rc = _native.qesgd_encode_batch(self._address, local, local_stride, anchor, d, K,
+                                        bucket, s, bits, scale_mode, fixed_delta, seed, worker0,
+                                        epoch, codes_out, code_stride, scales_out,
+                                        scale_stride)
+        if rc:
+            self._check(rc)
 
     def qesgd_requantize(self, u, anchor, d, bucket, s, bits, scale_mode, seed, worker, step, zsum,
                          codes_out, scales_out, fixed_delta=0.0):
-        self._check(lib.qesgd_requantize(self._h, _ptr(u), _ptr(anchor), d, bucket, s, bits,
-                                         scale_mode, fixed_delta, seed, worker, step, _ptr(zsum),
-                                         _ptr(codes_out), _ptr(scales_out)))
+        rc = _native.qesgd_requantize(self._address, u, anchor, d, bucket, s, bits,
+                                      scale_mode, fixed_delta, seed, worker, step, zsum,
+                                      codes_out, scales_out)
+        if rc:
+            self._check(rc)
 
     def qesgd_lr_qesgd_step(self, Xb, yb, m, d, lr, u, anchor, bucket, s, bits, scale_mode, seed, worker,
                             step, zsum, codes_out, scales_out, fixed_delta=0.0):
-        self._check(lib.qesgd_lr_qesgd_step(self._h, _ptr(Xb), _ptr(yb), m, d, lr, _ptr(u), _ptr(anchor),
-                                            bucket, s, bits, scale_mode, fixed_delta, seed, worker, step,
-                                            _ptr(zsum), _ptr(codes_out), _ptr(scales_out)))
+        rc = _native.qesgd_lr_qesgd_step(self._address, Xb, yb, m, d, lr, u, anchor,
+                                         bucket, s, bits, scale_mode, fixed_delta, seed, worker, step,
+                                         zsum, codes_out, scales_out)
+        if rc:
+            self._check(rc)
 
     # -- server side ---------------------------------------------------------
     def qesgd_decode_average_apply(self, param, d, K, codes, code_stride, scales, scale_stride,
                                    bucket, s, bits):
-        self._check(lib.qesgd_decode_average_apply(self._h, _ptr(param), d, K, _ptr(codes),
-                                                   code_stride, _ptr(scales), scale_stride,
-                                                   bucket, s, bits))
+        rc = _native.qesgd_decode_average_apply(self._address, param, d, K, codes,
+                                                code_stride, scales, scale_stride,
+                                                bucket, s, bits)
+        if rc:
+            self._check(rc)
 
     def qesgd_decode_average_axpy(self, param, d, K, codes, code_stride, scales, scale_stride,
                                   bucket, s, bits, alpha):
-        self._check(lib.qesgd_decode_average_axpy(self._h, _ptr(param), d, K, _ptr(codes),
-                                                  code_stride, _ptr(scales), scale_stride,
-                                                  bucket, s, bits, alpha))
+        rc = _native.qesgd_decode_average_axpy(self._address, param, d, K, codes,
+                                               code_stride, scales, scale_stride,
+                                               bucket, s, bits, alpha)
+        if rc:
+            self._check(rc)
 
     def qesgd_decode(self, codes, scales, d, bucket, s, bits, out):
-        self._check(lib.qesgd_decode(self._h, _ptr(codes), _ptr(scales), d, bucket, s, bits,
-                                     _ptr(out)))
+        rc = _native.qesgd_decode(self._address, codes, scales, d, bucket, s, bits,
+                                  out)
+        if rc:
+            self._check(rc)
 
     # -- local epoch ---------------------------------------------------------
     def qesgd_lr_sgd_step(self, Xb, yb, m, d, lr, u):
-        self._check(lib.qesgd_lr_sgd_step(self._h, _ptr(Xb), _ptr(yb), m, d, lr, _ptr(u)))
+        rc = _native.qesgd_lr_sgd_step(self._address, Xb, yb, m, d, lr, u)
+        if rc:
+            self._check(rc)
 
     def qesgd_lr_gradient(self, Xb, yb, m, d, w, g_out):
-        self._check(lib.qesgd_lr_gradient(self._h, _ptr(Xb), _ptr(yb), m, d, _ptr(w), _ptr(g_out)))
+        rc = _native.qesgd_lr_gradient(self._address, Xb, yb, m, d, w, g_out)
+        if rc:
+            self._check(rc)
 
     def qesgd_lr_local_epoch(self, X, y, n_local, d, batch, lr, u):
-        self._check(lib.qesgd_lr_local_epoch(self._h, _ptr(X), _ptr(y), n_local, d, batch, lr,
-                                             _ptr(u)))
+        rc = _native.qesgd_lr_local_epoch(self._address, X, y, n_local, d, batch, lr,
+                                          u)
+        if rc:
+            self._check(rc)
 
     def qesgd_lr_local_epoch_batch(self, X, y, n_local, d, K, batch, lr, u, u_stride):
-        self._check(lib.qesgd_lr_local_epoch_batch(self._h, _ptr(X), _ptr(y), n_local, d, K, batch,
-                                                   lr, _ptr(u), u_stride))
+        rc = _native.qesgd_lr_local_epoch_batch(self._address, X, y, n_local, d, K, batch,
+                                                lr, u, u_stride)
+        if rc:
+            self._check(rc)
 
     # -- bookkeeping ---------------------------------------------------------
     def qesgd_status(self):
@@ -202,8 +229,7 @@ def qesgd_lr_sgd_step_noalloc(stream, Xb, yb, m, d, lr, u):
     allocation by the library: for callers that must not allocate device memory when
     they take the step (the scratch is a fixed 64 KB array inside the library; at most
     NOALLOC_MAX_LR_BATCH rows; calls must not overlap on the GPU)."""
-    rc = lib.qesgd_lr_sgd_step_noalloc(C.c_void_p(stream.cuda_stream if stream is not None else 0),
-                                       _ptr(Xb), _ptr(yb), m, d, lr, _ptr(u))
+    rc = _native.qesgd_lr_sgd_step_noalloc(stream.cuda_stream if stream is not None else 0, Xb, yb, m, d, lr, u)
     if rc != OK:
         raise QesgdError(rc)
 
