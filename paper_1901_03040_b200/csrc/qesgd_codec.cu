@@ -585,6 +585,7 @@ template <int BITS, int MODE, bool ANCHOR, bool VEC, int V, int WARPS, bool REQ>
 __global__ void __launch_bounds__(WARPS * 32, QESGD_ENCODE_MIN_WARPS / WARPS)
     qesgd_encode_kernel(const EncodeArgs a)
 {
+    qesgd_wait_for_previous();
     __shared__ EncodeShared sh;
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t warp = threadIdx.x >> 5;
@@ -723,6 +724,7 @@ __global__ void __launch_bounds__(QS_THREADS, QESGD_QS_CTAS) qesgd_lr_qstep_kern
     __shared__ float s_coef[QESGD_MAX_LR_BATCH];
     __shared__ EncodeShared sh;
     const EncodeArgs &a = q.e;
+    qesgd_wait_for_previous();
     for (uint32_t j = threadIdx.x; j < q.m; j += blockDim.x) {
         const float margin = q.margins[j];
         const float yj = __ldg(q.y + j);
@@ -815,6 +817,7 @@ __device__ __forceinline__ void load_codes(const uint8_t *__restrict__ codes, ui
 template <int BITS, bool VEC>
 __global__ void __launch_bounds__(256) qesgd_decode_kernel(const DecodeArgs a)
 {
+    qesgd_wait_for_previous();
     constexpr int OPT = QESGD_DECODE_OCTETS;
     const uint64_t nthreads = (uint64_t)gridDim.x * blockDim.x;
     const uint64_t t0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -936,6 +939,7 @@ template <int BITS, bool VEC, int W, int KS = 0>
 __global__ void __launch_bounds__(QESGD_DAA_THREADS, BITS == 4 ? QESGD_DAA_MIN_CTAS + 4 : QESGD_DAA_MIN_CTAS)
     qesgd_decode_average_apply_kernel(const DecodeArgs a)
 {
+    qesgd_wait_for_previous();
     const uint32_t K = KS ? (uint32_t)KS : a.K;
     constexpr int OPL = 8 / BITS;                 // octets per lane and chunk: 4, 2, 1
     constexpr int LANE_ELEMS = 8 * OPL;
@@ -1124,10 +1128,8 @@ cudaError_t launch_encode_w(const EncodeArgs &a, uint32_t K, cudaStream_t stream
     if (tiles == 0 || tiles * K > 0x7FFFFFFFull) return cudaErrorInvalidValue;
     dim3 grid((unsigned)(tiles * K), 1, 1), block(WARPS * 32u, 1, 1);
     if (ANCHOR && a.u_out)   // per-step QESGD: write back u = anchor + Q(z)
-        qesgd_encode_kernel<BITS, MODE, ANCHOR, VEC, V, WARPS, ANCHOR><<<grid, block, 0, stream>>>(a);
-    else
-        qesgd_encode_kernel<BITS, MODE, ANCHOR, VEC, V, WARPS, false><<<grid, block, 0, stream>>>(a);
-    return cudaGetLastError();
+        return qesgd_launch(qesgd_encode_kernel<BITS, MODE, ANCHOR, VEC, V, WARPS, ANCHOR>, grid, block, stream, a);
+    return qesgd_launch(qesgd_encode_kernel<BITS, MODE, ANCHOR, VEC, V, WARPS, false>, grid, block, stream, a);
 }
 
 template <int BITS, int MODE, bool ANCHOR, bool VEC>
@@ -1204,11 +1206,10 @@ int QESGD_CAT(qesgd_launch_lr_qstep_, QESGD_BITS)(const QstepArgs &a, uint32_t s
     if (tiles == 0 || tiles > 0x7FFFFFFFull) return (int)cudaErrorInvalidValue;
     dim3 grid((unsigned)tiles), block(QS_THREADS);
     switch (scale_mode) {
-        case QESGD_SCALE_NORM: qesgd_lr_qstep_kernel<QESGD_BITS, 0><<<grid, block, 0, stream>>>(a); break;
-        case QESGD_SCALE_MAX: qesgd_lr_qstep_kernel<QESGD_BITS, 1><<<grid, block, 0, stream>>>(a); break;
-        default: qesgd_lr_qstep_kernel<QESGD_BITS, 2><<<grid, block, 0, stream>>>(a); break;
+        case QESGD_SCALE_NORM: return (int)qesgd_launch(qesgd_lr_qstep_kernel<QESGD_BITS, 0>, grid, block, stream, a);
+        case QESGD_SCALE_MAX: return (int)qesgd_launch(qesgd_lr_qstep_kernel<QESGD_BITS, 1>, grid, block, stream, a);
+        default: return (int)qesgd_launch(qesgd_lr_qstep_kernel<QESGD_BITS, 2>, grid, block, stream, a);
     }
-    return (int)cudaGetLastError();
 }
 
 int QESGD_CAT(qesgd_launch_decode_, QESGD_BITS)(const DecodeArgs &a, bool vec, cudaStream_t stream)
@@ -1217,9 +1218,8 @@ int QESGD_CAT(qesgd_launch_decode_, QESGD_BITS)(const DecodeArgs &a, bool vec, c
     const uint64_t blocks = (octets + 256 * QESGD_DECODE_OCTETS - 1) / (256 * QESGD_DECODE_OCTETS);
     if (blocks == 0 || blocks > 0x7FFFFFFFull) return (int)cudaErrorInvalidValue;
     dim3 grid((unsigned)blocks), block(256);
-    if (vec) qesgd_decode_kernel<QESGD_BITS, true><<<grid, block, 0, stream>>>(a);
-    else qesgd_decode_kernel<QESGD_BITS, false><<<grid, block, 0, stream>>>(a);
-    return (int)cudaGetLastError();
+    return (int)(vec ? qesgd_launch(qesgd_decode_kernel<QESGD_BITS, true>, grid, block, stream, a)
+                     : qesgd_launch(qesgd_decode_kernel<QESGD_BITS, false>, grid, block, stream, a));
 }
 
 int QESGD_CAT(qesgd_launch_decode_average_apply_, QESGD_BITS)(const DecodeArgs &a, bool vec,
@@ -1232,13 +1232,16 @@ int QESGD_CAT(qesgd_launch_decode_average_apply_, QESGD_BITS)(const DecodeArgs &
     const uint64_t blocks = (warps + wpc - 1) / wpc;
     if (blocks == 0 || blocks > 0x7FFFFFFFull) return (int)cudaErrorInvalidValue;
     dim3 grid((unsigned)blocks), block(QESGD_DAA_THREADS);
+    void (*kernel)(DecodeArgs);
     if (vec && a.K == 8)
-        qesgd_decode_average_apply_kernel<QESGD_BITS, true, W, 8><<<grid, block, 0, stream>>>(a);
+        kernel = qesgd_decode_average_apply_kernel<QESGD_BITS, true, W, 8>;
     else if (vec && QESGD_BITS != 2 && a.K == 4)
-        qesgd_decode_average_apply_kernel<QESGD_BITS, true, W, (QESGD_BITS != 2 ? 4 : 0)><<<grid, block, 0, stream>>>(a);
+        kernel = qesgd_decode_average_apply_kernel<QESGD_BITS, true, W, (QESGD_BITS != 2 ? 4 : 0)>;
     else if (vec && QESGD_BITS != 4 && a.K == 16)
-        qesgd_decode_average_apply_kernel<QESGD_BITS, true, W, (QESGD_BITS != 4 ? 16 : 0)><<<grid, block, 0, stream>>>(a);
-    else if (vec) qesgd_decode_average_apply_kernel<QESGD_BITS, true, W><<<grid, block, 0, stream>>>(a);
-    else qesgd_decode_average_apply_kernel<QESGD_BITS, false, W><<<grid, block, 0, stream>>>(a);
-    return (int)cudaGetLastError();
+        kernel = qesgd_decode_average_apply_kernel<QESGD_BITS, true, W, (QESGD_BITS != 4 ? 16 : 0)>;
+    else if (vec)
+        kernel = qesgd_decode_average_apply_kernel<QESGD_BITS, true, W>;
+    else
+        kernel = qesgd_decode_average_apply_kernel<QESGD_BITS, false, W>;
+    return (int)qesgd_launch(kernel, grid, block, stream, a);
 }

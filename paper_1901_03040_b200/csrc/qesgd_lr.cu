@@ -52,6 +52,7 @@ template <bool VEC>
 __global__ void __launch_bounds__(256) qesgd_lr_margin_kernel(const LrArgs a)
 {
     __shared__ float s_part[QESGD_MAX_LR_BATCH];
+    qesgd_wait_for_previous();
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     const uint32_t k = blockIdx.y, p = blockIdx.x, rg = blockIdx.z;
     const float *__restrict__ X = a.X + (uint64_t)k * a.x_stride;
@@ -164,6 +165,7 @@ __global__ void __launch_bounds__(UPD_THREADS) qesgd_lr_update_kernel(const LrAr
 {
     __shared__ float s_coef[QESGD_MAX_LR_BATCH];
     __shared__ float4 s_sum[UPD_ROWGROUPS][UPD_COLS / 4];
+    qesgd_wait_for_previous();
     const uint32_t k = blockIdx.y;
     const float *__restrict__ X = a.X + (uint64_t)k * a.x_stride;
     const float *__restrict__ y = a.y + (uint64_t)k * a.y_stride;
@@ -275,22 +277,19 @@ int launch_lr_passes(const float *Xb, uint64_t x_worker_stride, const float *yb,
     const bool vec = (d % 4 == 0) && (x_worker_stride % 4 == 0) && (u_stride % 4 == 0) &&
                      (((uintptr_t)Xb | (uintptr_t)u | (uintptr_t)dst) % 16 == 0);
     dim3 g1((unsigned)parts, K, a.row_groups), b1(256);
-    if (vec) qesgd_lr_margin_kernel<true><<<g1, b1, 0, stream>>>(a);
-    else qesgd_lr_margin_kernel<false><<<g1, b1, 0, stream>>>(a);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = vec ? qesgd_launch(qesgd_lr_margin_kernel<true>, g1, b1, stream, a)
+                        : qesgd_launch(qesgd_lr_margin_kernel<false>, g1, b1, stream, a);
     if (e != cudaSuccess) return (int)e;
     *launched = 1;
     const uint64_t ublocks = (d + UPD_COLS - 1) / UPD_COLS;
     if (ublocks > 0x7FFFFFFFull) return (int)cudaErrorInvalidValue;
     dim3 g2((unsigned)ublocks, K), b2(UPD_THREADS);
-    if (qesgd_second_pass_reversed((uint64_t)K * m, d)) {
-        if (vec) qesgd_lr_update_kernel<true, true><<<g2, b2, 0, stream>>>(a);
-        else qesgd_lr_update_kernel<false, true><<<g2, b2, 0, stream>>>(a);
-    } else {
-        if (vec) qesgd_lr_update_kernel<true, false><<<g2, b2, 0, stream>>>(a);
-        else qesgd_lr_update_kernel<false, false><<<g2, b2, 0, stream>>>(a);
-    }
-    e = cudaGetLastError();
+    void (*update)(LrArgs);
+    if (qesgd_second_pass_reversed((uint64_t)K * m, d))
+        update = vec ? qesgd_lr_update_kernel<true, true> : qesgd_lr_update_kernel<false, true>;
+    else
+        update = vec ? qesgd_lr_update_kernel<true, false> : qesgd_lr_update_kernel<false, false>;
+    e = qesgd_launch(update, g2, b2, stream, a);
     if (e == cudaSuccess) *launched = 2;
     return (int)e;
 }
@@ -312,10 +311,9 @@ int qesgd_launch_lr_margins(const float *Xb, const float *yb, uint32_t m, uint64
     a.nseg = (uint32_t)nseg;
     const bool vec = (d % 4 == 0) && (((uintptr_t)Xb | (uintptr_t)u) % 16 == 0);
     dim3 g1((unsigned)parts, 1, a.row_groups), b1(256);
-    if (vec) qesgd_lr_margin_kernel<true><<<g1, b1, 0, stream>>>(a);
-    else qesgd_lr_margin_kernel<false><<<g1, b1, 0, stream>>>(a);
     *margins_out = a.margins;
-    return (int)cudaGetLastError();
+    return (int)(vec ? qesgd_launch(qesgd_lr_margin_kernel<true>, g1, b1, stream, a)
+                     : qesgd_launch(qesgd_lr_margin_kernel<false>, g1, b1, stream, a));
 }
 
 int qesgd_launch_lr_step(const float *Xb, uint64_t x_worker_stride, const float *yb,

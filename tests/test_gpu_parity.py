@@ -800,6 +800,46 @@ def test_invalid_arguments_return_einval_and_launch_nothing():
     assert c.qesgd_status() == 0
 
 
+# ------------------------------------------------ ordering of dependent calls ----
+@pytest.mark.parametrize("K,d,bucket,bits,s", [(3, 5000, 64, 4, 7), (2, 300_001, 2048, 8, 127)])
+def test_calls_in_a_row_see_one_another_and_other_kernels_of_the_stream(K, d, bucket, bits, s):
+    """Kernels are set up while the one before still drains and wait for it before they touch memory.
+    Thirty rounds, each call reading what the one before wrote (the library's and torch's kernels in
+    turn, small grids that overlap most), give what the same calls give when each is waited for."""
+    c = G.ctx()
+    m = 8
+    X, y, _ = synthetic.logistic_problem(m, d, seed=5)
+    tX, ty = G.dev(X), G.dev(y)
+    w0 = G.dev(synthetic.anchor_vector(d, seed=6))
+    stride = (d + 7) // 8 * 8
+
+    def rounds(wait):
+        sync = torch.cuda.synchronize if wait else (lambda: None)
+        param, loc = w0.clone(), torch.zeros((K, stride), device="cuda")
+        u, z, out = w0.clone(), torch.zeros(d, device="cuda"), torch.zeros(d, device="cuda")
+        codes, scales = qesgd.alloc_stream_buffers(K, d, bucket, bits, "cuda")
+        torch.cuda.synchronize()
+        for r in range(30):
+            loc[:, :d] = param * 0.75 + out
+            sync()
+            c.qesgd_encode_batch(loc, stride, param, d, K, bucket, s, bits, qesgd.SCALE_MAX, 3, 0, r, codes,
+                                 codes.stride(0), scales, scales.stride(0))
+            sync()
+            c.qesgd_decode_average_apply(param, d, K, codes, codes.stride(0), scales, scales.stride(0), bucket, s, bits)
+            sync()
+            c.qesgd_decode(codes[1], scales[1], d, bucket, s, bits, out)
+            sync()
+            c.qesgd_lr_sgd_step(tX, ty, m, d, 0.1, u)
+            sync()
+            c.qesgd_requantize(u, param, d, bucket, s, bits, qesgd.SCALE_MAX, 3, 0, r, z, codes[0], scales[0])
+            sync()
+        torch.cuda.synchronize()
+        return param, u, z, out, codes, scales
+    for a, b in zip(rounds(True), rounds(False)):
+        assert torch.equal(a, b)
+    assert c.qesgd_status() == 0
+
+
 # ----------------------------------------------------------- graph replay ----
 def test_round_recorded_into_a_cuda_graph_replays_bit_identically():
     """The codec calls only enqueue kernels on the context's stream, so a round (encode of all
