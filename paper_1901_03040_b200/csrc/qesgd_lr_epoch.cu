@@ -21,8 +21,11 @@
 //                   their slots in step, right after the exchange, and refilled at once by all of them
 //                   the copies of one SM queue behind another's, the slowest of which everybody then
 //                   waits for.  At 0.6 of the interval at which HBM can serve every SM the first
-//                   shape takes 324 us, the HBM time of X (349 without a pause; 330 at 0.5, 347 at 0.7,
-//                   381 at 0.8); K = 8, n = 512, d = 65536: 183 -> 169
+//                   shape takes 330 us, the HBM time of X (349 without a pause; 330 at 0.5, 347 at 0.7,
+//                   381 at 0.8); K = 8, n = 512, d = 65536: 183 -> 169.  The pause is kept by the global
+//                   timer (32 ns a tick), not in clocks: under the power cap the SM clock falls by a
+//                   quarter, and a pause that grew with it would hold HBM back (a round of the first
+//                   shape, repeated for a second: 381 us by clocks, 373 by the timer, 377 without a pause)
 //   consumer chain  eight warps; tile i = minibatch i / Kg of the group's worker i % Kg:
 //     M(i)  warp w takes the sub-tiles w, w + 8, ...: partial margins of the rows over the slice;
 //           the values it reads go to tensor memory on the way (tcgen05.st), so the slot returns
@@ -92,7 +95,7 @@ constexpr int EP_BOX_COLS = 256;     // widest TMA box
 constexpr int EP_MAX_M = EP_CHAIN;   // rows per minibatch: a thread of the chain per row
 constexpr int EP_MAX_SLOTS = 64;     // ring slots
 constexpr uint32_t EP_FLAG_BYTES = (16 + EP_MAX_SLOTS) * 4;
-constexpr float EP_HBM_BYTES_PER_CLK = 3400.0f;      // 6.55 TB/s at 1.93 GHz
+constexpr float EP_HBM_BYTES_PER_NS = 6550.0f;
 constexpr int EP_PRODUCERS = 2;      // producer warps
 constexpr int EP_UNITS = 8;          // 8 x 128 blocks of a tile that the tensor memory holds per warp
 constexpr float EP_CHAIN_US = 2.5f, EP_UNIT_US = 0.25f;   // a tile's latency: exchange, and per block of a warp
@@ -119,7 +122,7 @@ struct EpochArgs {
     uint32_t nsub_max, nsub_last;
     uint32_t cols, nit;     // columns per CTA (a multiple of 4), blocks of 128 columns
     uint32_t nslots;        // sub-tiles the ring holds
-    uint32_t pace;          // clocks between two copies of a producer, at least
+    uint32_t pace;          // ns between two copies of a producer, at least
     uint32_t off_u, off_part, off_coef, off_bars, off_flags;   // shared-memory layout, bytes
     float rate, rate_last;  // lr / rows of a minibatch, of the last one (lr = -1 for the mean gradient)
     const float *u;         // where the epoch starts
@@ -398,7 +401,7 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + EP_PRODUCERS * 32, 1)
             uint32_t i = 0u, s = p, slot = p, turn = 0u;
             Tile T;
             T.start(a);
-            uint32_t issued = (uint32_t)clock() - a.pace;
+            uint32_t issued = (uint32_t)now_ns() - a.pace;
             for (;;) {
                 while (s >= T.nsub && i < ntiles) {
                     s -= T.nsub;
@@ -406,7 +409,7 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + EP_PRODUCERS * 32, 1)
                     ++i;
                 }
                 if (i >= ntiles) break;
-                while ((uint32_t)clock() - issued < a.pace) __nanosleep(20);
+                while ((uint32_t)now_ns() - issued < a.pace) __nanosleep(20);
                 // the slot's previous sub-tile has been taken
                 if (turn != 0u && !mbar_wait(&empty[slot], (turn - 1u) & 1u, &s_flag[0], a.wait_ns)) {
                     s_flag[0] = 1u;
@@ -415,7 +418,7 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + EP_PRODUCERS * 32, 1)
                 }
                 const uint32_t row = (uint32_t)((uint64_t)(grp + T.kk * a.G) * a.n_local + (uint64_t)T.t * a.batch) + s * SUB;
                 float *dst = ring + (size_t)slot * slot_floats;
-                issued = (uint32_t)clock();
+                issued = (uint32_t)now_ns();
                 mbar_arrive_expect_tx(&full[slot], slot_floats * 4u);
                 uint32_t c = 0u;
                 for (; c + EP_BOX_COLS <= a.cols; c += EP_BOX_COLS, dst += SUB * EP_BOX_COLS)
@@ -855,7 +858,7 @@ int qesgd_launch_lr_epoch_fused(const float *X, const float *y, uint64_t n_local
     // One group with one chain is late for the next tile whenever it was for this one, and gains from
     // copies spread a little wider (K = 4, n = 512, d = 131072: 260 us without a pace, 256 at 0.6, 245 at
     // 0.8, 248 at 1.0); all others are best at 0.6 (see the head of the file).
-    a.pace = (uint32_t)((s.G == 1u && s.NC == 1u ? 0.8f : 0.6f) * (float)(SUB * s.cols * 4u * EP_PRODUCERS) * (float)(s.G * s.P) / EP_HBM_BYTES_PER_CLK);
+    a.pace = (uint32_t)((s.G == 1u && s.NC == 1u ? 0.8f : 0.6f) * (float)(SUB * s.cols * 4u * EP_PRODUCERS) * (float)(s.G * s.P) / EP_HBM_BYTES_PER_NS);
     a.rate = lr / (float)m_full;
     a.rate_last = lr / (float)a.m_last;
     a.u = u; a.dst = dst; a.gradient = gradient ? 1u : 0u; a.u_stride = u_stride;
