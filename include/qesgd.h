@@ -214,12 +214,13 @@ int qesgd_lr_local_epoch(qesgd_ctx *ctx, const float *X, const float *y, uint64_
                          uint64_t d, uint32_t batch, float lr, float *u);
 /* K workers side by side: worker k owns rows [k*n_local, (k+1)*n_local) of X and
  * y and updates u + k*u_stride (elements).
- * Where the shape allows (d a multiple of 4, minibatches of at most 256 rows whose slices fit the
- * SMs' tensor memory -- 64 rows of 1024 columns per SM, 128 of 512, 256 of 256 --, X and u 16-byte
- * aligned, u_stride a multiple of 4) the whole epoch of all K workers is ONE persistent kernel,
- * launched cooperatively with at most one CTA per SM, that stages every minibatch in shared memory
- * by TMA and reads X from HBM once.  Its CTAs form groups that share the workers out; the CTAs of a
- * group own a slice of the columns each, and the
+ * Where the shape allows (minibatches of at most 256 rows whose slices fit the SMs' tensor memory --
+ * 64 rows of 1024 columns per SM, 128 of 512, 256 of 256) the whole epoch of all K workers is ONE
+ * persistent kernel, launched cooperatively with at most one CTA per SM, that stages every minibatch
+ * in shared memory and reads X from HBM once: by TMA where d and u_stride are multiples of 4 and X
+ * and u are 16-byte aligned, else by copies of one or two elements (about twice the time for large
+ * minibatches).  Its CTAs form groups that share the workers out; the CTAs of a group own a slice of
+ * the columns each, and the
  * CTAs exchange partial margins through the context's workspace, which the kernel leaves
  * cleared.  The partial margins of a row are summed across the CTAs as fixed-point integers
  * (units of 2^-28 below 2^17 in magnitude, units of 2^-6 from there to 2^49), so the sum

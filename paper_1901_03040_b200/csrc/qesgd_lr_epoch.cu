@@ -96,7 +96,8 @@ constexpr int EP_MAX_M = EP_CHAIN;   // rows per minibatch: a thread of the chai
 constexpr int EP_MAX_SLOTS = 64;     // ring slots
 constexpr uint32_t EP_FLAG_BYTES = (16 + EP_MAX_SLOTS) * 4;
 constexpr float EP_HBM_BYTES_PER_NS = 6550.0f;
-constexpr int EP_PRODUCERS = 2;      // producer warps
+constexpr int EP_PRODUCERS = 2;      // producer warps with TMA
+constexpr int EP_LOADERS = 8;        // producer warps with element-wise copies
 constexpr int EP_UNITS = 8;          // 8 x 128 blocks of a tile that the tensor memory holds per warp
 constexpr float EP_CHAIN_US = 2.5f, EP_UNIT_US = 0.25f;   // a tile's latency: exchange, and per block of a warp
 constexpr uint64_t DRAIN_LIMIT_NS = 2000000000ull;   // the producers' last wait for their own copies
@@ -113,6 +114,7 @@ constexpr unsigned long long FX_ONE = 1ull << 55;    // one contribution counted
 constexpr unsigned long long FX_SPECIAL = 1ull << 54;   // one of the row's other words is in use
 
 struct EpochArgs {
+    const float *X;         // element-wise copies only
     const float *y;
     uint64_t n_local;       // rows per worker
     uint64_t d;
@@ -295,6 +297,21 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float4 (&v)[8])
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
+// EB bytes from global to shared memory, asynchronously; zeros where `inside` does not hold (then
+// nothing is read).
+template <int EB>
+__device__ __forceinline__ void copy_elements(uint32_t dst, const float *src, bool inside)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(src), "n"(EB == 8 ? 8 : 4),
+                 "r"(inside ? (EB == 8 ? 8 : 4) : 0)
+                 : "memory");
+}
+// One arrival on the barrier when all copies of this thread so far have landed.
+__device__ __forceinline__ void arrive_when_copied(uint64_t *bar)
+{
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
 // Sum over the 32 lanes of 8 per-lane values at once: three halving exchanges leave one
 // value per lane, two plain butterflies finish.  Lane L ends with the total of value
 // 4*bit4(L) + 2*bit3(L) + bit2(L); the order of the additions is fixed.
@@ -356,11 +373,19 @@ extern __shared__ __align__(1024) unsigned char ep_smem[];
 // Shared memory: the ring of slots of SUB x cols floats (a slot holds its boxes of 256 columns one
 // after the other, the last one narrower), the slices of u of the group's workers, the warps'
 // partial updates, the step coefficients, the barriers, a few flag words.
-template <int NC>
-__global__ void __launch_bounds__(NC * EP_CHAIN + EP_PRODUCERS * 32, 1)
+// EB = 16: rows of X start on 16-byte boundaries and TMA fetches them.  EB = 4 or 8: they do not (d no
+// multiple of 4, or unaligned vectors); eight producer warps copy 4 or 8 bytes at a time instead
+// (cp.async, completion on the same barriers, elements outside the matrix as zeros) and u is read and
+// written element by element.  One chain.  Bound by the copies' instructions (128 or 256 bytes each),
+// but against two passes of scalar loads per minibatch: K = 4, n = 512, d = 16383: 196 -> 45 us; K = 8,
+// n = 1010, d = 10001: 461 -> 132; one minibatch of 64 x 65537: 22 -> 11.5; K = 4, n = 2048, d = 65538:
+// 1168 -> 696.
+template <int NC, int EB>
+__global__ void __launch_bounds__(NC * EP_CHAIN + (EB == 16 ? EP_PRODUCERS : EP_LOADERS) * 32, 1)
     qesgd_lr_epoch_kernel(const EpochArgs a, const __grid_constant__ CUtensorMap map_full,
                           const __grid_constant__ CUtensorMap map_rest)
 {
+    constexpr uint32_t PRODUCERS = EB == 16 ? EP_PRODUCERS : EP_LOADERS;
     const uint32_t slot_floats = SUB * a.cols, ucols = a.nit * 128u;
     float *const ring = reinterpret_cast<float *>(ep_smem);
     float *const s_u = reinterpret_cast<float *>(ep_smem + a.off_u);
@@ -380,7 +405,7 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + EP_PRODUCERS * 32, 1)
     const uint32_t ntiles = a.nsteps * kg;
 
     if (tid < 2u * a.nslots) {
-        mbar_init(&full[tid], 1u);
+        mbar_init(&full[tid], EB == 16 || tid >= a.nslots ? 1u : 32u);   // element-wise: every lane of the loader
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (tid < 16u + EP_MAX_SLOTS) s_flag[tid] = 0u;
@@ -397,7 +422,7 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + EP_PRODUCERS * 32, 1)
         // the slots p, p + EP_PRODUCERS, ... and each of them turn by turn: a slot that several warps
         // refilled could be looked at two turns early, where a barrier's parity reads the same.
         const uint32_t p = warp - NC * EP_WARPS;
-        if (lane == 0 && p < a.nslots) {
+        if ((EB != 16 || lane == 0) && p < a.nslots) {
             uint32_t i = 0u, s = p, slot = p, turn = 0u;
             Tile T;
             T.start(a);
@@ -409,25 +434,44 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + EP_PRODUCERS * 32, 1)
                     ++i;
                 }
                 if (i >= ntiles) break;
-                while ((uint32_t)now_ns() - issued < a.pace) __nanosleep(20);
+                while (EB == 16 && (uint32_t)now_ns() - issued < a.pace) __nanosleep(20);
                 // the slot's previous sub-tile has been taken
-                if (turn != 0u && !mbar_wait(&empty[slot], (turn - 1u) & 1u, &s_flag[0], a.wait_ns)) {
+                bool ok = turn == 0u || mbar_wait(&empty[slot], (turn - 1u) & 1u, &s_flag[0], a.wait_ns);
+                if (EB != 16) ok = __all_sync(0xFFFFFFFFu, ok) != 0;
+                if (!ok) {
                     s_flag[0] = 1u;
                     atomicOr(a.status, QESGD_STATUS_TIMEOUT);
                     break;
                 }
                 const uint32_t row = (uint32_t)((uint64_t)(grp + T.kk * a.G) * a.n_local + (uint64_t)T.t * a.batch) + s * SUB;
                 float *dst = ring + (size_t)slot * slot_floats;
-                issued = (uint32_t)now_ns();
-                mbar_arrive_expect_tx(&full[slot], slot_floats * 4u);
-                uint32_t c = 0u;
-                for (; c + EP_BOX_COLS <= a.cols; c += EP_BOX_COLS, dst += SUB * EP_BOX_COLS)
-                    tma_load_box(dst, &map_full, c0 + c, row, &full[slot]);
-                if (c < a.cols) tma_load_box(dst, &map_rest, c0 + c, row, &full[slot]);
-                s_turn[slot] = turn + 1u;
-                if (slot + EP_PRODUCERS < a.nslots) {
-                    slot += EP_PRODUCERS;
-                    s += EP_PRODUCERS;
+                if (EB == 16) {
+                    issued = (uint32_t)now_ns();
+                    mbar_arrive_expect_tx(&full[slot], slot_floats * 4u);
+                    uint32_t c = 0u;
+                    for (; c + EP_BOX_COLS <= a.cols; c += EP_BOX_COLS, dst += SUB * EP_BOX_COLS)
+                        tma_load_box(dst, &map_full, c0 + c, row, &full[slot]);
+                    if (c < a.cols) tma_load_box(dst, &map_rest, c0 + c, row, &full[slot]);
+                } else {
+                    constexpr uint32_t N = EB / 4;
+                    const uint32_t rows = min(T.m - s * SUB, (uint32_t)SUB);
+                    const float *const src = a.X + (uint64_t)row * a.d + c0;
+                    for (uint32_t b0 = 0u; b0 < a.cols; b0 += EP_BOX_COLS) {
+                        const uint32_t width = min(a.cols - b0, (uint32_t)EP_BOX_COLS);
+                        for (uint32_t r = 0; r < rows; ++r) {
+                            const float *const line = src + (uint64_t)r * a.d + b0;
+                            const uint32_t to = smem_u32(dst + SUB * b0 + r * width);
+#pragma unroll 4
+                            for (uint32_t c = lane * N; c < width; c += 32u * N)
+                                copy_elements<EB>(to + c * 4u, line + c, (uint64_t)c0 + b0 + c < a.d);
+                        }
+                    }
+                    arrive_when_copied(&full[slot]);
+                }
+                if (lane == 0) s_turn[slot] = turn + 1u;
+                if (slot + PRODUCERS < a.nslots) {
+                    slot += PRODUCERS;
+                    s += PRODUCERS;
                 } else {
                     s += a.nslots - slot + p;
                     slot = p;
@@ -440,7 +484,7 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + EP_PRODUCERS * 32, 1)
         // landed) or is waited for here, so that the CTA does not end -- and its shared memory
         // is not handed to another CTA -- while a copy is still writing it.  After a normal
         // epoch these waits end with the consumers' last tiles.
-        for (uint32_t q = p + EP_PRODUCERS * lane; q < a.nslots; q += EP_PRODUCERS * 32u)
+        for (uint32_t q = p + PRODUCERS * lane; q < a.nslots; q += PRODUCERS * 32u)
             if (s_turn[q] != 0u) mbar_wait(&full[q], (s_turn[q] - 1u) & 1u, &s_flag[3], DRAIN_LIMIT_NS);
         // The first producer warp then waits until the chains have read their last margins and counts
         // the CTA, while they update for the last time.  Counted last of the group: nobody adds or
@@ -488,10 +532,18 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + EP_PRODUCERS * 32, 1)
     // the slices of u of the group's workers, zeros past the slice
     for (uint32_t q = tid; q < kg * (ucols / 4u); q += NC * EP_CHAIN) {
         const uint32_t kk = q / (ucols / 4u), c = (q - kk * (ucols / 4u)) * 4u;
-        const bool in = c < a.cols && (uint64_t)c0 + c < a.d;
-        reinterpret_cast<float4 *>(s_u)[q] =
-            in ? *reinterpret_cast<const float4 *>(a.u + (uint64_t)(grp + kk * a.G) * a.u_stride + c0 + c)
-               : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float *const from = a.u + (uint64_t)(grp + kk * a.G) * a.u_stride + c0 + c;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (EB == 16) {
+            if (c < a.cols && (uint64_t)c0 + c < a.d) v = *reinterpret_cast<const float4 *>(from);
+        } else if (c < a.cols) {
+            const uint64_t left = (uint64_t)c0 + c < a.d ? a.d - c0 - c : 0u;
+            if (left > 0u) v.x = from[0];
+            if (left > 1u) v.y = from[1];
+            if (left > 2u) v.z = from[2];
+            if (left > 3u) v.w = from[3];
+        }
+        reinterpret_cast<float4 *>(s_u)[q] = v;
     }
     asm volatile("bar.sync 3, %0;" ::"n"(NC * EP_CHAIN) : "memory");
 
@@ -691,8 +743,18 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + EP_PRODUCERS * 32, 1)
             }
             t.x += o.x; t.y += o.y; t.z += o.z; t.w += o.w;
             *reinterpret_cast<float4 *>(us + c) = t;
-            if (T.t == a.nsteps - 1u && c < a.cols && (uint64_t)c0 + c < a.d)   // the worker's last minibatch
-                *reinterpret_cast<float4 *>(a.dst + (uint64_t)worker * a.u_stride + c0 + c) = t;
+            if (T.t == a.nsteps - 1u && c < a.cols && (uint64_t)c0 + c < a.d) {   // the worker's last minibatch
+                float *const to = a.dst + (uint64_t)worker * a.u_stride + c0 + c;
+                if (EB == 16) {
+                    *reinterpret_cast<float4 *>(to) = t;
+                } else {
+                    const uint64_t have = a.d - c0 - c;
+                    to[0] = t.x;
+                    if (have > 1u) to[1] = t.y;
+                    if (have > 2u) to[2] = t.z;
+                    if (have > 3u) to[3] = t.w;
+                }
+            }
         }
         chain_sync();                                     // u complete for the next minibatch
         if (NC == 2 && tg == 0) {
@@ -717,6 +779,10 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
                                   CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
                                   CUtensorMapFloatOOBfill);
 
+// one and two chains with TMA, one chain with copies of 8 and 4 bytes
+const void *const EPOCH_KERNELS[4] = {(const void *)qesgd_lr_epoch_kernel<1, 16>, (const void *)qesgd_lr_epoch_kernel<2, 16>,
+                                      (const void *)qesgd_lr_epoch_kernel<1, 8>, (const void *)qesgd_lr_epoch_kernel<1, 4>};
+
 // Per-device set-up: shared-memory limit of the kernels, the driver's tensor-map encoder.
 constexpr int MAX_DEVICES = 64;
 std::mutex g_epoch_mutex;
@@ -732,10 +798,9 @@ int epoch_smem_limit(int device)
         cudaError_t e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device);
         if (e == cudaSuccess)
             e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
-        if (e == cudaSuccess && coop && optin > 0)
-            e = cudaFuncSetAttribute(qesgd_lr_epoch_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
-        if (e == cudaSuccess && coop && optin > 0)
-            e = cudaFuncSetAttribute(qesgd_lr_epoch_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+        for (const void *kernel : EPOCH_KERNELS)
+            if (e == cudaSuccess && coop && optin > 0)
+                e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
         if (e == cudaSuccess && !g_encode_tiled) {
             void *fn = nullptr;
             cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
@@ -771,7 +836,7 @@ struct Split {
 };
 
 // Fills in the rest of a split with G groups and P CTAs each; false where it does not fit.
-bool complete_split(Split &s, uint64_t d, uint32_t K, uint32_t m, uint32_t nsub, uint32_t limit)
+bool complete_split(Split &s, uint64_t d, uint32_t K, uint32_t m, uint32_t nsub, bool tma, uint32_t limit)
 {
     const uint64_t cols = ((d + s.P - 1) / s.P + 3) / 4 * 4;
     if (cols > 1024) return false;
@@ -781,7 +846,7 @@ bool complete_split(Split &s, uint64_t d, uint32_t K, uint32_t m, uint32_t nsub,
     const uint32_t kg = (K + s.G - 1u) / s.G;
     const uint32_t units = (nsub + EP_WARPS - 1u) / EP_WARPS * s.nit;    // tensor-memory blocks per warp
     if (units > (uint32_t)EP_UNITS) return false;
-    s.NC = kg >= 2u && units <= (uint32_t)EP_UNITS / 2u ? 2u : 1u;
+    s.NC = tma && kg >= 2u && units <= (uint32_t)EP_UNITS / 2u ? 2u : 1u;
     const uint32_t slot = SUB * s.cols * 4u, ubytes = s.nit * 512u;
     const uint32_t fixed = kg * ubytes + s.NC * EP_WARPS * ubytes + s.NC * EP_MAX_M * 4u + 2u * EP_MAX_SLOTS * 8u + EP_FLAG_BYTES;
     if (fixed + 2u * slot > limit) return false;
@@ -801,7 +866,8 @@ bool complete_split(Split &s, uint64_t d, uint32_t K, uint32_t m, uint32_t nsub,
 }
 
 // The modelled time picks the split; ties go to fewer groups.
-bool choose_split(Split &best, uint64_t d, uint32_t K, uint32_t m, uint32_t nsub, uint32_t sm_count, uint32_t limit)
+bool choose_split(Split &best, uint64_t d, uint32_t K, uint32_t m, uint32_t nsub, bool tma, uint32_t sm_count,
+                  uint32_t limit)
 {
     bool any = false;
     for (uint32_t G = 1; G <= K && G <= sm_count; ++G) {
@@ -812,7 +878,7 @@ bool choose_split(Split &best, uint64_t d, uint32_t K, uint32_t m, uint32_t nsub
         s.P = sm_count / G;
         const uint64_t most = (d + 127u) / 128u;              // a warp takes 128 columns at a time
         if (s.P > most) s.P = (uint32_t)most;
-        if (!complete_split(s, d, K, m, nsub, limit)) continue;
+        if (!complete_split(s, d, K, m, nsub, tma, limit)) continue;
         if (!any || s.us < 0.99f * best.us) best = s;
         any = true;
     }
@@ -837,17 +903,18 @@ int qesgd_launch_lr_epoch_fused(const float *X, const float *y, uint64_t n_local
     const uint64_t nsteps64 = (n_local + m_full - 1) / m_full;
     if (nsteps64 * K > (1u << 20)) return -1;
     if ((uint64_t)K * n_local + EP_MAX_M >= (1ull << 31)) return -1;   // TMA row coordinates
-    if (d % 4 != 0 || u_stride % 4 != 0 || ((uintptr_t)X | (uintptr_t)u | (uintptr_t)dst) % 16 != 0) return -1;
+    const bool tma = d % 4 == 0 && u_stride % 4 == 0 && ((uintptr_t)X | (uintptr_t)u | (uintptr_t)dst) % 16 == 0;
+    const bool pairs = d % 2 == 0 && (uintptr_t)X % 8 == 0;
     if (sm_count < 1 || d > 1024ull * (uint64_t)sm_count) return -1;
     const int limit = epoch_smem_limit(device);
     if (limit <= 0) return -1;
     const uint32_t nsub = (m_full + SUB - 1) / SUB;
     Split s;
     // the accumulator word counts up to 256 contributions
-    if (!choose_split(s, d, K, m_full, nsub, (uint32_t)(sm_count < 256 ? sm_count : 256), (uint32_t)limit)) return -1;
+    if (!choose_split(s, d, K, m_full, nsub, tma, (uint32_t)(sm_count < 256 ? sm_count : 256), (uint32_t)limit)) return -1;
 
     EpochArgs a;
-    a.y = y; a.n_local = n_local;
+    a.X = X; a.y = y; a.n_local = n_local;
     a.d = d; a.K = K; a.G = s.G; a.P = s.P;
     a.batch = m_full; a.nsteps = (uint32_t)nsteps64;
     a.m_last = (uint32_t)(n_local - (nsteps64 - 1) * m_full);
@@ -871,16 +938,16 @@ int qesgd_launch_lr_epoch_fused(const float *X, const float *y, uint64_t n_local
     a.acc = reinterpret_cast<unsigned long long *>(work + QESGD_MAX_WORKERS * EP_HEADER_WORDS);
     a.wide = a.acc + (size_t)EP_RING * (QESGD_LR_EPOCH_ROWS / SUB) * EP_ACC_PITCH;
 
-    CUtensorMap map_full, map_rest;
+    CUtensorMap map_full = {}, map_rest = {};
     const uint32_t wide_box = s.cols < (uint32_t)EP_BOX_COLS ? s.cols : (uint32_t)EP_BOX_COLS;
     const uint32_t rest = s.cols % EP_BOX_COLS;
-    if (!make_map(&map_full, X, (uint64_t)K * n_local, d, wide_box)) return -1;
-    if (!make_map(&map_rest, X, (uint64_t)K * n_local, d, rest ? rest : wide_box)) return -1;
+    if (tma && !make_map(&map_full, X, (uint64_t)K * n_local, d, wide_box)) return -1;
+    if (tma && !make_map(&map_rest, X, (uint64_t)K * n_local, d, rest ? rest : wide_box)) return -1;
 
     void *params[] = {(void *)&a, (void *)&map_full, (void *)&map_rest};
-    const void *kernel = s.NC == 2u ? (const void *)qesgd_lr_epoch_kernel<2> : (const void *)qesgd_lr_epoch_kernel<1>;
-    const cudaError_t e = cudaLaunchCooperativeKernel(kernel, dim3(s.G * s.P), dim3(s.NC * EP_CHAIN + EP_PRODUCERS * 32), params,
-                                                      s.bytes, stream);
+    const void *const kernel = EPOCH_KERNELS[tma ? s.NC - 1u : (pairs ? 2u : 3u)];
+    const uint32_t threads = s.NC * EP_CHAIN + (tma ? EP_PRODUCERS : EP_LOADERS) * 32u;
+    const cudaError_t e = cudaLaunchCooperativeKernel(kernel, dim3(s.G * s.P), dim3(threads), params, s.bytes, stream);
     if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources ||
         e == cudaErrorInvalidConfiguration || e == cudaErrorNotSupported) {
         cudaGetLastError();   // the device cannot hold all CTAs at once as configured: two-pass steps

@@ -373,10 +373,18 @@ def test_lr_local_epoch_shapes_match_oracle(K, n_local, d, batch):
     (2, 150, 30000, 100),    # more rows than the warps of a chain take in one go
     (1, 2000, 784, 16),      # many short steps of one group: the accumulator ring goes round 15 times
     (2, 40, 160000, 16),     # above 1024 columns per SM: two-pass steps
+    (1, 8, 1, 8),            # rows on no 16-byte boundary from here on: one column
+    (1, 20, 3, 7),
+    (2, 100, 1001, 33),      # odd d, a last sub-tile of one row
+    (4, 130, 10003, 64),     # odd d over several CTAs, the last slice partly outside
+    (3, 77, 50002, 50),      # even d: copies of two elements
+    (1, 130, 140001, 64),    # ring shorter than a minibatch
+    (1, 300, 254, 256),
 ])
 def test_lr_local_epoch_splits_match_oracle(K, n_local, d, batch):
     """The ways the persistent kernel deals an epoch out (groups of CTAs, one or two chains, slices
-    of up to 1024 columns, rings shorter than a minibatch) at the edges of their ranges, twice: the
+    of up to 1024 columns, rings shorter than a minibatch, rows that TMA cannot fetch) at the edges of
+    their ranges, twice: the
     second call finds the workspace as the first one left it.  Bound: fp32 dot products of d terms
     against fp64, as for the other logistic steps (1e-5)."""
     X, y, _ = synthetic.logistic_problem(K * n_local, d, seed=K + n_local + d)
@@ -679,7 +687,7 @@ def test_fused_inner_step_at_the_edges_of_its_tiles(m, d, bucket, bits, s, mode,
 
 
 @pytest.mark.parametrize("m,d", [(200, 5001), (33, 65541), (17, 150001),    # rows split over 13, 2 and 1 CTAs per segment
-                                 (64, 150000), (256, 30000), (1, 4), (64, 419432)])
+                                 (64, 150000), (256, 30000), (1, 4), (64, 419432), (100, 250001), (64, 9999)])
 def test_lr_gradient_shapes_match_oracle(m, d):
     """Both forms of the gradient: two passes with the rows split over CTAs where segments are few, and
     the persistent kernel as an epoch of one step.  fp32 sums of d (margins) and m terms against fp64."""
