@@ -74,6 +74,28 @@ def test_encode_unaligned_pointer_takes_the_scalar_path():
         _assert_streams_equal(G.gpu_encode(z, None, *args, misalign=mis), want)
 
 
+@pytest.mark.parametrize("n", [1023, 1028, 2052, 3077, 8195, 16390])
+@pytest.mark.parametrize("bucket,bits,s,shift", [(64, 4, 7, 0), (512, 8, 127, 1), (4096, 2, 1, 2), (2048, 4, 7, 3)])
+def test_encode_batch_of_contiguous_rows_that_start_anywhere(n, bucket, bits, s, shift):
+    """Workers' vectors as rows of one [K, d] array: with d no multiple of 8 every row starts at another
+    alignment, and interior tiles are read in aligned pieces around them.  Sizes at the edges of the
+    1024-element tiles; the anchor starts `shift` floats off its boundary."""
+    K = 5
+    w = synthetic.anchor_vector(n, seed=1)
+    locs = synthetic.worker_locals(w, K, 1e-4, seed=2)
+    codes, scales = qesgd.alloc_stream_buffers(K, n, bucket, bits, "cuda")
+    anchor = torch.zeros(n + shift, dtype=torch.float32, device="cuda")
+    anchor[shift:] = G.dev(w)
+    c = G.ctx()
+    c.qesgd_encode_batch(G.dev(locs), n, anchor[shift:], n, K, bucket, s, bits, ref.SCALE_NORM, 42, 10, 3, codes,
+                         codes.stride(0), scales, scales.stride(0))
+    assert c.qesgd_status() == 0
+    gc, gs = codes.cpu().numpy().view(np.uint32), scales[:, :qesgd.num_buckets(n, bucket)].cpu().numpy()
+    for k in range(K):
+        wc, ws, _ = ref.encode(locs[k], w, bucket, s, bits, ref.SCALE_NORM, 42, 10 + k, 3)
+        assert (gc[k] == wc).all() and (gs[k].view(np.uint32) == ws.view(np.uint32)).all()
+
+
 def test_encode_batch_uses_worker_ids_and_strides():
     K, n, bucket = 5, 8192 + 520, 128
     w = synthetic.anchor_vector(n, seed=1)
