@@ -427,6 +427,24 @@ struct EncodeShared {
     uint32_t maxv[2][16];
 };
 
+// Where the quantised vector is written back (requantise), all three vectors of a tile are requested at
+// once and stay in registers: two chunks per warp and 20 warps per SM, or, for buckets that would then
+// span more than two warps, four and 16.  Bound by HBM then: d = 2^26 with 8-bit codes, buckets of 512 and
+// a given spacing 237 -> 205 us (1.41 GB), d = 2^22 15 -> 8.8; before, the anchor was read twice and the
+// running sum only after the rounding, a second round trip to memory in every warp's life.  Two chunks
+// with 24 or 32 warps: 206, 216; four for all: 206, but d = 10^6 4.4 -> 6.0; two chunks with buckets of 8192:
+// 243 against 198 with four.
+constexpr int REQ_CHUNKS = 2, REQ_WARPS = 20;
+constexpr int REQ_WIDE_CHUNKS = 4, REQ_WIDE_WARPS = 16;
+// What a warp tile that is written back needs besides its deltas, requested together with them: the
+// anchor and the running sum (of a tile inside the vector).
+template <int V, bool REQ>
+struct WriteBack {};
+template <int V>
+struct WriteBack<V, true> {
+    float w[V][8], zsum[V][8];
+};
+
 // Everything after the deltas z of one warp tile are in registers: bucket scale,
 // Philox draws, stochastic rounding, packing, stores.  `iter` selects the half of the
 // cross-warp scratch (callers alternate it between consecutive tiles of one CTA).
@@ -436,7 +454,7 @@ struct EncodeShared {
 // added to the running sum of the epoch average.
 template <int BITS, int MODE, int V, bool FULL, bool REQ>
 __device__ __forceinline__ void encode_warp_tile(const EncodeArgs &a, float (&z)[V][8],
-                                                 uint64_t warp_base, uint32_t k, uint32_t lane,
+                                                 WriteBack<V, REQ> &wb, uint64_t warp_base, uint32_t k, uint32_t lane,
                                                  uint32_t warp, EncodeShared &sh, uint32_t iter)
 {
     constexpr uint32_t LOG2_WARP_ELEMS = V == 4 ? 10 : (V == 2 ? 9 : 8);
@@ -563,15 +581,15 @@ __device__ __forceinline__ void encode_warp_tile(const EncodeArgs &a, float (&z)
             level_pair<MODE == 2>(z[c][j], z[c][j + 1], inv2, sf, x[j >> 1] & 0xFFFFu, x[j >> 1] >> 16,
                        X[j], X[j + 1]);
         }
-        if (REQ) {
+        if constexpr (REQ) {
             // decode what was just quantised: +-level * delta, the sign only where level > 0
             float v[8], w[8];
             const uint64_t e0 = warp_base + off;
             const uint64_t go = (uint64_t)k * a.local_stride + e0;
-            if (FULL) ld256(a.anchor + e0, w);
-            else load_octet<false>(a.anchor, e0, a.d, w);
+            if (!FULL) load_octet<false>(a.anchor, e0, a.d, w);
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
+                if (FULL) w[j] = wb.w[c][j];
                 const uint32_t lv = X[j] >> 16;
                 const float lf = __fsub_rn(__uint_as_float(0x4B000000u | lv), 8388608.0f);
                 const uint32_t sign31 = Z[j] & (lv + 0x7FFFFFFFu) & 0x80000000u;
@@ -587,10 +605,9 @@ __device__ __forceinline__ void encode_warp_tile(const EncodeArgs &a, float (&z)
             }
             if (a.zsum) {
                 float zs[8];
-                if (FULL) ld256_rw(a.zsum + go, zs);
-                else load_octet<false, true>(a.zsum, go, (uint64_t)k * a.local_stride + a.d, zs);
+                if (!FULL) load_octet<false, true>(a.zsum, go, (uint64_t)k * a.local_stride + a.d, zs);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) zs[j] = __fadd_rn(zs[j], v[j]);
+                for (int j = 0; j < 8; ++j) zs[j] = __fadd_rn(FULL ? wb.zsum[c][j] : zs[j], v[j]);
                 if (FULL) {
                     if (QESGD_IN_RANGE(a.status, e0 + 8 <= a.d)) st256(a.zsum + go, zs);
                 } else {
@@ -620,7 +637,8 @@ __device__ __forceinline__ void encode_warp_tile(const EncodeArgs &a, float (&z)
 // uses any of them, and several CTAs per SM overlap one another's load and arithmetic
 // phases.  VEC = false (pointers not 32-byte aligned) falls back to scalar loads.
 template <int BITS, int MODE, bool ANCHOR, bool VEC, int V, int WARPS, bool REQ>
-__global__ void __launch_bounds__(WARPS * 32, QESGD_ENCODE_MIN_WARPS / WARPS)
+__global__ void __launch_bounds__(WARPS * 32,
+                                  (!REQ ? QESGD_ENCODE_MIN_WARPS : (V == REQ_CHUNKS ? REQ_WARPS : REQ_WIDE_WARPS)) / WARPS)
     qesgd_encode_kernel(const EncodeArgs a)
 {
     qesgd_wait_for_previous();
@@ -635,6 +653,7 @@ __global__ void __launch_bounds__(WARPS * 32, QESGD_ENCODE_MIN_WARPS / WARPS)
     const uint64_t warp_base = ((uint64_t)tile * WARPS + warp) * (uint64_t)(V * CHUNK);
 
     float z[V][8];
+    WriteBack<V, REQ> wb;
     if (VEC && warp_base + V * CHUNK <= a.d) {   // the whole warp tile is inside the vector
         const float *__restrict__ p = local + warp_base + lane * 8u;
 #pragma unroll
@@ -642,7 +661,22 @@ __global__ void __launch_bounds__(WARPS * 32, QESGD_ENCODE_MIN_WARPS / WARPS)
             if (REQ) ld256_rw(p + c * CHUNK, z[c]);   // u is written back below
             else ld256(p + c * CHUNK, z[c]);
         }
-        if (ANCHOR) {
+        if constexpr (REQ) {
+            const float *__restrict__ q = a.anchor + warp_base + lane * 8u;
+#pragma unroll
+            for (int c = 0; c < V; ++c) ld256(q + c * CHUNK, wb.w[c]);
+            if (a.zsum) {
+                const float *r = a.zsum + (uint64_t)k * a.local_stride + warp_base + lane * 8u;
+#pragma unroll
+                for (int c = 0; c < V; ++c) ld256_rw(r + c * CHUNK, wb.zsum[c]);
+            }
+#pragma unroll
+            for (int c = 0; c < V; ++c)
+#pragma unroll
+                for (int j = 0; j < 8; j += 2)
+                    unpack2(sub2(pack2f(z[c][j], z[c][j + 1]), pack2f(wb.w[c][j], wb.w[c][j + 1])),
+                            z[c][j], z[c][j + 1]);
+        } else if (ANCHOR) {
             const float *__restrict__ q = a.anchor + warp_base + lane * 8u;
             float w[V][8];
 #pragma unroll
@@ -654,7 +688,7 @@ __global__ void __launch_bounds__(WARPS * 32, QESGD_ENCODE_MIN_WARPS / WARPS)
                     unpack2(sub2(pack2f(z[c][j], z[c][j + 1]), pack2f(w[c][j], w[c][j + 1])),
                             z[c][j], z[c][j + 1]);
         }
-        encode_warp_tile<BITS, MODE, V, true, REQ>(a, z, warp_base, k, lane, warp, sh, 0u);
+        encode_warp_tile<BITS, MODE, V, true, REQ>(a, z, wb, warp_base, k, lane, warp, sh, 0u);
         return;
     }
     if (!VEC && !REQ && warp_base >= 4 && warp_base + V * CHUNK + 4 <= a.d) {
@@ -678,7 +712,7 @@ __global__ void __launch_bounds__(WARPS * 32, QESGD_ENCODE_MIN_WARPS / WARPS)
                     unpack2(sub2(pack2f(z[c][j], z[c][j + 1]), pack2f(w[c][j], w[c][j + 1])),
                             z[c][j], z[c][j + 1]);
         }
-        encode_warp_tile<BITS, MODE, V, true, REQ>(a, z, warp_base, k, lane, warp, sh, 0u);
+        encode_warp_tile<BITS, MODE, V, true, REQ>(a, z, wb, warp_base, k, lane, warp, sh, 0u);
         return;
     }
 #pragma unroll
@@ -693,7 +727,7 @@ __global__ void __launch_bounds__(WARPS * 32, QESGD_ENCODE_MIN_WARPS / WARPS)
             for (int j = 0; j < 8; ++j) z[c][j] = __fsub_rn(z[c][j], w[j]);
         }
     }
-    encode_warp_tile<BITS, MODE, V, false, REQ>(a, z, warp_base, k, lane, warp, sh, 0u);
+    encode_warp_tile<BITS, MODE, V, false, REQ>(a, z, wb, warp_base, k, lane, warp, sh, 0u);
 }
 
 // ---------------------------------- update + requantise (Algorithm 2 inner step) ----
@@ -798,14 +832,16 @@ __global__ void __launch_bounds__(QS_THREADS, QESGD_QS_CTAS) qesgd_lr_qstep_kern
     const uint64_t tile0 = (uint64_t)(q.reverse ? gridDim.x - 1u - blockIdx.x : blockIdx.x) * QS_TILE, warp0 = tile0 + warp * (uint32_t)CHUNK;
     const uint64_t c = warp0 + lane * 8u;
     float z[1][8];
+    WriteBack<1, true> wb;
     if (tile0 + QS_TILE <= a.d && q.wide) {   // interior tile, everything 32-byte aligned
-        float t[8], u[8], w[8];
+        float t[8], u[8];
         sum_rows<true>(q.X + c, a.d, q.m, s_coef, t);
         ld256_rw(a.local + c, u);
-        ld256(a.anchor + c, w);
+        ld256(a.anchor + c, wb.w[0]);
+        if (a.zsum) ld256_rw(a.zsum + c, wb.zsum[0]);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) z[0][j] = __fsub_rn(__fadd_rn(u[j], t[j]), w[j]);
-        encode_warp_tile<BITS, MODE, 1, true, true>(a, z, warp0, 0u, lane, warp, sh, 0u);
+        for (int j = 0; j < 8; ++j) z[0][j] = __fsub_rn(__fadd_rn(u[j], t[j]), wb.w[0][j]);
+        encode_warp_tile<BITS, MODE, 1, true, true>(a, z, wb, warp0, 0u, lane, warp, sh, 0u);
         return;
     }
     float t[8];
@@ -838,7 +874,7 @@ __global__ void __launch_bounds__(QS_THREADS, QESGD_QS_CTAS) qesgd_lr_qstep_kern
     load_octet<false>(a.anchor, c, a.d, w);
 #pragma unroll
     for (int j = 0; j < 8; ++j) z[0][j] = c + j < a.d ? __fsub_rn(__fadd_rn(u[j], t[j]), w[j]) : 0.0f;
-    encode_warp_tile<BITS, MODE, 1, false, true>(a, z, warp0, 0u, lane, warp, sh, 0u);
+    encode_warp_tile<BITS, MODE, 1, false, true>(a, z, wb, warp0, 0u, lane, warp, sh, 0u);
 }
 
 // ------------------------------------------------------------- decode -------
@@ -1181,32 +1217,47 @@ __global__ void __launch_bounds__(QESGD_DAA_THREADS, BITS == 4 ? QESGD_DAA_MIN_C
 }
 
 // ------------------------------------------------------------ dispatch ------
-template <int BITS, int MODE, bool ANCHOR, bool VEC, int WARPS>
+template <int BITS, int MODE, bool ANCHOR, bool VEC, int V, int WARPS, bool REQ>
 cudaError_t launch_encode_w(const EncodeArgs &a, uint32_t K, cudaStream_t stream)
 {
-    constexpr int V = QESGD_ENCODE_CHUNKS;
     const uint64_t tile = (uint64_t)WARPS * V * CHUNK;
     const uint64_t tiles = (a.padded + tile - 1) / tile;
     if (tiles == 0 || tiles * K > 0x7FFFFFFFull) return cudaErrorInvalidValue;
     dim3 grid((unsigned)(tiles * K), 1, 1), block(WARPS * 32u, 1, 1);
-    if (ANCHOR && a.u_out)   // per-step QESGD: write back u = anchor + Q(z)
-        return qesgd_launch(qesgd_encode_kernel<BITS, MODE, ANCHOR, VEC, V, WARPS, ANCHOR>, grid, block, stream, a);
-    return qesgd_launch(qesgd_encode_kernel<BITS, MODE, ANCHOR, VEC, V, WARPS, false>, grid, block, stream, a);
+    return qesgd_launch(qesgd_encode_kernel<BITS, MODE, ANCHOR, VEC, V, WARPS, REQ>, grid, block, stream, a);
+}
+
+// A bucket never leaves its CTA: as many warps as it spans, no more; with a caller-given spacing nothing
+// is reduced over a bucket and one warp will do (requantise of 2^26 with buckets of 4096: 284 -> 205 us).
+template <int BITS, int MODE, bool ANCHOR, bool VEC, int V, bool REQ>
+cudaError_t launch_encode_n(const EncodeArgs &a, uint32_t K, cudaStream_t stream)
+{
+    constexpr uint32_t SMALL = QESGD_ENCODE_WARPS;        // warps of the usual CTA
+    const uint32_t need = MODE == 2 ? 1u : (1u << a.log2_bucket) / (uint32_t)(V * CHUNK);
+    if (need <= SMALL) return launch_encode_w<BITS, MODE, ANCHOR, VEC, V, SMALL, REQ>(a, K, stream);
+    if constexpr (MODE != 2) {
+        if (need <= 2u) return launch_encode_w<BITS, MODE, ANCHOR, VEC, V, (SMALL > 2 ? SMALL : 2), REQ>(a, K, stream);
+        if constexpr (V >= 4) {
+            if (need <= 4u) return launch_encode_w<BITS, MODE, ANCHOR, VEC, V, (SMALL > 4 ? SMALL : 4), REQ>(a, K, stream);
+            constexpr uint32_t LARGE = QESGD_MAX_BUCKET / (V * CHUNK);   // enough for the widest bucket
+            return launch_encode_w<BITS, MODE, ANCHOR, VEC, V, (LARGE > SMALL ? LARGE : SMALL), REQ>(a, K, stream);
+        }
+    }
+    return cudaErrorInvalidValue;
 }
 
 template <int BITS, int MODE, bool ANCHOR, bool VEC>
 cudaError_t launch_encode_v(const EncodeArgs &a, uint32_t K, int sm_count, cudaStream_t stream)
 {
     (void)sm_count;
-    constexpr int V = QESGD_ENCODE_CHUNKS;
-    constexpr uint32_t SMALL = QESGD_ENCODE_WARPS;        // warps of the usual CTA
-    // a bucket never leaves its CTA: as many warps as the bucket spans, no more
-    const uint32_t need = (1u << a.log2_bucket) / (uint32_t)(V * CHUNK);
-    if (need <= SMALL) return launch_encode_w<BITS, MODE, ANCHOR, VEC, SMALL>(a, K, stream);
-    if (need <= 2u) return launch_encode_w<BITS, MODE, ANCHOR, VEC, (SMALL > 2 ? SMALL : 2)>(a, K, stream);
-    if (need <= 4u) return launch_encode_w<BITS, MODE, ANCHOR, VEC, (SMALL > 4 ? SMALL : 4)>(a, K, stream);
-    constexpr uint32_t LARGE = QESGD_MAX_BUCKET / (V * CHUNK);   // enough for the widest bucket
-    return launch_encode_w<BITS, MODE, ANCHOR, VEC, (LARGE > SMALL ? LARGE : SMALL)>(a, K, stream);
+    if constexpr (ANCHOR) {   // per-step QESGD: write back u = anchor + Q(z)
+        if (a.u_out) {
+            if (MODE == 2 || (1u << a.log2_bucket) <= 2u * REQ_CHUNKS * CHUNK)
+                return launch_encode_n<BITS, MODE, true, VEC, REQ_CHUNKS, true>(a, K, stream);
+            return launch_encode_n<BITS, MODE, true, VEC, REQ_WIDE_CHUNKS, true>(a, K, stream);
+        }
+    }
+    return launch_encode_n<BITS, MODE, ANCHOR, VEC, QESGD_ENCODE_CHUNKS, false>(a, K, stream);
 }
 
 template <int BITS, int MODE>

@@ -587,6 +587,23 @@ def test_requantize_matches_oracle_bitwise(bits, s, mode, bucket):
     assert (got[0].view(np.uint32) == want[0].view(np.uint32)).all() and got[1] is None
 
 
+@pytest.mark.parametrize("n", [8, 504, 512, 1032, 4096 + 24, 20000])
+@pytest.mark.parametrize("bucket,mode", [(512, 0), (1024, 1), (2048, 0), (8192, 0), (8192, 2)])
+def test_requantize_at_the_edges_of_its_tiles(n, bucket, mode):
+    """Tiles of 512 elements per warp up to buckets of 1024 (and for every bucket with a given spacing),
+    of 1024 above, CTAs as wide as a bucket."""
+    w = synthetic.anchor_vector(n, seed=bucket)
+    u = (w + synthetic.delta_vector(n, 1e-3, seed=n, outlier_prob=0.01)).astype(np.float32)
+    zsum = synthetic.delta_vector(n, 1e-3, seed=n + 2)
+    for z in (zsum, None):
+        got = _gpu_requantize(u, w, z, bucket, 7, 4, mode, 99, 1, 6, 3e-4)
+        want = ref.requantize(u, w, bucket, 7, 4, mode, 99, 1, 6, zsum=z, fixed_delta=3e-4)
+        assert (got[0].view(np.uint32) == want[0].view(np.uint32)).all()
+        assert z is None or (got[1].view(np.uint32) == want[1].view(np.uint32)).all()
+        assert (got[2] == want[2]).all() and (got[3].view(np.uint32) == want[3].view(np.uint32)).all()
+        assert got[4] == want[4]
+
+
 def test_qesgd_inner_loop_on_the_gpu_follows_the_oracle():
     """Algorithm 2 on a logistic problem: gradient step, requantize, running sum; the GPU's
     u after every step is handed to the oracle's requantize, which must agree bit for bit."""
