@@ -337,11 +337,13 @@ struct MaxU32 {
 template <int V>
 __device__ __forceinline__ uint32_t chunk_of_lane(uint32_t lane)
 {
+    if (V == 8) return 4u * (lane & 1u) + 2u * ((lane >> 1) & 1u) + ((lane >> 2) & 1u);
     return V == 4 ? 2u * (lane & 1u) + ((lane >> 1) & 1u) : (V == 2 ? (lane & 1u) : 0u);
 }
 template <int V>
 __device__ __forceinline__ uint32_t lane_of_chunk(uint32_t lane, int c)
 {
+    if (V == 8) return (lane & 24u) | ((c >> 2) & 1) | (((c >> 1) & 1) << 1) | ((c & 1) << 2);
     return V == 4 ? ((lane & 28u) | ((c >> 1) & 1) | ((c & 1) << 1)) : (V == 2 ? ((lane & 30u) | (c & 1)) : lane);
 }
 
@@ -364,6 +366,34 @@ __device__ __forceinline__ typename R::T reduce_chunks(const typename R::T (&t)[
     if (lb >= 9) k = R::op(k, __shfl_xor_sync(FULL, k, 2));    // chunks (0,1) and (2,3)
     if (lb >= 10) k = R::op(k, __shfl_xor_sync(FULL, k, 1));   // all four chunks
     return k;
+}
+
+template <typename R>
+__device__ __forceinline__ typename R::T reduce_chunks(const typename R::T (&t)[8], uint32_t lane,
+                                                       uint32_t lb)
+{
+    typedef typename R::T T;
+    const bool b0 = lane & 1u, b1 = lane & 2u, b2 = lane & 4u;
+    T k[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const T keep = b0 ? t[i + 4] : t[i], send = b0 ? t[i] : t[i + 4];
+        k[i] = R::op(keep, __shfl_xor_sync(FULL, send, 1));
+    }
+    T l[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const T keep = b1 ? k[i + 2] : k[i], send = b1 ? k[i] : k[i + 2];
+        l[i] = R::op(keep, __shfl_xor_sync(FULL, send, 2));
+    }
+    const T keep = b2 ? l[1] : l[0], send = b2 ? l[0] : l[1];
+    T m = R::op(keep, __shfl_xor_sync(FULL, send, 4));
+    if (lb >= 7) m = R::op(m, __shfl_xor_sync(FULL, m, 8));
+    if (lb >= 8) m = R::op(m, __shfl_xor_sync(FULL, m, 16));
+    if (lb >= 9) m = R::op(m, __shfl_xor_sync(FULL, m, 4));    // chunks (0,1), (2,3), ...
+    if (lb >= 10) m = R::op(m, __shfl_xor_sync(FULL, m, 2));   // fours
+    if (lb >= 11) m = R::op(m, __shfl_xor_sync(FULL, m, 1));   // all eight
+    return m;
 }
 
 template <typename R>
@@ -434,6 +464,9 @@ struct EncodeShared {
 // running sum only after the rounding, a second round trip to memory in every warp's life.  Two chunks
 // with 24 or 32 warps: 206, 216; four for all: 206, but d = 10^6 4.4 -> 6.0; two chunks with buckets of 8192:
 // 243 against 198 with four.
+// Encode of wide buckets: eight chunks per warp, 16 warps per SM (12: 274 us where 16 take 263, 20: 272).
+constexpr int WIDE_CHUNKS = 8, WIDE_WARPS = 16;
+constexpr uint64_t WIDE_MIN_ELEMENTS = 8ull << 20;
 constexpr int REQ_CHUNKS = 2, REQ_WARPS = 20;
 constexpr int REQ_WIDE_CHUNKS = 4, REQ_WIDE_WARPS = 16;
 // What a warp tile that is written back needs besides its deltas, requested together with them: the
@@ -457,7 +490,7 @@ __device__ __forceinline__ void encode_warp_tile(const EncodeArgs &a, float (&z)
                                                  WriteBack<V, REQ> &wb, uint64_t warp_base, uint32_t k, uint32_t lane,
                                                  uint32_t warp, EncodeShared &sh, uint32_t iter)
 {
-    constexpr uint32_t LOG2_WARP_ELEMS = V == 4 ? 10 : (V == 2 ? 9 : 8);
+    constexpr uint32_t LOG2_WARP_ELEMS = V == 8 ? 11 : (V == 4 ? 10 : (V == 2 ? 9 : 8));
     constexpr int DRAWS = V > 1 ? 2 : 1;                        // Philox blocks advanced together
     const uint32_t lb = a.log2_bucket;
     const float sf = (float)a.s;
@@ -638,7 +671,7 @@ __device__ __forceinline__ void encode_warp_tile(const EncodeArgs &a, float (&z)
 // phases.  VEC = false (pointers not 32-byte aligned) falls back to scalar loads.
 template <int BITS, int MODE, bool ANCHOR, bool VEC, int V, int WARPS, bool REQ>
 __global__ void __launch_bounds__(WARPS * 32,
-                                  (!REQ ? QESGD_ENCODE_MIN_WARPS : (V == REQ_CHUNKS ? REQ_WARPS : REQ_WIDE_WARPS)) / WARPS)
+                                  (!REQ ? (V == 8 ? WIDE_WARPS : QESGD_ENCODE_MIN_WARPS) : (V == REQ_CHUNKS ? REQ_WARPS : REQ_WIDE_WARPS)) / WARPS)
     qesgd_encode_kernel(const EncodeArgs a)
 {
     qesgd_wait_for_previous();
@@ -1237,7 +1270,8 @@ cudaError_t launch_encode_n(const EncodeArgs &a, uint32_t K, cudaStream_t stream
     if (need <= SMALL) return launch_encode_w<BITS, MODE, ANCHOR, VEC, V, SMALL, REQ>(a, K, stream);
     if constexpr (MODE != 2) {
         if (need <= 2u) return launch_encode_w<BITS, MODE, ANCHOR, VEC, V, (SMALL > 2 ? SMALL : 2), REQ>(a, K, stream);
-        if constexpr (V >= 4) {
+        if constexpr (V == 8) return launch_encode_w<BITS, MODE, ANCHOR, VEC, V, 4, REQ>(a, K, stream);
+        if constexpr (V == 4) {
             if (need <= 4u) return launch_encode_w<BITS, MODE, ANCHOR, VEC, V, (SMALL > 4 ? SMALL : 4), REQ>(a, K, stream);
             constexpr uint32_t LARGE = QESGD_MAX_BUCKET / (V * CHUNK);   // enough for the widest bucket
             return launch_encode_w<BITS, MODE, ANCHOR, VEC, V, (LARGE > SMALL ? LARGE : SMALL), REQ>(a, K, stream);
@@ -1257,6 +1291,13 @@ cudaError_t launch_encode_v(const EncodeArgs &a, uint32_t K, int sm_count, cudaS
             return launch_encode_n<BITS, MODE, true, VEC, REQ_WIDE_CHUNKS, true>(a, K, stream);
         }
     }
+    // Buckets above 1024: a warp takes 2048 elements, so that a bucket spans one warp, two or four instead of
+    // two, four or eight that wait for one another with all their registers held (2^28 elements in all:
+    // buckets of 2048 291 -> 261 us, 4096 274 -> 263, 8192 309 -> 275).  Short inputs need the finer tiles to
+    // fill the device (2 x 2^21: 6.4 against 6.8).
+    if constexpr (VEC && MODE != 2)
+        if (a.log2_bucket >= 11 && a.padded * K >= WIDE_MIN_ELEMENTS)
+            return launch_encode_n<BITS, MODE, ANCHOR, VEC, WIDE_CHUNKS, false>(a, K, stream);
     return launch_encode_n<BITS, MODE, ANCHOR, VEC, QESGD_ENCODE_CHUNKS, false>(a, K, stream);
 }
 

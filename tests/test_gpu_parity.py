@@ -65,6 +65,21 @@ def test_encode_with_anchor_large(bits, s):
     _assert_streams_equal(G.gpu_encode(u, w, *args), ref.encode(u, w, *args))
 
 
+@pytest.mark.parametrize("bucket,bits,s,mode", [(2048, 4, 7, ref.SCALE_NORM), (4096, 2, 1, ref.SCALE_MAX),
+                                                (8192, 8, 127, ref.SCALE_NORM)])
+def test_encode_wide_buckets_of_long_vectors(bucket, bits, s, mode):
+    """From 8 Mi elements on a warp takes 2048 elements of buckets above 1024; every word and scale of two
+    workers, the last bucket of 40 elements."""
+    K, n = 2, (1 << 22) + 8192 + 40
+    w = synthetic.anchor_vector(n, seed=5)
+    locs = synthetic.worker_locals(w, K, 1e-3, seed=6, outlier_prob=0.01)
+    gc, gs, gst = G.gpu_encode_batch(locs, w, bucket, s, bits, mode, 7, 3, 1)
+    assert gst == 0
+    for k in range(K):
+        wc, ws, _ = ref.encode(locs[k], w, bucket, s, bits, mode, 7, 3 + k, 1)
+        assert (gc[k] == wc).all() and (gs[k].view(np.uint32) == ws.view(np.uint32)).all()
+
+
 def test_encode_unaligned_pointer_takes_the_scalar_path():
     n = 8192 + 77
     z = _delta(n, seed=31)
