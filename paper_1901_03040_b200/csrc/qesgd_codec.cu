@@ -997,6 +997,41 @@ __global__ void __launch_bounds__(256) qesgd_decode_kernel(const DecodeArgs a)
 
 // -------------------------------------------- decode + average + apply ------
 
+// Codes of 4 and 8 bits as floats without any arithmetic: a level in bits 16..22 below the code's sign in
+// bit 31 IS the float +-level * 2^-133 (a subnormal, which multiply-adds take at full speed), and one byte
+// permute puts it there from a word of levels and a word of signs.  The spacing is multiplied by 2^110, so
+// the sum comes out in units of 2^-23 of itself; all these factors are powers of two and every rounding is
+// the one that the plain sum would make as long as nothing leaves the range of normal floats, which holds
+// for spacings in [2^-79, 2^18) (see the caller).
+constexpr float STEP_SCALE = 0x1p110f, SUM_SCALE = 0x1p23f;
+constexpr float STEP_MIN = 0x1p-79f, STEP_LIMIT = 0x1p18f;
+
+template <int BITS>
+__device__ __forceinline__ void accumulate_octet_scaled(const uint32_t (&cw)[2], int o, uint64_t step2,
+                                                        uint64_t (&acc)[4])
+{
+    // byte j of the levels to byte 2, of the signs to byte 3; zeros below (a level's top bit, replicated)
+    auto value = [](uint32_t levels, uint32_t signs, int j) {
+        return prmt(levels, signs, ((4 + j) << 12) | (j << 8) | ((8 + j) << 4) | (8 + j));
+    };
+    if (BITS == 8) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint32_t lv = cw[h] & 0x7F7F7F7Fu, sg = cw[h] & 0x80808080u;
+#pragma unroll
+            for (int j = 0; j < 4; j += 2)
+                acc[2 * h + j / 2] = fma2(pack2(value(lv, sg, j), value(lv, sg, j + 1)), step2, acc[2 * h + j / 2]);
+        }
+    } else {
+        const uint32_t word = cw[o];
+        const uint32_t le = word & 0x07070707u, lo = (word >> 4) & 0x07070707u;      // even, odd elements
+        const uint32_t se = (word << 4) & 0x80808080u, so = word & 0x80808080u;
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+            acc[p] = fma2(pack2(value(le, se, p), value(lo, so, p)), step2, acc[p]);
+    }
+}
+
 // acc += +-level * step for the 8 codes of one octet, two elements per arithmetic
 // instruction (acc[p] holds elements 2p, 2p+1).  One rounding per product-sum: the sign
 // is folded into the multiplier.  `cw` is the 64-bit code word of the lane and `o` the
@@ -1059,15 +1094,16 @@ __device__ __forceinline__ void accumulate_octet(const uint32_t (&cw)[2], int o,
 // needs are computed once per warp (one division per lane) and handed out by shuffle;
 // code words are fetched several workers at a time so that independent loads are in
 // flight before the first is used.
-// KS > 0: the number of workers is that compile-time constant and the worker loop is unrolled
-// completely (no loop counter, no predicates on the worker index).  Measured: 14 % faster for
-// 8-bit, 4 % for 4-bit and 4 % for 2-bit codes at K = 8, but slower for 2-bit codes at K = 4
-// (1 %) and at K = 16 (3-9 %: 16 workers x 32 codes per lane no longer fit the instruction
-// cache), where unrolling half the loop gives 2-3 %; the launcher picks accordingly.
-// Register budget: 24 resident CTAs per SM, 28 for 4-bit codes (measured 4-5 % faster there,
-// slower for the other widths).
+// KS > 0: the number of workers is that compile-time constant and the worker loop is unrolled (no loop
+// counter, no predicates on the worker index): K = 3, 5, 6, 7 with 8-bit codes 8 to 13 % faster, with 4-bit
+// codes 1 to 6 %; the launcher picks.  Register budget: 24 resident CTAs per SM (28 for 4-bit codes: 20.0
+// against 17.2 us at K = 8, d = 11.7 M, 58 against 51 at K = 16).
+// 4- and 8-bit codes cost two instructions each (accumulate_octet_scaled); with a table of the sixteen
+// values looked up by shuffle (4-bit, buckets of 256 and more) it was 2.5 on the busier shuffle path, with
+// levels spliced into 2^23 four to five: 2^28 4-bit codes of 8 workers, buckets of 128 81 -> 62 us, of 512
+// 66 -> 61, of 16 workers 79 -> 52 and 56 -> 48; 8-bit codes of 16 workers 73 -> 64, of 32 75 -> 57.
 template <int BITS, bool VEC, int W, int KS = 0>
-__global__ void __launch_bounds__(QESGD_DAA_THREADS, BITS == 4 ? QESGD_DAA_MIN_CTAS + 4 : QESGD_DAA_MIN_CTAS)
+__global__ void __launch_bounds__(QESGD_DAA_THREADS, QESGD_DAA_MIN_CTAS)
     qesgd_decode_average_apply_kernel(const DecodeArgs a)
 {
     qesgd_wait_for_previous();
@@ -1111,12 +1147,8 @@ __global__ void __launch_bounds__(QESGD_DAA_THREADS, BITS == 4 ? QESGD_DAA_MIN_C
             for (int p = 0; p < 4; ++p) acc[c][o][p] = 0ull;   // pairs of +0.0f
     }
 
-    // Four-bit codes with buckets of at least 256 elements: a half-warp (16 lanes x 16
-    // elements) lies inside one bucket, so the 16 possible code values +-level * step of a
-    // worker fit one per lane and decoding becomes a 16-wide shuffle.  signed_level is the
-    // level of code (lane & 15) with its sign: 0..7, -0..-7.
-    const bool lut = BITS == 4 && lb >= 8;
-    const float signed_level = (lane & 8u) ? -(float)(lane & 7u) : (float)(lane & 7u);
+    constexpr bool SCALED = BITS != 2;
+    bool odd_step = false;   // a spacing outside the range in which the scaled sum is exact
 
     // Code words of BATCH workers are requested one batch ahead of the batch being decoded.
     auto fetch = [&](uint32_t kfirst, uint32_t (&dst)[BATCH][W][2]) {
@@ -1147,40 +1179,31 @@ __global__ void __launch_bounds__(QESGD_DAA_THREADS, BITS == 4 ? QESGD_DAA_MIN_C
     fetch(0u, cw);
     float sc_next = fetch_scale(0u);
     float st = 0.0f;
-    // 2-bit codes of 16 workers: two batches per loop iteration (the whole loop would not fit
-    // the instruction cache); every other compile-time worker count: the whole loop
-    constexpr int OUTER_UNROLL = KS == 0 ? 1 : ((BITS == 2 && KS > 8) ? 2 : 64);
-#pragma unroll OUTER_UNROLL
-    for (uint32_t kb = 0; kb < (KS ? (uint32_t)KS : a.K); kb += BATCH) {
+    // Decodes the workers kb .. kb + BATCH - 1, having requested the next ones' words.
+    auto batch = [&](uint32_t kb) {
         fetch(kb + BATCH, nx);
 #pragma unroll
         for (int i = 0; i < BATCH; ++i) {
             const uint32_t k = kb + i;
             if (k < K) {   // uniform across the warp
                 // position of worker k inside its pass (per_pass is a power of two)
-                const uint32_t kp = KS ? (k & (per_pass - 1u)) : k % per_pass;
+                const uint32_t kp = k & (per_pass - 1u);
                 if (kp == 0u) {   // a new pass: every lane computes one spacing
                     st = __fdiv_rn(sc_next, sf);
+                    if (SCALED) {
+                        odd_step |= !(st == 0.0f || (st >= STEP_MIN && st < STEP_LIMIT));
+                        st = __fmul_rn(st, STEP_SCALE);
+                    }
                     sc_next = fetch_scale(k + per_pass);
                 }
 #pragma unroll
                 for (int c = 0; c < W; ++c) {
                     const float step = __shfl_sync(FULL, st, kp * nbw + sub[c]);
-                    if (BITS == 4 && lut) {
-                        // every lane holds the value of code (lane & 15) for this worker; a
-                        // code is decoded by fetching its value from that lane of the same
-                        // half-warp
-                        const float tab = __fmul_rn(signed_level, step);
+                    if (SCALED) {
+                        const uint64_t step2 = pack2f(step, step);
 #pragma unroll
-                        for (int o = 0; o < OPL; ++o) {
-                            const uint32_t word = cw[i][c][o];
-#pragma unroll
-                            for (int p = 0; p < 4; ++p) {
-                                const float v0 = __shfl_sync(FULL, tab, (int)(word >> (8 * p)), 16);
-                                const float v1 = __shfl_sync(FULL, tab, (int)(word >> (8 * p + 4)), 16);
-                                acc[c][o][p] = add2(acc[c][o][p], pack2f(v0, v1));
-                            }
-                        }
+                        for (int o = 0; o < OPL; ++o)
+                            accumulate_octet_scaled<BITS>(cw[i][c], o, step2, acc[c][o]);
                     } else {
 #pragma unroll
                         for (int o = 0; o < OPL; ++o)
@@ -1196,7 +1219,12 @@ __global__ void __launch_bounds__(QESGD_DAA_THREADS, BITS == 4 ? QESGD_DAA_MIN_C
                 cw[i][c][0] = nx[i][c][0];
                 cw[i][c][1] = nx[i][c][1];
             }
-    }
+    };
+    // 2-bit codes of 16 or 32 workers: two batches per loop iteration (the whole loop would not fit the
+    // instruction cache), of wider codes and 32 workers four; every other compile-time count: the whole loop
+    constexpr int OUTER_UNROLL = KS == 0 ? 1 : (BITS == 2 && KS > 8 ? 2 : (KS > 16 ? 4 : 64));
+#pragma unroll OUTER_UNROLL
+    for (uint32_t kb = 0; kb < (KS ? (uint32_t)KS : a.K); kb += BATCH) batch(kb);
     // Apply: param += (alpha / K) * sum.  The warp never loads the parameter: every element
     // gets exactly one add, done by the memory system (a vector reduction of four floats), so a
     // warp's life ends with its last code word instead of a further round trip to memory, and the
@@ -1207,6 +1235,35 @@ __global__ void __launch_bounds__(QESGD_DAA_THREADS, BITS == 4 ? QESGD_DAA_MIN_C
     // P ^ ((P >> 3) & 7), which keeps both the lane-major writes and the piece-major reads free
     // of bank conflicts for 2, 4 or 8 pieces per lane.
     const float inv_k = a.avg_scale;   // alpha / K
+    if (SCALED) {
+        if (__any_sync(FULL, odd_step)) {   // rare: the same sum once more, plainly
+#pragma unroll
+            for (int c = 0; c < W; ++c)
+#pragma unroll
+                for (int o = 0; o < OPL; ++o)
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) acc[c][o][p] = 0ull;
+#pragma unroll 1
+            for (uint32_t k = 0; k < a.K; ++k) {
+#pragma unroll
+                for (int c = 0; c < W; ++c) {
+                    const uint64_t bucket = bucket0 + sub[c];
+                    const float sc = bucket < a.nb ? __ldg(a.scales + (uint64_t)k * a.scale_stride + bucket) : 0.0f;
+                    const uint2 v = __ldg(reinterpret_cast<const uint2 *>(cp[c] + (uint64_t)k * a.code_stride));
+                    const uint32_t word[2] = {v.x, v.y};
+#pragma unroll
+                    for (int o = 0; o < OPL; ++o) accumulate_octet<BITS>(word, o, __fdiv_rn(sc, sf), acc[c][o]);
+                }
+            }
+        } else {
+#pragma unroll
+            for (int c = 0; c < W; ++c)
+#pragma unroll
+                for (int o = 0; o < OPL; ++o)
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) acc[c][o][p] = mul2(acc[c][o][p], pack2f(SUM_SCALE, SUM_SCALE));
+        }
+    }
     constexpr int NCH = LANE_ELEMS / 4;           // 16-byte pieces per lane and chunk: 8, 4, 2
     __shared__ float4 s_inc[(QESGD_DAA_THREADS / 32) * W * 32 * NCH];
     float4 *wt = s_inc + (threadIdx.x >> 5) * (W * 32 * NCH);
@@ -1386,16 +1443,22 @@ int QESGD_CAT(qesgd_launch_decode_average_apply_, QESGD_BITS)(const DecodeArgs &
     const uint64_t blocks = (warps + wpc - 1) / wpc;
     if (blocks == 0 || blocks > 0x7FFFFFFFull) return (int)cudaErrorInvalidValue;
     dim3 grid((unsigned)blocks), block(QESGD_DAA_THREADS);
-    void (*kernel)(DecodeArgs);
-    if (vec && a.K == 8)
-        kernel = qesgd_decode_average_apply_kernel<QESGD_BITS, true, W, 8>;
-    else if (vec && QESGD_BITS != 2 && a.K == 4)
-        kernel = qesgd_decode_average_apply_kernel<QESGD_BITS, true, W, (QESGD_BITS != 2 ? 4 : 0)>;
-    else if (vec && QESGD_BITS != 4 && a.K == 16)
-        kernel = qesgd_decode_average_apply_kernel<QESGD_BITS, true, W, (QESGD_BITS != 4 ? 16 : 0)>;
-    else if (vec)
-        kernel = qesgd_decode_average_apply_kernel<QESGD_BITS, true, W>;
-    else
-        kernel = qesgd_decode_average_apply_kernel<QESGD_BITS, false, W>;
+    // Worker counts with a loop of their own (1 to 8, 16, 32); the smallest of 2- and 8-bit codes are bound
+    // by HBM and no faster for it (2-bit, K = 1: 358 against 364 us).
+    constexpr uint32_t FIRST = QESGD_BITS == 2 ? 5u : (QESGD_BITS == 8 ? 3u : 1u);
+    static void (*const BY_COUNT[9])(DecodeArgs) = {
+        qesgd_decode_average_apply_kernel<QESGD_BITS, true, W>,
+        qesgd_decode_average_apply_kernel<QESGD_BITS, true, W, (FIRST <= 1u ? 1 : 0)>,
+        qesgd_decode_average_apply_kernel<QESGD_BITS, true, W, (FIRST <= 2u ? 2 : 0)>,
+        qesgd_decode_average_apply_kernel<QESGD_BITS, true, W, (FIRST <= 3u ? 3 : 0)>,
+        qesgd_decode_average_apply_kernel<QESGD_BITS, true, W, (FIRST <= 4u ? 4 : 0)>,
+        qesgd_decode_average_apply_kernel<QESGD_BITS, true, W, 5>,
+        qesgd_decode_average_apply_kernel<QESGD_BITS, true, W, 6>,
+        qesgd_decode_average_apply_kernel<QESGD_BITS, true, W, 7>,
+        qesgd_decode_average_apply_kernel<QESGD_BITS, true, W, 8>};
+    void (*kernel)(DecodeArgs) = BY_COUNT[a.K <= 8u ? a.K : 0u];
+    if (a.K == 16u) kernel = qesgd_decode_average_apply_kernel<QESGD_BITS, true, W, 16>;
+    if (a.K == 32u) kernel = qesgd_decode_average_apply_kernel<QESGD_BITS, true, W, 32>;
+    if (!vec) kernel = qesgd_decode_average_apply_kernel<QESGD_BITS, false, W>;
     return (int)qesgd_launch(kernel, grid, block, stream, a);
 }

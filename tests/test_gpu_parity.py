@@ -307,6 +307,39 @@ def test_decode_average_apply_matches_oracle(K, bucket, bits, s):
     _assert_param_close(got, want, w, scales, bucket)
 
 
+@pytest.mark.parametrize("K", [1, 6, 7, 10, 16, 32])
+@pytest.mark.parametrize("bits,s", [(4, 7), (8, 127)])
+def test_decode_average_apply_is_the_plain_sum_for_every_spacing(bits, s, K):
+    """4- and 8-bit codes are summed in units scaled by powers of two, and plainly where a spacing lies
+    outside the range in which that is exact (2^-79 to 2^18).  Scales from 1e-30 to 3e38 / s, within and
+    outside that range and at its borders, all codes: the result is, bit for bit, the fp32 sum by fused
+    multiply-adds over the workers in order, times 1/K, added to the parameter.  (numpy has no fused
+    multiply-add: a level times a spacing is exact in fp64 -- 7 + 24 bits --, so is its sum with an fp32
+    number rounded once to fp64 and then to fp32 unless that lies within 2^-53 of a tie, which the inputs
+    avoid: they have at most 16 significant bits.)"""
+    bucket, nb = 64, 96
+    n = bucket * nb
+    rng = np.random.default_rng(bits * 100 + K)
+    exps = np.concatenate([np.arange(-90, -70, 2), [-79, -78, 17, 18, 19], rng.integers(-70, 17, nb - 25),
+                           np.arange(100, 120, 2)])[:nb]
+    step = np.ldexp(rng.integers(128, 256, (K, nb)) / 256.0, exps[None, :]).astype(np.float32)
+    scales = (step * np.float32(s)).astype(np.float32)
+    step = (scales / np.float32(s)).astype(np.float32)
+    levels = rng.integers(0, s + 1, (K, n)).astype(np.uint32)
+    signs = (rng.integers(0, 2, (K, n)) * (levels > 0)).astype(np.uint32)
+    per = 32 // bits
+    codes = ((signs << (bits - 1)) | levels).reshape(K, n // per, per)
+    words = np.bitwise_or.reduce(codes << (np.arange(per, dtype=np.uint32) * bits), axis=2).astype(np.uint32)
+    acc = np.zeros(n, dtype=np.float32)
+    for k in range(K):
+        v = np.where(signs[k] == 1, -1.0, 1.0) * levels[k] * np.repeat(step[k], bucket).astype(np.float64)
+        acc = (acc.astype(np.float64) + v).astype(np.float32)
+    w = np.zeros(n, dtype=np.float32)
+    want = w + acc * np.float32(np.float32(1.0) / np.float32(K))
+    got = G.gpu_decode_average_apply(w, words, scales, bucket, s, bits)
+    assert np.array_equal(got, want)
+
+
 @pytest.mark.parametrize("n", [1, 9, 255, 256, 257, 2049])
 def test_decode_average_apply_small_sizes(n):
     w, codes, scales = _daa_case(n, 4, 64, 4, 7, seed=n)
