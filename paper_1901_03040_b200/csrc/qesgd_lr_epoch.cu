@@ -410,11 +410,6 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + (EB == 16 ? EP_PRODUCERS : EP_
     }
     if (tid < 16u + EP_MAX_SLOTS) s_flag[tid] = 0u;
     __syncthreads();
-    if (warp == 0) tmem_alloc_all(const_cast<uint32_t *>(&s_flag[8]));
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem_base = s_flag[8];
 
     // ----------------------------------------------------------- producers ----
     if (warp >= NC * EP_WARPS) {
@@ -500,9 +495,7 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + (EB == 16 ? EP_PRODUCERS : EP_
             uint32_t before = 0u;
             if (lane == 0) {
                 if (s_flag[0] != 0u) atomicExch(header, 1u);   // gave up: so shall the others
-                __threadfence();
-                before = atomicAdd(header + 1, 1u);
-                __threadfence();
+                asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(before) : "l"(header + 1) : "memory");
             }
             if (__shfl_sync(0xFFFFFFFFu, before, 0) == a.P - 1u) {
                 for (uint32_t j = lane; j < EP_RING * mpad; j += 32u) {
@@ -521,14 +514,12 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + (EB == 16 ? EP_PRODUCERS : EP_
     float *const coef = s_coef + g * EP_MAX_M;
     float *const part = s_part + (size_t)g * EP_WARPS * ucols;
     auto chain_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1u + g), "n"(EP_CHAIN) : "memory"); };
-    // this thread's lane of the tensor memory, this warp's columns
-    const uint32_t taddr = tmem_base + ((32u * (wg & 3u)) << 16) +
-                           (NC == 2 ? 256u * g + 128u * (wg >> 2) : 256u * (wg >> 2));
     const uint32_t mpad = SUB * a.nsub_max;
     unsigned long long *const acc_g = a.acc + (size_t)grp * EP_RING * a.nsub_max * EP_ACC_PITCH;
     unsigned long long *const wide_g = a.wide + (size_t)grp * EP_RING * mpad * EP_WIDE_WORDS;
     uint32_t *const header = a.header + grp * EP_HEADER_WORDS;
 
+    if (warp == 0) tmem_alloc_all(const_cast<uint32_t *>(&s_flag[8]));
     // the slices of u of the group's workers, zeros past the slice
     for (uint32_t q = tid; q < kg * (ucols / 4u); q += NC * EP_CHAIN) {
         const uint32_t kk = q / (ucols / 4u), c = (q - kk * (ucols / 4u)) * 4u;
@@ -545,7 +536,14 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + (EB == 16 ? EP_PRODUCERS : EP_
         }
         reinterpret_cast<float4 *>(s_u)[q] = v;
     }
+    // (the producers are under way meanwhile)
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     asm volatile("bar.sync 3, %0;" ::"n"(NC * EP_CHAIN) : "memory");
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem_base = s_flag[8];
+    // this thread's lane of the tensor memory, this warp's columns
+    const uint32_t taddr = tmem_base + ((32u * (wg & 3u)) << 16) +
+                           (NC == 2 ? 256u * g + 128u * (wg >> 2) : 256u * (wg >> 2));
 
     Tile T;
     T.start(a);
