@@ -368,6 +368,40 @@ struct Tile {
     }
 };
 
+// The warps' sums of a tile (minibatch t of `worker`) onto the worker's slice of u, which goes out with the
+// last minibatch.
+template <int EB>
+__device__ __forceinline__ void add_to_u(const EpochArgs &a, float *us, const float *part, uint32_t ucols, uint32_t tg,
+                                         uint32_t c0, uint32_t worker, uint32_t nsub, uint32_t t_step)
+{
+    if (tg < ucols / 4u) {
+        const uint32_t c = tg * 4u;
+        float4 o = make_float4(0.f, 0.f, 0.f, 0.f), t = o;
+        if (!a.gradient) o = *reinterpret_cast<const float4 *>(us + c);
+#pragma unroll
+        for (uint32_t w = 0; w < (uint32_t)EP_WARPS; ++w) {
+            if (w < nsub) {
+                const float4 v = *reinterpret_cast<const float4 *>(part + (size_t)w * ucols + c);
+                t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
+            }
+        }
+        t.x += o.x; t.y += o.y; t.z += o.z; t.w += o.w;
+        *reinterpret_cast<float4 *>(us + c) = t;
+        if (t_step == a.nsteps - 1u && c < a.cols && (uint64_t)c0 + c < a.d) {   // the worker's last minibatch
+            float *const to = a.dst + (uint64_t)worker * a.u_stride + c0 + c;
+            if (EB == 16) {
+                *reinterpret_cast<float4 *>(to) = t;
+            } else {
+                const uint64_t have = a.d - c0 - c;
+                to[0] = t.x;
+                if (have > 1u) to[1] = t.y;
+                if (have > 2u) to[2] = t.z;
+                if (have > 3u) to[3] = t.w;
+            }
+        }
+    }
+}
+
 extern __shared__ __align__(1024) unsigned char ep_smem[];
 
 // Shared memory: the ring of slots of SUB x cols floats (a slot holds its boxes of 256 columns one
@@ -549,6 +583,12 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + (EB == 16 ? EP_PRODUCERS : EP_
     T.start(a);
     if (g == 1u) T.next(a, kg);
     uint32_t base = 0u, turn0 = 0u, first0 = 0u;           // the tile's first sub-tile: its slot and turn in the ring, its number
+    // With one chain the next tile, if it is another worker's, does not need this tile's update: its
+    // margins go out first, and the warps' sums are added up while they travel, off the chain of
+    // dependent steps and with one barrier less.  K = 4, n = 512, d = 131072: 246 -> 239 us; K = 3,
+    // n = 640, d = 100000: 152 -> 147.5; K = 4, n = 512, d = 40000, batch 128: 83.5 -> 80.  With two chains the
+    // other one's work lies there already.
+    uint32_t due_kk = 0u, due_nsub = 0u, due_t = 0u;       // the tile whose sums are still to be added (none: no sub-tiles)
     bool read_all = false;                                 // the producer warp knows that this chain needs no margins any more
     for (uint32_t i = g; i < ntiles; i += NC) {
         for (base += T.first - first0; base >= a.nslots; base -= a.nslots) ++turn0;
@@ -634,6 +674,11 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + (EB == 16 ? EP_PRODUCERS : EP_
             }
         }
         tmem_wait_st();
+        if (NC == 1 && due_nsub != 0u) {
+            chain_sync();
+            add_to_u<EB>(a, s_u + (size_t)due_kk * ucols, part, ucols, tg, c0, grp + due_kk * a.G, due_nsub, due_t);   // complete for all at the barrier in W(i)
+            due_nsub = 0u;
+        }
 
         // ---- W(i): all CTAs' partial margins -> step coefficients in shared memory ----
         if (rank == i % a.P) {   // this CTA clears the slot that tile i + RING/2 will add into
@@ -727,39 +772,55 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + (EB == 16 ? EP_PRODUCERS : EP_
                 if (NC == 1 && two) *reinterpret_cast<float4 *>(pw + 128) = s1;
             }
         }
-        chain_sync();
-        if (tg < ucols / 4u) {
-            const uint32_t c = tg * 4u;
-            float4 o = make_float4(0.f, 0.f, 0.f, 0.f), t = o;
-            if (!a.gradient) o = *reinterpret_cast<const float4 *>(us + c);
+        if constexpr (NC == 1) {
+            if (kg > 1u) {
+                due_kk = T.kk;
+                due_nsub = T.nsub;
+                due_t = T.t;
+            } else {
+                chain_sync();
+                add_to_u<EB>(a, us, part, ucols, tg, c0, worker, T.nsub, T.t);
+                chain_sync();                                 // u complete for the next minibatch
+            }
+        } else {   // written out: through the function K = 8, n = 600, d = 30000, batch 100 takes 133.5 us instead of 131.4
+            chain_sync();
+            if (tg < ucols / 4u) {
+                const uint32_t c = tg * 4u;
+                float4 o = make_float4(0.f, 0.f, 0.f, 0.f), t = o;
+                if (!a.gradient) o = *reinterpret_cast<const float4 *>(us + c);
 #pragma unroll
-            for (uint32_t w = 0; w < (uint32_t)EP_WARPS; ++w) {
-                if (w < T.nsub) {
-                    const float4 v = *reinterpret_cast<const float4 *>(part + (size_t)w * ucols + c);
-                    t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
+                for (uint32_t w = 0; w < (uint32_t)EP_WARPS; ++w) {
+                    if (w < T.nsub) {
+                        const float4 v = *reinterpret_cast<const float4 *>(part + (size_t)w * ucols + c);
+                        t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w;
+                    }
+                }
+                t.x += o.x; t.y += o.y; t.z += o.z; t.w += o.w;
+                *reinterpret_cast<float4 *>(us + c) = t;
+                if (T.t == a.nsteps - 1u && c < a.cols && (uint64_t)c0 + c < a.d) {   // the worker's last minibatch
+                    float *const to = a.dst + (uint64_t)worker * a.u_stride + c0 + c;
+                    if (EB == 16) {
+                        *reinterpret_cast<float4 *>(to) = t;
+                    } else {
+                        const uint64_t have = a.d - c0 - c;
+                        to[0] = t.x;
+                        if (have > 1u) to[1] = t.y;
+                        if (have > 2u) to[2] = t.z;
+                        if (have > 3u) to[3] = t.w;
+                    }
                 }
             }
-            t.x += o.x; t.y += o.y; t.z += o.z; t.w += o.w;
-            *reinterpret_cast<float4 *>(us + c) = t;
-            if (T.t == a.nsteps - 1u && c < a.cols && (uint64_t)c0 + c < a.d) {   // the worker's last minibatch
-                float *const to = a.dst + (uint64_t)worker * a.u_stride + c0 + c;
-                if (EB == 16) {
-                    *reinterpret_cast<float4 *>(to) = t;
-                } else {
-                    const uint64_t have = a.d - c0 - c;
-                    to[0] = t.x;
-                    if (have > 1u) to[1] = t.y;
-                    if (have > 2u) to[2] = t.z;
-                    if (have > 3u) to[3] = t.w;
-                }
-            }
+            chain_sync();                                     // u complete for the next minibatch
         }
-        chain_sync();                                     // u complete for the next minibatch
         if (NC == 2 && tg == 0) {
             __threadfence_block();
             s_flag[4u + g] = (i >> 1) + 1u;               // this chain's tiles completed
         }
         for (uint32_t n = 0; n < (uint32_t)NC && i + n + 1u < ntiles; ++n) T.next(a, kg);
+    }
+    if (NC == 1 && due_nsub != 0u) {
+        chain_sync();
+        add_to_u<EB>(a, s_u + (size_t)due_kk * ucols, part, ucols, tg, c0, grp + due_kk * a.G, due_nsub, due_t);
     }
     if (!read_all && wg == 0u)                             // a chain without tiles, or one that gave up
         asm volatile("bar.arrive %0, 64;" ::"r"(4u + g) : "memory");

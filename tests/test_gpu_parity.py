@@ -473,6 +473,29 @@ def test_lr_local_epoch_splits_match_oracle(K, n_local, d, batch):
         _lr_close(got[k], ref.lr_local_epoch(X[rows], y[rows], batch, 0.5, u0))
 
 
+@pytest.mark.parametrize("K,n_local,d,batch", [
+    (2, 40, 131072, 64),     # one step of two workers: every update waits for the other's margins or the end
+    (2, 130, 131072, 64),    # the tile after next is the same worker's again; last minibatch of two rows
+    (5, 70, 100000, 16),     # two sub-tiles a minibatch, fewer than the chain has warps
+    (3, 200, 40000, 128),    # two rounds of sub-tiles per warp
+    (3, 33, 131073, 32),     # element-wise copies, the slice of the last CTA partly outside
+])
+def test_lr_local_epoch_updates_behind_the_next_margins_match_oracle(K, n_local, d, batch):
+    """One chain with several workers: a tile's update is added up after the next tile's margins have
+    gone out.  Every worker is compared, twice for the workspace.  Bound as above (1e-5)."""
+    X, y, _ = synthetic.logistic_problem(K * n_local, d, seed=K + n_local + d)
+    u0 = (0.1 * synthetic.normal_f32(K * d, 1.0, 23)).astype(np.float32).reshape(K, d)
+    c, tX, ty = G.ctx(), G.dev(X), G.dev(y)
+    for _ in range(2):
+        tu = G.dev(u0)
+        c.qesgd_lr_local_epoch_batch(tX, ty, n_local, d, K, batch, 0.5, tu, d)
+        assert c.qesgd_status() == 0
+        got = tu.cpu().numpy()
+        for k in range(K):
+            rows = slice(k * n_local, (k + 1) * n_local)
+            _lr_close(got[k], ref.lr_local_epoch(X[rows], y[rows], batch, 0.5, u0[k]))
+
+
 @pytest.mark.parametrize("gain", [2e7, 1e9])
 def test_local_epoch_partial_margins_beyond_the_fine_fixed_point_range(gain):
     """The CTAs of the persistent kernel add their partial margins as fixed-point integers: units
