@@ -6,7 +6,9 @@
 // took 2.1 us (decode) to 4.2 us (encode_batch, sixteen of them), here 0.3 to 0.6 us.
 //
 // The library is loaded by the Python module (release or debug build), which hands the addresses of
-// its functions to bind(); nothing is linked.
+// its functions to bind(); nothing is linked.  A call with an argument that is not taken here goes back
+// to that module, which makes it through ctypes: what ctypes converts is accepted, what it refuses is
+// refused with its errors.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
@@ -17,33 +19,44 @@
 namespace {
 
 PyObject *g_data_ptr;   // "data_ptr"
+PyObject *g_by_ctypes;  // by_ctypes(name, arguments): the same call through ctypes
 
-// What ctypes took: integers of any size, of which the low bits count; ints or floats for a float.
+// Taken here: integers of any size, of which the low bits count, and what has __index__ (numpy integers,
+// tensors of one integer); what has __float__ for a float.
 struct Args {
     PyObject *const *a;
     Py_ssize_t n, i;
-    bool ok;
-    Args(PyObject *const *args, Py_ssize_t have, Py_ssize_t want) : a(args), n(have), i(0), ok(have == want)
+    bool ok, hand_over;   // hand_over: an argument that is not taken here (no exception is set)
+    Args(PyObject *const *args, Py_ssize_t have, Py_ssize_t want) : a(args), n(have), i(0), ok(have == want), hand_over(false)
     {
         if (!ok) PyErr_Format(PyExc_TypeError, "%zd arguments expected, got %zd", want, have);
+    }
+    void not_taken()
+    {
+        PyErr_Clear();
+        ok = false;
+        hand_over = true;
     }
     uint64_t u64()
     {
         if (!ok) return 0;
         PyObject *const o = a[i++];
-        if (!PyLong_Check(o)) {
-            PyErr_Format(PyExc_TypeError, "argument %zd: int expected instead of %s", i, Py_TYPE(o)->tp_name);
-            ok = false;
+        if (PyLong_Check(o)) return PyLong_AsUnsignedLongLongMask(o);
+        PyObject *const v = PyNumber_Index(o);
+        if (!v) {
+            not_taken();
             return 0;
         }
-        return PyLong_AsUnsignedLongLongMask(o);
+        const uint64_t u = PyLong_AsUnsignedLongLongMask(v);
+        Py_DECREF(v);
+        return u;
     }
     uint32_t u32() { return (uint32_t)u64(); }
     float f32()
     {
         if (!ok) return 0.0f;
         const double v = PyFloat_AsDouble(a[i++]);
-        if (v == -1.0 && PyErr_Occurred()) ok = false;
+        if (v == -1.0 && PyErr_Occurred()) not_taken();
         return (float)v;
     }
     // address held by an int (the context) ...
@@ -60,9 +73,10 @@ struct Args {
             ok = false;
             return nullptr;
         }
-        const uint64_t v = PyLong_AsUnsignedLongLongMask(p);
+        uint64_t v = 0;
+        if (PyLong_Check(p)) v = PyLong_AsUnsignedLongLongMask(p);
+        else not_taken();
         Py_DECREF(p);
-        if (PyErr_Occurred()) ok = false;
         return (T *)(uintptr_t)v;
     }
 };
@@ -77,8 +91,16 @@ ENTRIES(DECLARE)
 
 // Runs the call without the interpreter lock, as ctypes did.
 template <typename F>
-PyObject *result(Args &args, F call)
+PyObject *result(const char *name, Args &args, F call)
 {
+    if (args.hand_over) {
+        PyObject *const all = PyTuple_New(args.n);
+        if (!all) return nullptr;
+        for (Py_ssize_t i = 0; i < args.n; ++i) PyTuple_SET_ITEM(all, i, Py_NewRef(args.a[i]));
+        PyObject *const rc = PyObject_CallFunction(g_by_ctypes, "sO", name, all);
+        Py_DECREF(all);
+        return rc;
+    }
     if (!args.ok) return nullptr;
     int rc;
     Py_BEGIN_ALLOW_THREADS
@@ -91,7 +113,7 @@ PyObject *result(Args &args, F call)
     {                                                                                     \
         Args x(args, n, count);
 #define CALL(name, ...)                                                                   \
-        return result(x, [&] { return f_##name(__VA_ARGS__); });                          \
+        return result(#name, x, [&] { return f_##name(__VA_ARGS__); });                          \
     }
 
 ENTRY(qesgd_encode, 14)
@@ -235,9 +257,11 @@ ENTRY(qesgd_lr_sgd_step_noalloc, 7)
     auto *u = x.tensor<float>();
 CALL(qesgd_lr_sgd_step_noalloc, stream, X, y, m, d, lr, u)
 
-// bind({name: address}): every entry point, before the first call
-PyObject *py_bind(PyObject *, PyObject *table)
+// bind({name: address}, by_ctypes): every entry point, before the first call
+PyObject *py_bind(PyObject *, PyObject *args)
 {
+    PyObject *table, *by_ctypes;
+    if (!PyArg_ParseTuple(args, "OO", &table, &by_ctypes)) return nullptr;
 #define BIND(name)                                                                              \
     {                                                                                           \
         PyObject *v = PyDict_Check(table) ? PyDict_GetItemString(table, #name) : nullptr;       \
@@ -246,11 +270,12 @@ PyObject *py_bind(PyObject *, PyObject *table)
     }
     ENTRIES(BIND)
 #undef BIND
+    Py_XSETREF(g_by_ctypes, Py_NewRef(by_ctypes));
     Py_RETURN_NONE;
 }
 
 #define METHOD(name) {#name, (PyCFunction)(void (*)(void))py_##name, METH_FASTCALL, nullptr},
-PyMethodDef g_methods[] = {ENTRIES(METHOD){"bind", py_bind, METH_O, nullptr}, {nullptr, nullptr, 0, nullptr}};
+PyMethodDef g_methods[] = {ENTRIES(METHOD){"bind", py_bind, METH_VARARGS, nullptr}, {nullptr, nullptr, 0, nullptr}};
 #undef METHOD
 
 PyModuleDef g_module = {PyModuleDef_HEAD_INIT, "_qesgd_py", nullptr, -1, g_methods, nullptr, nullptr, nullptr, nullptr};

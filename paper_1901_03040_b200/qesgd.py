@@ -72,7 +72,15 @@ for _name, (_res, _args) in SIGNATURES.items():
 
 from paper_1901_03040_b200 import _qesgd_py as _native      # noqa: E402  (built with the library)
 
-_native.bind({_name: C.cast(getattr(lib, _name), C.c_void_p).value for _name in SIGNATURES})
+
+def _by_ctypes(name, args):
+    """The call of an entry point some argument of which the native module does not take as it is: an
+    address (the context or a stream), then numbers and tensors."""
+    return getattr(lib, name)(_vp(args[0]), *[
+        _vp(a.data_ptr()) if kind is _vp and a is not None else a for kind, a in zip(SIGNATURES[name][1][1:], args[1:])])
+
+
+_native.bind({_name: C.cast(getattr(lib, _name), _vp).value for _name in SIGNATURES}, _by_ctypes)
 
 
 class QesgdError(RuntimeError):
