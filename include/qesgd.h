@@ -203,9 +203,12 @@ int qesgd_lr_sgd_step(qesgd_ctx *ctx, const float *Xb, const float *yb, uint32_t
                       float lr, float *u);
 /* The summand of Eq. 2 alone: g_out = (1/m) * sum_j grad f_j(w) on the m rows of Xb, for
  * workers that push (quantised) gradients instead of parameters.  w and g_out are float[d]
- * and must not overlap.  One launch of the persistent local-epoch kernel where it takes the shape
- * (see qesgd_lr_local_epoch_batch; its waits are bounded, QESGD_STATUS_TIMEOUT), else one margin pass
- * and one pass that writes the gradient; fp32 arithmetic and accumulation as for qesgd_lr_sgd_step. */
+ * and must not overlap.  One launch of the persistent local-epoch kernel where that takes the shape
+ * on fifteen SMs of sixteen (see qesgd_lr_local_epoch_batch; its waits are bounded,
+ * QESGD_STATUS_TIMEOUT), else one margin pass and one pass that writes the gradient; fp32 arithmetic
+ * and accumulation as for qesgd_lr_sgd_step.  The persistent kernel starts when the SMs it takes are
+ * free of other streams' kernels: a few of those run beside it, gradients of several contexts follow
+ * one another (one of 64 x 65536 on each of four streams: 28 us together, 52 by the two passes). */
 int qesgd_lr_gradient(qesgd_ctx *ctx, const float *Xb, const float *yb, uint32_t m, uint64_t d,
                       const float *w, float *g_out);
 /* Rows [0, n_local) of X in consecutive minibatches of `batch` rows, in row

@@ -969,8 +969,15 @@ int qesgd_launch_lr_epoch_fused(const float *X, const float *y, uint64_t n_local
     if (limit <= 0) return -1;
     const uint32_t nsub = (m_full + SUB - 1) / SUB;
     Split s;
-    // the accumulator word counts up to 256 contributions
-    if (!choose_split(s, d, K, m_full, nsub, tma, (uint32_t)(sm_count < 256 ? sm_count : 256), (uint32_t)limit)) return -1;
+    // A CTA takes a whole SM and none starts before all can, so a call that takes every SM waits for any
+    // kernel of another stream that holds one.  A single step leaves one SM in sixteen free, which costs it
+    // nothing (148, 140, 132 and 128 SMs: 64 x 65536 8.4, 8.3, 8.5, 8.3 us; 64 x 131072 out of HBM 12.4, 12.4,
+    // 12.4, 12.5).  A gradient never takes more: where it only fits all SMs (256 x 37888: 14.4 us), two passes
+    // of small kernels (28.9) run on whatever is free.  The accumulator word counts up to 256 contributions.
+    const uint32_t sms = (uint32_t)(sm_count < 256 ? sm_count : 256);
+    bool fits = nsteps64 * K == 1u && choose_split(s, d, K, m_full, nsub, tma, sms - sms / 16u, (uint32_t)limit);
+    if (!fits && !gradient) fits = choose_split(s, d, K, m_full, nsub, tma, sms, (uint32_t)limit);
+    if (!fits) return -1;
 
     EpochArgs a;
     a.X = X; a.y = y; a.n_local = n_local;

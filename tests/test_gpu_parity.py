@@ -1,6 +1,8 @@
 """GPU parity: the CUDA library, called through its C ABI, against the CPU oracle
 on the same seeded inputs.  Codes and scales must match bit for bit; applied
 parameters within 1e-6 relative; the logistic step within 1e-5 relative."""
+import time
+
 import numpy as np
 import pytest
 
@@ -807,6 +809,43 @@ def test_lr_gradient_shapes_match_oracle(m, d):
     G.ctx().qesgd_lr_gradient(G.dev(X), G.dev(y), m, d, G.dev(w), tg)
     assert G.ctx().qesgd_status() == 0 and (tg[d:] == 9.0).all().item()
     _lr_close(tg[:d].cpu().numpy(), ref.lr_gradient(X, y, w))
+
+
+@pytest.mark.parametrize("m,d,step", [
+    (16, 1000, True), (64, 65536, True), (64, 131072, True), (128, 65536, True),   # TMA, up to one CTA on 15 SMs of 16
+    (33, 100002, True), (64, 65537, True), (256, 4097, True),                      # element-wise copies
+    (64, 142336, True), (256, 35584, True),                                        # the widest on 139 SMs
+    (64, 142340, False), (256, 35588, False), (256, 37888, False), (16, 151552, False),   # the gradient by two passes from here on
+    (300, 5000, True)])
+def test_lr_gradient_and_single_step_run_beside_a_kernel_of_another_stream(m, d, step):
+    """A kernel of one warp holds an SM for some 50 ms; a gradient and, where it leaves an SM in sixteen
+    free, a step on another stream are done before it ends."""
+    X, y, _ = synthetic.logistic_problem(m, d, seed=m + d)
+    w = (0.3 * synthetic.normal_f32(d, 1.0, 8)).astype(np.float32)
+    tX, ty, tw = G.dev(X), G.dev(y), G.dev(w)
+    own, other = torch.cuda.Stream(), torch.cuda.Stream()
+    c = qesgd.Context(0, own)
+    results = []
+    for busy in (False, True):
+        tg, tu = torch.zeros(d, device="cuda"), tw.clone()
+        torch.cuda.synchronize()
+        if busy:
+            with torch.cuda.stream(other):
+                torch.cuda._sleep(100_000_000)
+            time.sleep(0.005)
+        c.qesgd_lr_gradient(tX, ty, m, d, tw, tg)
+        if step:
+            c.qesgd_lr_sgd_step(tX, ty, m, d, 0.5, tu)
+        own.synchronize()
+        assert not busy or not other.query(), "waited for the other stream's kernel"
+        torch.cuda.synchronize()
+        assert c.qesgd_status() == 0
+        results.append((tg, tu))
+    assert torch.equal(results[0][0], results[1][0]) and torch.equal(results[0][1], results[1][1])
+    _lr_close(results[1][0].cpu().numpy(), ref.lr_gradient(X, y, w))
+    if step:
+        _lr_close(results[1][1].cpu().numpy(), ref.lr_sgd_step(X, y, 0.5, w))
+    c.close()
 
 
 @pytest.mark.parametrize("alpha", [-0.1, 1.0, -3.5])
