@@ -988,10 +988,14 @@ int qesgd_launch_lr_epoch_fused(const float *X, const float *y, uint64_t n_local
     a.nsub_last = (a.m_last + SUB - 1) / SUB;
     a.cols = s.cols; a.nit = s.nit; a.nslots = s.nslots;
     a.off_u = s.off_u; a.off_part = s.off_part; a.off_coef = s.off_coef; a.off_bars = s.off_bars; a.off_flags = s.off_flags;
-    // One group with one chain is late for the next tile whenever it was for this one, and gains from
-    // copies spread a little wider (K = 4, n = 512, d = 131072: 260 us without a pace, 256 at 0.6, 245 at
-    // 0.8, 248 at 1.0); all others are best at 0.6 (see the head of the file).
-    a.pace = (uint32_t)((s.G == 1u && s.NC == 1u ? 0.8f : 0.6f) * (float)(SUB * s.cols * 4u * EP_PRODUCERS) * (float)(s.G * s.P) / EP_HBM_BYTES_PER_NS);
+    // Pause between a producer's copies, in parts of the interval at which HBM serves all SMs (see the head of
+    // the file).  One group with one chain is late for the next tile whenever it was for this one, and gains
+    // from copies spread a little wider: 0.6 -> 0.8, K = 4, n = 512, d = 131072 251.9 -> 238.8 us, K = 8,
+    // n = 128 132.5 -> 125.4, K = 1, d = 65536 36.3 -> 35.0, minibatches of 128, d = 75776 35.0 -> 33.9 (K = 4:
+    // 120.0 -> 112.6); only where all of X stays in L2 from call to call is it slower (K = 1, d = 50000,
+    // minibatches of 128 24.7 -> 26.7).  A single tile is late for none: 128 x 75776 11.2 us against 12.4.
+    const float pace = s.G == 1u && s.NC == 1u && nsteps64 * K > 1u ? 0.8f : 0.6f;
+    a.pace = (uint32_t)(pace * (float)(SUB * s.cols * 4u * EP_PRODUCERS) * (float)(s.G * s.P) / EP_HBM_BYTES_PER_NS);
     a.rate = lr / (float)m_full;
     a.rate_last = lr / (float)a.m_last;
     a.u = u; a.dst = dst; a.gradient = gradient ? 1u : 0u; a.u_stride = u_stride;
