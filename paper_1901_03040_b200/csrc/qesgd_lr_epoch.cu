@@ -994,7 +994,11 @@ int qesgd_launch_lr_epoch_fused(const float *X, const float *y, uint64_t n_local
     // n = 128 132.5 -> 125.4, K = 1, d = 65536 36.3 -> 35.0, minibatches of 128, d = 75776 35.0 -> 33.9 (K = 4:
     // 120.0 -> 112.6); only where all of X stays in L2 from call to call is it slower (K = 1, d = 50000,
     // minibatches of 128 24.7 -> 26.7).  A single tile is late for none: 128 x 75776 11.2 us against 12.4.
-    const float pace = s.G == 1u && s.NC == 1u && nsteps64 * K > 1u ? 0.8f : 0.6f;
+    // Two chains whose ring holds no more than half a minibatch (many workers: their slices of u take the
+    // room) leave no slot free for long and wait for one another's copies: 0.6 -> 0.9, K = 64, n = 64,
+    // d = 65536 (four slots) 261 -> 253 us, d = 75776 (three) 334 -> 330; with five slots the copies already
+    // run ahead and a wider pace only costs (K = 48, d = 75776 176 -> 201, K = 56, d = 65536 200 -> 217).
+    const float pace = s.G == 1u && s.NC == 1u && nsteps64 * K > 1u ? 0.8f : s.NC == 2u && 2u * s.nslots <= nsub ? 0.9f : 0.6f;
     a.pace = (uint32_t)(pace * (float)(SUB * s.cols * 4u * EP_PRODUCERS) * (float)(s.G * s.P) / EP_HBM_BYTES_PER_NS);
     a.rate = lr / (float)m_full;
     a.rate_last = lr / (float)a.m_last;

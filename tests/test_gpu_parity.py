@@ -475,6 +475,29 @@ def test_lr_local_epoch_splits_match_oracle(K, n_local, d, batch):
         _lr_close(got[k], ref.lr_local_epoch(X[rows], y[rows], batch, 0.5, u0))
 
 
+@pytest.mark.parametrize("K,n_local,d", [(64, 70, 65536),     # two chains and a ring of four slots
+                                         (64, 65, 75776),     # three slots
+                                         (32, 66, 131072)])   # one chain, three slots
+def test_lr_local_epoch_of_many_workers_with_a_ring_shorter_than_a_minibatch(K, n_local, d):
+    """The slices of u of all workers of a group stay in shared memory and leave the ring fewer slots than a
+    minibatch of 64 rows has sub-tiles.  X is drawn on the device (1.2 GB); bound as above (1e-5)."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(K + d)
+    tX = torch.randn(K * n_local, d, device="cuda", generator=g) / d ** 0.5
+    ty = torch.where(torch.rand(K * n_local, device="cuda", generator=g) < 0.5, -1.0, 1.0)
+    u0 = (0.1 * synthetic.normal_f32(d, 1.0, 22)).astype(np.float32)
+    c, runs = G.ctx(), []
+    for _ in range(2):
+        tu = G.dev(u0).repeat(K, 1)
+        c.qesgd_lr_local_epoch_batch(tX, ty, n_local, d, K, 64, 0.5, tu, d)
+        assert c.qesgd_status() == 0
+        runs.append(tu)
+    assert torch.equal(runs[0], runs[1])
+    for k in (0, K // 2 + 1, K - 1):
+        rows = slice(k * n_local, (k + 1) * n_local)
+        _lr_close(runs[0][k].cpu().numpy(), ref.lr_local_epoch(tX[rows].cpu().numpy(), ty[rows].cpu().numpy(), 64, 0.5, u0))
+
+
 @pytest.mark.parametrize("K,n_local,d,batch", [
     (2, 40, 131072, 64),     # one step of two workers: every update waits for the other's margins or the end
     (2, 130, 131072, 64),    # the tile after next is the same worker's again; last minibatch of two rows
