@@ -162,9 +162,11 @@ int qesgd_launch_lr_step(const float *Xb, uint64_t x_worker_stride, const float 
                          float *u, uint64_t u_stride, float *work, uint64_t work_floats,
                          cudaStream_t stream, int *launched);
 // A minibatch that does not fit L2 is read a second time from its end: what the margin pass, which walks
-// the columns upwards, read last is still there.  Measured (second pass included): 64 x 2^22 sgd_step 324 ->
-// 318 us, qstep 343 -> 337; 64 x 2^19 54 -> 50; where the minibatch fits, the plain order is the better
-// one (16 x 2^20, 67 MB: 31.8 against 33.8).
+// the workers and their columns upwards, read last is still there.  Measured (second pass included): 64 x 2^22
+// sgd_step 324 -> 318 us, qstep 343 -> 337; 64 x 2^19 54 -> 50; where the minibatch fits, the plain order is the
+// better one (16 x 2^20, 67 MB: 31.8 against 33.8).  Several workers, m the rows of all of them, against the
+// columns alone turned round: K = 4, n = 256, d = 160000, minibatches of 64 258 -> 233 us, K = 8, n = 64,
+// d = 400000, of 16 374 -> 347, K = 16, n = 600, d = 20000, of 300 302 -> 298; K = 32, n = 512, of 512 404 -> 409.
 inline bool qesgd_second_pass_reversed(uint64_t m, uint64_t d) { return m * d * 4u > (96ull << 20); }
 // The margin pass alone (pass 1 of a step) for one worker; *parts_out receives the number of
 // partial margins per row that the pass leaves in `work` ([parts][m]).

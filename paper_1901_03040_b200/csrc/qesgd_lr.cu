@@ -159,14 +159,15 @@ __global__ void __launch_bounds__(256) qesgd_lr_margin_kernel(const LrArgs a)
 // Pass 2.  A CTA updates UPD_COLS consecutive columns: 64 column groups of 4 columns
 // times UPD_ROWGROUPS row groups; row group g sums rows g, g + G, g + 2G, ... (coalesced
 // 1 KB per row), the G partial sums meet in shared memory in fixed order.
-// REV: from the last columns to the first (see qesgd_second_pass_reversed).
+// REV: from the last worker to the first and from the last columns to the first (see
+// qesgd_second_pass_reversed).
 template <bool VEC, bool REV>
 __global__ void __launch_bounds__(UPD_THREADS) qesgd_lr_update_kernel(const LrArgs a)
 {
     __shared__ float s_coef[QESGD_MAX_LR_BATCH];
     __shared__ float4 s_sum[UPD_ROWGROUPS][UPD_COLS / 4];
     qesgd_wait_for_previous();
-    const uint32_t k = blockIdx.y;
+    const uint32_t k = REV ? gridDim.y - 1u - blockIdx.y : blockIdx.y;
     const float *__restrict__ X = a.X + (uint64_t)k * a.x_stride;
     const float *__restrict__ y = a.y + (uint64_t)k * a.y_stride;
     float *__restrict__ u = a.dst + (uint64_t)k * a.u_stride;

@@ -499,6 +499,26 @@ def test_lr_local_epoch_of_many_workers_with_a_ring_shorter_than_a_minibatch(K, 
 
 
 @pytest.mark.parametrize("K,n_local,d,batch", [
+    (3, 40, 300001, 32),     # element by element, a last minibatch in forward order
+    (4, 24, 280000, 24),     # 107 MB in one step
+    (2, 260, 50004, 257),    # more than 256 rows of two workers, 103 MB, and three rows
+    (2, 300, 1001, 300),     # element by element, small: forward
+])
+def test_lr_two_pass_steps_of_several_workers_match_oracle(K, n_local, d, batch):
+    """Two passes per minibatch; above 96 MiB in all the second one goes from the last worker and column to
+    the first.  Every worker from a point of its own, every row of the result.  Bound as above (1e-5)."""
+    X, y, _ = synthetic.logistic_problem(K * n_local, d, seed=K + n_local + d)
+    u0 = (0.1 * synthetic.normal_f32(K * d, 1.0, 23)).astype(np.float32).reshape(K, d)
+    c, tu = G.ctx(), G.dev(u0)
+    c.qesgd_lr_local_epoch_batch(G.dev(X), G.dev(y), n_local, d, K, batch, 0.5, tu, d)
+    assert c.qesgd_status() == 0
+    got = tu.cpu().numpy()
+    for k in range(K):
+        rows = slice(k * n_local, (k + 1) * n_local)
+        _lr_close(got[k], ref.lr_local_epoch(X[rows], y[rows], batch, 0.5, u0[k]))
+
+
+@pytest.mark.parametrize("K,n_local,d,batch", [
     (2, 40, 131072, 64),     # one step of two workers: every update waits for the other's margins or the end
     (2, 130, 131072, 64),    # the tile after next is the same worker's again; last minibatch of two rows
     (5, 70, 100000, 16),     # two sub-tiles a minibatch, fewer than the chain has warps
