@@ -309,37 +309,56 @@ def test_decode_average_apply_matches_oracle(K, bucket, bits, s):
     _assert_param_close(got, want, w, scales, bucket)
 
 
+def _fused_sums(codes_signed, step, bucket, order, fmaf):
+    """sum_k code * spacing in fp32, one rounding per worker, in the order given."""
+    acc = np.zeros(codes_signed.shape[1], dtype=np.float32)
+    for k in order:
+        acc = fmaf(codes_signed[k].astype(np.float32), np.repeat(step[k], bucket), acc)
+    return acc
+
+
+def _spacing_case(bits, s, K, bucket=64, nb=112):
+    """Streams of K workers whose spacings have all 24 bits and, within a bucket, exponents up to 8 apart
+    (so that additions round); buckets from 2^-113 to 2^100, several at either border of the range
+    in which 4- and 8-bit codes are summed scaled, in tiles wholly inside it, wholly outside and mixed."""
+    rng = np.random.default_rng(bits * 100 + K)
+    centre = np.concatenate([np.full(8, -109), np.arange(-103, -80, 4), np.full(12, -79), np.full(12, 17), [-80, -78, 16, 18, 19], np.arange(20, 100, 8),
+                             rng.integers(-70, 10, nb)])[:nb]
+    centre[8:64] = rng.permutation(centre[8:64])
+    exps = centre[None, :] + np.where(centre < -90, rng.integers(-4, 1, (K, nb)), rng.integers(-4, 5, (K, nb)))
+    scales = np.ldexp(rng.integers(1 << 23, 1 << 24, (K, nb)) / float(1 << 23), exps).astype(np.float32) * np.float32(s)
+    step = (scales / np.float32(s)).astype(np.float32)
+    levels = rng.integers(0, s + 1, (K, bucket * nb)).astype(np.uint32)
+    signs = (rng.integers(0, 2, levels.shape) * (levels > 0)).astype(np.uint32)
+    per = 32 // bits
+    codes = ((signs << (bits - 1)) | levels).reshape(K, -1, per)
+    words = np.bitwise_or.reduce(codes << (np.arange(per, dtype=np.uint32) * bits), axis=2).astype(np.uint32)
+    return words, scales, step, np.where(signs == 1, -1.0, 1.0) * levels
+
+
 @pytest.mark.parametrize("K", [1, 6, 7, 10, 16, 32])
 @pytest.mark.parametrize("bits,s", [(4, 7), (8, 127)])
 def test_decode_average_apply_is_the_plain_sum_for_every_spacing(bits, s, K):
     """4- and 8-bit codes are summed in units scaled by powers of two, and plainly where a spacing lies
-    outside the range in which that is exact (2^-79 to 2^18).  Scales from 1e-30 to 3e38 / s, within and
-    outside that range and at its borders, all codes: the result is, bit for bit, the fp32 sum by fused
-    multiply-adds over the workers in order, times 1/K, added to the parameter.  (numpy has no fused
-    multiply-add: a level times a spacing is exact in fp64 -- 7 + 24 bits --, so is its sum with an fp32
-    number rounded once to fp64 and then to fp32 unless that lies within 2^-53 of a tie, which the inputs
-    avoid: they have at most 16 significant bits.)"""
-    bucket, nb = 64, 96
-    n = bucket * nb
-    rng = np.random.default_rng(bits * 100 + K)
-    exps = np.concatenate([np.arange(-90, -70, 2), [-79, -78, 17, 18, 19], rng.integers(-70, 17, nb - 25),
-                           np.arange(100, 120, 2)])[:nb]
-    step = np.ldexp(rng.integers(128, 256, (K, nb)) / 256.0, exps[None, :]).astype(np.float32)
-    scales = (step * np.float32(s)).astype(np.float32)
-    step = (scales / np.float32(s)).astype(np.float32)
-    levels = rng.integers(0, s + 1, (K, n)).astype(np.uint32)
-    signs = (rng.integers(0, 2, (K, n)) * (levels > 0)).astype(np.uint32)
-    per = 32 // bits
-    codes = ((signs << (bits - 1)) | levels).reshape(K, n // per, per)
-    words = np.bitwise_or.reduce(codes << (np.arange(per, dtype=np.uint32) * bits), axis=2).astype(np.uint32)
-    acc = np.zeros(n, dtype=np.float32)
-    for k in range(K):
-        v = np.where(signs[k] == 1, -1.0, 1.0) * levels[k] * np.repeat(step[k], bucket).astype(np.float64)
-        acc = (acc.astype(np.float64) + v).astype(np.float32)
-    w = np.zeros(n, dtype=np.float32)
-    want = w + acc * np.float32(np.float32(1.0) / np.float32(K))
-    got = G.gpu_decode_average_apply(w, words, scales, bucket, s, bits)
-    assert np.array_equal(got, want)
+    outside [2^-79, 2^18).  The result is, bit for bit, the fp32 sum by fused multiply-adds (the C
+    library's) over the workers in order, times 1/K, added to the parameter.  The inputs tell it from a
+    sum in another order and from a sum that stays scaled below the range (both computed here)."""
+    import ctypes
+    import ctypes.util
+    libm = ctypes.CDLL(ctypes.util.find_library("m"))
+    libm.fmaf.restype, libm.fmaf.argtypes = ctypes.c_float, [ctypes.c_float] * 3
+    fmaf = np.vectorize(libm.fmaf, otypes=[np.float32])
+    bucket = 64
+    words, scales, step, codes = _spacing_case(bits, s, K, bucket)
+    acc = _fused_sums(codes, step, bucket, range(K), fmaf)
+    got = G.gpu_decode_average_apply(np.zeros(acc.size, dtype=np.float32), words, scales, bucket, s, bits)
+    assert np.array_equal(got, acc * np.float32(np.float32(1.0) / np.float32(K)))
+    if K > 2:
+        assert (_fused_sums(codes, step, bucket, range(K - 1, -1, -1), fmaf) != acc).mean() > 0.2
+    low = slice(0, 8 * bucket)               # spacings below 2^-108
+    with np.errstate(under="ignore"):
+        scaled = _fused_sums(codes[:, low] * 2.0 ** -133, step[:, :8] * np.float32(2.0) ** 110, bucket, range(K), fmaf)
+        assert (scaled * np.float32(2.0 ** 23) != acc[low]).mean() > 0.1
 
 
 @pytest.mark.parametrize("n", [1, 9, 255, 256, 257, 2049])
@@ -403,14 +422,14 @@ def test_lr_local_epoch_and_batch_match_oracle():
     (4, 96, 65536, 32),      # the benchmark's width (444 columns per CTA, two TMA boxes)
     (5, 77, 1000, 20),       # odd K, rows not a multiple of 8, ragged last minibatch of 17
     (3, 300, 2048, 256),     # the largest minibatch the persistent kernel takes
-    (2, 40, 75776, 8),       # the widest slice (512 columns per CTA)
+    (2, 40, 75776, 8),       # slices of 512 columns
     (2, 600, 1024, 300),     # minibatch above 256 rows: two-pass steps
-    (2, 64, 1002, 32),       # d not a multiple of 4: two-pass steps
-    (2, 64, 80000, 32),      # d above 512 columns per SM: two-pass steps
+    (2, 64, 1002, 32),       # d not a multiple of 4: element-wise copies
+    (2, 64, 80000, 32),      # slices of 544 columns
 ])
 def test_lr_local_epoch_shapes_match_oracle(K, n_local, d, batch):
     """The local epoch through the C ABI against the fp64 oracle, over shapes that take the
-    persistent kernel (shared-memory tiles, inter-CTA margins) and shapes that fall back to
+    persistent kernel (tiles on chip, inter-CTA margins) and shapes that fall back to
     one margin pass and one update pass per minibatch."""
     X, y, _ = synthetic.logistic_problem(K * n_local, d, seed=K + n_local + d)
     u0 = (0.1 * synthetic.normal_f32(d, 1.0, 21)).astype(np.float32)
@@ -600,8 +619,12 @@ def _epoch_once(c, X, y, n_local, d, K, batch, u0):
 
 
 @pytest.mark.parametrize("K,n_local,d,batch", [
-    (2, 96, 8192, 32),       # minibatches stashed in tensor memory between their two uses
-    (3, 200, 4096, 100),     # minibatches that stay in shared memory, odd K
+    (2, 96, 8192, 32),       # two chains
+    (3, 200, 4096, 100),     # two chains, odd K, 13 sub-tiles
+    (2, 40, 131072, 64),     # one chain, several workers: sums added up behind the next margins
+    (1, 100, 20000, 64),     # one chain, one worker
+    (2, 70, 10003, 32),      # element by element: 4-byte copies, several CTAs
+    (1, 70, 50002, 32),      # 8-byte copies
 ])
 def test_local_epoch_wait_runs_out_and_the_context_recovers(K, n_local, d, batch):
     """One CTA never announces its partial margins of the first minibatch (a flag nothing
@@ -631,12 +654,34 @@ def test_local_epoch_wait_runs_out_and_the_context_recovers(K, n_local, d, batch
     c.close()
 
 
-def test_local_epoch_with_a_wait_limit_below_the_timer_resolution():
+@pytest.mark.parametrize("m,d", [(64, 65536), (40, 10003)])
+def test_lr_gradient_wait_runs_out_and_the_context_recovers(m, d):
+    """The same for the mean gradient, by TMA and element by element."""
+    X, y, _ = synthetic.logistic_problem(m, d, seed=m)
+    w = (0.1 * synthetic.normal_f32(d, 1.0, 22)).astype(np.float32)
+    tX, ty, tw = G.dev(X), G.dev(y), G.dev(w)
+    c, g = qesgd.Context(0, None), torch.zeros(d, device="cuda")
+    c.qesgd_set_wait_limit(3_000_000)
+    c.qesgd_debug_drop_signal(5)
+    c.qesgd_lr_gradient(tX, ty, m, d, tw, g)
+    assert c.qesgd_status() == qesgd.STATUS_TIMEOUT
+    c.qesgd_debug_drop_signal(-1)
+    c.qesgd_set_wait_limit(0)
+    c.qesgd_lr_gradient(tX, ty, m, d, tw, g)
+    assert c.qesgd_status() == 0
+    _lr_close(g.cpu().numpy(), ref.lr_gradient(X, y, w))
+    want = torch.zeros(d, device="cuda")
+    G.ctx().qesgd_lr_gradient(tX, ty, m, d, tw, want)
+    assert torch.equal(g, want)
+    c.close()
+
+
+@pytest.mark.parametrize("K,n_local,d,batch", [(4, 256, 16384, 32), (2, 200, 131072, 64), (2, 100, 10003, 32), (1, 100, 50002, 32)])
+def test_local_epoch_with_a_wait_limit_below_the_timer_resolution(K, n_local, d, batch):
     """A limit under a microsecond means "look once more, then give up": ordinary latency
     between CTAs and of the TMA copies exhausts it at whatever point each CTA happens to be,
     so the give-up path is entered from many places at once.  The call must return either way;
     a run that happened to need no second look is a complete epoch.  The context recovers."""
-    K, n_local, d, batch = 4, 256, 16384, 32
     X, y, _ = synthetic.logistic_problem(K * n_local, d, seed=9)
     u0 = (0.1 * synthetic.normal_f32(d, 1.0, 23)).astype(np.float32)
     tX, ty = G.dev(X), G.dev(y)
@@ -753,6 +798,8 @@ def test_qesgd_inner_loop_on_the_gpu_follows_the_oracle():
     (33, 4100, 64, 4, 7, ref.SCALE_MAX, True),         # ragged last tile, odd row count
     (256, 8192, 1024, 2, 1, ref.SCALE_FIXED, True),    # widest bucket the fused kernel takes
     (16, 524288, 256, 4, 7, ref.SCALE_NORM, True),     # 512 column segments: 296 CTAs in the margin pass
+    (64, 400004, 512, 8, 127, ref.SCALE_NORM, True),   # 102 MB: tiles from the last, which is ragged; rows 16-byte aligned
+    (64, 400384, 1024, 4, 7, ref.SCALE_MAX, True),     # the same, rows 32-byte aligned
     (64, 8192, 4096, 8, 100, ref.SCALE_NORM, False),   # bucket above 1024: the two calls
     (20, 1002, 128, 4, 7, ref.SCALE_NORM, False),      # d not a multiple of 4: the two calls
 ])
@@ -770,9 +817,9 @@ def test_fused_inner_step_equals_step_then_requantize(m, d, bucket, bits, s, mod
     tX, ty = G.dev(X), G.dev(y)
     # the gradient step alone, in the arithmetic the fused call uses
     u1 = G.dev(u0)
-    if fused:
+    if fused and d <= 151552:
         qesgd.qesgd_lr_sgd_step_noalloc(None, tX, ty, m, d, lr, u1)      # always the two-pass form
-    else:
+    else:                                                                # beyond, the context's step too
         c.qesgd_lr_sgd_step(tX, ty, m, d, lr, u1)
     torch.cuda.synchronize()
     u1 = u1.cpu().numpy()
@@ -841,8 +888,11 @@ def test_fused_inner_step_at_the_edges_of_its_tiles(m, d, bucket, bits, s, mode,
     assert (codes.cpu().numpy().view(np.uint32) == want[2]).all()
 
 
-@pytest.mark.parametrize("m,d", [(200, 5001), (33, 65541), (17, 150001),    # rows split over 13, 2 and 1 CTAs per segment
-                                 (64, 150000), (256, 30000), (1, 4), (64, 419432), (100, 250001), (64, 9999)])
+@pytest.mark.parametrize("m,d", [
+    (200, 5001), (33, 65541), (256, 30000), (1, 4), (64, 9999),     # the persistent kernel
+    (300, 5001), (1000, 20000), (17, 150001), (64, 150000),         # two passes, rows split over 19, 7, 1 and 1 CTAs per segment
+    (64, 419432), (100, 250001),                                    # 107 MB backwards, 100.0 MB (below 96 MiB) forwards
+    (100, 260001)])                                                 # backwards, element by element
 def test_lr_gradient_shapes_match_oracle(m, d):
     """Both forms of the gradient: two passes with the rows split over CTAs where segments are few, and
     the persistent kernel as an epoch of one step.  fp32 sums of d (margins) and m terms against fp64."""
