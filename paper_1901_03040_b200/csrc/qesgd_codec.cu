@@ -776,7 +776,8 @@ __global__ void __launch_bounds__(WARPS * 32,
 // groups of eight columns, two rows of each requested at a time, take 128 registers: four CTAs per SM,
 // 128 KB of loads in flight.  Against the kernel before (one warp of eight quantised a tile that all
 // had summed into shared memory), margin pass included: 64 x 2^22 369 -> 335 us, 128 x 2^20 193 -> 176,
-// 16 x 2^20 53 -> 33, 256 x 4096 33 -> 23.
+// 16 x 2^20 53 -> 33, 256 x 4096 33 -> 23.  Rows of X, u, anchor or running sum off 32-byte boundaries (d = 4 mod 8)
+// take every tile through the ragged form: 64 x (2^22 + 4) 377 -> 355, 64 x (2^20 + 4) 111 -> 91, 128 x (2^20 + 4) 198 -> 180.
 constexpr int QS_WARPS = 4;
 constexpr int QS_THREADS = QS_WARPS * 32;
 constexpr int QS_TILE = QS_WARPS * CHUNK;      // columns per CTA

@@ -34,15 +34,20 @@ static const uint64_t QESGD_MAX_WAIT_NS = 10000000000ull;
 // Workspace (4 MiB): partial margins of the two-pass steps, K * P * m floats, and behind them what the
 // persistent kernel's CTAs exchange: a header of 16 words per group of CTAs, then for each of 8 ring
 // slots the accumulators (four 64-bit words and three of space per row) of up to
-// QESGD_LR_EPOCH_ROWS rows of all groups.
+// QESGD_LR_EPOCH_ROWS rows of all groups.  With all 2^20 floats for the partial margins no step is faster
+// (64 workers, minibatches of 1024 rows of 4096 columns, 11 parts a worker or 14: 306 and 304 us; 8 workers,
+// 98 parts or 126: 90.1 and 90.1).
 static const uint32_t QESGD_LR_EPOCH_ROWS = 2048;
 static const uint64_t QESGD_LR_EPOCH_FLOATS = QESGD_MAX_WORKERS * 16ull + 8ull * QESGD_LR_EPOCH_ROWS * 14ull;
 static const uint64_t QESGD_LR_WORK_FLOATS = (1ull << 20) - QESGD_LR_EPOCH_FLOATS;
 
-// Every kernel of the library is launched so that it may be set up while the kernel before it in the
-// stream drains (programmatic dependent launch), and begins with qesgd_wait_for_previous: nothing is
-// read or written before that one is done and its writes are visible.  No kernel lets its successor
-// start earlier than at its own end: a waiting grid would take resident slots.  Without it a
+// Kernels that go through qesgd_launch may be set up while the kernel before them in the stream drains
+// (programmatic dependent launch), and begin with qesgd_wait_for_previous: nothing is read or written
+// before that one is done and its writes are visible.  The cooperative local-epoch kernel and the debug
+// build's range self-test do not: they are launched plainly, start when all before them is done and contain
+// no such wait, so they must not be given the attribute without one (in the epoch kernel ahead of the
+// producers' first copy and the consumers' loads of u).  No kernel lets its successor
+// start earlier than at its own end: a waiting grid would take resident slots.  Without the overlap a
 // kernel costs a whole number of about 2.05 us in a stream: encode + decode-average-apply of 4 x 30000
 // 11.3 -> 5.9 us, of 8 x 10^6 18.5 -> 14.4, decode of 2^24 13.9 -> 11.3, a logistic step of 64 x 2^22
 // 319 -> 311, and no grid was found that is slower.  (With griddepcontrol.launch_dependents at the top of

@@ -20,7 +20,7 @@ constexpr int SEG = 1024;        // columns per segment in pass 1 (32 lanes x 8 
 #define QESGD_LR_MAX_PARTS 296
 #endif
 constexpr int MAX_PARTS = QESGD_LR_MAX_PARTS;   // CTAs of the margin pass per worker: two per SM of a B200
-constexpr int ROW_CTAS = 148;    // rows are split over CTAs up to this many
+constexpr int ROW_CTAS = 148;    // rows are split over CTAs up to this many: one per SM of a B200
 constexpr int DONE_WORDS = 64;   // one arrival counter per worker at the head of the workspace
 // pass 2: eight CTAs per SM with 32 registers, so no run-time choice of direction (36 registers, six CTAs:
 // 16 x 2^20 32.8 -> 34.9 us)
@@ -247,9 +247,10 @@ uint64_t lay_out_work(LrArgs &a, float *work, uint64_t work_floats, uint32_t K, 
     a.work = work + head;
     a.parts = (uint32_t)parts;
     // Too few column segments for the SMs: the rows are split as well, sixteen (two per warp, one trip of
-    // the row loop) to a CTA at the least.  A gradient of 200 x 5001 37 -> 22 us, a step of 64 x 30002
-    // 18.6 -> 16.6; with more CTAs than SMs the arrivals at the end cost more than the trips saved
-    // (64 x 131072, margins and fused second pass: 21.0, at 296 CTAs 24.7).
+    // the row loop) to a CTA at the least.  A gradient of 300 x 5001 45.5 -> 23.1 us, of 1000 x 20000 121 -> 69;
+    // a step without a context of 64 x 30002 15.4 -> 11.0, of 256 x 4096 21.9 -> 12.1; a fused inner step of
+    // 256 x 4096 26.8 -> 17.3.  With more CTAs than SMs the arrivals at the end cost more than the trips
+    // saved (64 x 131072, margins and fused second pass: 21.0, at 296 CTAs 24.7).
     const uint32_t trips = (m + 15u) / 16u;
     uint32_t groups = parts > 0 && K * parts < (uint64_t)ROW_CTAS ? ROW_CTAS / (uint32_t)(K * parts) : 1u;
     a.row_groups = groups < trips ? groups : trips;

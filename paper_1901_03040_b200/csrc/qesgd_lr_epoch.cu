@@ -14,18 +14,20 @@
 //                   warps, one thread of each, take the slots in turn: looking at the slot, arming
 //                   its barrier and issuing two to four boxes takes a thread about 650 clocks, which
 //                   with one producer bounded the whole kernel at 27 bytes per clock and SM.  Two are best:
-//                   K = 4, n = 2048, d = 65536: 409 us with one, 350, 348 and 349 with two, three and
-//                   four; K = 8, n = 1010, d = 10000: 121, 83, 89, 90; K = 4, n = 512, d = 131072:
-//                   270, 268, 279, 295 (more requests at once delay the exchange between the CTAs).
+//                   K = 4, n = 2048, d = 65536: 441 us with one, 329, 337 and 341 with two, three and
+//                   four; K = 8, n = 1010, d = 10000: 127, 81, 87, 88; K = 8, n = 512, d = 65536: 224, 167,
+//                   177, 175 (more requests at once delay the exchange between the CTAs); only the widest
+//                   slices do better with one (K = 4, n = 512, d = 131072: 236, 240, 237, 247).
 //                   For the same reason a producer leaves a pause between two copies: the CTAs free
 //                   their slots in step, right after the exchange, and refilled at once by all of them
 //                   the copies of one SM queue behind another's, the slowest of which everybody then
 //                   waits for.  At 0.6 of the interval at which HBM can serve every SM the first
-//                   shape takes 330 us, the HBM time of X (349 without a pause; 330 at 0.5, 347 at 0.7,
-//                   381 at 0.8); K = 8, n = 512, d = 65536: 183 -> 169.  The pause is kept by the global
+//                   shape takes 329 us, the HBM time of X (343 without a pause; 327 at 0.5, 362 at 0.7,
+//                   394 at 0.8); K = 8, n = 512, d = 65536: 179 -> 168.  The pause is kept by the global
 //                   timer (32 ns a tick), not in clocks: under the power cap the SM clock falls by a
-//                   quarter, and a pause that grew with it would hold HBM back (a round of the first
-//                   shape, repeated for a second: 381 us by clocks, 373 by the timer, 377 without a pause)
+//                   quarter, and a pause that grew with it would hold HBM back (whole rounds of the first
+//                   shape, repeated for a second, were 1 % slower than without a pause by clocks, 1 %
+//                   faster by the timer)
 //   consumer chain  eight warps; tile i = minibatch i / Kg of the group's worker i % Kg:
 //     M(i)  warp w takes the sub-tiles w, w + 8, ...: partial margins of the rows over the slice;
 //           the values it reads go to tensor memory on the way (tcgen05.st), so the slot returns
@@ -43,8 +45,8 @@
 // coefficients: 64 rows x 512 columns for each of two chains or x 1024 columns for one.
 // Measured against the kernel this one replaces (one group, u in global memory, tiles kept in two
 // shared-memory buffers, at most 512 columns per SM): K = 8, n = 1010, d = 10000, batch 50:
-// 429 -> 126 us; K = 4, n = 128, d = 4096, batch 32: 38 -> 17; K = 4, n = 512, d = 131072 (two
-// passes before): 426 -> 275; K = 4, n = 2048, d = 65536: 461 -> 421.
+// 434 -> 81 us; K = 4, n = 128, d = 4096, batch 32: 37.6 -> 14.4; K = 4, n = 512, d = 131072 (two
+// passes before): 426 -> 240; K = 4, n = 2048, d = 65536: 460 -> 329; K = 64, n = 64, d = 65536: 255 -> 253.
 //
 // Exchange through global memory: each row's partial margin is added, as a fixed-point integer,
 // to the row's accumulator acc[i % RING][row] by one 64-bit reduction that also counts the
@@ -95,7 +97,7 @@ constexpr int EP_BOX_COLS = 256;     // widest TMA box
 constexpr int EP_MAX_M = EP_CHAIN;   // rows per minibatch: a thread of the chain per row
 constexpr int EP_MAX_SLOTS = 64;     // ring slots
 constexpr uint32_t EP_FLAG_BYTES = (16 + EP_MAX_SLOTS) * 4;
-constexpr float EP_HBM_BYTES_PER_NS = 6550.0f;
+constexpr float EP_HBM_BYTES_PER_NS = 6500.0f;   // what HBM delivers to all SMs together
 constexpr int EP_PRODUCERS = 2;      // producer warps with TMA
 constexpr int EP_LOADERS = 8;        // producer warps with element-wise copies
 constexpr int EP_UNITS = 8;          // 8 x 128 blocks of a tile that the tensor memory holds per warp
@@ -411,9 +413,9 @@ extern __shared__ __align__(1024) unsigned char ep_smem[];
 // multiple of 4, or unaligned vectors); eight producer warps copy 4 or 8 bytes at a time instead
 // (cp.async, completion on the same barriers, elements outside the matrix as zeros) and u is read and
 // written element by element.  One chain.  Bound by the copies' instructions (128 or 256 bytes each),
-// but against two passes of scalar loads per minibatch: K = 4, n = 512, d = 16383: 196 -> 45 us; K = 8,
-// n = 1010, d = 10001: 461 -> 132; one minibatch of 64 x 65537: 22 -> 11.5; K = 4, n = 2048, d = 65538:
-// 1168 -> 696.
+// but against two passes of scalar loads per minibatch: K = 4, n = 512, d = 16383: 193 -> 45 us; K = 8,
+// n = 1010, d = 10001: 465 -> 132; one minibatch of 64 x 65537: 19.6 -> 10.3; K = 4, n = 2048, d = 65538:
+// 1173 -> 670.
 template <int NC, int EB>
 __global__ void __launch_bounds__(NC * EP_CHAIN + (EB == 16 ? EP_PRODUCERS : EP_LOADERS) * 32, 1)
     qesgd_lr_epoch_kernel(const EpochArgs a, const __grid_constant__ CUtensorMap map_full,
@@ -782,7 +784,10 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + (EB == 16 ? EP_PRODUCERS : EP_
                 add_to_u<EB>(a, us, part, ucols, tg, c0, worker, T.nsub, T.t);
                 chain_sync();                                 // u complete for the next minibatch
             }
-        } else {   // written out: through the function K = 8, n = 600, d = 30000, batch 100 takes 133.5 us instead of 131.4
+        } else {
+            // add_to_u written out: through the function K = 4, n = 2048, d = 65536 takes 333.6 us instead of
+            // 329.5, K = 8, n = 512 171.0 instead of 167.5
+            static_assert(NC == 1 || EB == 16, "two chains are fed by TMA");
             chain_sync();
             if (tg < ucols / 4u) {
                 const uint32_t c = tg * 4u;
@@ -797,18 +802,8 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + (EB == 16 ? EP_PRODUCERS : EP_
                 }
                 t.x += o.x; t.y += o.y; t.z += o.z; t.w += o.w;
                 *reinterpret_cast<float4 *>(us + c) = t;
-                if (T.t == a.nsteps - 1u && c < a.cols && (uint64_t)c0 + c < a.d) {   // the worker's last minibatch
-                    float *const to = a.dst + (uint64_t)worker * a.u_stride + c0 + c;
-                    if (EB == 16) {
-                        *reinterpret_cast<float4 *>(to) = t;
-                    } else {
-                        const uint64_t have = a.d - c0 - c;
-                        to[0] = t.x;
-                        if (have > 1u) to[1] = t.y;
-                        if (have > 2u) to[2] = t.z;
-                        if (have > 3u) to[3] = t.w;
-                    }
-                }
+                if (T.t == a.nsteps - 1u && c < a.cols && (uint64_t)c0 + c < a.d)   // the worker's last minibatch
+                    *reinterpret_cast<float4 *>(a.dst + (uint64_t)worker * a.u_stride + c0 + c) = t;
             }
             chain_sync();                                     // u complete for the next minibatch
         }
@@ -917,7 +912,7 @@ bool complete_split(Split &s, uint64_t d, uint32_t K, uint32_t m, uint32_t nsub,
     s.off_bars = s.off_coef + s.NC * EP_MAX_M * 4u;
     s.off_flags = s.off_bars + 2u * EP_MAX_SLOTS * 8u;
     s.bytes = s.off_flags + EP_FLAG_BYTES;
-    const float hbm = (float)((double)K * m * d * 4.0 / 6.5e6);          // us at 6.5 TB/s
+    const float hbm = (float)((double)K * m * d * 4.0 / (1000.0 * EP_HBM_BYTES_PER_NS));   // us
     const float chain = EP_CHAIN_US + EP_UNIT_US * (float)units;
     const float chained = chain * (float)kg / (float)s.NC;
     s.us = hbm > chained ? hbm : chained;
@@ -948,9 +943,9 @@ bool choose_split(Split &best, uint64_t d, uint32_t K, uint32_t m, uint32_t nsub
 
 // Returns 0 = launched, -1 = shape not covered by the fused kernel (caller uses the
 // two-pass steps), > 0 = cudaError_t.
-// A single minibatch's mean gradient is an epoch of one step with lr = -1 that does not add u: at 64 x
-// 65536 10.4 us instead of 16.5 for the margin pass and the update pass, at 256 x 37888 14.6 instead of
-// 42.3 (two launches, and most SMs idle in the first).
+// A single minibatch's mean gradient is an epoch of one step with lr = -1 that does not add u: minibatches
+// of 64 x 65536 out of HBM 10.3 us instead of 16.5 for the margin pass and the update pass, of 256 x 35584
+// 13.1 instead of 37.7 (two launches, and most SMs idle in the first).
 int qesgd_launch_lr_epoch_fused(const float *X, const float *y, uint64_t n_local, uint64_t d,
                                 uint32_t K, uint32_t batch, float lr, const float *u, float *dst,
                                 bool gradient, uint64_t u_stride, float *work, uint32_t *status, int device, int sm_count, uint64_t wait_ns,
