@@ -911,7 +911,7 @@ def test_lr_gradient_shapes_match_oracle(m, d):
     (64, 142340, False), (256, 35588, False), (256, 37888, False), (16, 151552, False),   # the gradient by two passes from here on
     (300, 5000, True)])
 def test_lr_gradient_and_single_step_run_beside_a_kernel_of_another_stream(m, d, step):
-    """A kernel of one warp holds an SM for some 50 ms; a gradient and, where it leaves an SM in sixteen
+    """A kernel of one warp holds an SM for some 200 ms; a gradient and, where it leaves an SM in sixteen
     free, a step on another stream are done before it ends."""
     X, y, _ = synthetic.logistic_problem(m, d, seed=m + d)
     w = (0.3 * synthetic.normal_f32(d, 1.0, 8)).astype(np.float32)
@@ -924,7 +924,7 @@ def test_lr_gradient_and_single_step_run_beside_a_kernel_of_another_stream(m, d,
         torch.cuda.synchronize()
         if busy:
             with torch.cuda.stream(other):
-                torch.cuda._sleep(100_000_000)
+                torch.cuda._sleep(400_000_000)
             time.sleep(0.005)
         c.qesgd_lr_gradient(tX, ty, m, d, tw, tg)
         if step:
