@@ -191,52 +191,78 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
     return d;
 }
-__device__ __forceinline__ uint64_t fma2_ru(uint64_t a, uint64_t b, uint64_t c)   // toward +inf
+__device__ __forceinline__ uint64_t add2_ru(uint64_t a, uint64_t b)   // toward +inf
 {
     uint64_t d;
-    asm("fma.rp.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    asm("add.rp.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
     return d;
 }
 
 // ------------------------------------------------------- rounding (Eq. 4) ----
 // level = floor(r) + [h + 1/2 < frac(r) * 2^16] for r = min(|z|*inv, s), 0 <= r <= 127.
 //
-// With U = ceil(r * 2^16 - 1/2) the level is (U + 65535 - h) >> 16: writing U =
-// floor(r) * 2^16 + T, T = ceil(frac(r) * 2^16 - 1/2) in [0, 2^16], the draw rounds
-// up iff h < T.  U comes from ONE fused multiply-add rounded toward +infinity:
-// r * 2^16 + (2^23 - 1/2) lies in [2^23, 2^24) where floats are the integers, so
-// the bit pattern of the result is 0x4B000000 + U.  r is kept >= 2^-30 so that
-// r = 0 (where the sum would be 2^23 - 1/2 exactly, below the integer binade)
-// gives U = 0 like every r with r * 2^16 <= 1/2; the same clamp turns the NaN of
-// an invalid bucket (inv = 0) into level 0.
-// Two neighbouring elements at a time: the multiply and the fused multiply-add run on
-// packed pairs, the clamp stays scalar (it takes |.| for free).  x0, x1 receive the level
-// in bits 16..22 (what is below is of no interest).
+// Codes of 2 and 4 bits (s <= 7).  With V = ceil(r * 2^17) the level is (V + 131070 - 2h) >> 17: writing
+// V = floor(r) * 2^17 + ceil(f), f = frac(r) * 2^17, the sum carries iff ceil(f) >= 2h + 2, that is iff
+// f > 2h + 1.  inv comes multiplied by 2^17 (a power of two: the product is r * 2^17 bit for bit, or both
+// are too small to matter), and ONE addition of 2^23 + 131070 rounded toward +infinity leaves
+// 0x4B000000 + 131070 + V as bit pattern, because floats in [2^23, 2^24) are the integers.
+// Codes of 8 bits: seven bits of level and seventeen below do not fit the 23 bits of that binade.  With
+// U = ceil(r * 2^16 - 1/2) the level is (U + 65535 - h) >> 16 by the same argument.  |t| - 1/2 is exact where
+// t = r * 2^16 is at least 1/2 (it has t's spacing or more and is no larger) and otherwise lies in [-1/2, 0],
+// rounded up or not; adding 2^23 + 65535 rounded toward +infinity leaves 0x4B000000 + 65535 + U either way.
+// The scalar additions take |t| as an operand modifier, so there is neither a clamp at zero nor an operation for
+// the magnitude; and the draw, one 16-bit half of a Philox word, is subtracted by a dot product of the word's
+// halves with (-2, 0) or (0, -2), so the halves are never taken apart.  Against multiply, clamp, multiply-add,
+// mask or shift, and a three-input addition: 2.5 or 3 instructions per element for 4, and the shorter chain shows
+// (encode + apply: 16 x 25.6 M 2-bit 459 -> 443 us, 8 x 2^28 4-bit 2706 -> 2611, 5 x 10^6 4-bit 11.19 -> 10.83).
+//
 // CLIP: only a caller-given spacing needs the upper clamp min(r, s).  With a scale taken
 // from the bucket itself |z| <= scale, and inv = fl32(s/scale) is at most (s/scale) *
 // (1 + 2^-24), so the exact product is below s + ulp(s) and its fp32 rounding is s or
 // s + ulp(s).  (Where s/scale is subnormal -- scale > s * 2^126, so s < 4 -- inv is off by
 // at most 2^-150 and the product by at most 2^128 * 2^-150 = 2^-22.)  Either way r - s <=
-// 2^-17 for s <= 127, i.e. at most 1/2 after the scaling by 2^16, and ceil(s * 2^16 + 1/2
-// - 1/2) is still s * 2^16: the overshoot never reaches a level, so the clamp would change
-// nothing.
-template <bool CLIP>
-__device__ __forceinline__ void level_pair(float z0, float z1, uint64_t inv2, float sf,
-                                           uint32_t h0, uint32_t h1, uint32_t &x0, uint32_t &x1)
+// 2^-17 for s <= 127, so V <= s * 2^17 + 1 and U = s * 2^16: the overshoot never reaches a level, and the clamp
+// would change nothing.  The lower clamp of that mode turns a NaN into level 0; without CLIP no z is NaN or
+// infinite here (encode_warp_tile takes them out with their bucket).
+// x0, x1 receive the level in bits 17..19 (2- and 4-bit codes) or 16..22 under 0x4B in byte 3 and a zero bit
+// 23; what is below is of no interest.
+template <int BITS>
+struct Level {
+    static constexpr float UNIT = BITS == 8 ? 65536.0f : 131072.0f;                     // r is taken in units of 1 / UNIT
+    static constexpr float BASE = 8388608.0f + (BITS == 8 ? 65535.0f : 131070.0f);
+    static constexpr uint32_t SHIFT = BITS == 8 ? 16u : 17u;
+    static constexpr uint32_t DRAW = BITS == 8 ? 0xFFu : 0xFEu;                         // -1 or -2 in a signed byte
+};
+// c + a.low half * b.byte 0 + a.high half * b.byte 1, halves unsigned, bytes signed
+__device__ __forceinline__ uint32_t dot2(uint32_t a, uint32_t b, uint32_t c)
 {
-    float t0, t1;
+    uint32_t d;
+    asm("dp2a.lo.u32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+    return d;
+}
+// Two neighbouring elements at a time; h = their two draws, `top` = s * UNIT.
+template <int BITS, bool CLIP>
+__device__ __forceinline__ void level_pair(float z0, float z1, uint64_t inv2, float top, uint32_t h,
+                                           uint32_t &x0, uint32_t &x1)
+{
+    typedef Level<BITS> L;
+    float t0, t1, f0, f1;
     unpack2(mul2(pack2f(z0, z1), inv2), t0, t1);           // sign rides along, removed by |.|
-    float r0 = fmaxf(fabsf(t0), 0x1p-30f);
-    float r1 = fmaxf(fabsf(t1), 0x1p-30f);
     if (CLIP) {
-        r0 = fminf(r0, sf);
-        r1 = fminf(r1, sf);
+        t0 = fminf(fmaxf(fabsf(t0), 0.0f), top);
+        t1 = fminf(fmaxf(fabsf(t1), 0.0f), top);
+        uint64_t t = pack2f(t0, t1);
+        if (BITS == 8) t = add2_ru(t, pack2f(-0.5f, -0.5f));
+        unpack2(add2_ru(t, pack2f(L::BASE, L::BASE)), f0, f1);
+    } else if (BITS == 8) {
+        unpack2(add2_ru(pack2f(__fadd_ru(fabsf(t0), -0.5f), __fadd_ru(fabsf(t1), -0.5f)), pack2f(L::BASE, L::BASE)),
+                f0, f1);
+    } else {
+        f0 = __fadd_ru(fabsf(t0), L::BASE);
+        f1 = __fadd_ru(fabsf(t1), L::BASE);
     }
-    float u0, u1;
-    unpack2(fma2_ru(pack2f(r0, r1), pack2f(65536.0f, 65536.0f), pack2f(8388607.5f, 8388607.5f)),
-            u0, u1);
-    x0 = __float_as_uint(u0) - h0 + (65535u - 0x4B000000u);
-    x1 = __float_as_uint(u1) - h1 + (65535u - 0x4B000000u);
+    x0 = dot2(h, L::DRAW, __float_as_uint(f0));
+    x1 = dot2(h, L::DRAW << 8, __float_as_uint(f1));
 }
 
 // (a & b) | c and (a & b) ^ c as one three-input logic operation each
@@ -253,12 +279,11 @@ __device__ __forceinline__ uint32_t and_xor(uint32_t a, uint32_t b, uint32_t c)
     return d;
 }
 
-// Packing.  X[j] holds the level of element j in byte 2 (bits 16..22) and Z[j] the
-// sign of z_j in bit 31.  Bytes are gathered with PRMT, fields merged with
+// Packing.  X[j] holds the level of element j in byte 2 (bits 16..22, or 17..19 above a bit of no interest) and
+// Z[j] the sign of z_j in bit 31.  Bytes are gathered with PRMT, fields merged with
 // multiply-adds; the sign is kept only where the level is not zero, which is
 // tested on whole words (a field plus its largest level never carries).
-// X[j] = U + 65535 - h lies in [0, 2^23), so its byte 3 is always zero and serves as the
-// source of zero bytes.  PRMT's replicate mode (selector nibble 8 + n) turns the top bit of
+// PRMT's replicate mode (selector nibble 8 + n) turns the top bit of
 // byte n into a whole byte of ones or zeros, so a sign lands on any bit of its byte by a
 // mask alone, without a shift.
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
@@ -267,7 +292,7 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel)
     asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(sel));
     return d;
 }
-__device__ __forceinline__ uint32_t bytes2(uint32_t a, uint32_t b)   // [a.b2, b.b2, 0, 0]
+__device__ __forceinline__ uint32_t bytes2(uint32_t a, uint32_t b)   // [a.b2, b.b2, ., .]
 {
     return prmt(a, b, 0x3362u);
 }
@@ -297,7 +322,7 @@ __device__ __forceinline__ void pack_octet(const uint32_t (&X)[8], const uint32_
         // even elements fill the low nibbles, odd elements the high nibbles
         const uint32_t le = __byte_perm(__byte_perm(X[0], X[2], 0x0062), __byte_perm(X[4], X[6], 0x0062), 0x5410);
         const uint32_t lo = __byte_perm(__byte_perm(X[1], X[3], 0x0062), __byte_perm(X[5], X[7], 0x0062), 0x5410);
-        const uint32_t lv = le + lo * 16u;
+        const uint32_t lv = ((le + lo * 16u) >> 1) & 0x77777777u;
         const uint32_t se = __byte_perm(signs2(Z[0], Z[2]), signs2(Z[4], Z[6]), 0x5410);
         const uint32_t so = __byte_perm(signs2(Z[1], Z[3]), signs2(Z[5], Z[7]), 0x5410);
         const uint32_t sg = and_or(se, 0x08080808u, so & 0x80808080u);
@@ -307,11 +332,11 @@ __device__ __forceinline__ void pack_octet(const uint32_t (&X)[8], const uint32_
         // element j sits at bits 2j, 2j+1: byte 0 holds elements 0..3, byte 1 elements 4..7
         const uint32_t g0 = bytes2(X[0], X[4]), g1 = bytes2(X[1], X[5]);
         const uint32_t g2 = bytes2(X[2], X[6]), g3 = bytes2(X[3], X[7]);
-        const uint32_t lv = (g0 + g1 * 4u) + (g2 * 16u + g3 * 64u);
+        const uint32_t lv = (g0 + g1 * 4u) + (g2 * 16u + g3 * 64u);   // a level on each odd bit, the rest above bit 16
         const uint32_t h0 = signs2(Z[0], Z[4]), h1 = signs2(Z[1], Z[5]);
         const uint32_t h2 = signs2(Z[2], Z[6]), h3 = signs2(Z[3], Z[7]);
         const uint32_t sg = and_or(h3, 0x8080u, and_or(h2, 0x2020u, and_or(h1, 0x0808u, h0 & 0x0202u)));
-        out[0] = lv | (sg & (lv << 1));
+        out[0] = and_or(sg, lv, (lv >> 1) & 0x5555u);
         out[1] = 0u;
     }
 }
@@ -562,11 +587,19 @@ __device__ __forceinline__ void encode_warp_tile(const EncodeArgs &a, float (&z)
     {
         const bool nonfinite = !(my_scale <= 3.402823466e38f);   // Inf or NaN (scales are >= 0)
         const bool ok = !nonfinite && my_scale >= 0x1p-100f;
-        my_inv = ok ? __fdiv_rn(sf, my_scale) : 0.0f;
+        my_inv = ok ? __fmul_rn(__fdiv_rn(sf, my_scale), Level<BITS>::UNIT) : 0.0f;
         my_scale = ok ? my_scale : 0.0f;
         if (REQ) my_delta = __fdiv_rn(my_scale, sf);   // grid spacing of the decoder
         // Lanes past the padded length hold zeros, so a set flag always belongs to real data.
         flag = nonfinite;
+    }
+    // Rare: the codes of a bucket that is not finite are 0.  Its inv is 0, so its finite elements come out so.
+    if (MODE != 2 && __any_sync(0xFFFFFFFFu, flag)) {
+#pragma unroll
+        for (int c = 0; c < V; ++c)
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                if ((__float_as_uint(z[c][j]) & 0x7FFFFFFFu) >= 0x7F800000u) z[c][j] = 0.0f;
     }
 
     // ---- rounding, packing, stores ---------------------------------------------
@@ -577,9 +610,9 @@ __device__ __forceinline__ void encode_warp_tile(const EncodeArgs &a, float (&z)
         float scale = my_scale, inv = my_inv, delta = my_delta;
         if (MODE != 2 && V > 1) {   // fetch chunk c's bucket scale from the neighbour lane that carried it
             const int src = (int)lane_of_chunk<V>(lane, c);
-            scale = __shfl_sync(FULL, my_scale, src);
-            inv = __shfl_sync(FULL, my_inv, src);
-            if (REQ) delta = __shfl_sync(FULL, my_delta, src);
+            scale = __shfl_sync(0xFFFFFFFFu, my_scale, src);
+            inv = __shfl_sync(0xFFFFFFFFu, my_inv, src);
+            if (REQ) delta = __shfl_sync(0xFFFFFFFFu, my_delta, src);
         }
         if (inside) {      // the first lane of every bucket writes its scale
             if (!wide) {
@@ -611,8 +644,7 @@ __device__ __forceinline__ void encode_warp_tile(const EncodeArgs &a, float (&z)
             Z[j + 1] = __float_as_uint(z[c][j + 1]);
             if (MODE == 2)   // NaN has no place on the grid: flagged (and encoded as 0 by the clamp)
                 flag |= (Z[j] & 0x7FFFFFFFu) > 0x7F800000u || (Z[j + 1] & 0x7FFFFFFFu) > 0x7F800000u;
-            level_pair<MODE == 2>(z[c][j], z[c][j + 1], inv2, sf, x[j >> 1] & 0xFFFFu, x[j >> 1] >> 16,
-                       X[j], X[j + 1]);
+            level_pair<BITS, MODE == 2>(z[c][j], z[c][j + 1], inv2, sf * Level<BITS>::UNIT, x[j >> 1], X[j], X[j + 1]);
         }
         if constexpr (REQ) {
             // decode what was just quantised: +-level * delta, the sign only where level > 0
@@ -623,9 +655,10 @@ __device__ __forceinline__ void encode_warp_tile(const EncodeArgs &a, float (&z)
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 if (FULL) w[j] = wb.w[c][j];
-                const uint32_t lv = X[j] >> 16;
-                const float lf = __fsub_rn(__uint_as_float(0x4B000000u | lv), 8388608.0f);
-                const uint32_t sign31 = Z[j] & (lv + 0x7FFFFFFFu) & 0x80000000u;
+                // the bits below the level cleared: the float 2^23 + level << SHIFT
+                const uint32_t lv = X[j] & ~((1u << Level<BITS>::SHIFT) - 1u);
+                const float lf = fmaf(__uint_as_float(lv), 1.0f / Level<BITS>::UNIT, -8388608.0f / Level<BITS>::UNIT);
+                const uint32_t sign31 = Z[j] & (lv + (0x7FFFFFFFu - 0x4B000000u)) & 0x80000000u;
                 v[j] = __uint_as_float(__float_as_uint(__fmul_rn(lf, delta)) | sign31);
                 w[j] = __fadd_rn(w[j], v[j]);
             }

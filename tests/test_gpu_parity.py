@@ -254,6 +254,30 @@ def test_negative_zero_and_exact_ties_match_the_oracle():
         _assert_streams_equal(got, want)
 
 
+@pytest.mark.parametrize("bits,s", [(2, 1), (4, 1), (4, 7), (8, 1), (8, 64), (8, 127)])
+@pytest.mark.parametrize("mode", [ref.SCALE_MAX, ref.SCALE_FIXED])
+def test_levels_at_the_boundary_of_their_own_draw(bits, s, mode):
+    """Every element lies exactly where its own draw decides, |z|/spacing = level + (2h + 1)/2^17, one fp32 number
+    above or one below, for levels from 0 to s - 1, between zeros of both signs, tiny values and the top level.
+    The spacing is a power of two (the first element of a bucket is s of them), so the quotient is exact."""
+    bucket, nb, delta = 64, 64, np.float32(2.0 ** -9)
+    n = bucket * nb
+    h = np.array([ref.draw16(5, 3, 2, i) for i in range(n)], dtype=np.float64)
+    rng = np.random.default_rng(bits * 1000 + s)
+    level = rng.integers(0, s, n)
+    r = (level + (2 * h + 1) / 131072.0).astype(np.float32)
+    kind = np.arange(n) % 8
+    r = np.where(kind == 1, np.nextafter(r, np.float32(200)), np.where(kind == 2, np.nextafter(r, np.float32(0)), r))
+    r = np.where(kind == 3, np.float32(0), np.where(kind == 4, np.float32(2.0 ** -40), r))
+    r = np.where(kind == 5, np.float32(s), r).astype(np.float32)
+    z = (r * delta * rng.choice(np.float32([-1, 1]), n)).astype(np.float32)
+    z[::bucket] = s * delta
+    args = (bucket, s, bits, mode, 5, 3, 2)
+    got, want = G.gpu_encode(z, None, *args, fixed_delta=float(delta)), ref.encode(z, None, *args, fixed_delta=float(delta))
+    _assert_streams_equal(got, want)
+    assert got[2] == 0
+
+
 def test_on_grid_input_round_trips_exactly_on_the_gpu():
     s, bits, bucket = 127, 8, 256
     rng = np.random.default_rng(4)
