@@ -26,6 +26,7 @@ UNITS = [
     ("qesgd_codec.cu", "qesgd_codec_8.o", ["-fmad=false", "-DQESGD_BITS=8"]),
     ("qesgd_lr.cu", "qesgd_lr.o", []),
     ("qesgd_lr_epoch.cu", "qesgd_lr_epoch.o", []),
+    ("qesgd_lr_tile.cu", "qesgd_lr_tile.o", []),
     ("qesgd_api.cu", "qesgd_api.o", []),
 ]
 
@@ -59,7 +60,8 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False) -> st
     -DQESGD_DEBUG (the codec kernels check their indices and set QESGD_STATUS_RANGE)."""
     os.makedirs(OBJ, exist_ok=True)
     build_py_module(force)
-    headers = [os.path.join(CSRC, "qesgd_internal.h"), os.path.join(ROOT, "include", "qesgd.h"),
+    headers = [os.path.join(CSRC, "qesgd_internal.h"), os.path.join(CSRC, "qesgd_lr_device.cuh"),
+               os.path.join(CSRC, "qesgd_lr_tile.h"), os.path.join(ROOT, "include", "qesgd.h"),
                os.path.abspath(__file__)]
     nvcc = _nvcc()
     objs = []

@@ -43,6 +43,7 @@
 // where one group holds several workers two chains (NC = 2) alternate over its tiles, one
 // computing while the other waits.  The tensor memory (256 KB) holds what waits for its
 // coefficients: 64 rows x 512 columns for each of two chains or x 1024 columns for one.
+// Epochs of few columns per CTA, where that chain is all the time there is, go to qesgd_lr_tile.cu.
 // Measured against the kernel this one replaces (one group, u in global memory, tiles kept in two
 // shared-memory buffers, at most 512 columns per SM): K = 8, n = 1010, d = 10000, batch 50:
 // 434 -> 81 us; K = 4, n = 128, d = 4096, batch 32: 37.6 -> 14.4; K = 4, n = 512, d = 131072 (two
@@ -81,19 +82,16 @@
 // memory.  The one wait without a bound is the tensor-memory allocation at the start, which
 // blocks while another kernel resident on the same SM holds tensor memory (until that kernel
 // ends).
-#include <cuda.h>
-
 #include <mutex>
 
-#include "qesgd_internal.h"
+#include "qesgd_lr_device.cuh"
+#include "qesgd_lr_tile.h"
 
 namespace {
 
 constexpr int EP_WARPS = 8;                       // consumer warps of a chain
 constexpr int EP_CHAIN = EP_WARPS * 32;
-constexpr int SUB = 8;               // rows per sub-tile
-constexpr int EP_RING = 8;           // accumulator slots; a slot is cleared RING/2 tiles before its use
-constexpr int EP_BOX_COLS = 256;     // widest TMA box
+constexpr int EP_BOX_COLS = 256;     // widest TMA box; element-wise copies keep whole rows together
 constexpr int EP_MAX_M = EP_CHAIN;   // rows per minibatch: a thread of the chain per row
 constexpr int EP_MAX_SLOTS = 64;     // ring slots
 constexpr uint32_t EP_FLAG_BYTES = (16 + EP_MAX_SLOTS) * 4;
@@ -102,19 +100,6 @@ constexpr int EP_PRODUCERS = 2;      // producer warps with TMA
 constexpr int EP_LOADERS = 8;        // producer warps with element-wise copies
 constexpr int EP_UNITS = 8;          // 8 x 128 blocks of a tile that the tensor memory holds per warp
 constexpr float EP_CHAIN_US = 2.5f, EP_UNIT_US = 0.25f;   // a tile's latency: exchange, and per block of a warp
-constexpr uint64_t DRAIN_LIMIT_NS = 2000000000ull;   // the producers' last wait for their own copies
-constexpr uint64_t COARSE_TIMER_NS = 1024ull;        // limits below this mean "one look, then give up"
-constexpr uint32_t EP_HEADER_WORDS = 16;             // per group: [0] abort flag, [1] CTAs that have read their last margins
-constexpr uint32_t EP_ACC_PITCH = 32;                // 64-bit words from one 8-row group of accumulators to the next
-constexpr uint32_t EP_WIDE_WORDS = 3;                // rarely used 64-bit words per accumulator row
-constexpr float FX_SCALE = 268435456.0f;             // 2^28: unit of the first word
-constexpr float FX_LIMIT = 131072.0f;                // 2^17: partials below go to the first word
-constexpr float FX_WIDE_SCALE = 64.0f;               // 2^6: unit of the second word
-constexpr float FX_WIDE_LIMIT = 562949953421312.0f;  // 2^49: partials below go to the second word
-constexpr unsigned long long FX_BIAS = 1ull << 45;   // makes every contribution to the first word positive
-constexpr unsigned long long FX_ONE = 1ull << 55;    // one contribution counted
-constexpr unsigned long long FX_SPECIAL = 1ull << 54;   // one of the row's other words is in use
-
 struct EpochArgs {
     const float *X;         // element-wise copies only
     const float *y;
@@ -141,120 +126,6 @@ struct EpochArgs {
     uint32_t poll_mask;     // the clock is read every (poll_mask + 1) looks at a counter
     uint32_t drop_cta;      // test hook: this CTA does not count itself for tile 0 (none: ~0)
 };
-
-// ------------------------------------------------------------- primitives ----
-__device__ __forceinline__ uint32_t smem_u32(const void *p)
-{
-    return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ uint64_t now_ns()
-{
-    uint64_t t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-                 "r"(bytes)
-                 : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n"
-        ".reg .pred p;\n"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        "selp.u32 %0, 1, 0, p;\n"
-        "}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0u;
-}
-// Has a wait that began at t0 used up `limit`?  The global timer may tick as coarsely as a
-// microsecond, so a smaller limit is read as "give up after one round of looks".
-__device__ __forceinline__ bool expired(uint64_t t0, uint64_t limit)
-{
-    return limit < COARSE_TIMER_NS || now_ns() - t0 > limit;
-}
-// Bounded wait for phase `parity` of a barrier; gives up early when `*stop` is set.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, const volatile uint32_t *stop,
-                                          uint64_t limit)
-{
-    if (mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = now_ns();
-    for (;;) {
-        for (int n = 0; n < 32; ++n)
-            if (mbar_try_wait(bar, parity)) return true;
-        if (*stop != 0u || expired(t0, limit)) return false;
-    }
-}
-// Bounded wait until the counter *flag, which another warp of this CTA advances, exceeds `value`.
-__device__ __forceinline__ bool flag_above(const volatile uint32_t *flag, uint32_t value,
-                                           const volatile uint32_t *stop, uint64_t limit)
-{
-    if (*flag > value) return true;
-    const uint64_t t0 = now_ns();
-    for (;;) {
-        for (int n = 0; n < 32; ++n)
-            if (*flag > value) return true;
-        if (*stop != 0u || expired(t0, limit)) return false;
-    }
-}
-// One 2-D box of the row-major matrix X: columns [x, x + box width), rows [y, y + SUB).
-// x * 4 bytes is a multiple of 16; dst is 128-byte aligned.  The copy goes to this CTA alone.
-__device__ __forceinline__ void tma_load_box(float *dst, const CUtensorMap *map, uint32_t x, uint32_t y,
-                                             uint64_t *bar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::
-            "r"(smem_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_u32(bar))
-        : "memory");
-}
-__device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p)
-{
-    uint32_t v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long *p)
-{
-    unsigned long long v;
-    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-
-// Barrier `id` of `count` threads that also answers one question the same way for all of them:
-// has any of them seen `flag` set?  (Each thread reads the flag for itself; a plain barrier
-// followed by separate reads could send the threads different ways while another warp sets it,
-// and the ones that stay would then wait at the next barrier for the ones that left.)
-__device__ __forceinline__ bool sync_any(uint32_t id, uint32_t count, uint32_t flag)
-{
-    uint32_t r;
-    asm volatile(
-        "{\n"
-        ".reg .pred p, q;\n"
-        "setp.ne.u32 q, %1, 0;\n"
-        "bar.red.or.pred p, %2, %3, q;\n"
-        "selp.u32 %0, 1, 0, p;\n"
-        "}"
-        : "=r"(r)
-        : "r"(flag), "r"(id), "r"(count)
-        : "memory");
-    return r != 0u;
-}
 
 // ---- tensor memory as a stash for a tile between its two uses --------------------------
 // The SM's 256 KB of tensor memory (128 lanes x 512 columns of 32 bits) is not needed for
@@ -298,52 +169,6 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float4 (&v)[8])
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-// EB bytes from global to shared memory, asynchronously; zeros where `inside` does not hold (then
-// nothing is read).
-template <int EB>
-__device__ __forceinline__ void copy_elements(uint32_t dst, const float *src, bool inside)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(dst), "l"(src), "n"(EB == 8 ? 8 : 4),
-                 "r"(inside ? (EB == 8 ? 8 : 4) : 0)
-                 : "memory");
-}
-// One arrival on the barrier when all copies of this thread so far have landed.
-__device__ __forceinline__ void arrive_when_copied(uint64_t *bar)
-{
-    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
-// Sum over the 32 lanes of 8 per-lane values at once: three halving exchanges leave one
-// value per lane, two plain butterflies finish.  Lane L ends with the total of value
-// 4*bit4(L) + 2*bit3(L) + bit2(L); the order of the additions is fixed.
-__device__ __forceinline__ float reduce8(float (&v)[8], uint32_t lane)
-{
-    const bool h4 = lane & 16u, h3 = lane & 8u, h2 = lane & 4u;
-    float a[4], b[2];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        const float keep = h4 ? v[r + 4] : v[r], send = h4 ? v[r] : v[r + 4];
-        a[r] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, 16);
-    }
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        const float keep = h3 ? a[r + 2] : a[r], send = h3 ? a[r] : a[r + 2];
-        b[r] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, 8);
-    }
-    const float keep = h2 ? b[1] : b[0], send = h2 ? b[0] : b[1];
-    float c = keep + __shfl_xor_sync(0xFFFFFFFFu, send, 4);
-    c += __shfl_xor_sync(0xFFFFFFFFu, c, 2);
-    c += __shfl_xor_sync(0xFFFFFFFFu, c, 1);
-    return c;
-}
-__device__ __forceinline__ uint32_t reduce8_row(uint32_t lane)
-{
-    return ((lane >> 4) & 1u) * 4u + ((lane >> 3) & 1u) * 2u + ((lane >> 2) & 1u);
-}
-
-// Where row j's accumulator lies within its ring slot: eight rows in a row, the eights 256 bytes apart.
-__device__ __forceinline__ uint32_t acc_index(uint32_t j) { return (j / SUB) * EP_ACC_PITCH + j % SUB; }
 
 // A tile of a group: minibatch t of the group's worker kk; `first` is the number of its first
 // sub-tile.  Stepped, not divided out: an integer division takes 240 clocks, a small step 3500.
@@ -421,6 +246,7 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + (EB == 16 ? EP_PRODUCERS : EP_
     qesgd_lr_epoch_kernel(const EpochArgs a, const __grid_constant__ CUtensorMap map_full,
                           const __grid_constant__ CUtensorMap map_rest)
 {
+    constexpr uint32_t BOX = EB == 16 ? EP_BOX_COLS : 1024u, BOX_UNITS = BOX / 128u;   // columns that lie together in a slot
     constexpr uint32_t PRODUCERS = EB == 16 ? EP_PRODUCERS : EP_LOADERS;
     const uint32_t slot_floats = SUB * a.cols, ucols = a.nit * 128u;
     float *const ring = reinterpret_cast<float *>(ep_smem);
@@ -487,15 +313,12 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + (EB == 16 ? EP_PRODUCERS : EP_
                     constexpr uint32_t N = EB / 4;
                     const uint32_t rows = min(T.m - s * SUB, (uint32_t)SUB);
                     const float *const src = a.X + (uint64_t)row * a.d + c0;
-                    for (uint32_t b0 = 0u; b0 < a.cols; b0 += EP_BOX_COLS) {
-                        const uint32_t width = min(a.cols - b0, (uint32_t)EP_BOX_COLS);
-                        for (uint32_t r = 0; r < rows; ++r) {
-                            const float *const line = src + (uint64_t)r * a.d + b0;
-                            const uint32_t to = smem_u32(dst + SUB * b0 + r * width);
+                    for (uint32_t r = 0; r < rows; ++r) {
+                        const float *const line = src + (uint64_t)r * a.d;
+                        const uint32_t to = smem_u32(dst + r * a.cols);
 #pragma unroll 4
-                            for (uint32_t c = lane * N; c < width; c += 32u * N)
-                                copy_elements<EB>(to + c * 4u, line + c, (uint64_t)c0 + b0 + c < a.d);
-                        }
+                        for (uint32_t c = lane * N; c < a.cols; c += 32u * N)
+                            copy_elements<EB>(to + c * 4u, line + c, (uint64_t)c0 + c < a.d);
                     }
                     arrive_when_copied(&full[slot]);
                 }
@@ -633,8 +456,8 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + (EB == 16 ? EP_PRODUCERS : EP_
             for (int r = 0; r < SUB; ++r) acc[r] = 0.0f;
 #pragma unroll 1
             for (uint32_t it = 0; it < a.nit; ++it) {
-                const uint32_t b0 = (it >> 1) * EP_BOX_COLS, c = it * 128u + lane * 4u;
-                const uint32_t pitch = min(a.cols - b0, (uint32_t)EP_BOX_COLS);
+                const uint32_t b0 = it / BOX_UNITS * BOX, c = it * 128u + lane * 4u;
+                const uint32_t pitch = min(a.cols - b0, BOX);
                 const float *const base = xs + SUB * b0 + (c - b0);
                 const float4 uu = *reinterpret_cast<const float4 *>(us + c);
                 float4 x[SUB];
@@ -868,19 +691,22 @@ int epoch_smem_limit(int device)
     return g_epoch_smem_limit[device];
 }
 
-// Row-major float matrix [rows][d] seen as a 2-D tensor; a box is SUB rows of box_cols columns.
-// Elements outside the matrix read as zero.
-bool make_map(CUtensorMap *map, const float *X, uint64_t rows, uint64_t d, uint32_t box_cols)
+// Row-major float matrix [rows][d] seen as a 2-D tensor; a box is SUB rows of box_cols columns.  As a tensor of pairs of
+// floats (d and box_cols are even) the widest box, 256 elements, is 512 columns.  Elements outside the matrix read as zero.
+}  // namespace
+bool qesgd_lr_tensor_map(CUtensorMap *map, const float *X, uint64_t rows, uint64_t d, uint32_t box_cols, bool pairs)
 {
-    const cuuint64_t dims[2] = {d, rows};
+    const uint32_t n = pairs ? 2u : 1u;
+    const cuuint64_t dims[2] = {d / n, rows};
     const cuuint64_t strides[1] = {d * sizeof(float)};
-    const cuuint32_t box[2] = {box_cols, (cuuint32_t)SUB};
+    const cuuint32_t box[2] = {box_cols / n, (cuuint32_t)SUB};
     const cuuint32_t elem[2] = {1u, 1u};
-    return g_encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2u, const_cast<float *>(X), dims, strides, box,
+    return g_encode_tiled(map, pairs ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2u, const_cast<float *>(X), dims, strides, box,
                           elem, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
+namespace {
 
 // One way to deal the epoch out: G groups of P CTAs, NC chains per CTA.
 struct Split {
@@ -972,6 +798,16 @@ int qesgd_launch_lr_epoch_fused(const float *X, const float *y, uint64_t n_local
     const uint32_t sms = (uint32_t)(sm_count < 256 ? sm_count : 256);
     bool fits = nsteps64 * K == 1u && choose_split(s, d, K, m_full, nsub, tma, sms - sms / 16u, (uint32_t)limit);
     if (!fits && !gradient) fits = choose_split(s, d, K, m_full, nsub, tma, sms, (uint32_t)limit);
+    // workspace, all zero between launches: headers | accumulators | their rarely used words
+    uint32_t *const header = reinterpret_cast<uint32_t *>(work);
+    unsigned long long *const acc = reinterpret_cast<unsigned long long *>(work + QESGD_MAX_WORKERS * EP_HEADER_WORDS);
+    unsigned long long *const wide = acc + (size_t)EP_RING * (QESGD_LR_EPOCH_ROWS / SUB) * EP_ACC_PITCH;
+    {
+        const QesgdTileCall q = {X, y, n_local, d, nsteps64, K, m_full, lr, u, dst, gradient, u_stride, tma ? 16 : (pairs ? 8 : 4),
+                                 header, acc, wide, status, device, nsteps64 * K == 1u ? sms - sms / 16u : sms, wait_ns, drop_cta, stream};
+        const int e = qesgd_launch_lr_tile(q, (uint32_t)limit, fits ? s.us : 1e30f, launched);
+        if (e >= 0) return e;
+    }
     if (!fits) return -1;
 
     EpochArgs a;
@@ -1002,16 +838,15 @@ int qesgd_launch_lr_epoch_fused(const float *X, const float *y, uint64_t n_local
     a.wait_ns = wait_ns;
     a.poll_mask = wait_ns < COARSE_TIMER_NS ? 0u : 31u;
     a.drop_cta = drop_cta;
-    // workspace, all zero between launches: headers | accumulators | their rarely used words
-    a.header = reinterpret_cast<uint32_t *>(work);
-    a.acc = reinterpret_cast<unsigned long long *>(work + QESGD_MAX_WORKERS * EP_HEADER_WORDS);
-    a.wide = a.acc + (size_t)EP_RING * (QESGD_LR_EPOCH_ROWS / SUB) * EP_ACC_PITCH;
+    a.header = header;
+    a.acc = acc;
+    a.wide = wide;
 
     CUtensorMap map_full = {}, map_rest = {};
     const uint32_t wide_box = s.cols < (uint32_t)EP_BOX_COLS ? s.cols : (uint32_t)EP_BOX_COLS;
     const uint32_t rest = s.cols % EP_BOX_COLS;
-    if (tma && !make_map(&map_full, X, (uint64_t)K * n_local, d, wide_box)) return -1;
-    if (tma && !make_map(&map_rest, X, (uint64_t)K * n_local, d, rest ? rest : wide_box)) return -1;
+    if (tma && !qesgd_lr_tensor_map(&map_full, X, (uint64_t)K * n_local, d, wide_box, false)) return -1;
+    if (tma && !qesgd_lr_tensor_map(&map_rest, X, (uint64_t)K * n_local, d, rest ? rest : wide_box, false)) return -1;
 
     void *params[] = {(void *)&a, (void *)&map_full, (void *)&map_rest};
     const void *const kernel = EPOCH_KERNELS[tma ? s.NC - 1u : (pairs ? 2u : 3u)];

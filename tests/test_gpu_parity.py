@@ -584,6 +584,77 @@ def test_lr_local_epoch_updates_behind_the_next_margins_match_oracle(K, n_local,
             _lr_close(got[k], ref.lr_local_epoch(X[rows], y[rows], batch, 0.5, u0[k]))
 
 
+@pytest.mark.parametrize("K,n_local,d,batch", [
+    (1, 70, 100, 16),        # a CTA of its own, nothing to exchange
+    (2, 1000, 200, 64),      # clusters of two CTAs, one block of columns, the ring goes round
+    (3, 101, 384, 33),       # of four, one of them without columns; sub-tiles of one row
+    (2, 90, 900, 50),        # of eight
+    (9, 70, 1999, 20),       # of sixteen, element by element
+    (3, 70, 1002, 40),       # pairs of elements
+    (4, 160, 4096, 32),      # two blocks of columns
+    (1, 200, 6000, 64),      # three and more
+    (2, 100, 8000, 8),       # one sub-tile
+    (1, 90, 9998, 16),       # five blocks, pairs
+    (2, 250, 500, 100),      # sixteen warps
+    (3, 300, 1900, 128),
+    (1, 270, 2002, 121),
+    (24, 40, 2000, 32),      # more clusters than are resident at once
+    (1, 150, 17000, 64),     # groups of a cooperative grid: one block, 133 CTAs
+    (1, 90, 20001, 24),      # element by element
+    (8, 170, 10000, 50),     # five blocks, a ring of little more than a minibatch
+    (4, 200, 16384, 32),     # four blocks
+    (2, 300, 7000, 128),     # sixteen warps
+])
+def test_lr_epochs_with_the_minibatch_in_registers_match_oracle(K, n_local, d, batch):
+    """The kernel that keeps a minibatch's slice in registers, over its blocks of columns, warps, cluster sizes and
+    kinds of copies, every worker from a point of its own.  Twice: the workspace and shared memory are as found.
+    Bound as above (1e-5)."""
+    X, y, _ = synthetic.logistic_problem(K * n_local, d, seed=K + n_local + d)
+    u0 = (0.1 * synthetic.normal_f32(K * d, 1.0, 26)).astype(np.float32).reshape(K, d)
+    c, tX, ty = G.ctx(), G.dev(X), G.dev(y)
+    runs = []
+    for _ in range(2):
+        tu = G.dev(u0)
+        c.qesgd_lr_local_epoch_batch(tX, ty, n_local, d, K, batch, 0.5, tu, d)
+        assert c.qesgd_status() == 0
+        runs.append(tu)
+    assert torch.equal(runs[0], runs[1])
+    got = runs[0].cpu().numpy()
+    for k in sorted({0, 1, K // 2, K - 1} & set(range(K))):
+        rows = slice(k * n_local, (k + 1) * n_local)
+        _lr_close(got[k], ref.lr_local_epoch(X[rows], y[rows], batch, 0.5, u0[k]))
+
+
+@pytest.mark.parametrize("d", [700, 1500, 20000])    # clusters, a group through global memory
+def test_lr_epoch_in_registers_carries_extreme_and_nonfinite_margins(d):
+    """Partial margins of 1e30 that cancel over the CTAs but for a remainder the size of one, rows of infinite and of
+    NaN margins: the sum over the CTAs keeps the remainder, infinities saturate the step coefficient, NaN spreads."""
+    m, lr = 16, 0.5
+    X = np.zeros((m, d), dtype=np.float32)
+    u0 = np.zeros(d, dtype=np.float32)
+    u0[:3], u0[-3:] = (1.0, 1.0, 0.5), (1.0, -1.0, 0.25)
+    X[:, 2] = 1.0
+    big = np.float32(2.0 ** 20)
+    X[0, 0], X[0, -3] = big, -big                # cancels exactly
+    X[1, 0], X[1, -2] = big, big
+    X[2, 0], X[3, 0] = np.inf, -np.inf
+    y = np.where(np.arange(m) % 2 == 0, 1.0, -1.0).astype(np.float32)
+    tu = G.dev(u0)
+    c = G.ctx()
+    c.qesgd_lr_sgd_step(G.dev(X), G.dev(y), m, d, lr, tu)
+    assert c.qesgd_status() == 0
+    with np.errstate(all="ignore"):
+        want = ref.lr_sgd_step(X, y, lr, u0)
+    got = tu.cpu().numpy()
+    fin = np.isfinite(want)
+    assert np.array_equal(fin, np.isfinite(got)) and fin.sum() >= d - 1
+    _lr_close(got[fin], want[fin])
+    X[4, 1] = np.nan
+    tu = G.dev(u0)
+    c.qesgd_lr_sgd_step(G.dev(X), G.dev(y), m, d, lr, tu)
+    assert np.isnan(tu.cpu().numpy()).all()
+
+
 @pytest.mark.parametrize("gain", [2e7, 1e9])
 def test_local_epoch_partial_margins_beyond_the_fine_fixed_point_range(gain):
     """The CTAs of the persistent kernel add their partial margins as fixed-point integers: units
@@ -643,8 +714,11 @@ def _epoch_once(c, X, y, n_local, d, K, batch, u0):
 
 
 @pytest.mark.parametrize("K,n_local,d,batch", [
-    (2, 96, 8192, 32),       # two chains
-    (3, 200, 4096, 100),     # two chains, odd K, 13 sub-tiles
+    (2, 96, 8192, 32),       # a cluster of sixteen for each worker
+    (3, 200, 4096, 100),     # 13 sub-tiles
+    (4, 130, 65536, 64),     # two chains
+    (3, 130, 65536, 64),     # two chains, odd K
+    (1, 100, 1000, 32),      # a cluster of eight
     (2, 40, 131072, 64),     # one chain, several workers: sums added up behind the next margins
     (1, 100, 20000, 64),     # one chain, one worker
     (2, 70, 10003, 32),      # element by element: 4-byte copies, several CTAs
