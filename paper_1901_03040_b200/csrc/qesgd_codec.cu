@@ -526,11 +526,10 @@ __device__ __forceinline__ void encode_warp_tile(const EncodeArgs &a, float (&z)
     // V*256, so the Philox block index (warp_base/8 + lane + 32c) never carries into
     // its high word when c advances.
     const uint32_t loff = lane * 8u;
-    uint8_t *const cbase = reinterpret_cast<uint8_t *>(a.codes) + (uint64_t)k * a.code_stride +
-                           ((warp_base + loff) >> 3) * (uint64_t)BITS;
+    uint8_t *const cbase = reinterpret_cast<uint8_t *>(a.codes) + (uint64_t)k * a.code_stride + (warp_base >> 3) * (uint64_t)BITS +
+                           lane * (uint32_t)BITS;
     float *const sbase = a.scales + (uint64_t)k * a.scale_stride + (warp_base >> lb);
-    const uint64_t blk0 = (warp_base >> 3) + lane;
-    const uint32_t blk_lo = (uint32_t)blk0, blk_hi = (uint32_t)(blk0 >> 32);
+    const uint32_t blk_lo = (uint32_t)(warp_base >> 3) + lane, blk_hi = (uint32_t)(warp_base >> 35);
     const uint32_t bucket_mask = (1u << lb) - 1u;
     const bool wide = lb > LOG2_WARP_ELEMS;                     // bucket spans several warps
     const bool wide_first = ((uint32_t)warp_base & bucket_mask) == 0u;   // this warp starts it
@@ -602,28 +601,42 @@ __device__ __forceinline__ void encode_warp_tile(const EncodeArgs &a, float (&z)
                 if ((__float_as_uint(z[c][j]) & 0x7FFFFFFFu) >= 0x7F800000u) z[c][j] = 0.0f;
     }
 
+    // Every bucket's scale, by the first of the lanes that hold its total (with a caller-given spacing: of its elements).
+    if (!wide) {
+        // lane's chunk and eight elements of it; a total lies in all lanes that agree with the holder outside `same`:
+        // the bucket's own lanes but for the bits that tell its chunks apart, which are the lowest (chunk_of_lane)
+        constexpr uint32_t CHUNK_BITS = MODE == 2 || V == 1 ? 0u : (V == 8 ? 7u : (V == 4 ? 3u : 1u));
+        const uint32_t lanes = lb >= 8u ? 31u : (1u << (lb - 3u)) - 1u;       // of a chunk that a bucket covers
+        if (MODE != 2) {
+            const uint32_t off = chunk_of_lane<V>(lane) * (uint32_t)CHUNK + (loff & ~(CHUNK_BITS * 8u));
+            if ((lane & lanes & ~CHUNK_BITS) == 0u && (off & bucket_mask) == 0u && (FULL || warp_base + off < a.padded) &&
+                QESGD_IN_RANGE(a.status, ((warp_base + off) >> lb) < (a.padded >> lb)))
+                sbase[off >> lb] = my_scale;
+        } else {
+#pragma unroll
+            for (int c = 0; c < V; ++c) {
+                const uint32_t off = (uint32_t)c * CHUNK + loff;
+                if ((off & bucket_mask) == 0u && (FULL || warp_base + off < a.padded) &&
+                    QESGD_IN_RANGE(a.status, ((warp_base + off) >> lb) < (a.padded >> lb)))
+                    sbase[off >> lb] = my_scale;
+            }
+        }
+    } else if (lane == 0u && wide_first && (FULL || warp_base < a.padded) &&
+               QESGD_IN_RANGE(a.status, (warp_base >> lb) < (a.padded >> lb))) {
+        sbase[0] = my_scale;
+    }
+
     // ---- rounding, packing, stores ---------------------------------------------
 #pragma unroll
     for (int c = 0; c < V; ++c) {
         const uint32_t off = (uint32_t)c * CHUNK + loff;        // element offset inside the tile
         const bool inside = FULL || warp_base + off < a.padded;
-        float scale = my_scale, inv = my_inv, delta = my_delta;
+        float inv = my_inv, delta = my_delta;
         if (MODE != 2 && V > 1) {   // fetch chunk c's bucket scale from the neighbour lane that carried it
             const int src = (int)lane_of_chunk<V>(lane, c);
-            scale = __shfl_sync(0xFFFFFFFFu, my_scale, src);
             inv = __shfl_sync(0xFFFFFFFFu, my_inv, src);
             if (REQ) delta = __shfl_sync(0xFFFFFFFFu, my_delta, src);
         }
-        if (inside) {      // the first lane of every bucket writes its scale
-            if (!wide) {
-                if ((off & bucket_mask) == 0u &&
-                    QESGD_IN_RANGE(a.status, ((warp_base + off) >> lb) < (a.padded >> lb)))
-                    sbase[off >> lb] = scale;
-            } else if (off == 0u && wide_first && QESGD_IN_RANGE(a.status, (warp_base >> lb) < (a.padded >> lb))) {
-                sbase[0] = scale;
-            }
-        }
-
         if ((c & 1) == 0 && c > 0) {   // draws for this chunk and the next, interleaved
 #pragma unroll
             for (int n = 0; n < DRAWS; ++n) {
@@ -709,8 +722,9 @@ __global__ void __launch_bounds__(WARPS * 32,
 {
     qesgd_wait_for_previous();
     __shared__ EncodeShared sh;
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t warp = threadIdx.x >> 5;
+    // (with one warp per CTA the tile's position is the same for the whole warp, and the compiler is told so)
+    const uint32_t lane = WARPS == 1 ? threadIdx.x : threadIdx.x & 31u;
+    const uint32_t warp = WARPS == 1 ? 0u : threadIdx.x >> 5;
     // Workers vary fastest over the grid: the K CTAs that share a tile of the anchor run
     // close together in time, so the anchor comes from HBM once and from L2 K-1 times.
     const uint32_t k = blockIdx.x % a.K;
