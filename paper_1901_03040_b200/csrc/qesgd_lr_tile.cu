@@ -4,7 +4,7 @@
 // update -- behind copies of many columns and behind a second chain.  With few columns per CTA nothing hides
 // it, and the chain itself is the time: there every phase goes through shared or tensor memory with four
 // barriers a step, about 3500 clocks of which the exchange is 400 to 1000.  Here a worker has its own CTAs
-// (one cluster of up to 16, or a group of the cooperative grid), and a warp its own eight rows of U x 128
+// (one cluster of up to 16, a group of the cooperative grid, or for one minibatch a grid launched plainly), and a warp its own eight rows of U x 128
 // columns: the rows live in registers from the margins to the update, a lane always holds the same columns,
 // and the row whose sum a lane ends up with is the row it exchanges and finishes, so between the margins and the
 // update nothing crosses the warp.  Two barriers a step are left, around the sum of the warps' updates.
@@ -51,7 +51,11 @@ struct TileArgs {
     uint32_t *status;
     uint64_t wait_ns;
     uint32_t poll_mask, drop_cta;
+    uint32_t *claims;            // one minibatch, plain launch: [P] slices that a CTA has begun; else null
+    uint32_t off_claims;         // shared memory: the coefficients, then how many slices this CTA took over and which
 };
+constexpr uint64_t TL_STEAL_NS = 20000ull;   // a wait longer than this looks for slices that nobody has begun
+constexpr uint32_t TL_ROWS = 128;            // coefficients kept for them
 
 __device__ __forceinline__ uint32_t cluster_address(uint32_t addr, uint32_t rank)
 {
@@ -136,14 +140,90 @@ __device__ __forceinline__ uint32_t kept(uint32_t v)
     return v;
 }
 
-template <int U, int W, int EB, bool CL>
-__global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
-    qesgd_lr_tile_kernel(const TileArgs a, const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap map_rest)
+// Slices that nobody has begun.  The grid of one minibatch is launched like any other kernel, so that it is set up while the
+// one before it drains (a cooperative launch is not, and occupies the stream for a whole number of 2.05 us: 64 x 65536 from L2
+// 8.2 us, launched plainly 6.2, from HBM 10.2 and 8.0; 64 x 20000 8.2 and 5.1; 16 x 80000 8.1 and 5.0).  Then nothing promises that all its CTAs are resident at once: beside other streams' kernels
+// some may start late.  So a CTA never waits for one that has not started: each claims its slice when it starts, a wait
+// longer than 20 us claims one that is still free and does its margins here, by the same operations in the same order, and
+// after its own update the CTA does theirs.  A CTA that finds its slice claimed has nothing left to do.
+//
+// A warp looks for a free slice and adds its partial margins to the rows' accumulators.
+template <int U>
+__device__ __noinline__ void take_over(const TileArgs &a, uint32_t *list, uint32_t lane)
 {
+    uint32_t slice = ~0u;
+    for (uint32_t b = 0; b < a.P && slice == ~0u; b += 32u) {
+        const uint32_t free = __ballot_sync(0xFFFFFFFFu, b + lane < a.P && ld_acquire(a.claims + b + lane) == 0u);
+        if (free == 0u) continue;
+        const uint32_t first = b + (uint32_t)__ffs((int)free) - 1u;
+        uint32_t before = 1u;
+        if (lane == 0) before = atomicCAS(a.claims + first, 0u, 1u);
+        if (__shfl_sync(0xFFFFFFFFu, before, 0) == 0u) slice = first;
+    }
+    if (slice == ~0u) return;
+    if (lane == 0) list[1u + atomicAdd(list, 1u)] = slice;
+    const uint32_t m = a.m_last;
+    for (uint32_t s = 0; s < a.nsub_last; ++s) {
+        float acc[SUB];
+        for (int r = 0; r < SUB; ++r) acc[r] = 0.0f;
+        for (uint32_t it = 0; it < (uint32_t)U; ++it)
+            for (int r = 0; r < SUB; ++r)
+                for (uint32_t e = 0; e < 4u; ++e) {
+                    const uint64_t c = (uint64_t)slice * (U * 128u) + it * 128u + lane * 4u + e;
+                    const bool in = s * SUB + r < m && c < a.d;
+                    acc[r] = fmaf(in ? a.X[(uint64_t)(s * SUB + r) * a.d + c] : 0.0f, c < a.d ? a.u[c] : 0.0f, acc[r]);
+                }
+        const float tot = reduce8(acc, lane);
+        const uint32_t row = s * SUB + (lane >> 2);
+        if ((lane & 3u) == 0u && row < m) exchange_add(a.acc + acc_index(row), a.wide + (size_t)row * EP_WIDE_WORDS, tot);
+    }
+}
+// Counted last of the group: nobody adds or reads any more.  By a warp; the accumulators that the epoch has used.
+__device__ __noinline__ void leave_clear(const TileArgs &a, uint32_t lane)
+{
+    const uint32_t worker = blockIdx.x / a.P, mpad = SUB * a.nsub, used = min(a.nsteps, (uint32_t)EP_RING);
+    uint32_t *const header = a.header + worker * EP_HEADER_WORDS;
+    for (uint32_t j = lane; j < used * mpad; j += 32u) {
+        a.acc[(size_t)worker * EP_RING * a.nsub * EP_ACC_PITCH + acc_index(j)] = 0ull;   // slots follow one another at the same pitch
+#pragma unroll
+        for (uint32_t v = 0; v < EP_WIDE_WORDS; ++v) a.wide[((size_t)worker * EP_RING * mpad + j) * EP_WIDE_WORDS + v] = 0ull;
+    }
+    if (a.claims != nullptr)
+        for (uint32_t j = lane; j < a.P; j += 32u) a.claims[j] = 0u;
+    if (lane < 2u) header[lane] = 0u;
+}
+// The update of a slice that this CTA has taken over, by all its threads.
+template <int U, int W>
+__device__ __noinline__ void finish_slice(const TileArgs &a, uint32_t slice, const float *coef)
+{
+    for (uint32_t q = threadIdx.x; q < U * 128u; q += W * 32u) {
+        const uint64_t c = (uint64_t)slice * (U * 128u) + q;
+        if (c >= a.d) continue;
+        float s = 0.0f;
+        for (uint32_t v = 0; v < a.nsub_last; ++v) {
+            float p = 0.0f;
+            for (uint32_t r = 0; r < (uint32_t)SUB; ++r) {
+                const uint32_t row = v * SUB + r;
+                p = fmaf(coef[row], row < a.m_last ? a.X[(uint64_t)row * a.d + c] : 0.0f, p);
+            }
+            s += p;
+        }
+        if (a.gradient == 0u) s += a.u[c];
+        a.dst[c] = s;
+    }
+}
+
+// EX: how a worker's CTAs meet -- a group of a cooperative grid, a cluster, or a plain grid of one minibatch.
+enum Exchange { GROUP = 0, CLUSTER = 1, PLAIN = 2 };
+template <int U, int W, int EB, int EX>
+__global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
+    qesgd_lr_tile_kernel(const __grid_constant__ TileArgs a, const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap map_rest)
+{
+    constexpr bool CL = EX == CLUSTER, plain = EX == PLAIN;
     constexpr uint32_t COLS = U * 128u, SLOT = SUB * COLS;
     // The slot of the warp's own sub-tile, once that is in the registers, takes the next copy: right away where blocks are
     // wide and the ring holds little more than a minibatch, else while the margins travel.
-    constexpr bool EARLY = U >= 3;
+    constexpr bool EARLY = U >= 3 && EX != PLAIN;
     float *const ring = reinterpret_cast<float *>(tl_smem);
     float *const us = reinterpret_cast<float *>(tl_smem + a.off_u);
     float *const part = reinterpret_cast<float *>(tl_smem + a.off_part);
@@ -153,7 +233,7 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
     volatile uint32_t *const flag = reinterpret_cast<volatile uint32_t *>(tl_smem + a.off_flags);
 
     const uint32_t tid = threadIdx.x, lane = tid & 31u, w = tid >> 5;
-    const uint32_t P = kept(a.P), nsteps = kept(a.nsteps), batch = kept(a.batch), nsub = kept(a.nsub), nslots = kept(a.nslots);
+    const uint32_t P = kept(a.P), nsteps = plain ? 1u : kept(a.nsteps), batch = kept(a.batch), nsub = kept(a.nsub), nslots = kept(a.nslots);
     const uint32_t worker = blockIdx.x / P, rank = blockIdx.x - worker * P;
     const uint32_t c0 = rank * COLS;
 
@@ -165,11 +245,14 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
     if (CL)                      // no word of the exchange carries a tile's number yet
         for (uint32_t q = tid; q < 2u * P * a.x_pitch; q += W * 32u)
             reinterpret_cast<unsigned long long *>(tl_smem + a.off_x)[q] = 0ull;
+    float *const kept_coef = reinterpret_cast<float *>(tl_smem + a.off_claims);
+    uint32_t *const list = reinterpret_cast<uint32_t *>(kept_coef + TL_ROWS);
+    if (plain && tid == 0) list[0] = 0u;
     __syncthreads();
-    if (CL) {
-        cluster_arrive();        // waited for before the first store into another CTA
-        qesgd_wait_for_previous();
-    }
+    if (CL) cluster_arrive();    // waited for before the first store into another CTA
+    if (CL || plain) qesgd_wait_for_previous();
+    uint32_t taken = 0u;
+    if (plain && tid == 0) taken = atomicExch(a.claims + rank, 1u);
 
     const uint32_t row0 = (uint32_t)((uint64_t)worker * a.n_local);
     auto rows_of = [&](uint32_t t) { return t + 1u == nsteps ? a.m_last : batch; };
@@ -245,7 +328,14 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
         if (tid + e * W * 32u < COLS) us[tid + e * W * 32u] = u0[e];
     if (CL) cluster_wait();
     if (w < subs_of(0u)) take(false, slot, 0u, rows_of(0u) - w * SUB);
-    __syncthreads();
+    if (!plain) {
+        __syncthreads();
+    } else if (__syncthreads_or((int)taken) != 0) {               // another CTA does this slice; every copy requested has been taken
+        uint32_t before = 0u;
+        if (tid == 0) asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(before) : "l"(a.header + 1) : "memory");
+        if (w == 0u && __shfl_sync(0xFFFFFFFFu, before, 0) == P - 1u) leave_clear(a, lane);
+        return;
+    }
 
     const uint32_t mpad = SUB * nsub;
     unsigned long long *const acc_g = a.acc + (size_t)worker * EP_RING * nsub * EP_ACC_PITCH + acc_index(my_row);
@@ -311,7 +401,7 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
         const bool more = !last && w < next_subs;
         const float next_y = more && my_row < next_m ? __ldg(label + batch) : 0.0f;
         const bool landed = more && mbar_try_wait(&full[next_slot], next_parity);
-        if (!CL && rank == clears) {                       // this CTA clears the accumulators that minibatch t + RING/2 will use
+        if (!CL && rank == clears && t + EP_RING / 2 < nsteps) {                       // this CTA clears the accumulators that minibatch t + RING/2 will use
             const uint32_t zs = (t + EP_RING / 2) % EP_RING;
             unsigned long long *const az = a.acc + ((size_t)worker * EP_RING + zs) * nsub * EP_ACC_PITCH;
             unsigned long long *const wz = a.wide + ((size_t)worker * EP_RING + zs) * mpad * EP_WIDE_WORDS;
@@ -364,14 +454,34 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
                     e += d;
                 }
                 margin = fabsf(s) <= 3.402823466e38f ? s + e : s;   // the errors of an infinite sum are NaN
-            } else if ((lane & 3u) == 0u && my_row < m) {
-                unsigned long long v;
-                while (((v = ld_relaxed(acc_t)) >> 55) < P)
-                    if (give_up()) break;
-                margin = exchange_margin(v, wide_t, P);
+            } else if (!plain) {
+                if ((lane & 3u) == 0u && my_row < m) {
+                    unsigned long long v;
+                    while (((v = ld_relaxed(acc_t)) >> 55) < P)
+                        if (give_up()) break;
+                    margin = exchange_margin(v, wide_t, P);
+                }
+            } else {
+                // the warp together, so that it can take over a slice
+                unsigned long long v = 0ull;
+                bool done = (lane & 3u) != 0u || my_row >= m;
+                const bool reads = !done;
+                for (;;) {
+                    for (uint32_t n = 0; !done && n <= a.poll_mask; ++n) done = ((v = ld_relaxed(acc_t)) >> 55) >= P;
+                    if (__all_sync(0xFFFFFFFFu, done)) break;
+                    if (looks++ == 0u) t0 = now_ns();
+                    const bool stop = flag[0] != 0u || ld_acquire(header) != 0u || expired(t0, a.wait_ns);
+                    if (__any_sync(0xFFFFFFFFu, stop)) {
+                        flag[0] = 1u;
+                        break;
+                    }
+                    if (__any_sync(0xFFFFFFFFu, now_ns() - t0 > TL_STEAL_NS)) take_over<U>(a, list, lane);
+                }
+                if (reads) margin = exchange_margin(v, wide_t, P);
             }
             // -(lr/m) * c_j with c_j = -y_j / (1 + exp(y_j m_j))
             const float cj = my_row < m ? ry / (1.0f + expf(yj * margin)) : 0.0f;
+            if (plain && (lane & 3u) == 0u) kept_coef[my_row] = cj;
             __syncwarp();
             if (!CL && last && lane == 0) {                // the last warp counts the CTA
                 __threadfence_block();
@@ -431,7 +541,11 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
                 if (last && (uint64_t)c0 + c + e < a.d) a.dst[(uint64_t)worker * a.u_stride + c0 + c + e] = s[e];
             }
         }
-        if (last) break;
+        if (last) {
+            if constexpr (plain)
+                for (uint32_t n = 0; n < list[0]; ++n) finish_slice<U, W>(a, list[1u + n], kept_coef);
+            break;
+        }
         asm volatile("bar.sync 2, %0;" ::"n"(W * 32) : "memory");   // u complete for the next minibatch
         ++t;
         m = next_m;
@@ -460,27 +574,19 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
     }
     if (CL) return;
     __syncwarp();
-    // Counted last of the group: nobody adds or reads any more.
-    if (__shfl_sync(0xFFFFFFFFu, counted, 0) == P - 1u) {
-        for (uint32_t j = lane; j < EP_RING * mpad; j += 32u) {
-            a.acc[(size_t)worker * EP_RING * nsub * EP_ACC_PITCH + acc_index(j)] = 0ull;   // slots follow one another at the same pitch
-#pragma unroll
-            for (uint32_t v = 0; v < EP_WIDE_WORDS; ++v) a.wide[((size_t)worker * EP_RING * mpad + j) * EP_WIDE_WORDS + v] = 0ull;
-        }
-        if (lane < 2u) header[lane] = 0u;
-    }
+    if (__shfl_sync(0xFFFFFFFFu, counted, 0) == P - 1u) leave_clear(a, lane);
 }
 
 // ------------------------------------------------------------------ host ----
 typedef void (*TileKernel)(TileArgs, CUtensorMap, CUtensorMap);
 struct Variant {
     uint32_t U, W;
-    TileKernel kernel[2][3];     // a group of the grid, a cluster; copies of 16 (TMA), 8, 4 bytes
+    TileKernel kernel[3][3];     // by Exchange; copies of 16 (TMA), 8, 4 bytes
 };
-#define TL_VARIANT(U, W) \
-    {U, W, {{qesgd_lr_tile_kernel<U, W, 16, false>, qesgd_lr_tile_kernel<U, W, 8, false>, qesgd_lr_tile_kernel<U, W, 4, false>}, \
-            {qesgd_lr_tile_kernel<U, W, 16, true>, qesgd_lr_tile_kernel<U, W, 8, true>, qesgd_lr_tile_kernel<U, W, 4, true>}}}
-// Registers: 32 U for the rows.  A block of eight warps has 255 a thread, one of sixteen 128.
+#define TL_COPIES(U, W, EX) {qesgd_lr_tile_kernel<U, W, 16, EX>, qesgd_lr_tile_kernel<U, W, 8, EX>, qesgd_lr_tile_kernel<U, W, 4, EX>}
+#define TL_VARIANT(U, W) {U, W, {TL_COPIES(U, W, GROUP), TL_COPIES(U, W, CLUSTER), TL_COPIES(U, W, PLAIN)}}
+// Registers: 32 U for the rows.  A block of eight warps has 255 a thread, one of sixteen 128.  (Six blocks of columns
+// spill: a gradient of 64 x 100000 10.4 us against 10.3 for the other kernel.)
 const Variant VARIANTS[] = {TL_VARIANT(1, 8), TL_VARIANT(2, 8), TL_VARIANT(3, 8), TL_VARIANT(4, 8),
                             TL_VARIANT(5, 8), TL_VARIANT(1, 16), TL_VARIANT(2, 16)};
 constexpr uint32_t NVARIANTS = sizeof(VARIANTS) / sizeof(VARIANTS[0]);
@@ -513,15 +619,16 @@ uint32_t budget(const Variant &v, uint32_t limit) { return v.U == 1u && v.W == 8
 
 struct Plan {
     const Variant *v;
-    uint32_t P, cluster, nslots, bytes, x_pitch;
-    uint32_t off_u, off_part, off_x, off_bars, off_flags;
+    uint32_t P, exchange, nslots, bytes, x_pitch;
+    uint32_t off_u, off_part, off_x, off_bars, off_flags, off_claims;
 };
 bool lay_out(Plan &p, uint32_t nsub, uint64_t subtiles, uint32_t limit)
 {
     const uint32_t cols = p.v->U * 128u, slot = SUB * cols * 4u;
     p.x_pitch = SUB * nsub + (nsub % 2u ? 12u : 4u);
-    const uint32_t xbytes = p.cluster ? 2u * p.P * p.x_pitch * 8u : 0u;
-    const uint32_t fixed = cols * 4u + p.v->W * cols * 4u + xbytes + TL_MAX_SLOTS * 8u + (4u + TL_MAX_SLOTS) * 4u;
+    const uint32_t xbytes = p.exchange == CLUSTER ? 2u * p.P * p.x_pitch * 8u : 0u;
+    const uint32_t cbytes = p.exchange == PLAIN ? (TL_ROWS + 1u + 256u) * 4u : 0u;
+    const uint32_t fixed = cols * 4u + p.v->W * cols * 4u + xbytes + TL_MAX_SLOTS * 8u + (4u + TL_MAX_SLOTS) * 4u + cbytes;
     const uint32_t have = budget(*p.v, limit);
     if (fixed + nsub * slot > have) return false;
     p.nslots = (have - fixed) / slot;
@@ -532,7 +639,8 @@ bool lay_out(Plan &p, uint32_t nsub, uint64_t subtiles, uint32_t limit)
     p.off_x = p.off_part + p.v->W * cols * 4u;
     p.off_bars = p.off_x + xbytes;
     p.off_flags = p.off_bars + TL_MAX_SLOTS * 8u;
-    p.bytes = p.off_flags + (4u + TL_MAX_SLOTS) * 4u;
+    p.off_claims = p.off_flags + (4u + TL_MAX_SLOTS) * 4u;
+    p.bytes = p.off_claims + cbytes;
     return true;
 }
 
@@ -542,10 +650,10 @@ bool prepare_device(int device, uint32_t limit)
     std::lock_guard<std::mutex> lock(g_tile_mutex);
     if (g_tile_ready[device]) return true;
     for (uint32_t i = 0; i < NVARIANTS; ++i) {
-        for (uint32_t j = 0; j < 6u; ++j) {
+        for (uint32_t j = 0; j < 9u; ++j) {
             const void *const k = (const void *)VARIANTS[i].kernel[j / 3u][j % 3u];
             if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit) != cudaSuccess ||
-                (j >= 3u && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
+                (j / 3u == CLUSTER && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
                 cudaGetLastError();
                 return false;
             }
@@ -554,7 +662,7 @@ bool prepare_device(int device, uint32_t limit)
             cudaLaunchAttribute at[2];
             const cudaLaunchConfig_t c = cluster_config(1u << l, 1u << l, VARIANTS[i].W * 32u, budget(VARIANTS[i], limit), nullptr, at);
             int n = 0, least = 1 << 30;
-            for (const TileKernel k : VARIANTS[i].kernel[1]) {
+            for (const TileKernel k : VARIANTS[i].kernel[CLUSTER]) {
                 if (cudaOccupancyMaxActiveClusters(&n, k, &c) != cudaSuccess) {
                     cudaGetLastError();
                     n = 0;
@@ -577,9 +685,9 @@ float modelled_us(const Plan &p, const QesgdTileCall &q, uint32_t nsub, uint32_t
 {
     const float hbm = (float)((double)q.K * q.m * q.d * 4.0 / 6.5e6), U = (float)p.v->U, rows = (float)nsub;
     const float copy = q.copy == 16 ? 0.0f : (q.copy == 8 ? 0.045f : 0.085f) * U * rows;
-    const float chain = (waves > 1u ? 1.2f * (float)waves : 1.0f) * ((p.cluster ? 0.85f : 1.3f) + U * (0.03f + 0.026f * rows) + copy + (p.v->W == 16u ? 0.3f : 0.0f));
+    const float chain = (waves > 1u ? 1.2f * (float)waves : 1.0f) * ((p.exchange == CLUSTER ? 0.85f : 1.3f) + U * (0.03f + 0.026f * rows) + copy + (p.v->W == 16u ? 0.3f : 0.0f));
     const float fetch = hbm * (p.v->U > 2u ? 1.3f : 1.1f);
-    const float start = p.cluster ? 2.0f * (float)waves - 0.5f : (p.v->U > 2u && q.nsteps > 1u ? 5.0f : 4.0f);
+    const float start = p.exchange != GROUP ? 2.0f * (float)waves - 0.5f : (p.v->U > 2u ? 5.0f : 4.0f);
     return (float)q.nsteps * (chain > fetch ? chain : fetch) + start;
 }
 
@@ -590,7 +698,7 @@ float modelled_us(const Plan &p, const QesgdTileCall &q, uint32_t nsub, uint32_t
 //   K = 4, n = 128, d = 4096, batch 32 (cluster of 16, two blocks): 14.4 -> 7.0 us;  K = 4, n = 1000, d = 1000, batch 32 (8, one)
 //   71.8 -> 34.1;  K = 2, n = 800, d = 300, batch 64 (4, one) 41.0 -> 16.6;  K = 8, n = 500, d = 2000, batch 100 (8, two, sixteen
 //   warps) 28.7 -> 12.4;  K = 8, n = 2000, d = 128, batch 16 (one CTA) 271 -> 126;  one gradient of 64 x 4096 (16, two) 6.7 -> 3.5;
-//   K = 1, n = 1010, d = 10000, batch 50 (79 CTAs of a group, one) 44.7 -> 36.9;  K = 8 of them (16 CTAs, five) 80.8 -> 71.1;
+//   gradients of 64 x 65536 (128 CTAs, four) 8.2 -> 6.2;  K = 1, n = 1010, d = 10000, batch 50 (79 CTAs of a group, one) 44.7 -> 36.9;  K = 8 of them (16 CTAs, five) 80.8 -> 71.1;
 //   K = 4, n = 1000, d = 16384, batch 32 (32 CTAs, four) 89.5 -> 72.3.
 // Where it loses and is not taken: more clusters than the device holds at once (K = 16, n = 200, d = 8000, batch 64: 32.5 in three
 // turns against 28.7); element-wise copies of many columns (K = 6, n = 700, d = 8003, batch 50: 57 against 49).
@@ -604,12 +712,12 @@ int qesgd_launch_lr_tile(const QesgdTileCall &q, uint32_t smem_limit, float othe
         const Variant &v = VARIANTS[i];
         if (v.W != W) continue;
         const uint64_t need = (q.d + v.U * 128u - 1u) / (v.U * 128u);        // CTAs that hold a row
-        for (uint32_t cluster = 0; cluster < 2u; ++cluster) {
+        for (const uint32_t exchange : {(uint32_t)CLUSTER, (uint32_t)(q.nsteps * q.K == 1u ? PLAIN : GROUP)}) {
             Plan c = {};
             c.v = &v;
-            c.cluster = cluster;
+            c.exchange = exchange;
             uint32_t waves = 1u;
-            if (cluster) {
+            if (exchange == CLUSTER) {
                 uint32_t l = 0;
                 while ((1u << l) < need && l < 5u) ++l;
                 if (l > 4u || g_room[q.device][i][l] == 0u) continue;
@@ -643,16 +751,25 @@ int qesgd_launch_lr_tile(const QesgdTileCall &q, uint32_t smem_limit, float othe
     a.header = q.header; a.acc = q.acc; a.wide = q.wide;
     a.status = q.status; a.wait_ns = q.wait_ns; a.poll_mask = q.wait_ns < COARSE_TIMER_NS ? 0u : 31u;
     a.drop_cta = q.drop_cta;
+    a.claims = p.exchange == PLAIN ? q.header + EP_HEADER_WORDS : nullptr;       // the headers of other workers' groups, of which there are none
+    a.off_claims = p.off_claims;
+    static_assert(QESGD_MAX_WORKERS * EP_HEADER_WORDS >= EP_HEADER_WORDS + 256u, "a word for each CTA");
     CUtensorMap map = {}, map_rest = {};
     const uint32_t cols = p.v->U * 128u, rest = cols > 512u ? cols - 512u : cols;
     if (q.copy == 16 && !qesgd_lr_tensor_map(&map, q.X, (uint64_t)q.K * q.n_local, q.d, cols < 512u ? cols : 512u, true)) return -1;
     if (q.copy == 16 && cols > 512u && !qesgd_lr_tensor_map(&map_rest, q.X, (uint64_t)q.K * q.n_local, q.d, rest, true)) return -1;
-    const TileKernel kernel = p.v->kernel[p.cluster][q.copy == 16 ? 0 : (q.copy == 8 ? 1 : 2)];
+    const TileKernel kernel = p.v->kernel[p.exchange][q.copy == 16 ? 0 : (q.copy == 8 ? 1 : 2)];
     const uint32_t threads = W * 32u;
     cudaError_t err;
-    if (p.cluster) {
+    if (p.exchange == CLUSTER) {
         cudaLaunchAttribute at[2];
         const cudaLaunchConfig_t c = cluster_config(q.K * p.P, p.P, threads, p.bytes, q.stream, at);
+        err = cudaLaunchKernelEx(&c, kernel, a, map, map_rest);
+    } else if (p.exchange == PLAIN) {
+        cudaLaunchAttribute at[2];
+        cudaLaunchConfig_t c = cluster_config(p.P, 1u, threads, p.bytes, q.stream, at);
+        at[0] = at[1];           // no cluster
+        c.numAttrs = 1;
         err = cudaLaunchKernelEx(&c, kernel, a, map, map_rest);
     } else {
         void *params[] = {(void *)&a, (void *)&map, (void *)&map_rest};

@@ -1039,6 +1039,40 @@ def test_lr_gradient_and_single_step_run_beside_a_kernel_of_another_stream(m, d,
     c.close()
 
 
+@pytest.mark.parametrize("m,d,step", [(64, 65536, False), (40, 50002, True), (100, 30001, False), (16, 100000, True), (64, 80000, True)])
+def test_lr_gradient_takes_over_slices_whose_ctas_cannot_start(m, d, step):
+    """The grid of one minibatch is launched plainly, so some of its CTAs may start late.  Here 120 other streams'
+    kernels hold an SM each for some 100 ms: those CTAs that can start take the slices of the others over, the call is
+    done before the others' kernels end, and the result is the one of an idle device bit for bit.  Then once more,
+    idle: the workspace is as it was found."""
+    X, y, _ = synthetic.logistic_problem(m, d, seed=m + d)
+    w = (0.3 * synthetic.normal_f32(d, 1.0, 8)).astype(np.float32)
+    tX, ty, tw = G.dev(X), G.dev(y), G.dev(w)
+    own, others = torch.cuda.Stream(), [torch.cuda.Stream() for _ in range(120)]
+    c = qesgd.Context(0, own)
+    results = []
+    for busy in (False, True, False):
+        out = tw.clone() if step else torch.zeros(d, device="cuda")
+        torch.cuda.synchronize()
+        if busy:
+            for s in others:
+                with torch.cuda.stream(s):
+                    torch.cuda._sleep(200_000_000)
+            time.sleep(0.005)
+        if step:
+            c.qesgd_lr_sgd_step(tX, ty, m, d, 0.5, out)
+        else:
+            c.qesgd_lr_gradient(tX, ty, m, d, tw, out)
+        own.synchronize()
+        assert not busy or not others[-1].query(), "waited for the other streams' kernels"
+        torch.cuda.synchronize()
+        assert c.qesgd_status() == 0
+        results.append(out)
+    assert torch.equal(results[0], results[1]) and torch.equal(results[0], results[2])
+    _lr_close(results[1].cpu().numpy(), ref.lr_sgd_step(X, y, 0.5, w) if step else ref.lr_gradient(X, y, w))
+    c.close()
+
+
 @pytest.mark.parametrize("alpha", [-0.1, 1.0, -3.5])
 @pytest.mark.parametrize("K,bucket,bits,s", [(4, 128, 4, 7), (16, 256, 2, 1), (3, 1024, 8, 127)])
 def test_decode_average_axpy_matches_oracle(K, bucket, bits, s, alpha):
