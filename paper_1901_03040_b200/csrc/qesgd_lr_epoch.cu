@@ -454,26 +454,78 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + (EB == 16 ? EP_PRODUCERS : EP_
             float acc[SUB];
 #pragma unroll
             for (int r = 0; r < SUB; ++r) acc[r] = 0.0f;
+            if constexpr (NC == 1 && EB == 16) {
+                // Two blocks are requested at a time: one chain has the registers, and where slices are wide the time
+                // until a slot is free again is what the last sub-tiles of a minibatch wait for (six slots for eight
+                // sub-tiles: the margins of the six take 2330 clocks for 2940).  K = 4, n = 512, d = 131072 238.6 ->
+                // 230.8 us, n = 256, d = 140000, batch 32 138.4 -> 132.3; with element-wise copies, whose blocks have
+                // 128 registers a thread, 152.8 -> 164.2 (K = 3, n = 300, d = 131073).
+                auto load = [&](uint32_t it, float4 (&x)[SUB]) {
+                    const uint32_t b0 = it / BOX_UNITS * BOX, c = it * 128u + lane * 4u;
+                    const uint32_t pitch = min(a.cols - b0, BOX);
+                    const float *const from = xs + SUB * b0 + (c - b0);
+                    if (rows >= (uint32_t)SUB && it * 128u + 128u <= a.cols) {
+#pragma unroll
+                        for (uint32_t r = 0; r < (uint32_t)SUB; ++r) x[r] = *reinterpret_cast<const float4 *>(from + r * pitch);
+                    } else {
+#pragma unroll
+                        for (uint32_t r = 0; r < (uint32_t)SUB; ++r)
+                            x[r] = (c < a.cols && r < rows) ? *reinterpret_cast<const float4 *>(from + r * pitch)
+                                                            : make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+                };
+                auto margins = [&](const float4 uu, const float4 (&x)[SUB]) {
+#pragma unroll
+                    for (int r = 0; r < SUB; ++r) {
+                        acc[r] = fmaf(x[r].x, uu.x, acc[r]);
+                        acc[r] = fmaf(x[r].y, uu.y, acc[r]);
+                        acc[r] = fmaf(x[r].z, uu.z, acc[r]);
+                        acc[r] = fmaf(x[r].w, uu.w, acc[r]);
+                    }
+                };
+                const float *const ul = us + lane * 4u;
+                float4 x0[SUB], x1[SUB];
+                uint32_t it = 0u;
 #pragma unroll 1
-            for (uint32_t it = 0; it < a.nit; ++it) {
-                const uint32_t b0 = it / BOX_UNITS * BOX, c = it * 128u + lane * 4u;
-                const uint32_t pitch = min(a.cols - b0, BOX);
-                const float *const base = xs + SUB * b0 + (c - b0);
-                const float4 uu = *reinterpret_cast<const float4 *>(us + c);
-                float4 x[SUB];
-#pragma unroll
-                for (uint32_t r = 0; r < (uint32_t)SUB; ++r)
-                    x[r] = (c < a.cols && r < rows) ? *reinterpret_cast<const float4 *>(base + r * pitch)
-                                                    : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                for (int r = 0; r < SUB; ++r) {
-                    acc[r] = fmaf(x[r].x, uu.x, acc[r]);
-                    acc[r] = fmaf(x[r].y, uu.y, acc[r]);
-                    acc[r] = fmaf(x[r].z, uu.z, acc[r]);
-                    acc[r] = fmaf(x[r].w, uu.w, acc[r]);
+                for (; it + 1u < a.nit; it += 2u) {
+                    load(it, x0);
+                    const float4 u0 = *reinterpret_cast<const float4 *>(ul + it * 128u);
+                    load(it + 1u, x1);
+                    const float4 u1 = *reinterpret_cast<const float4 *>(ul + it * 128u + 128u);
+                    margins(u0, x0);
+                    margins(u1, x1);
+                    tmem_st32(taddr + 32u * unit, x0);
+                    tmem_st32(taddr + 32u * (unit + 1u), x1);
+                    unit += 2u;
                 }
-                tmem_st32(taddr + 32u * unit, x);
-                ++unit;
+                if (it < a.nit) {
+                    load(it, x0);
+                    margins(*reinterpret_cast<const float4 *>(ul + it * 128u), x0);
+                    tmem_st32(taddr + 32u * unit, x0);
+                    ++unit;
+                }
+            } else {
+#pragma unroll 1
+                for (uint32_t it = 0; it < a.nit; ++it) {
+                    const uint32_t b0 = it / BOX_UNITS * BOX, c = it * 128u + lane * 4u;
+                    const uint32_t pitch = min(a.cols - b0, BOX);
+                    const float *const base = xs + SUB * b0 + (c - b0);
+                    const float4 uu = *reinterpret_cast<const float4 *>(us + c);
+                    float4 x[SUB];
+#pragma unroll
+                    for (uint32_t r = 0; r < (uint32_t)SUB; ++r)
+                        x[r] = (c < a.cols && r < rows) ? *reinterpret_cast<const float4 *>(base + r * pitch)
+                                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                    for (int r = 0; r < SUB; ++r) {
+                        acc[r] = fmaf(x[r].x, uu.x, acc[r]);
+                        acc[r] = fmaf(x[r].y, uu.y, acc[r]);
+                        acc[r] = fmaf(x[r].z, uu.z, acc[r]);
+                        acc[r] = fmaf(x[r].w, uu.w, acc[r]);
+                    }
+                    tmem_st32(taddr + 32u * unit, x);
+                    ++unit;
+                }
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty[slot]);
