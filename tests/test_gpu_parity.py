@@ -1039,32 +1039,64 @@ def test_lr_gradient_and_single_step_run_beside_a_kernel_of_another_stream(m, d,
     c.close()
 
 
-@pytest.mark.parametrize("m,d,step", [(64, 65536, False), (40, 50002, True), (100, 30001, False), (16, 100000, True), (64, 80000, True)])
+_HOLD = r"""
+extern "C" __global__ void hold(int us)
+{
+    unsigned long long begin, now;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(begin));
+    for (int n = 0; n < us; ++n) {
+        __nanosleep(2000);
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+        if (now - begin > 1000ull * us) break;
+    }
+}
+"""
+
+
+class _Holder:
+    """Holds `sms` SMs for `ms` milliseconds, one block with most of the shared memory on each, on a stream that is
+    none of `own`."""
+    SMEM = 200 << 10
+
+    def __init__(self):
+        self.kernel = torch.cuda._compile_kernel(_HOLD, "hold")
+        self.kernel.set_shared_memory_config(self.SMEM)
+
+    def start(self, sms, ms, *own):
+        self.stream = torch.cuda.Stream()
+        while self.stream.cuda_stream in [s.cuda_stream for s in own]:     # they come out of a pool
+            self.stream = torch.cuda.Stream()
+        self.kernel((sms, 1, 1), (32, 1, 1), [int(ms * 1000)], self.SMEM, self.stream)
+        time.sleep(0.005)
+        assert not self.stream.query()
+
+    def holds(self):
+        return not self.stream.query()
+
+
+@pytest.mark.parametrize("m,d,step", [(64, 65536, False), (40, 50002, True), (100, 30001, False), (16, 80000, True), (64, 80000, True)])
 def test_lr_gradient_takes_over_slices_whose_ctas_cannot_start(m, d, step):
-    """The grid of one minibatch is launched plainly, so some of its CTAs may start late.  Here 120 other streams'
-    kernels hold an SM each for some 100 ms: those CTAs that can start take the slices of the others over, the call is
-    done before the others' kernels end, and the result is the one of an idle device bit for bit.  Then once more,
+    """The grid of one minibatch is launched plainly, so some of its CTAs may start late.  Here 100 SMs are held for
+    some 100 ms, so of the 98 to 131 CTAs at most 48 can start: those take the slices of the others over, the call is
+    done before the SMs are free again, and the result is the one of an idle device bit for bit.  Then once more,
     idle: the workspace is as it was found."""
     X, y, _ = synthetic.logistic_problem(m, d, seed=m + d)
     w = (0.3 * synthetic.normal_f32(d, 1.0, 8)).astype(np.float32)
     tX, ty, tw = G.dev(X), G.dev(y), G.dev(w)
-    own, others = torch.cuda.Stream(), [torch.cuda.Stream() for _ in range(120)]
+    own, holder = torch.cuda.Stream(), _Holder()
     c = qesgd.Context(0, own)
     results = []
     for busy in (False, True, False):
         out = tw.clone() if step else torch.zeros(d, device="cuda")
         torch.cuda.synchronize()
         if busy:
-            for s in others:
-                with torch.cuda.stream(s):
-                    torch.cuda._sleep(200_000_000)
-            time.sleep(0.005)
+            holder.start(100, 100, own)
         if step:
             c.qesgd_lr_sgd_step(tX, ty, m, d, 0.5, out)
         else:
             c.qesgd_lr_gradient(tX, ty, m, d, tw, out)
         own.synchronize()
-        assert not busy or not others[-1].query(), "waited for the other streams' kernels"
+        assert not busy or holder.holds(), "waited for the SMs that another stream's kernel holds"
         torch.cuda.synchronize()
         assert c.qesgd_status() == 0
         results.append(out)
