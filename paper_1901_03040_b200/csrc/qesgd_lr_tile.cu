@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
     float *const part = reinterpret_cast<float *>(tl_smem + a.off_part);
     uint64_t *const full = reinterpret_cast<uint64_t *>(tl_smem + a.off_bars);
     // [0] a wait ran out in this CTA, [1] always zero, [2] warps that have read their last margins, [3] the CTA is counted,
-    // [4 + slot] the slot's copy did not land in time, so no other was requested
+    // [4 + slot] bits: 1 the slot's copy did not land in time, 2 nor did its very first one, so no other is requested
     volatile uint32_t *const flag = reinterpret_cast<volatile uint32_t *>(tl_smem + a.off_flags);
 
     const uint32_t tid = threadIdx.x, lane = tid & 31u, w = tid >> 5;
@@ -284,8 +284,11 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
     };
     // a warp's rows of a landed slot into registers, zeros past the minibatch
     float4 x[U][SUB];
-    auto take = [&](bool landed, uint32_t slot, uint32_t parity, uint32_t rows) {
-        if (!landed && !mbar_wait(&full[slot], parity, &flag[0], a.wait_ns)) flag[0] = flag[4u + slot] = 1u;
+    auto take = [&](bool landed, uint32_t slot, uint32_t parity, uint32_t rows, uint32_t late) {
+        if (!landed && !mbar_wait(&full[slot], parity, &flag[0], a.wait_ns)) {
+            flag[0] = 1u;
+            flag[4u + slot] = flag[4u + slot] | late;
+        }
         const float *const from = ring + slot * SLOT + lane * 4u;
 #pragma unroll
         for (uint32_t it = 0; it < U; ++it) {
@@ -327,7 +330,7 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
     for (uint32_t e = 0; e < UPT; ++e)
         if (tid + e * W * 32u < COLS) us[tid + e * W * 32u] = u0[e];
     if (CL) cluster_wait();
-    if (w < subs_of(0u)) take(false, slot, 0u, rows_of(0u) - w * SUB);
+    if (w < subs_of(0u)) take(false, slot, 0u, rows_of(0u) - w * SUB, 2u);
     if (!plain) {
         __syncthreads();
     } else if (__syncthreads_or((int)taken) != 0) {               // another CTA does this slice; every copy requested has been taken
@@ -345,11 +348,11 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
     const uint32_t pitch = kept(a.x_pitch * 8u), words = smem_u32(tl_smem + a.off_x), odd = kept(P * pitch), send_r = send_row(P, lane);
     const uint32_t send_to = !CL || send_rank(P, lane) >= P ? 0u : cluster_address(words + rank * pitch + (w * SUB + send_r) * 8u, send_rank(P, lane));
     const uint32_t read_at = words + (lane & 3u) * pitch + my_row * 8u;
-    auto refill = [&](uint32_t t) {
+    auto refill = [&](uint32_t t, uint32_t late) {
         __syncwarp();            // every lane's rows are in its registers
-        if ((!EARLY || flag[4u + slot] == 0u) && t + next_t < nsteps && next_s < subs_of(t + next_t)) request(slot, t + next_t, next_s);
+        if ((!EARLY || (flag[4u + slot] & late) == 0u) && t + next_t < nsteps && next_s < subs_of(t + next_t)) request(slot, t + next_t, next_s);
     };
-    if (EARLY && w < subs_of(0u)) refill(0u);
+    if (EARLY && w < subs_of(0u)) refill(0u, 2u);          // (bit 1 here would be the next turn's, by another warp)
     bool gave_up = false;
     uint32_t gave_up_at = 0u, clears = 0u;
     uint32_t counted = ~0u;                                // by the warp that counted the CTA: how many were before it
@@ -357,6 +360,10 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
     uint32_t t = 0u, m = nsteps == 1u ? m_last : batch, subs = nsteps == 1u ? nsub_last : nsub;
     float ry = (nsteps == 1u ? a.rate_last : a.rate) * yj;
     bool signal = blockIdx.x != a.drop_cta;
+    if ((flag[4u + slot] & 2u) != 0u) {    // the first copy is not there: nothing goes out, and the block leaves after this step
+        signal = false;
+        if (!EARLY) next_t = nsteps;       // no refill (EARLY: refused above)
+    }
 
     for (;;) {
         const bool last = t + 1u == nsteps;
@@ -386,7 +393,7 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
             } else if ((lane & 3u) == 0u && my_row < m && signal) {
                 exchange_add(acc_t, wide_t, tot);
             }
-            if (!EARLY) refill(t);
+            if (!EARLY) refill(t, 0u);
             if (t == 0u)         // the rest of the ring's first turn
                 for (uint32_t n = w + 2u * nsub, v = 2u; n < nslots && v < nsteps; n += nsub, ++v)
                     if (w < subs_of(v)) request(n, v, w);
@@ -511,8 +518,8 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
         slot = next_slot;
         parity = next_parity;
         if (more) {
-            take(landed, slot, parity, next_m - w * SUB);
-            if (EARLY) refill(t + 1u);
+            take(landed, slot, parity, next_m - w * SUB, 1u);
+            if (EARLY) refill(t + 1u, 3u);
         }
         if (sync_any(1u, W * 32u, flag[0])) {
             gave_up = true;
@@ -559,11 +566,16 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
 
     if (gave_up) {
         if (tid == 0) atomicOr(a.status, QESGD_STATUS_TIMEOUT);
-        // every copy requested: sub-tile n goes to slot n % nslots, and the warps have requested all below `requested`
-        const uint32_t total = (nsteps - 1u) * nsub + nsub_last;
-        const uint32_t requested = min(total, (gave_up_at + EARLY) * nsub + subs_of(min(gave_up_at + EARLY, nsteps - 1u)) + nslots);
-        for (uint32_t q = tid; q < nslots && q < requested; q += W * 32u)
-            mbar_wait(&full[q], ((requested - 1u - q) / nslots - (EARLY ? flag[4u + q] : 0u)) & 1u, &flag[1], DRAIN_LIMIT_NS);
+        // Every slot's last copy has landed before the block ends, so that none is on its way into memory that another block
+        // then owns.  Sub-tile n goes to slot n % nslots, and all below `requested` have been requested, but for those that
+        // would have followed a late one: `next` is the minibatch taken last.
+        const uint32_t total = (nsteps - 1u) * nsub + nsub_last, next = min(gave_up_at + EARLY, nsteps - 1u);
+        const uint32_t requested = min(total, (gave_up_at + EARLY) * nsub + subs_of(next) + nslots);
+        for (uint32_t q = tid; q < nslots && q < requested; q += W * 32u) {
+            const uint32_t late = flag[4u + q];
+            const uint32_t turn = late & 2u ? 0u : (EARLY && late != 0u ? next * nsub + nslots - 1u - q : requested - 1u - q) / nslots;
+            mbar_wait(&full[q], turn & 1u, &flag[1], DRAIN_LIMIT_NS);
+        }
         if (CL) {
             cluster_arrive();
             cluster_wait();

@@ -801,6 +801,42 @@ def test_local_epoch_with_a_wait_limit_below_the_timer_resolution(K, n_local, d,
     c.close()
 
 
+@pytest.mark.parametrize("K,n_local,d,batch", [
+    (2, 1000, 200, 64),      # one block of columns, a ring of a few of the epoch's minibatches
+    (1, 2000, 784, 16),
+    (4, 1500, 1999, 32),     # the same by element-wise copies
+    (3, 900, 3000, 40),      # two blocks
+    (8, 1010, 10000, 50),    # five blocks, a ring shorter than two minibatches
+    (4, 700, 9998, 50),
+    (1, 1010, 10000, 50),    # groups through global memory: one block
+    (4, 400, 16384, 32),     # four
+])
+@pytest.mark.parametrize("limit", [100, 1100, 2500])
+def test_lr_epoch_in_registers_whose_first_copies_are_late(K, n_local, d, batch, limit):
+    """Limits that the first copies out of HBM exceed or just meet, rings that are shorter than the epoch: a block
+    that leaves then must not refill a slot whose copy has not landed, and must wait for what it has requested and
+    no longer, 2 seconds at the most being its own bound for that.  Then the context recovers, bit for bit."""
+    X, y, _ = synthetic.logistic_problem(K * n_local, d, seed=9)
+    u0 = (0.1 * synthetic.normal_f32(d, 1.0, 23)).astype(np.float32)
+    tX, ty = G.dev(X), G.dev(y)
+    want, status = _epoch_once(G.ctx(), tX, ty, n_local, d, K, batch, u0)
+    assert status == 0
+    _lr_close(want[K - 1].cpu().numpy(), ref.lr_local_epoch(X[-n_local:], y[-n_local:], batch, 0.5, u0))
+    c = qesgd.Context(0, None)
+    for _ in range(4):
+        c.qesgd_set_wait_limit(limit)
+        torch.zeros(64 << 20, device="cuda").add_(1.0)     # X is not in L2
+        torch.cuda.synchronize()
+        start = time.time()
+        got, status = _epoch_once(c, tX, ty, n_local, d, K, batch, u0)
+        assert time.time() - start < 1.0
+        assert status == qesgd.STATUS_TIMEOUT or (status == 0 and torch.equal(got, want))
+        c.qesgd_set_wait_limit(0)
+        got, status = _epoch_once(c, tX, ty, n_local, d, K, batch, u0)
+        assert status == 0 and torch.equal(got, want)
+    c.close()
+
+
 # ----------------------------------------------- per-step QESGD (Algorithm 2) ---
 def _gpu_requantize(u, w, zsum, bucket, s, bits, mode, seed, worker, step, fixed_delta=0.0,
                     misalign=0):
