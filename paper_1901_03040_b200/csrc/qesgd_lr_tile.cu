@@ -333,7 +333,9 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
     if (w < subs_of(0u)) take(false, slot, 0u, rows_of(0u) - w * SUB, 2u);
     if (!plain) {
         __syncthreads();
-    } else if (__syncthreads_or((int)taken) != 0) {               // another CTA does this slice; every copy requested has been taken
+    } else if (__syncthreads_or((int)taken) != 0) {               // another CTA does this slice
+        // every copy requested has been taken, or was late and is waited for here as at the end
+        if (tid < nslots && flag[4u + tid] != 0u) mbar_wait(&full[tid], 0u, &flag[1], DRAIN_LIMIT_NS);
         uint32_t before = 0u;
         if (tid == 0) asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(before) : "l"(a.header + 1) : "memory");
         if (w == 0u && __shfl_sync(0xFFFFFFFFu, before, 0) == P - 1u) leave_clear(a, lane);
