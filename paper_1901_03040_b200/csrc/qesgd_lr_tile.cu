@@ -51,10 +51,12 @@ struct TileArgs {
     uint32_t *status;
     uint64_t wait_ns;
     uint32_t poll_mask, drop_cta;
-    uint32_t *claims;            // one minibatch, plain launch: [P] slices that a CTA has begun; else null
+    uint32_t *claims;            // one minibatch, plain launch: [P] Claim of each slice; else null
     uint32_t off_claims;         // shared memory: the coefficients, then how many slices this CTA took over and which
 };
 constexpr uint64_t TL_STEAL_NS = 20000ull;   // a wait longer than this looks for slices that nobody has begun
+constexpr uint64_t TL_BEGIN_NS = 2000000000ull;   // by then every slice has been begun
+enum Claim { FREE = 0, BEGUN = 1, TAKEN = 2 };    // of a slice: BEGUN by a CTA that runs, or its margins are out; TAKEN over, not yet out
 constexpr uint32_t TL_ROWS = 128;            // coefficients kept for them
 
 __device__ __forceinline__ uint32_t cluster_address(uint32_t addr, uint32_t rank)
@@ -147,20 +149,28 @@ __device__ __forceinline__ uint32_t kept(uint32_t v)
 // longer than 20 us claims one that is still free and does its margins here, by the same operations in the same order, and
 // after its own update the CTA does theirs.  A CTA that finds its slice claimed has nothing left to do.
 //
-// A warp looks for a free slice and adds its partial margins to the rows' accumulators.
+// The wait limit is about CTAs that run and do not answer.  Time in which slices have not been begun, because other
+// streams' kernels hold the SMs, or are being made up for, does not count: a limit of 100 us is no reason to give a call
+// up that takes 131 us beside 120 kernels.  It counts from when a look finds every slice BEGUN.
+//
+// A warp looks whether every slice has been begun (then true); where that is `due` it takes a free one and adds its
+// partial margins to the rows' accumulators.
 template <int U>
-__device__ __noinline__ void take_over(const TileArgs &a, uint32_t *list, uint32_t lane)
+__device__ __noinline__ bool take_over(const TileArgs &a, uint32_t *list, bool due, uint32_t lane)
 {
     uint32_t slice = ~0u;
+    bool begun = true;
     for (uint32_t b = 0; b < a.P && slice == ~0u; b += 32u) {
-        const uint32_t free = __ballot_sync(0xFFFFFFFFu, b + lane < a.P && ld_acquire(a.claims + b + lane) == 0u);
-        if (free == 0u) continue;
+        const uint32_t claim = b + lane < a.P ? ld_acquire(a.claims + b + lane) : (uint32_t)BEGUN;
+        if (__any_sync(0xFFFFFFFFu, claim != BEGUN)) begun = false;
+        const uint32_t free = __ballot_sync(0xFFFFFFFFu, claim == FREE);
+        if (free == 0u || !due) continue;
         const uint32_t first = b + (uint32_t)__ffs((int)free) - 1u;
-        uint32_t before = 1u;
-        if (lane == 0) before = atomicCAS(a.claims + first, 0u, 1u);
-        if (__shfl_sync(0xFFFFFFFFu, before, 0) == 0u) slice = first;
+        uint32_t before = BEGUN;
+        if (lane == 0) before = atomicCAS(a.claims + first, (uint32_t)FREE, (uint32_t)TAKEN);
+        if (__shfl_sync(0xFFFFFFFFu, before, 0) == FREE) slice = first;
     }
-    if (slice == ~0u) return;
+    if (slice == ~0u) return begun;
     if (lane == 0) list[1u + atomicAdd(list, 1u)] = slice;
     const uint32_t m = a.m_last;
     for (uint32_t s = 0; s < a.nsub_last; ++s) {
@@ -177,6 +187,10 @@ __device__ __noinline__ void take_over(const TileArgs &a, uint32_t *list, uint32
         const uint32_t row = s * SUB + (lane >> 2);
         if ((lane & 3u) == 0u && row < m) exchange_add(a.acc + acc_index(row), a.wide + (size_t)row * EP_WIDE_WORDS, tot);
     }
+    __threadfence();
+    __syncwarp();
+    if (lane == 0) atomicExch(a.claims + slice, (uint32_t)BEGUN);
+    return false;
 }
 // Counted last of the group: nobody adds or reads any more.  By a warp; the accumulators that the epoch has used.
 __device__ __noinline__ void leave_clear(const TileArgs &a, uint32_t lane)
@@ -252,7 +266,7 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
     if (CL) cluster_arrive();    // waited for before the first store into another CTA
     if (CL || plain) qesgd_wait_for_previous();
     uint32_t taken = 0u;
-    if (plain && tid == 0) taken = atomicExch(a.claims + rank, 1u);
+    if (plain && tid == 0) taken = atomicCAS(a.claims + rank, (uint32_t)FREE, (uint32_t)BEGUN);
 
     const uint32_t row0 = (uint32_t)((uint64_t)worker * a.n_local);
     auto rows_of = [&](uint32_t t) { return t + 1u == nsteps ? a.m_last : batch; };
@@ -475,16 +489,21 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
                 unsigned long long v = 0ull;
                 bool done = (lane & 3u) != 0u || my_row >= m;
                 const bool reads = !done;
+                bool begun = false;          // every slice: from then on the limit counts
                 for (;;) {
                     for (uint32_t n = 0; !done && n <= a.poll_mask; ++n) done = ((v = ld_relaxed(acc_t)) >> 55) >= P;
                     if (__all_sync(0xFFFFFFFFu, done)) break;
                     if (looks++ == 0u) t0 = now_ns();
-                    const bool stop = flag[0] != 0u || ld_acquire(header) != 0u || expired(t0, a.wait_ns);
+                    const bool stop = flag[0] != 0u || ld_acquire(header) != 0u || (begun && expired(t0, a.wait_ns));
                     if (__any_sync(0xFFFFFFFFu, stop)) {
                         flag[0] = 1u;
                         break;
                     }
-                    if (__any_sync(0xFFFFFFFFu, now_ns() - t0 > TL_STEAL_NS)) take_over<U>(a, list, lane);
+                    const bool due = __any_sync(0xFFFFFFFFu, now_ns() - t0 > TL_STEAL_NS) != 0;
+                    if (!begun && (due || __any_sync(0xFFFFFFFFu, expired(t0, a.wait_ns)) != 0)) {
+                        begun = take_over<U>(a, list, due, lane) || __any_sync(0xFFFFFFFFu, now_ns() - t0 > TL_BEGIN_NS) != 0;
+                        if (begun) t0 = now_ns();
+                    }
                 }
                 if (reads) margin = exchange_margin(v, wide_t, P);
             }

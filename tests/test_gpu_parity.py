@@ -1141,6 +1141,45 @@ def test_lr_gradient_takes_over_slices_whose_ctas_cannot_start(m, d, step):
     c.close()
 
 
+@pytest.mark.parametrize("limit", [30_000, 100_000])
+@pytest.mark.parametrize("m,d,step", [(64, 65536, False), (40, 50002, True), (100, 30001, True), (16, 80000, False)])
+def test_lr_gradient_wait_limit_leaves_out_ctas_that_cannot_start(m, d, step, limit):
+    """The limit is about CTAs that run: with 130 SMs held the few that can start take over slice after slice, which
+    takes longer than the limit, and the call is done all the same.  A CTA that runs and does not answer exhausts it,
+    beside the other kernel too."""
+    X, y, _ = synthetic.logistic_problem(m, d, seed=m + d)
+    w = (0.3 * synthetic.normal_f32(d, 1.0, 8)).astype(np.float32)
+    tX, ty, tw = G.dev(X), G.dev(y), G.dev(w)
+    own, holder = torch.cuda.Stream(), _Holder()
+    c = qesgd.Context(0, own)
+
+    def call(busy):
+        out = tw.clone() if step else torch.zeros(d, device="cuda")
+        torch.cuda.synchronize()
+        if busy:
+            holder.start(130, 100, own)
+        if step:
+            c.qesgd_lr_sgd_step(tX, ty, m, d, 0.5, out)
+        else:
+            c.qesgd_lr_gradient(tX, ty, m, d, tw, out)
+        status = c.qesgd_status()
+        assert not busy or holder.holds(), "waited for the SMs that another stream's kernel holds"
+        torch.cuda.synchronize()
+        return out, status
+
+    want, status = call(False)
+    assert status == 0
+    c.qesgd_set_wait_limit(limit)
+    got, status = call(True)
+    assert status == 0 and torch.equal(got, want)
+    c.qesgd_debug_drop_signal(0)
+    assert call(True)[1] == qesgd.STATUS_TIMEOUT
+    c.qesgd_debug_drop_signal(-1)
+    got, status = call(False)
+    assert status == 0 and torch.equal(got, want)
+    c.close()
+
+
 @pytest.mark.parametrize("alpha", [-0.1, 1.0, -3.5])
 @pytest.mark.parametrize("K,bucket,bits,s", [(4, 128, 4, 7), (16, 256, 2, 1), (3, 1024, 8, 127)])
 def test_decode_average_axpy_matches_oracle(K, bucket, bits, s, alpha):
