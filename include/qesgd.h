@@ -256,6 +256,17 @@ int qesgd_set_wait_limit(qesgd_ctx *ctx, uint64_t nanoseconds);
  * for them runs out after the wait limit, the kernel returns and QESGD_STATUS_TIMEOUT is
  * set.  Nothing faults or hangs.  cta = -1 (the default) switches the hook off. */
 int qesgd_debug_drop_signal(qesgd_ctx *ctx, int64_t cta);
+/* Test hook: how the context's last local epoch, single step or gradient was launched (tests that aim at one
+ * kernel ask, so that a change of the rules does not move them elsewhere unnoticed).  plan[0] is one of
+ * QESGD_LR_*; the rest describes the kernel and is 0 for two passes: [1] CTAs that share a worker's columns,
+ * [2] columns of each, [3] its chains of eight warps (PERSISTENT) or its warps, [4] slots of its ring, [5] bytes of
+ * a copy (16 = TMA), [6] CTAs in all, [7] workers that a CTA runs at most. */
+#define QESGD_LR_TWO_PASSES 0u /* a margin pass and an update pass per minibatch */
+#define QESGD_LR_PERSISTENT 1u /* groups of a cooperative grid, minibatches in tensor memory */
+#define QESGD_LR_CLUSTER 2u    /* a cluster for each worker, minibatches in registers */
+#define QESGD_LR_GROUP 3u      /* a group of a cooperative grid for each worker, minibatches in registers */
+#define QESGD_LR_PLAIN 4u      /* one minibatch by a grid that is launched plainly */
+int qesgd_debug_lr_plan(const qesgd_ctx *ctx, uint32_t plan[8]);
 
 /*
  * The paper has no counterpart for this entry point; it exists for callers that are

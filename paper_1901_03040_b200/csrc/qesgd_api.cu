@@ -72,6 +72,7 @@ int qesgd_create(qesgd_ctx **out, int device, void *cuda_stream)
     ctx->lr_work_floats = QESGD_LR_WORK_FLOATS;
     ctx->wait_ns = QESGD_DEFAULT_WAIT_NS;
     ctx->drop_cta = 0xFFFFFFFFu;
+    for (uint32_t &v : ctx->lr_plan) v = 0u;
     DeviceGuard guard(device);
     if (!guard.ok) { delete ctx; return QESGD_ECUDA; }
     cudaError_t e = cudaMalloc((void **)&ctx->d_status, 256);
@@ -125,6 +126,13 @@ int qesgd_debug_drop_signal(qesgd_ctx *ctx, int64_t cta)
 {
     if (!ctx || cta < -1 || cta > 0x7FFFFFFF) return QESGD_EINVAL;
     ctx->drop_cta = cta < 0 ? 0xFFFFFFFFu : (uint32_t)cta;
+    return QESGD_OK;
+}
+
+int qesgd_debug_lr_plan(const qesgd_ctx *ctx, uint32_t plan[8])
+{
+    if (!ctx || !plan) return QESGD_EINVAL;
+    for (int i = 0; i < 8; ++i) plan[i] = ctx->lr_plan[i];
     return QESGD_OK;
 }
 
@@ -393,7 +401,7 @@ int qesgd_lr_local_epoch_batch(qesgd_ctx *ctx, const float *X, const float *y, u
         int launched = 0;
         const int e = qesgd_launch_lr_epoch_fused(X, y, n_local, d, K, batch, lr, u, u, false, K > 1 ? u_stride : 0,
                                                   ctx->d_lr_epoch, ctx->d_status, ctx->device, ctx->sm_count,
-                                                  ctx->wait_ns, ctx->drop_cta, ctx->stream, &launched);
+                                                  ctx->wait_ns, ctx->drop_cta, ctx->stream, &launched, ctx->lr_plan);
         ctx->launches += (uint64_t)launched;
         if (e > 0) return cuda_fail(ctx, e);
         if (e == 0) return QESGD_OK;
@@ -435,7 +443,7 @@ int qesgd_lr_gradient(qesgd_ctx *ctx, const float *Xb, const float *yb, uint32_t
     if (!guard.ok) return cuda_fail(ctx, (int)cudaErrorInvalidDevice);
     int launched = 0;
     int e = qesgd_launch_lr_epoch_fused(Xb, yb, m, d, 1, m, -1.0f, w, g_out, true, 0, ctx->d_lr_epoch, ctx->d_status,
-                                        ctx->device, ctx->sm_count, ctx->wait_ns, ctx->drop_cta, ctx->stream, &launched);
+                                        ctx->device, ctx->sm_count, ctx->wait_ns, ctx->drop_cta, ctx->stream, &launched, ctx->lr_plan);
     ctx->launches += (uint64_t)launched;
     if (e > 0) return cuda_fail(ctx, e);
     if (e == 0) return QESGD_OK;

@@ -26,7 +26,8 @@ struct qesgd_ctx {
     int last_cuda_error;
     int sm_count;
     uint64_t wait_ns;       // limit of each wait inside the local-epoch kernel
-    uint32_t drop_cta;      // give-up-path test hook of the local-epoch kernel (none: ~0)
+    uint32_t drop_cta;      // give-up-path test hook of the local-epoch kernels (none: ~0)
+    uint32_t lr_plan[8];    // qesgd_debug_lr_plan
 };
 static const uint64_t QESGD_DEFAULT_WAIT_NS = 1000000000ull;
 static const uint64_t QESGD_MAX_WAIT_NS = 10000000000ull;
@@ -190,4 +191,4 @@ int qesgd_launch_lr_epoch_fused(const float *X, const float *y, uint64_t n_local
                                 uint32_t K, uint32_t batch, float lr, const float *u, float *dst,
                                 bool gradient, uint64_t u_stride, float *work, uint32_t *status, int device,
                                 int sm_count, uint64_t wait_ns, uint32_t drop_cta, cudaStream_t stream,
-                                int *launched);
+                                int *launched, uint32_t (&plan)[8]);

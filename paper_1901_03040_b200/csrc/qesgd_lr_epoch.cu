@@ -827,9 +827,10 @@ bool choose_split(Split &best, uint64_t d, uint32_t K, uint32_t m, uint32_t nsub
 int qesgd_launch_lr_epoch_fused(const float *X, const float *y, uint64_t n_local, uint64_t d,
                                 uint32_t K, uint32_t batch, float lr, const float *u, float *dst,
                                 bool gradient, uint64_t u_stride, float *work, uint32_t *status, int device, int sm_count, uint64_t wait_ns,
-                                uint32_t drop_cta, cudaStream_t stream, int *launched)
+                                uint32_t drop_cta, cudaStream_t stream, int *launched, uint32_t (&plan)[8])
 {
     *launched = 0;
+    for (uint32_t &v : plan) v = 0u;          // two passes, unless a kernel is launched here
     const uint32_t m_full = (uint32_t)(n_local < batch ? n_local : batch);
     if (m_full > (uint32_t)EP_MAX_M) return -1;
     const uint64_t nsteps64 = (n_local + m_full - 1) / m_full;
@@ -857,7 +858,7 @@ int qesgd_launch_lr_epoch_fused(const float *X, const float *y, uint64_t n_local
     {
         const QesgdTileCall q = {X, y, n_local, d, nsteps64, K, m_full, lr, u, dst, gradient, u_stride, tma ? 16 : (pairs ? 8 : 4),
                                  header, acc, wide, status, device, nsteps64 * K == 1u ? sms - sms / 16u : sms, wait_ns, drop_cta, stream};
-        const int e = qesgd_launch_lr_tile(q, (uint32_t)limit, fits ? s.us : 1e30f, launched);
+        const int e = qesgd_launch_lr_tile(q, (uint32_t)limit, fits ? s.us : 1e30f, launched, plan);
         if (e >= 0) return e;
     }
     if (!fits) return -1;
@@ -911,5 +912,8 @@ int qesgd_launch_lr_epoch_fused(const float *X, const float *y, uint64_t n_local
     }
     if (e != cudaSuccess) return (int)e;
     *launched = 1;
+    const uint32_t shape[8] = {QESGD_LR_PERSISTENT, s.P, s.cols, s.NC, s.nslots, tma ? 16u : (pairs ? 8u : 4u), s.G * s.P,
+                               (K + s.G - 1u) / s.G};
+    for (int i = 0; i < 8; ++i) plan[i] = shape[i];
     return 0;
 }

@@ -735,7 +735,8 @@ float modelled_us(const Plan &p, const QesgdTileCall &q, uint32_t nsub, uint32_t
 //   K = 4, n = 1000, d = 16384, batch 32 (32 CTAs, four) 89.5 -> 72.3.
 // Where it loses and is not taken: more clusters than the device holds at once (K = 16, n = 200, d = 8000, batch 64: 32.5 in three
 // turns against 28.7); element-wise copies of many columns (K = 6, n = 700, d = 8003, batch 50: 57 against 49).
-int qesgd_launch_lr_tile(const QesgdTileCall &q, uint32_t smem_limit, float other_us, int *launched)
+int qesgd_launch_lr_tile(const QesgdTileCall &q, uint32_t smem_limit, float other_us, int *launched,
+                         uint32_t (&plan)[8])
 {
     const uint32_t nsub = (q.m + SUB - 1u) / SUB, W = nsub <= 8u ? 8u : 16u;
     if (nsub > 16u || !prepare_device(q.device, smem_limit)) return -1;
@@ -815,5 +816,8 @@ int qesgd_launch_lr_tile(const QesgdTileCall &q, uint32_t smem_limit, float othe
     }
     if (err != cudaSuccess) return (int)err;
     *launched = 1;
+    const uint32_t kind = p.exchange == PLAIN ? QESGD_LR_PLAIN : (p.exchange == CLUSTER ? QESGD_LR_CLUSTER : QESGD_LR_GROUP);
+    const uint32_t shape[8] = {kind, p.P, cols, W, p.nslots, (uint32_t)q.copy, q.K * p.P, 1u};
+    for (int i = 0; i < 8; ++i) plan[i] = shape[i];
     return 0;
 }

@@ -23,5 +23,7 @@ struct QesgdTileCall {
     uint32_t drop_cta;
     cudaStream_t stream;
 };
-// 0 = launched, -1 = not covered, or `the other kernel is modelled to be faster (`other_us` a step), > 0 = cudaError_t.
-int qesgd_launch_lr_tile(const QesgdTileCall &q, uint32_t smem_limit, float other_us, int *launched);
+// 0 = launched (`plan`: see qesgd_debug_lr_plan), -1 = not covered, or the other kernel is modelled to be faster
+// (`other_us` a step), > 0 = cudaError_t.
+int qesgd_launch_lr_tile(const QesgdTileCall &q, uint32_t smem_limit, float other_us, int *launched,
+                         uint32_t (&plan)[8]);

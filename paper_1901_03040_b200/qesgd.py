@@ -19,6 +19,7 @@ SCALE_NORM, SCALE_MAX, SCALE_FIXED = 0, 1, 2
 STATUS_NONFINITE = 1
 STATUS_TIMEOUT = 2
 STATUS_RANGE = 4
+LR_TWO_PASSES, LR_PERSISTENT, LR_CLUSTER, LR_GROUP, LR_PLAIN = range(5)
 OK, EINVAL, ECUDA, ENOMEM, ELIMIT = 0, -1, -2, -3, -4
 MAX_WORKERS, MIN_BUCKET, MAX_BUCKET, MAX_LR_BATCH = 64, 64, 8192, 1024
 NOALLOC_MAX_LR_BATCH = 256
@@ -38,6 +39,7 @@ SIGNATURES = {
     "qesgd_set_stream": (_int, [_vp, _vp]),
     "qesgd_set_wait_limit": (_int, [_vp, _u64]),
     "qesgd_debug_drop_signal": (_int, [_vp, C.c_int64]),
+    "qesgd_debug_lr_plan": (_int, [_vp, C.POINTER(_u32)]),
     "qesgd_num_buckets": (_u64, [_u64, _u32]),
     "qesgd_code_bytes": (_u64, [_u64, _u32, _u32]),
     "qesgd_encode": (_int, [_vp, _vp, _vp, _u64, _u32, _u32, _u32, _u32, _f32, _u64, _u32, _u32,
@@ -140,6 +142,12 @@ class Context:
 
     def qesgd_debug_drop_signal(self, cta):
         self._check(lib.qesgd_debug_drop_signal(self._h, cta))
+
+    def qesgd_debug_lr_plan(self):
+        """How the last local epoch, step or gradient was launched: LR_*, then the seven words that describe it."""
+        plan = (_u32 * 8)()
+        self._check(lib.qesgd_debug_lr_plan(self._h, plan))
+        return tuple(plan)
 
     # -- worker side ---------------------------------------------------------
     def qesgd_encode(self, local, anchor, d, bucket, s, bits, scale_mode, seed, worker, epoch,
