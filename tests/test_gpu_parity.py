@@ -486,7 +486,9 @@ def test_lr_local_epoch_shapes_match_oracle(K, n_local, d, batch):
     (4, 200, 65536, 64),     # two chains, last minibatch of eight rows
     (3, 130, 65536, 64),     # two chains over an odd number of workers
     (2, 150, 30000, 100),    # more rows than the warps of a chain take in one go
-    (1, 2000, 784, 16),      # many short steps of one group: the accumulator ring goes round 15 times
+    (1, 2000, 784, 16),      # many short steps
+    (3, 400, 65536, 32),     # the accumulator ring goes round five times
+    (1, 400, 20000, 16),     # three times, in registers
     (2, 40, 160000, 16),     # above 1024 columns per SM: two-pass steps
     (1, 8, 1, 8),            # rows on no 16-byte boundary from here on: one column
     (1, 20, 3, 7),
@@ -497,9 +499,9 @@ def test_lr_local_epoch_shapes_match_oracle(K, n_local, d, batch):
     (1, 300, 254, 256),
 ])
 def test_lr_local_epoch_splits_match_oracle(K, n_local, d, batch):
-    """The ways the persistent kernel deals an epoch out (groups of CTAs, one or two chains, slices
-    of up to 1024 columns, rings shorter than a minibatch, rows that TMA cannot fetch) at the edges of
-    their ranges, twice: the
+    """The ways an epoch is dealt out (by the persistent kernel over groups of CTAs, one or two chains, slices of up
+    to 1024 columns, rings shorter than a minibatch, rows that TMA cannot fetch; the short ones in registers) at the
+    edges of their ranges, twice: the
     second call finds the workspace as the first one left it.  Bound: fp32 dot products of d terms
     against fp64, as for the other logistic steps (1e-5)."""
     X, y, _ = synthetic.logistic_problem(K * n_local, d, seed=K + n_local + d)
@@ -584,28 +586,28 @@ def test_lr_local_epoch_updates_behind_the_next_margins_match_oracle(K, n_local,
             _lr_close(got[k], ref.lr_local_epoch(X[rows], y[rows], batch, 0.5, u0[k]))
 
 
-@pytest.mark.parametrize("K,n_local,d,batch", [
-    (1, 70, 100, 16),        # a CTA of its own, nothing to exchange
-    (2, 1000, 200, 64),      # clusters of two CTAs, one block of columns, the ring goes round
-    (3, 101, 384, 33),       # of four, one of them without columns; sub-tiles of one row
-    (2, 90, 900, 50),        # of eight
-    (9, 70, 1999, 20),       # of sixteen, element by element
-    (3, 70, 1002, 40),       # pairs of elements
-    (4, 160, 4096, 32),      # two blocks of columns
-    (1, 200, 6000, 64),      # three and more
-    (2, 100, 8000, 8),       # one sub-tile
-    (1, 90, 9998, 16),       # five blocks, pairs
-    (2, 250, 500, 100),      # sixteen warps
-    (3, 300, 1900, 128),
-    (1, 270, 2002, 121),
-    (24, 40, 2000, 32),      # more clusters than are resident at once
-    (1, 150, 17000, 64),     # groups of a cooperative grid: one block, 133 CTAs
-    (1, 90, 20001, 24),      # element by element
-    (8, 170, 10000, 50),     # five blocks, a ring of little more than a minibatch
-    (4, 200, 16384, 32),     # four blocks
-    (2, 300, 7000, 128),     # sixteen warps
+@pytest.mark.parametrize("K,n_local,d,batch,kind,columns,warps", [
+    (1, 70, 100, 16, qesgd.LR_CLUSTER, 128, 8),        # a CTA of its own, nothing to exchange
+    (2, 1000, 200, 64, qesgd.LR_CLUSTER, 128, 8),      # clusters of two CTAs, one block of columns, the ring goes round
+    (3, 101, 384, 33, qesgd.LR_CLUSTER, 128, 8),       # of four, one of them without columns; sub-tiles of one row
+    (2, 90, 900, 50, qesgd.LR_CLUSTER, 128, 8),        # of eight
+    (9, 70, 1999, 20, qesgd.LR_CLUSTER, 128, 8),       # of sixteen, element by element
+    (3, 70, 1002, 40, qesgd.LR_CLUSTER, 128, 8),       # pairs of elements
+    (4, 160, 4096, 32, qesgd.LR_CLUSTER, 256, 8),      # two blocks of columns
+    (1, 200, 6000, 64, qesgd.LR_CLUSTER, 384, 8),      # three and more
+    (2, 100, 8000, 8, qesgd.LR_CLUSTER, 512, 8),       # one sub-tile
+    (1, 90, 9998, 16, qesgd.LR_CLUSTER, 640, 8),       # five blocks, pairs
+    (2, 250, 500, 100, qesgd.LR_CLUSTER, 128, 16),     # sixteen warps
+    (3, 300, 1900, 128, qesgd.LR_CLUSTER, 128, 16),
+    (1, 270, 2002, 121, qesgd.LR_CLUSTER, 128, 16),
+    (64, 20, 2000, 16, qesgd.LR_CLUSTER, 512, 8),      # 256 CTAs: clusters that take turns
+    (1, 150, 17000, 64, qesgd.LR_GROUP, 128, 8),       # groups of a cooperative grid: one block, 133 CTAs
+    (1, 90, 20001, 24, qesgd.LR_GROUP, 256, 8),        # element by element
+    (8, 1010, 10000, 50, qesgd.LR_GROUP, 640, 8),      # five blocks, a ring of little more than a minibatch
+    (4, 200, 16384, 32, qesgd.LR_GROUP, 512, 8),       # four blocks
+    (2, 300, 7000, 128, qesgd.LR_GROUP, 128, 16),      # sixteen warps
 ])
-def test_lr_epochs_with_the_minibatch_in_registers_match_oracle(K, n_local, d, batch):
+def test_lr_epochs_with_the_minibatch_in_registers_match_oracle(K, n_local, d, batch, kind, columns, warps):
     """The kernel that keeps a minibatch's slice in registers, over its blocks of columns, warps, cluster sizes and
     kinds of copies, every worker from a point of its own.  Twice: the workspace and shared memory are as found.
     Bound as above (1e-5)."""
@@ -617,6 +619,8 @@ def test_lr_epochs_with_the_minibatch_in_registers_match_oracle(K, n_local, d, b
         tu = G.dev(u0)
         c.qesgd_lr_local_epoch_batch(tX, ty, n_local, d, K, batch, 0.5, tu, d)
         assert c.qesgd_status() == 0
+        plan = c.qesgd_debug_lr_plan()
+        assert (plan[0], plan[2], plan[3]) == (kind, columns, warps)
         runs.append(tu)
     assert torch.equal(runs[0], runs[1])
     got = runs[0].cpu().numpy()
@@ -625,8 +629,8 @@ def test_lr_epochs_with_the_minibatch_in_registers_match_oracle(K, n_local, d, b
         _lr_close(got[k], ref.lr_local_epoch(X[rows], y[rows], batch, 0.5, u0[k]))
 
 
-@pytest.mark.parametrize("d", [700, 1500, 20000])    # clusters, a group through global memory
-def test_lr_epoch_in_registers_carries_extreme_and_nonfinite_margins(d):
+@pytest.mark.parametrize("d,kind", [(700, qesgd.LR_CLUSTER), (1500, qesgd.LR_CLUSTER), (20000, qesgd.LR_PLAIN)])
+def test_lr_epoch_in_registers_carries_extreme_and_nonfinite_margins(d, kind):
     """Partial margins of 1e30 that cancel over the CTAs but for a remainder the size of one, rows of infinite and of
     NaN margins: the sum over the CTAs keeps the remainder, infinities saturate the step coefficient, NaN spreads."""
     m, lr = 16, 0.5
@@ -642,7 +646,7 @@ def test_lr_epoch_in_registers_carries_extreme_and_nonfinite_margins(d):
     tu = G.dev(u0)
     c = G.ctx()
     c.qesgd_lr_sgd_step(G.dev(X), G.dev(y), m, d, lr, tu)
-    assert c.qesgd_status() == 0
+    assert c.qesgd_status() == 0 and c.qesgd_debug_lr_plan()[0] == kind
     with np.errstate(all="ignore"):
         want = ref.lr_sgd_step(X, y, lr, u0)
     got = tu.cpu().numpy()
@@ -655,13 +659,20 @@ def test_lr_epoch_in_registers_carries_extreme_and_nonfinite_margins(d):
     assert np.isnan(tu.cpu().numpy()).all()
 
 
-@pytest.mark.parametrize("gain", [2e7, 1e9])
-def test_local_epoch_partial_margins_beyond_the_fine_fixed_point_range(gain):
-    """The CTAs of the persistent kernel add their partial margins as fixed-point integers: units
-    of 2^-28 below 2^17, units of 2^-6 from there on.  With features scaled by 2e7 about half of
-    the partial margins of a row take the coarse word and half the fine one; scaled by 1e9 all
+@pytest.mark.parametrize("half", [True, False])
+@pytest.mark.parametrize("K,n_local,d,batch,kind,large", [
+    (2, 64, 8192, 32, qesgd.LR_CLUSTER, 1e9),          # no fixed point here: sums of floats with their errors
+    (2, 400, 65536, 32, qesgd.LR_PERSISTENT, 1e9),     # 26 tiles: the ring of accumulators is cleared three times
+    (1, 400, 20000, 32, qesgd.LR_GROUP, 1e8),          # 13 minibatches, the last ones' partial margins near 2^49 with 1e9
+    (1, 70, 131073, 32, qesgd.LR_PERSISTENT, 1e9),     # element by element
+    (1, 64, 131074, 16, qesgd.LR_PERSISTENT, 1e9),
+])
+def test_local_epoch_partial_margins_beyond_the_fine_fixed_point_range(K, n_local, d, batch, kind, large, half):
+    """The CTAs of a cooperative grid add their partial margins as fixed-point integers: units
+    of 2^-28 below 2^17, units of 2^-6 from there to 2^49.  With features scaled by 2e7 about half of
+    the partial margins of a row take the coarse word and half the fine one; scaled by 1e8 and 1e9 all
     take the coarse one (and the second step's reach 1e13).  The oracle knows no such split."""
-    K, n_local, d, batch = 2, 64, 8192, 32
+    gain = 2e7 if half else large
     X, y, _ = synthetic.logistic_problem(K * n_local, d, seed=31)
     X = (X * np.float32(gain)).astype(np.float32)
     u0 = (0.1 * synthetic.normal_f32(d, 1.0, 24)).astype(np.float32)
@@ -669,7 +680,7 @@ def test_local_epoch_partial_margins_beyond_the_fine_fixed_point_range(gain):
     tu = torch.zeros((K, d), dtype=torch.float32, device="cuda")
     tu[:] = G.dev(u0)
     c.qesgd_lr_local_epoch_batch(G.dev(X), G.dev(y), n_local, d, K, batch, 0.5, tu, d)
-    assert c.qesgd_status() == 0
+    assert c.qesgd_status() == 0 and c.qesgd_debug_lr_plan()[0] == kind
     got = tu.cpu().numpy()
     assert np.isfinite(got).all()
     for k in range(K):
@@ -677,22 +688,26 @@ def test_local_epoch_partial_margins_beyond_the_fine_fixed_point_range(gain):
         _lr_close(got[k], ref.lr_local_epoch(X[rows], y[rows], batch, 0.5, u0))
 
 
-def test_local_epoch_nonfinite_features_spread_as_in_floating_point():
+@pytest.mark.parametrize("n_local,d,kind", [(96, 8192, qesgd.LR_CLUSTER), (96, 65536, qesgd.LR_PERSISTENT),
+                                            (500, 30000, qesgd.LR_GROUP), (70, 65537, qesgd.LR_PERSISTENT)])
+def test_local_epoch_nonfinite_features_spread_as_in_floating_point(n_local, d, kind):
     """A NaN feature makes its row's margin NaN and with it the worker's whole parameter; an
     infinite feature makes the margin that infinity, the step coefficient saturates, and only the
     feature's own column becomes non-finite.  Same pattern as the fp64 oracle; the other worker
-    and the finite entries stay within tolerance."""
-    K, n_local, d, batch = 2, 96, 8192, 32
+    and the finite entries stay within tolerance.  Then finite features: the words that count such margins are clear."""
+    K, batch = 2, 32
     X, y, _ = synthetic.logistic_problem(K * n_local, d, seed=32)
+    clean = X.copy()
     u0 = (0.1 * synthetic.normal_f32(d, 1.0, 25)).astype(np.float32)
+    last = n_local + (n_local - 1) // batch * batch
     X[40, 1234] = np.nan                     # worker 0, second minibatch
-    X[n_local + 70, 77] = np.inf             # worker 1, last minibatch
-    X[n_local + 80, 4000] = -np.inf
+    X[last + 2, 77] = np.inf                 # worker 1, last minibatch
+    X[last + 4, 4000] = -np.inf
     c = G.ctx()
     tu = torch.zeros((K, d), dtype=torch.float32, device="cuda")
     tu[:] = G.dev(u0)
     c.qesgd_lr_local_epoch_batch(G.dev(X), G.dev(y), n_local, d, K, batch, 0.5, tu, d)
-    assert c.qesgd_status() == 0
+    assert c.qesgd_status() == 0 and c.qesgd_debug_lr_plan()[0] == kind
     got = tu.cpu().numpy()
     with np.errstate(all="ignore"):
         want = [ref.lr_local_epoch(X[k * n_local:(k + 1) * n_local], y[k * n_local:(k + 1) * n_local],
@@ -703,9 +718,12 @@ def test_local_epoch_nonfinite_features_spread_as_in_floating_point():
     assert np.array_equal(np.isnan(got[1]), np.isnan(want[1]))
     assert np.array_equal(got[1][np.isinf(want[1])], want[1][np.isinf(want[1])])
     _lr_close(got[1][fin], want[1][fin])
+    tu[:] = G.dev(u0)
+    c.qesgd_lr_local_epoch_batch(G.dev(clean), G.dev(y), n_local, d, K, batch, 0.5, tu, d)
+    _lr_close(tu[0].cpu().numpy(), ref.lr_local_epoch(clean[:n_local], y[:n_local], batch, 0.5, u0))
 
 
-# ------------------------------ the local-epoch kernel gives up and recovers ---
+# ----------------------------- the local-epoch kernels give up and recover ---
 def _epoch_once(c, X, y, n_local, d, K, batch, u0):
     tu = torch.zeros((K, d), dtype=torch.float32, device="cuda")
     tu[:] = G.dev(u0)
@@ -713,18 +731,21 @@ def _epoch_once(c, X, y, n_local, d, K, batch, u0):
     return tu, c.qesgd_status()
 
 
-@pytest.mark.parametrize("K,n_local,d,batch", [
-    (2, 96, 8192, 32),       # a cluster of sixteen for each worker
-    (3, 200, 4096, 100),     # 13 sub-tiles
-    (4, 130, 65536, 64),     # two chains
-    (3, 130, 65536, 64),     # two chains, odd K
-    (1, 100, 1000, 32),      # a cluster of eight
-    (2, 40, 131072, 64),     # one chain, several workers: sums added up behind the next margins
-    (1, 100, 20000, 64),     # one chain, one worker
-    (2, 70, 10003, 32),      # element by element: 4-byte copies, several CTAs
-    (1, 70, 50002, 32),      # 8-byte copies
+@pytest.mark.parametrize("K,n_local,d,batch,kind,chains,copy", [
+    (2, 96, 8192, 32, qesgd.LR_CLUSTER, 8, 16),         # a cluster of sixteen for each worker
+    (3, 200, 4096, 100, qesgd.LR_CLUSTER, 16, 16),      # 13 sub-tiles
+    (4, 130, 65536, 64, qesgd.LR_PERSISTENT, 2, 16),    # two chains
+    (3, 130, 65536, 64, qesgd.LR_PERSISTENT, 2, 16),    # two chains, odd K
+    (1, 100, 1000, 32, qesgd.LR_CLUSTER, 8, 16),        # a cluster of eight
+    (2, 40, 131072, 64, qesgd.LR_PERSISTENT, 1, 16),    # one chain, several workers: sums added up behind the next margins
+    (1, 100, 140000, 64, qesgd.LR_PERSISTENT, 1, 16),   # one chain, one worker
+    (1, 100, 131073, 64, qesgd.LR_PERSISTENT, 1, 4),    # element by element: 4-byte copies
+    (1, 100, 131074, 64, qesgd.LR_PERSISTENT, 1, 8),    # 8-byte copies
+    (1, 100, 20000, 64, qesgd.LR_GROUP, 8, 16),         # groups, in registers
+    (2, 70, 10003, 32, qesgd.LR_GROUP, 8, 4),
+    (1, 70, 50002, 32, qesgd.LR_GROUP, 8, 8),
 ])
-def test_local_epoch_wait_runs_out_and_the_context_recovers(K, n_local, d, batch):
+def test_local_epoch_wait_runs_out_and_the_context_recovers(K, n_local, d, batch, kind, chains, copy):
     """One CTA never announces its partial margins of the first minibatch (a flag nothing
     sets), so every CTA's bounded wait for them runs out: the call returns, the status word
     reports the time-out, nothing faults, and the next call on the same context -- hook off,
@@ -737,6 +758,8 @@ def test_local_epoch_wait_runs_out_and_the_context_recovers(K, n_local, d, batch
     c.qesgd_debug_drop_signal(5)
     _, status = _epoch_once(c, tX, ty, n_local, d, K, batch, u0)
     assert status == qesgd.STATUS_TIMEOUT
+    plan = c.qesgd_debug_lr_plan()
+    assert (plan[0], plan[3], plan[5]) == (kind, chains, copy)
     assert c.qesgd_status() == 0                   # reading the status word cleared it
     c.qesgd_debug_drop_signal(-1)
     c.qesgd_set_wait_limit(0)                      # back to the default
@@ -752,8 +775,10 @@ def test_local_epoch_wait_runs_out_and_the_context_recovers(K, n_local, d, batch
     c.close()
 
 
-@pytest.mark.parametrize("m,d", [(64, 65536), (40, 10003)])
-def test_lr_gradient_wait_runs_out_and_the_context_recovers(m, d):
+@pytest.mark.parametrize("m,d,kind", [(64, 65536, qesgd.LR_PLAIN), (40, 10003, qesgd.LR_PLAIN), (64, 4096, qesgd.LR_CLUSTER),
+                                      (128, 65536, qesgd.LR_PERSISTENT), (33, 100002, qesgd.LR_PERSISTENT),
+                                      (200, 5001, qesgd.LR_PERSISTENT)])
+def test_lr_gradient_wait_runs_out_and_the_context_recovers(m, d, kind):
     """The same for the mean gradient, by TMA and element by element."""
     X, y, _ = synthetic.logistic_problem(m, d, seed=m)
     w = (0.1 * synthetic.normal_f32(d, 1.0, 22)).astype(np.float32)
@@ -762,7 +787,7 @@ def test_lr_gradient_wait_runs_out_and_the_context_recovers(m, d):
     c.qesgd_set_wait_limit(3_000_000)
     c.qesgd_debug_drop_signal(5)
     c.qesgd_lr_gradient(tX, ty, m, d, tw, g)
-    assert c.qesgd_status() == qesgd.STATUS_TIMEOUT
+    assert c.qesgd_status() == qesgd.STATUS_TIMEOUT and c.qesgd_debug_lr_plan()[0] == kind
     c.qesgd_debug_drop_signal(-1)
     c.qesgd_set_wait_limit(0)
     c.qesgd_lr_gradient(tX, ty, m, d, tw, g)
@@ -774,8 +799,11 @@ def test_lr_gradient_wait_runs_out_and_the_context_recovers(m, d):
     c.close()
 
 
-@pytest.mark.parametrize("K,n_local,d,batch", [(4, 256, 16384, 32), (2, 200, 131072, 64), (2, 100, 10003, 32), (1, 100, 50002, 32)])
-def test_local_epoch_with_a_wait_limit_below_the_timer_resolution(K, n_local, d, batch):
+@pytest.mark.parametrize("K,n_local,d,batch,kind", [
+    (4, 256, 16384, 32, qesgd.LR_GROUP), (2, 100, 10003, 32, qesgd.LR_GROUP), (1, 100, 50002, 32, qesgd.LR_GROUP),
+    (2, 200, 131072, 64, qesgd.LR_PERSISTENT), (3, 130, 65536, 64, qesgd.LR_PERSISTENT),
+    (1, 100, 131073, 64, qesgd.LR_PERSISTENT), (2, 70, 65538, 32, qesgd.LR_PERSISTENT)])
+def test_local_epoch_with_a_wait_limit_below_the_timer_resolution(K, n_local, d, batch, kind):
     """A limit under a microsecond means "look once more, then give up": ordinary latency
     between CTAs and of the TMA copies exhausts it at whatever point each CTA happens to be,
     so the give-up path is entered from many places at once.  The call must return either way;
@@ -789,7 +817,7 @@ def test_local_epoch_with_a_wait_limit_below_the_timer_resolution(K, n_local, d,
     for attempt in range(3):
         c.qesgd_set_wait_limit(100)
         got, status = _epoch_once(c, tX, ty, n_local, d, K, batch, u0)
-        assert status in (0, qesgd.STATUS_TIMEOUT)
+        assert status in (0, qesgd.STATUS_TIMEOUT) and c.qesgd_debug_lr_plan()[0] == kind
         if status == 0:
             for k in range(K):
                 _lr_close(got[k].cpu().numpy(), want[k])
@@ -801,18 +829,19 @@ def test_local_epoch_with_a_wait_limit_below_the_timer_resolution(K, n_local, d,
     c.close()
 
 
-@pytest.mark.parametrize("K,n_local,d,batch", [
-    (2, 1000, 200, 64),      # one block of columns, a ring of a few of the epoch's minibatches
-    (1, 2000, 784, 16),
-    (4, 1500, 1999, 32),     # the same by element-wise copies
-    (3, 900, 3000, 40),      # two blocks
-    (8, 1010, 10000, 50),    # five blocks, a ring shorter than two minibatches
-    (4, 700, 9998, 50),
-    (1, 1010, 10000, 50),    # groups through global memory: one block
-    (4, 400, 16384, 32),     # four
+@pytest.mark.parametrize("K,n_local,d,batch,kind", [
+    (2, 1000, 200, 64, qesgd.LR_CLUSTER),      # one block of columns, a ring of a few of the epoch's minibatches
+    (1, 2000, 784, 16, qesgd.LR_CLUSTER),
+    (4, 1500, 1999, 32, qesgd.LR_CLUSTER),     # the same by element-wise copies
+    (3, 900, 3000, 40, qesgd.LR_CLUSTER),      # two blocks
+    (2, 300, 8000, 8, qesgd.LR_CLUSTER),       # four, one sub-tile
+    (8, 1010, 10000, 50, qesgd.LR_GROUP),      # groups through global memory: five, a ring shorter than two minibatches
+    (4, 700, 9998, 50, qesgd.LR_GROUP),        # three
+    (1, 1010, 10000, 50, qesgd.LR_GROUP),      # one
+    (4, 400, 16384, 32, qesgd.LR_GROUP),       # four
 ])
 @pytest.mark.parametrize("limit", [100, 1100, 2500])
-def test_lr_epoch_in_registers_whose_first_copies_are_late(K, n_local, d, batch, limit):
+def test_lr_epoch_in_registers_whose_first_copies_are_late(K, n_local, d, batch, kind, limit):
     """Limits that the first copies out of HBM exceed or just meet, rings that are shorter than the epoch: a block
     that leaves then must not refill a slot whose copy has not landed, and must wait for what it has requested and
     no longer, 2 seconds at the most being its own bound for that.  Then the context recovers, bit for bit."""
@@ -821,6 +850,8 @@ def test_lr_epoch_in_registers_whose_first_copies_are_late(K, n_local, d, batch,
     tX, ty = G.dev(X), G.dev(y)
     want, status = _epoch_once(G.ctx(), tX, ty, n_local, d, K, batch, u0)
     assert status == 0
+    plan, subtiles = G.ctx().qesgd_debug_lr_plan(), -(-n_local // batch) * -(-batch // 8)
+    assert plan[0] == kind and plan[4] < subtiles
     _lr_close(want[K - 1].cpu().numpy(), ref.lr_local_epoch(X[-n_local:], y[-n_local:], batch, 0.5, u0))
     c = qesgd.Context(0, None)
     for _ in range(4):
@@ -1023,13 +1054,13 @@ def test_fused_inner_step_at_the_edges_of_its_tiles(m, d, bucket, bits, s, mode,
 
 
 @pytest.mark.parametrize("m,d", [
-    (200, 5001), (33, 65541), (256, 30000), (1, 4), (64, 9999),     # the persistent kernel
+    (200, 5001), (256, 30000), (33, 65541), (64, 9999), (1, 4),     # one launch: persistent kernel, plain grid, cluster
     (300, 5001), (1000, 20000), (17, 150001), (64, 150000),         # two passes, rows split over 19, 7, 1 and 1 CTAs per segment
     (64, 419432), (100, 250001),                                    # 107 MB backwards, 100.0 MB (below 96 MiB) forwards
     (100, 260001)])                                                 # backwards, element by element
 def test_lr_gradient_shapes_match_oracle(m, d):
-    """Both forms of the gradient: two passes with the rows split over CTAs where segments are few, and
-    the persistent kernel as an epoch of one step.  fp32 sums of d (margins) and m terms against fp64."""
+    """The forms of the gradient: two passes with the rows split over CTAs where segments are few, and
+    the kernels of local epochs for an epoch of one step.  fp32 sums of d (margins) and m terms against fp64."""
     X, y, _ = synthetic.logistic_problem(m, d, seed=m + d)
     w = (0.3 * synthetic.normal_f32(d, 1.0, 8)).astype(np.float32)
     tg = torch.full((d + 4,), 9.0, dtype=torch.float32, device="cuda")
@@ -1135,6 +1166,8 @@ def test_lr_gradient_takes_over_slices_whose_ctas_cannot_start(m, d, step):
         assert not busy or holder.holds(), "waited for the SMs that another stream's kernel holds"
         torch.cuda.synchronize()
         assert c.qesgd_status() == 0
+        plan = c.qesgd_debug_lr_plan()
+        assert plan[0] == qesgd.LR_PLAIN and plan[6] > 2 * 48      # two CTAs share an SM at most
         results.append(out)
     assert torch.equal(results[0], results[1]) and torch.equal(results[0], results[2])
     _lr_close(results[1].cpu().numpy(), ref.lr_sgd_step(X, y, 0.5, w) if step else ref.lr_gradient(X, y, w))
@@ -1168,7 +1201,7 @@ def test_lr_gradient_wait_limit_leaves_out_ctas_that_cannot_start(m, d, step, li
         return out, status
 
     want, status = call(False)
-    assert status == 0
+    assert status == 0 and c.qesgd_debug_lr_plan()[0] == qesgd.LR_PLAIN
     c.qesgd_set_wait_limit(limit)
     got, status = call(True)
     assert status == 0 and torch.equal(got, want)
