@@ -172,16 +172,18 @@ __device__ __noinline__ bool take_over(const TileArgs &a, uint32_t *list, bool d
     }
     if (slice == ~0u) return begun;
     if (lane == 0) list[1u + atomicAdd(list, 1u)] = slice;
-    const uint32_t m = a.m_last;
-    for (uint32_t s = 0; s < a.nsub_last; ++s) {
+    const uint32_t m = a.m_last, nsub = a.nsub_last;
+    const float *const X = a.X, *const u = a.u;
+    const uint64_t d = a.d;
+    for (uint32_t s = 0; s < nsub; ++s) {
         float acc[SUB];
         for (int r = 0; r < SUB; ++r) acc[r] = 0.0f;
         for (uint32_t it = 0; it < (uint32_t)U; ++it)
             for (int r = 0; r < SUB; ++r)
                 for (uint32_t e = 0; e < 4u; ++e) {
                     const uint64_t c = (uint64_t)slice * (U * 128u) + it * 128u + lane * 4u + e;
-                    const bool in = s * SUB + r < m && c < a.d;
-                    acc[r] = fmaf(in ? a.X[(uint64_t)(s * SUB + r) * a.d + c] : 0.0f, c < a.d ? a.u[c] : 0.0f, acc[r]);
+                    const bool in = s * SUB + r < m && c < d;
+                    acc[r] = fmaf(in ? X[(uint64_t)(s * SUB + r) * d + c] : 0.0f, c < d ? u[c] : 0.0f, acc[r]);
                 }
         const float tot = reduce8(acc, lane);
         const uint32_t row = s * SUB + (lane >> 2);
