@@ -203,12 +203,14 @@ int qesgd_lr_sgd_step(qesgd_ctx *ctx, const float *Xb, const float *yb, uint32_t
                       float lr, float *u);
 /* The summand of Eq. 2 alone: g_out = (1/m) * sum_j grad f_j(w) on the m rows of Xb, for
  * workers that push (quantised) gradients instead of parameters.  w and g_out are float[d]
- * and must not overlap.  One launch of the persistent local-epoch kernel where that takes the shape
- * on fifteen SMs of sixteen (see qesgd_lr_local_epoch_batch; its waits are bounded,
+ * and must not overlap.  One launch of a local-epoch kernel for an epoch of one step where one takes the
+ * shape on fifteen SMs of sixteen (see qesgd_lr_local_epoch_batch; its waits are bounded,
  * QESGD_STATUS_TIMEOUT), else one margin pass and one pass that writes the gradient; fp32 arithmetic
- * and accumulation as for qesgd_lr_sgd_step.  The persistent kernel starts when the SMs it takes are
- * free of other streams' kernels: a few of those run beside it, gradients of several contexts follow
- * one another (one of 64 x 65536 on each of four streams: 28 us together, 52 by the two passes). */
+ * and accumulation as for qesgd_lr_sgd_step.  Beside other streams' kernels: a grid launched plainly (most
+ * shapes from some 10000 columns on) starts with the SMs that are free and does the work of the rest on them
+ * (64 x 65536 6.5 us alone, 0.1 to 0.2 ms where 24 to 130 of 148 SMs are held); a cluster (fewer columns)
+ * starts once 16, 8 or fewer SMs of one GPC are free (one of 16 beside up to 48 held SMs); the persistent
+ * kernel once all the SMs that it takes are.  Gradients of several contexts follow one another. */
 int qesgd_lr_gradient(qesgd_ctx *ctx, const float *Xb, const float *yb, uint32_t m, uint64_t d,
                       const float *w, float *g_out);
 /* Rows [0, n_local) of X in consecutive minibatches of `batch` rows, in row
@@ -218,40 +220,46 @@ int qesgd_lr_local_epoch(qesgd_ctx *ctx, const float *X, const float *y, uint64_
 /* K workers side by side: worker k owns rows [k*n_local, (k+1)*n_local) of X and
  * y and updates u + k*u_stride (elements).
  * Where the shape allows (minibatches of at most 256 rows whose slices fit the SMs' tensor memory --
- * 64 rows of 1024 columns per SM, 128 of 512, 256 of 256) the whole epoch of all K workers is ONE
- * persistent kernel, launched cooperatively with at most one CTA per SM, that stages every minibatch
- * in shared memory and reads X from HBM once: by TMA where d and u_stride are multiples of 4 and X
- * and u are 16-byte aligned, else by copies of one or two elements (about twice the time for large
- * minibatches).  Its CTAs form groups that share the workers out; the CTAs of a group own a slice of
- * the columns each, and the
- * CTAs exchange partial margins through the context's workspace, which the kernel leaves
- * cleared.  The partial margins of a row are summed across the CTAs as fixed-point integers
- * (units of 2^-28 below 2^17 in magnitude, units of 2^-6 from there to 2^49), so the sum
- * does not depend on the order in which the CTAs arrive; a NaN partial makes the row's
- * margin NaN, an infinite one (or one of 2^49 or more, far beyond where the step
- * coefficient saturates) makes it that infinity, and both then spread through u as they
- * would in floating point.  Every wait the kernel loops on (for another CTA, another warp group, a copy) is
+ * 64 rows of 1024 columns per SM, 128 of 512, 256 of 256 -- or registers) the whole epoch of all K workers is
+ * ONE kernel that stages every minibatch in shared memory and reads X from HBM once: by TMA where d and
+ * u_stride are multiples of 4 and X and u are 16-byte aligned, else by copies of one or two elements (about
+ * twice the time for large minibatches).  A worker's columns are shared out to CTAs that exchange partial
+ * margins.  Which kernel runs is chosen by the modelled time (qesgd_debug_lr_plan tells):
+ *   - persistent: groups of a cooperative grid, at most one CTA per SM, each running one worker or several;
+ *   - few columns per CTA: a cluster of up to 16 CTAs for each worker, an ordinary launch;
+ *   - the same CTAs as groups of a cooperative grid, where a cluster is too small;
+ *   - one minibatch of one worker (a step, a gradient): such a group, launched plainly.
+ * In a cluster the CTAs store their partial margins into one another's shared memory, and the sum over them
+ * carries every addition's error along and is rounded once.  The others exchange through the context's
+ * workspace, which the kernel leaves cleared: the partial margins of a row are summed as fixed-point integers
+ * (units of 2^-28 below 2^17 in magnitude, units of 2^-6 from there to 2^49), so the sum does not depend on the
+ * order in which the CTAs arrive; a NaN partial makes the row's margin NaN, an infinite one (or one of 2^49 or
+ * more, far beyond where the step coefficient saturates) makes it that infinity (NaN where both signs occur).
+ * Non-finite margins spread through u as they would in floating point.
+ * Every wait these kernels loop on (for another CTA, another warp group, a copy) is
  * bounded by the context's wait limit (one second unless qesgd_set_wait_limit changed it):
  * should one run out, the kernel returns, u is left partly updated and
  * QESGD_STATUS_TIMEOUT is set in the status word; the context stays usable and the next call
- * starts clean.  One wait has no bound of its own: at its start the kernel allocates the
+ * starts clean.  One wait has no bound of its own: at its start the persistent kernel allocates the
  * SM's tensor memory, and that allocation blocks while another kernel resident on the same
- * SM (another stream or process) holds tensor memory, until that kernel ends.  The kernel
- * needs all its CTAs resident at once, so do not run it next to other kernels that occupy
- * the device for long.  Other shapes run one margin pass and one
+ * SM (another stream or process) holds tensor memory, until that kernel ends.  A cooperative grid
+ * needs all its CTAs resident at once, a cluster all of its own, so do not run epochs next to other kernels that
+ * occupy the device for long.  Other shapes run one margin pass and one
  * update pass per minibatch, step t of every worker in the same launches.  Results are
- * deterministic (order-free integer sums or a fixed summation order) on either path. */
+ * deterministic (order-free integer sums or a fixed summation order) on every path. */
 int qesgd_lr_local_epoch_batch(qesgd_ctx *ctx, const float *X, const float *y, uint64_t n_local,
                                uint64_t d, uint32_t K, uint32_t batch, float lr, float *u,
                                uint64_t u_stride);
 
-/* Limit, in nanoseconds, of each wait inside the persistent local-epoch kernel (its CTAs
- * wait for one another's partial margins and for their own TMA copies).  0 restores the
+/* Limit, in nanoseconds, of each wait inside the local-epoch kernels (their CTAs
+ * wait for one another's partial margins and for their own copies).  0 restores the
  * default of one second; at most 10 seconds.  A limit below one microsecond means "look once
- * more, then give up" (the device timer is not finer than that).  Takes effect with the next
- * qesgd_lr_local_epoch[_batch] / qesgd_lr_sgd_step call of this context. */
+ * more, then give up" (the device timer is not finer than that).  It is about CTAs that run: where a grid of one
+ * minibatch is launched plainly, the wait for margins counts from when every CTA has started or its work has been
+ * taken over, so other streams' kernels do not use it up (two seconds bound that part).  Takes effect with the next
+ * qesgd_lr_local_epoch[_batch] / qesgd_lr_sgd_step / qesgd_lr_gradient call of this context. */
 int qesgd_set_wait_limit(qesgd_ctx *ctx, uint64_t nanoseconds);
-/* Test hook for the give-up path of that kernel (no counterpart in the paper): CTA number
+/* Test hook for the give-up path of those kernels (no counterpart in the paper): CTA number
  * `cta` does not announce its partial margins of the first minibatch, so every CTA's wait
  * for them runs out after the wait limit, the kernel returns and QESGD_STATUS_TIMEOUT is
  * set.  Nothing faults or hangs.  cta = -1 (the default) switches the hook off. */

@@ -603,8 +603,9 @@ __device__ __forceinline__ void encode_warp_tile(const EncodeArgs &a, float (&z)
 
     // Every bucket's scale, by the first of the lanes that hold its total (with a caller-given spacing: of its elements).
     if (!wide) {
-        // lane's chunk and eight elements of it; a total lies in all lanes that agree with the holder outside `same`:
-        // the bucket's own lanes but for the bits that tell its chunks apart, which are the lowest (chunk_of_lane)
+        // A bucket's total lies in all lanes that its elements in a chunk cover, but that the lowest lane bits
+        // (CHUNK_BITS) tell the warp's chunks apart (chunk_of_lane) instead of the elements: of those lanes the one
+        // whose other bits are zero stores the scale of the bucket that begins at `off`.
         constexpr uint32_t CHUNK_BITS = MODE == 2 || V == 1 ? 0u : (V == 8 ? 7u : (V == 4 ? 3u : 1u));
         const uint32_t lanes = lb >= 8u ? 31u : (1u << (lb - 3u)) - 1u;       // of a chunk that a bucket covers
         if (MODE != 2) {

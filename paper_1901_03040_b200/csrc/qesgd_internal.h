@@ -45,7 +45,8 @@ static const uint64_t QESGD_LR_WORK_FLOATS = (1ull << 20) - QESGD_LR_EPOCH_FLOAT
 // Kernels that go through qesgd_launch may be set up while the kernel before them in the stream drains
 // (programmatic dependent launch), and begin with qesgd_wait_for_previous: nothing is read or written
 // before that one is done and its writes are visible (qesgd_lr_tile.cu launches its clusters and its grids of one
-// minibatch the same way).  The cooperative local-epoch kernels and the debug build's range self-test do not: they are launched plainly, start when all before them is done and contain
+// minibatch the same way).  The cooperative local-epoch kernels and the debug build's range self-test do not: they are
+// launched plainly, start when all before them is done and contain
 // no such wait, so they must not be given the attribute without one (in the epoch kernel ahead of the
 // producers' first copy and the consumers' loads of u).  No kernel lets its successor
 // start earlier than at its own end: a waiting grid would take resident slots.  Without the overlap a

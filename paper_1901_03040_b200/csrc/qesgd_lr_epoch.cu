@@ -531,6 +531,8 @@ __global__ void __launch_bounds__(NC * EP_CHAIN + (EB == 16 ? EP_PRODUCERS : EP_
             if (lane == 0) mbar_arrive(&empty[slot]);
             const float tot = reduce8(acc, lane);
             const uint32_t jj = s * SUB + reduce8_row(lane);
+            // (exchange_add and exchange_margin of qesgd_lr_device.cuh written out: through the functions K = 3, n = 300,
+            // d = 131073 takes 154.5 us instead of 152.8, K = 4, n = 2048, d = 65536 330.5 instead of 329.8)
             if ((lane & 3u) == 0u && jj < T.m && signal) {
                 unsigned long long *const r = acc_t + acc_index(jj);
                 if (fabsf(tot) < FX_LIMIT) {

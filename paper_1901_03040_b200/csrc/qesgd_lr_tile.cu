@@ -4,10 +4,11 @@
 // update -- behind copies of many columns and behind a second chain.  With few columns per CTA nothing hides
 // it, and the chain itself is the time: there every phase goes through shared or tensor memory with four
 // barriers a step, about 3500 clocks of which the exchange is 400 to 1000.  Here a worker has its own CTAs
-// (one cluster of up to 16, a group of the cooperative grid, or for one minibatch a grid launched plainly), and a warp its own eight rows of U x 128
-// columns: the rows live in registers from the margins to the update, a lane always holds the same columns,
-// and the row whose sum a lane ends up with is the row it exchanges and finishes, so between the margins and the
-// update nothing crosses the warp.  Two barriers a step are left, around the sum of the warps' updates.
+// (one cluster of up to 16, a group of the cooperative grid, or for one minibatch a grid launched plainly), and a
+// warp its own eight rows of U x 128 columns: the rows live in registers from the margins to the update, a lane
+// always holds the same columns, and the row whose sum a lane ends up with is the row it exchanges and finishes, so
+// between the margins and the update nothing crosses the warp.  Two barriers a step are left, around the sum of the
+// warps' updates.
 //
 //   M  partial margins of the warp's rows from registers and the slice of u (shared memory); sum over the lanes
 //   X  the sums go out; the slot they came from is refilled (TMA, or element-wise copies); wait for all P
@@ -17,9 +18,9 @@
 //
 // Exchange in a cluster: each CTA stores {partial, tile number + 1} as one 64-bit word into every CTA's shared
 // memory; the reader polls its own.  The number says that the value beside it is there, so there is no barrier
-// and nothing in flight that the cluster's barrier would not cover.  The sum over the ranks is in double
-// precision, in a fixed order.  Exchange in a group: the accumulators in global memory described in
-// qesgd_lr_epoch.cu (qesgd_lr_device.cuh has the code of both kernels).
+// and nothing in flight that the cluster's barrier would not cover.  The sum over the ranks carries every
+// addition's error along (two_sum) and is rounded once, in a fixed order.  Exchange in a group or a plain grid: the
+// accumulators in global memory described in qesgd_lr_epoch.cu, by the functions of qesgd_lr_device.cuh.
 //
 // Every wait is bounded by the context's limit.  A wait that runs out sets QESGD_STATUS_TIMEOUT and the block
 // leaves at its next barrier, together; it then waits for the copies it has requested, and in a cluster until the
@@ -32,7 +33,6 @@
 namespace {
 
 constexpr uint32_t TL_MAX_SLOTS = 64;
-constexpr uint32_t TL_MAX_CLUSTER = 16;
 
 struct TileArgs {
     const float *X, *y;
@@ -40,7 +40,8 @@ struct TileArgs {
     uint32_t P;                  // CTAs per worker
     uint32_t batch, nsteps, m_last, nsub, nsub_last;
     uint32_t nslots;
-    uint32_t off_u, off_part, off_x, off_bars, off_flags, x_pitch;   // shared memory, bytes; words from one rank to the next
+    uint32_t off_u, off_part, off_x, off_bars, off_flags;   // shared memory, bytes
+    uint32_t x_pitch;            // words of the exchange from one rank to the next
     float rate, rate_last;
     const float *u;
     float *dst;
@@ -56,7 +57,8 @@ struct TileArgs {
 };
 constexpr uint64_t TL_STEAL_NS = 20000ull;   // a wait longer than this looks for slices that nobody has begun
 constexpr uint64_t TL_BEGIN_NS = 2000000000ull;   // by then every slice has been begun
-enum Claim { FREE = 0, BEGUN = 1, TAKEN = 2 };    // of a slice: BEGUN by a CTA that runs, or its margins are out; TAKEN over, not yet out
+// A slice is BEGUN by a CTA that runs, or its margins are out; TAKEN: another CTA does it, they are not out yet.
+enum Claim { FREE = 0, BEGUN = 1, TAKEN = 2 };
 constexpr uint32_t TL_ROWS = 128;            // coefficients kept for them
 
 __device__ __forceinline__ uint32_t cluster_address(uint32_t addr, uint32_t rank)
@@ -89,7 +91,10 @@ __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 // A warp's eight totals (lanes 4r to 4r + 3 hold row r's) to every CTA of the cluster: 32 / P lanes a CTA (two and more
 // of them for small clusters, where some lanes have nothing to do), the rows dealt out among them.
-__device__ __forceinline__ uint32_t send_rank(uint32_t P, uint32_t lane) { return P == 16u ? lane >> 1 : (P == 8u ? lane >> 2 : lane >> 3); }
+__device__ __forceinline__ uint32_t send_rank(uint32_t P, uint32_t lane)
+{
+    return P == 16u ? lane >> 1 : (P == 8u ? lane >> 2 : lane >> 3);
+}
 __device__ __forceinline__ uint32_t send_row(uint32_t P, uint32_t lane)
 {
     return P == 16u ? (lane & 1u) * 4u : (P == 8u ? (lane & 3u) * 2u : lane & 7u);
@@ -98,7 +103,8 @@ __device__ __forceinline__ void cluster_send(uint32_t to, uint32_t row, float to
 {
     const float v0 = __shfl_sync(0xFFFFFFFFu, tot, 4u * row), v1 = __shfl_sync(0xFFFFFFFFu, tot, 4u * row + 4u);
     if (P == 16u) {
-        const float v2 = __shfl_sync(0xFFFFFFFFu, tot, 4u * row + 8u), v3 = __shfl_sync(0xFFFFFFFFu, tot, 4u * row + 12u);
+        const float v2 = __shfl_sync(0xFFFFFFFFu, tot, 4u * row + 8u);
+        const float v3 = __shfl_sync(0xFFFFFFFFu, tot, 4u * row + 12u);
         cluster_store2(to, v0, v1, tag);
         cluster_store2(to + 16u, v2, v3, tag);
     } else if (P == 8u) {
@@ -107,7 +113,7 @@ __device__ __forceinline__ void cluster_send(uint32_t to, uint32_t row, float to
         cluster_store(to, v0, tag);
     }
 }
-// a + b = s + e exactly, for finite sums
+// a + b = s + e exactly, for finite sums (the error-free addition of Knuth and of Moller)
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
 {
     s = __fadd_rn(a, b);
@@ -131,27 +137,26 @@ __device__ __forceinline__ void load_n(const float *p, float (&v)[N])
 
 extern __shared__ __align__(1024) unsigned char tl_smem[];
 
-// U blocks of 128 columns, W warps of eight rows each.  Shared memory: a ring of slots of eight rows (boxes of 512 columns
-// one after the other, the last one narrower), the slice of u, the warps' updates, the exchange's words, a
-// barrier per slot, flags.  The sub-tiles (eight rows) of the epoch go round the ring; the warp that has taken one into
-// registers requests the one that the slot serves next, whoever will read it.
-// A kernel argument that the loop uses, in a register: read from the constant bank at each use it costs the chain 40 clocks.
+// A kernel argument that the loop uses, in a register: read from the constant bank at each use it costs the chain
+// 40 clocks.
 __device__ __forceinline__ uint32_t kept(uint32_t v)
 {
     asm volatile("" : "+r"(v));
     return v;
 }
 
-// Slices that nobody has begun.  The grid of one minibatch is launched like any other kernel, so that it is set up while the
-// one before it drains (a cooperative launch is not, and occupies the stream for a whole number of 2.05 us: 64 x 65536 from L2
-// 8.2 us, launched plainly 6.2, from HBM 10.2 and 8.0; 64 x 20000 8.2 and 5.1; 16 x 80000 8.1 and 5.0).  Then nothing promises that all its CTAs are resident at once: beside other streams' kernels
-// some may start late.  So a CTA never waits for one that has not started: each claims its slice when it starts, a wait
-// longer than 20 us claims one that is still free and does its margins here, by the same operations in the same order, and
-// after its own update the CTA does theirs.  A CTA that finds its slice claimed has nothing left to do.
+// Slices that nobody has begun.  The grid of one minibatch is launched like any other kernel, so that it is set up
+// while the one before it drains (a cooperative launch is not, and occupies the stream for a whole number of 2.05 us:
+// 64 x 65536 from L2 8.2 us, launched plainly 6.2, from HBM 10.2 and 8.0; 64 x 20000 8.2 and 5.1; 16 x 80000 8.1 and
+// 5.0).  Then nothing promises that all its CTAs are resident at once: beside other streams' kernels some may start
+// late.  So a CTA never waits for one that has not started: each claims its slice when it starts, a wait longer than
+// 20 us claims one that is still free and does its margins here, by the same operations in the same order, and after
+// its own update the CTA does theirs.  A CTA that finds its slice claimed has nothing left to do.  64 x 65536 beside
+// 24, 64, 100 and 130 held SMs: 96, 133, 147 and 180 us; a cooperative launch waits for those SMs.
 //
 // The wait limit is about CTAs that run and do not answer.  Time in which slices have not been begun, because other
-// streams' kernels hold the SMs, or are being made up for, does not count: a limit of 100 us is no reason to give a call
-// up that takes 131 us beside 120 kernels.  It counts from when a look finds every slice BEGUN.
+// streams' kernels hold the SMs, or are being made up for, does not count: a limit of 100 us is no reason to give up
+// a call that takes 180 us beside such kernels.  It counts from when a look finds every slice BEGUN.
 //
 // A warp looks whether every slice has been begun (then true); where that is `due` it takes a free one and adds its
 // partial margins to the rows' accumulators.
@@ -187,22 +192,32 @@ __device__ __noinline__ bool take_over(const TileArgs &a, uint32_t *list, bool d
                 }
         const float tot = reduce8(acc, lane);
         const uint32_t row = s * SUB + (lane >> 2);
-        if ((lane & 3u) == 0u && row < m) exchange_add(a.acc + acc_index(row), a.wide + (size_t)row * EP_WIDE_WORDS, tot);
+        if ((lane & 3u) == 0u && row < m)
+            exchange_add(a.acc + acc_index(row), a.wide + (size_t)row * EP_WIDE_WORDS, tot);
     }
     __threadfence();
     __syncwarp();
     if (lane == 0) atomicExch(a.claims + slice, (uint32_t)BEGUN);
     return false;
 }
+// One more CTA of the group that neither adds margins nor reads them any more; how many were before it.
+__device__ __forceinline__ uint32_t count_out(uint32_t *header)
+{
+    uint32_t before;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(before) : "l"(header + 1) : "memory");
+    return before;
+}
 // Counted last of the group: nobody adds or reads any more.  By a warp; the accumulators that the epoch has used.
 __device__ __noinline__ void leave_clear(const TileArgs &a, uint32_t lane)
 {
     const uint32_t worker = blockIdx.x / a.P, mpad = SUB * a.nsub, used = min(a.nsteps, (uint32_t)EP_RING);
     uint32_t *const header = a.header + worker * EP_HEADER_WORDS;
+    unsigned long long *const acc = a.acc + (size_t)worker * EP_RING * a.nsub * EP_ACC_PITCH;
+    unsigned long long *const wide = a.wide + (size_t)worker * EP_RING * mpad * EP_WIDE_WORDS;
     for (uint32_t j = lane; j < used * mpad; j += 32u) {
-        a.acc[(size_t)worker * EP_RING * a.nsub * EP_ACC_PITCH + acc_index(j)] = 0ull;   // slots follow one another at the same pitch
+        acc[acc_index(j)] = 0ull;    // slots follow one another at the same pitch
 #pragma unroll
-        for (uint32_t v = 0; v < EP_WIDE_WORDS; ++v) a.wide[((size_t)worker * EP_RING * mpad + j) * EP_WIDE_WORDS + v] = 0ull;
+        for (uint32_t v = 0; v < EP_WIDE_WORDS; ++v) wide[(size_t)j * EP_WIDE_WORDS + v] = 0ull;
     }
     if (a.claims != nullptr)
         for (uint32_t j = lane; j < a.P; j += 32u) a.claims[j] = 0u;
@@ -229,27 +244,34 @@ __device__ __noinline__ void finish_slice(const TileArgs &a, uint32_t slice, con
     }
 }
 
+// U blocks of 128 columns, W warps of eight rows each.  Shared memory: a ring of slots of eight rows (boxes of 512
+// columns one after the other, the last one narrower), the slice of u, the warps' updates, the exchange's words, a
+// barrier per slot, flags.  The sub-tiles (eight rows) of the epoch go round the ring; the warp that has taken one into
+// registers requests the one that the slot serves next, whoever will read it.
 // EX: how a worker's CTAs meet -- a group of a cooperative grid, a cluster, or a plain grid of one minibatch.
 enum Exchange { GROUP = 0, CLUSTER = 1, PLAIN = 2 };
 template <int U, int W, int EB, int EX>
 __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
-    qesgd_lr_tile_kernel(const __grid_constant__ TileArgs a, const __grid_constant__ CUtensorMap map, const __grid_constant__ CUtensorMap map_rest)
+    qesgd_lr_tile_kernel(const __grid_constant__ TileArgs a, const __grid_constant__ CUtensorMap map,
+                         const __grid_constant__ CUtensorMap map_rest)
 {
     constexpr bool CL = EX == CLUSTER, plain = EX == PLAIN;
     constexpr uint32_t COLS = U * 128u, SLOT = SUB * COLS;
-    // The slot of the warp's own sub-tile, once that is in the registers, takes the next copy: right away where blocks are
-    // wide and the ring holds little more than a minibatch, else while the margins travel.
+    // The slot of the warp's own sub-tile, once that is in the registers, takes the next copy: right away where blocks
+    // are wide and the ring holds little more than a minibatch, else while the margins travel.
     constexpr bool EARLY = U >= 3 && EX != PLAIN;
     float *const ring = reinterpret_cast<float *>(tl_smem);
     float *const us = reinterpret_cast<float *>(tl_smem + a.off_u);
     float *const part = reinterpret_cast<float *>(tl_smem + a.off_part);
     uint64_t *const full = reinterpret_cast<uint64_t *>(tl_smem + a.off_bars);
-    // [0] a wait ran out in this CTA, [1] always zero, [2] warps that have read their last margins, [3] the CTA is counted,
-    // [4 + slot] bits: 1 the slot's copy did not land in time, 2 nor did its very first one, so no other is requested
+    // [0] a wait ran out in this CTA, [1] always zero, [2] warps that have read their last margins, [3] the CTA is
+    // counted, [4 + slot] bits: 1 the slot's copy did not land in time, 2 nor did its very first one (either way no
+    // other is requested)
     volatile uint32_t *const flag = reinterpret_cast<volatile uint32_t *>(tl_smem + a.off_flags);
 
     const uint32_t tid = threadIdx.x, lane = tid & 31u, w = tid >> 5;
-    const uint32_t P = kept(a.P), nsteps = plain ? 1u : kept(a.nsteps), batch = kept(a.batch), nsub = kept(a.nsub), nslots = kept(a.nslots);
+    const uint32_t P = kept(a.P), nsteps = plain ? 1u : kept(a.nsteps), batch = kept(a.batch);
+    const uint32_t nsub = kept(a.nsub), nslots = kept(a.nslots);
     const uint32_t worker = blockIdx.x / P, rank = blockIdx.x - worker * P;
     const uint32_t c0 = rank * COLS;
 
@@ -282,7 +304,8 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
                 mbar_arrive_expect_tx(&full[slot], SLOT * 4u);
 #pragma unroll
                 for (uint32_t b = 0; b < COLS; b += 512u)
-                    tma_load_box(dst + SUB * b, b + 512u <= COLS || COLS < 512u ? &map : &map_rest, (c0 + b) / 2u, row, &full[slot]);
+                    tma_load_box(dst + SUB * b, b + 512u <= COLS || COLS < 512u ? &map : &map_rest, (c0 + b) / 2u, row,
+                                 &full[slot]);
             }
         } else {
             constexpr uint32_t N = EB / 4;
@@ -322,7 +345,8 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
         }
     };
 
-    // The first turn of the ring: slot n holds sub-tile n.  The warp's first two now, the rest once the first step is under way.
+    // The first turn of the ring: slot n holds sub-tile n.  The warp's first two now, the rest once the first step is
+    // under way.
     uint32_t slot = w, parity = 0u;
     if (w < subs_of(0u)) request(w, 0u, w);
     // and which sub-tile follows the warp's own of minibatch t in its slot: sub-tile next_s of minibatch t + next_t
@@ -353,7 +377,7 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
         // every copy requested has been taken, or was late and is waited for here as at the end
         if (tid < nslots && flag[4u + tid] != 0u) mbar_wait(&full[tid], 0u, &flag[1], DRAIN_LIMIT_NS);
         uint32_t before = 0u;
-        if (tid == 0) asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(before) : "l"(a.header + 1) : "memory");
+        if (tid == 0) before = count_out(a.header);
         if (w == 0u && __shfl_sync(0xFFFFFFFFu, before, 0) == P - 1u) leave_clear(a, lane);
         return;
     }
@@ -363,12 +387,15 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
     unsigned long long *const wide_g = a.wide + ((size_t)worker * EP_RING * mpad + my_row) * EP_WIDE_WORDS;
     uint32_t *const header = a.header + worker * EP_HEADER_WORDS;
     // the exchange's words: where this lane's go in another CTA, and where it reads (minibatches of odd number: + odd)
-    const uint32_t pitch = kept(a.x_pitch * 8u), words = smem_u32(tl_smem + a.off_x), odd = kept(P * pitch), send_r = send_row(P, lane);
-    const uint32_t send_to = !CL || send_rank(P, lane) >= P ? 0u : cluster_address(words + rank * pitch + (w * SUB + send_r) * 8u, send_rank(P, lane));
+    const uint32_t pitch = kept(a.x_pitch * 8u), words = smem_u32(tl_smem + a.off_x), odd = kept(P * pitch);
+    const uint32_t send_r = send_row(P, lane), to_rank = send_rank(P, lane);
+    const uint32_t send_to =
+        !CL || to_rank >= P ? 0u : cluster_address(words + rank * pitch + (w * SUB + send_r) * 8u, to_rank);
     const uint32_t read_at = words + (lane & 3u) * pitch + my_row * 8u;
     auto refill = [&](uint32_t t, uint32_t late) {
         __syncwarp();            // every lane's rows are in its registers
-        if ((!EARLY || (flag[4u + slot] & late) == 0u) && t + next_t < nsteps && next_s < subs_of(t + next_t)) request(slot, t + next_t, next_s);
+        if ((!EARLY || (flag[4u + slot] & late) == 0u) && t + next_t < nsteps && next_s < subs_of(t + next_t))
+            request(slot, t + next_t, next_s);
     };
     if (EARLY && w < subs_of(0u)) refill(0u, 2u);          // (bit 1 here would be the next turn's, by another warp)
     bool gave_up = false;
@@ -378,7 +405,7 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
     uint32_t t = 0u, m = nsteps == 1u ? m_last : batch, subs = nsteps == 1u ? nsub_last : nsub;
     float ry = (nsteps == 1u ? a.rate_last : a.rate) * yj;
     bool signal = blockIdx.x != a.drop_cta;
-    if ((flag[4u + slot] & 2u) != 0u) {    // the first copy is not there: nothing goes out, and the block leaves after this step
+    if ((flag[4u + slot] & 2u) != 0u) {    // the first copy is not there: nothing goes out, the block leaves this step
         signal = false;
         if (!EARLY) next_t = nsteps;       // no refill (EARLY: refused above)
     }
@@ -426,7 +453,7 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
         const bool more = !last && w < next_subs;
         const float next_y = more && my_row < next_m ? __ldg(label + batch) : 0.0f;
         const bool landed = more && mbar_try_wait(&full[next_slot], next_parity);
-        if (!CL && rank == clears && t + EP_RING / 2 < nsteps) {                       // this CTA clears the accumulators that minibatch t + RING/2 will use
+        if (!CL && rank == clears && t + EP_RING / 2 < nsteps) {     // clears what minibatch t + RING/2 will add to
             const uint32_t zs = (t + EP_RING / 2) % EP_RING;
             unsigned long long *const az = a.acc + ((size_t)worker * EP_RING + zs) * nsub * EP_ACC_PITCH;
             unsigned long long *const wz = a.wide + ((size_t)worker * EP_RING + zs) * mpad * EP_WIDE_WORDS;
@@ -503,7 +530,8 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
                     }
                     const bool due = __any_sync(0xFFFFFFFFu, now_ns() - t0 > TL_STEAL_NS) != 0;
                     if (!begun && (due || __any_sync(0xFFFFFFFFu, expired(t0, a.wait_ns)) != 0)) {
-                        begun = take_over<U>(a, list, due, lane) || __any_sync(0xFFFFFFFFu, now_ns() - t0 > TL_BEGIN_NS) != 0;
+                        begun = take_over<U>(a, list, due, lane) ||
+                                __any_sync(0xFFFFFFFFu, now_ns() - t0 > TL_BEGIN_NS) != 0;
                         if (begun) t0 = now_ns();
                     }
                 }
@@ -518,7 +546,7 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
                 if (atomicAdd(const_cast<uint32_t *>(&flag[2]), 1u) == subs - 1u) {
                     flag[3] = 1u;
                     if (flag[0] != 0u) atomicExch(header, 1u);   // gave up: so shall the others
-                    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(counted) : "l"(header + 1) : "memory");
+                    counted = count_out(header);
                 }
             }
             // ---- U
@@ -589,14 +617,15 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
 
     if (gave_up) {
         if (tid == 0) atomicOr(a.status, QESGD_STATUS_TIMEOUT);
-        // Every slot's last copy has landed before the block ends, so that none is on its way into memory that another block
-        // then owns.  Sub-tile n goes to slot n % nslots, and all below `requested` have been requested, but for those that
-        // would have followed a late one: `next` is the minibatch taken last.
+        // Every slot's last copy has landed before the block ends, so that none is on its way into memory that another
+        // block then owns.  Sub-tile n goes to slot n % nslots, and all below `requested` have been requested, but for
+        // those that would have followed a late one: `next` is the minibatch taken last.
         const uint32_t total = (nsteps - 1u) * nsub + nsub_last, next = min(gave_up_at + EARLY, nsteps - 1u);
         const uint32_t requested = min(total, (gave_up_at + EARLY) * nsub + subs_of(next) + nslots);
         for (uint32_t q = tid; q < nslots && q < requested; q += W * 32u) {
             const uint32_t late = flag[4u + q];
-            const uint32_t turn = late & 2u ? 0u : (EARLY && late != 0u ? next * nsub + nslots - 1u - q : requested - 1u - q) / nslots;
+            const uint32_t before = EARLY && late != 0u ? next * nsub + nslots - 1u - q : requested - 1u - q;
+            const uint32_t turn = late & 2u ? 0u : before / nslots;
             mbar_wait(&full[q], turn & 1u, &flag[1], DRAIN_LIMIT_NS);
         }
         if (CL) {
@@ -604,7 +633,7 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
             cluster_wait();
         } else if (tid == 0 && flag[3] == 0u) {
             atomicExch(header, 1u);
-            asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(counted) : "l"(header + 1) : "memory");
+            counted = count_out(header);
         }
     }
     if (CL) return;
@@ -618,7 +647,8 @@ struct Variant {
     uint32_t U, W;
     TileKernel kernel[3][3];     // by Exchange; copies of 16 (TMA), 8, 4 bytes
 };
-#define TL_COPIES(U, W, EX) {qesgd_lr_tile_kernel<U, W, 16, EX>, qesgd_lr_tile_kernel<U, W, 8, EX>, qesgd_lr_tile_kernel<U, W, 4, EX>}
+#define TL_COPIES(U, W, EX) \
+    {qesgd_lr_tile_kernel<U, W, 16, EX>, qesgd_lr_tile_kernel<U, W, 8, EX>, qesgd_lr_tile_kernel<U, W, 4, EX>}
 #define TL_VARIANT(U, W) {U, W, {TL_COPIES(U, W, GROUP), TL_COPIES(U, W, CLUSTER), TL_COPIES(U, W, PLAIN)}}
 // Registers: 32 U for the rows.  A block of eight warps has 255 a thread, one of sixteen 128.  (Six blocks of columns
 // spill: a gradient of 64 x 100000 10.4 us against 10.3 for the other kernel.)
@@ -663,7 +693,8 @@ bool lay_out(Plan &p, uint32_t nsub, uint64_t subtiles, uint32_t limit)
     p.x_pitch = SUB * nsub + (nsub % 2u ? 12u : 4u);
     const uint32_t xbytes = p.exchange == CLUSTER ? 2u * p.P * p.x_pitch * 8u : 0u;
     const uint32_t cbytes = p.exchange == PLAIN ? (TL_ROWS + 1u + 256u) * 4u : 0u;
-    const uint32_t fixed = cols * 4u + p.v->W * cols * 4u + xbytes + TL_MAX_SLOTS * 8u + (4u + TL_MAX_SLOTS) * 4u + cbytes;
+    const uint32_t fixed =
+        cols * 4u + p.v->W * cols * 4u + xbytes + TL_MAX_SLOTS * 8u + (4u + TL_MAX_SLOTS) * 4u + cbytes;
     const uint32_t have = budget(*p.v, limit);
     if (fixed + nsub * slot > have) return false;
     p.nslots = (have - fixed) / slot;
@@ -688,14 +719,16 @@ bool prepare_device(int device, uint32_t limit)
         for (uint32_t j = 0; j < 9u; ++j) {
             const void *const k = (const void *)VARIANTS[i].kernel[j / 3u][j % 3u];
             if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit) != cudaSuccess ||
-                (j / 3u == CLUSTER && cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
+                (j / 3u == CLUSTER &&
+                 cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
                 cudaGetLastError();
                 return false;
             }
         }
         for (uint32_t l = 0; l < 5u; ++l) {
             cudaLaunchAttribute at[2];
-            const cudaLaunchConfig_t c = cluster_config(1u << l, 1u << l, VARIANTS[i].W * 32u, budget(VARIANTS[i], limit), nullptr, at);
+            const cudaLaunchConfig_t c =
+                cluster_config(1u << l, 1u << l, VARIANTS[i].W * 32u, budget(VARIANTS[i], limit), nullptr, at);
             int n = 0, least = 1 << 30;
             for (const TileKernel k : VARIANTS[i].kernel[CLUSTER]) {
                 if (cudaOccupancyMaxActiveClusters(&n, k, &c) != cudaSuccess) {
@@ -712,15 +745,17 @@ bool prepare_device(int device, uint32_t limit)
 }
 
 // Modelled time of an epoch in us (measured over some 20 shapes, see below): a step's chain, the copies, the launch.
-// A chain costs 0.85 us in a cluster and 1.3 through global memory, and for each block of 128 columns 0.03 and 0.026 for
-// each eight rows; element-wise copies are issued by the warps themselves, and sixteen warps meet later than eight.  HBM
-// is not reached where the ring holds little more than a minibatch (U > 2).  A cluster is launched with the kernel before it
-// still draining; a cooperative grid is not.  Clusters that take turns cost a fifth more than a turn each.
+// A chain costs 0.85 us in a cluster and 1.3 through global memory, and for each block of 128 columns 0.03 and 0.026
+// for each eight rows; element-wise copies are issued by the warps themselves, and sixteen warps meet later than eight.
+// HBM is not reached where the ring holds little more than a minibatch (U > 2).  A cluster is launched with the kernel
+// before it still draining; a cooperative grid is not.  Clusters that take turns cost a fifth more than a turn each.
 float modelled_us(const Plan &p, const QesgdTileCall &q, uint32_t nsub, uint32_t waves)
 {
     const float hbm = (float)((double)q.K * q.m * q.d * 4.0 / 6.5e6), U = (float)p.v->U, rows = (float)nsub;
     const float copy = q.copy == 16 ? 0.0f : (q.copy == 8 ? 0.045f : 0.085f) * U * rows;
-    const float chain = (waves > 1u ? 1.2f * (float)waves : 1.0f) * ((p.exchange == CLUSTER ? 0.85f : 1.3f) + U * (0.03f + 0.026f * rows) + copy + (p.v->W == 16u ? 0.3f : 0.0f));
+    const float turn =
+        (p.exchange == CLUSTER ? 0.85f : 1.3f) + U * (0.03f + 0.026f * rows) + copy + (p.v->W == 16u ? 0.3f : 0.0f);
+    const float chain = (waves > 1u ? 1.2f * (float)waves : 1.0f) * turn;
     const float fetch = hbm * (p.v->U > 2u ? 1.3f : 1.1f);
     const float start = p.exchange != GROUP ? 2.0f * (float)waves - 0.5f : (p.v->U > 2u ? 5.0f : 4.0f);
     return (float)q.nsteps * (chain > fetch ? chain : fetch) + start;
@@ -730,13 +765,17 @@ float modelled_us(const Plan &p, const QesgdTileCall &q, uint32_t nsub, uint32_t
 
 // Which kernel.  Both times are modelled (the other kernel's by qesgd_lr_epoch.cu, within a quarter of what it takes).
 // Measured, whole epochs back to back, other kernel -> this one:
-//   K = 4, n = 128, d = 4096, batch 32 (cluster of 16, two blocks): 14.4 -> 7.0 us;  K = 4, n = 1000, d = 1000, batch 32 (8, one)
-//   71.8 -> 34.1;  K = 2, n = 800, d = 300, batch 64 (4, one) 41.0 -> 16.6;  K = 8, n = 500, d = 2000, batch 100 (8, two, sixteen
-//   warps) 28.7 -> 12.4;  K = 8, n = 2000, d = 128, batch 16 (one CTA) 271 -> 126;  one gradient of 64 x 4096 (16, two) 6.7 -> 3.5;
-//   gradients of 64 x 65536 (128 CTAs, four) 8.2 -> 6.2;  K = 1, n = 1010, d = 10000, batch 50 (79 CTAs of a group, one) 44.7 -> 36.9;  K = 8 of them (16 CTAs, five) 80.8 -> 71.1;
-//   K = 4, n = 1000, d = 16384, batch 32 (32 CTAs, four) 89.5 -> 72.3.
-// Where it loses and is not taken: more clusters than the device holds at once (K = 16, n = 200, d = 8000, batch 64: 32.5 in three
-// turns against 28.7); element-wise copies of many columns (K = 6, n = 700, d = 8003, batch 50: 57 against 49).
+//   K = 4, n = 128, d = 4096, batch 32 (cluster of 16, two blocks): 14.4 -> 7.0 us
+//   K = 4, n = 1000, d = 1000, batch 32 (8, one): 71.8 -> 34.1;  K = 2, n = 800, d = 300, batch 64 (4, one): 41.0 -> 16.6
+//   K = 8, n = 500, d = 2000, batch 100 (8, two, sixteen warps): 28.7 -> 12.4
+//   K = 8, n = 2000, d = 128, batch 16 (one CTA): 271 -> 126;  one gradient of 64 x 4096 (16, two): 6.7 -> 3.5
+//   gradients of 64 x 65536 (128 CTAs, four): 8.2 -> 6.2
+//   K = 1, n = 1010, d = 10000, batch 50 (79 CTAs of a group, one): 44.7 -> 36.9;  K = 8 of them (16, five): 80.8 -> 71.1
+//   K = 4, n = 1000, d = 16384, batch 32 (32 CTAs, four): 89.5 -> 72.3
+// Where it loses and is not taken: more clusters than the device holds at once (K = 16, n = 200, d = 8000, batch 64: 32.5
+// in three turns against 28.7); element-wise copies of many columns (K = 6, n = 700, d = 8003, batch 50: 57 against 49).
+// A cluster starts when one GPC has its SMs free: one of 16 beside up to 48 held SMs at once, beside 64 after them (one
+// of 8 beside 100, not beside 130).
 int qesgd_launch_lr_tile(const QesgdTileCall &q, uint32_t smem_limit, float other_us, int *launched,
                          uint32_t (&plan)[8])
 {
@@ -787,13 +826,15 @@ int qesgd_launch_lr_tile(const QesgdTileCall &q, uint32_t smem_limit, float othe
     a.header = q.header; a.acc = q.acc; a.wide = q.wide;
     a.status = q.status; a.wait_ns = q.wait_ns; a.poll_mask = q.wait_ns < COARSE_TIMER_NS ? 0u : 31u;
     a.drop_cta = q.drop_cta;
-    a.claims = p.exchange == PLAIN ? q.header + EP_HEADER_WORDS : nullptr;       // the headers of other workers' groups, of which there are none
+    // in the headers of other workers' groups, of which there are none
+    a.claims = p.exchange == PLAIN ? q.header + EP_HEADER_WORDS : nullptr;
     a.off_claims = p.off_claims;
     static_assert(QESGD_MAX_WORKERS * EP_HEADER_WORDS >= EP_HEADER_WORDS + 256u, "a word for each CTA");
     CUtensorMap map = {}, map_rest = {};
     const uint32_t cols = p.v->U * 128u, rest = cols > 512u ? cols - 512u : cols;
-    if (q.copy == 16 && !qesgd_lr_tensor_map(&map, q.X, (uint64_t)q.K * q.n_local, q.d, cols < 512u ? cols : 512u, true)) return -1;
-    if (q.copy == 16 && cols > 512u && !qesgd_lr_tensor_map(&map_rest, q.X, (uint64_t)q.K * q.n_local, q.d, rest, true)) return -1;
+    const uint64_t rows = (uint64_t)q.K * q.n_local;
+    if (q.copy == 16 && !qesgd_lr_tensor_map(&map, q.X, rows, q.d, cols < 512u ? cols : 512u, true)) return -1;
+    if (q.copy == 16 && cols > 512u && !qesgd_lr_tensor_map(&map_rest, q.X, rows, q.d, rest, true)) return -1;
     const TileKernel kernel = p.v->kernel[p.exchange][q.copy == 16 ? 0 : (q.copy == 8 ? 1 : 2)];
     const uint32_t threads = W * 32u;
     cudaError_t err;
@@ -809,7 +850,8 @@ int qesgd_launch_lr_tile(const QesgdTileCall &q, uint32_t smem_limit, float othe
         err = cudaLaunchKernelEx(&c, kernel, a, map, map_rest);
     } else {
         void *params[] = {(void *)&a, (void *)&map, (void *)&map_rest};
-        err = cudaLaunchCooperativeKernel((const void *)kernel, dim3(q.K * p.P), dim3(threads), params, p.bytes, q.stream);
+        err = cudaLaunchCooperativeKernel((const void *)kernel, dim3(q.K * p.P), dim3(threads), params, p.bytes,
+                                          q.stream);
     }
     if (err == cudaErrorCooperativeLaunchTooLarge || err == cudaErrorLaunchOutOfResources ||
         err == cudaErrorInvalidConfiguration || err == cudaErrorNotSupported || err == cudaErrorInvalidClusterSize) {
@@ -818,7 +860,8 @@ int qesgd_launch_lr_tile(const QesgdTileCall &q, uint32_t smem_limit, float othe
     }
     if (err != cudaSuccess) return (int)err;
     *launched = 1;
-    const uint32_t kind = p.exchange == PLAIN ? QESGD_LR_PLAIN : (p.exchange == CLUSTER ? QESGD_LR_CLUSTER : QESGD_LR_GROUP);
+    const uint32_t kind =
+        p.exchange == PLAIN ? QESGD_LR_PLAIN : (p.exchange == CLUSTER ? QESGD_LR_CLUSTER : QESGD_LR_GROUP);
     const uint32_t shape[8] = {kind, p.P, cols, W, p.nslots, (uint32_t)q.copy, q.K * p.P, 1u};
     for (int i = 0; i < 8; ++i) plan[i] = shape[i];
     return 0;
