@@ -322,9 +322,10 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
         }
     };
     // a warp's rows of a landed slot into registers, zeros past the minibatch
+    // (`late` in the slot's flag word if the copy did not land in time)
     float4 x[U][SUB];
     auto take = [&](bool landed, uint32_t slot, uint32_t parity, uint32_t rows, uint32_t late) {
-        if (!landed && !mbar_wait(&full[slot], parity, &flag[0], a.wait_ns)) {
+        if (!landed && __builtin_expect(!mbar_wait(&full[slot], parity, &flag[0], a.wait_ns), 0)) {
             flag[0] = 1u;
             flag[4u + slot] = flag[4u + slot] | late;
         }
@@ -405,7 +406,11 @@ __global__ void __launch_bounds__(W * 32, U == 1 && W == 8 ? 2 : 1)
     uint32_t t = 0u, m = nsteps == 1u ? m_last : batch, subs = nsteps == 1u ? nsub_last : nsub;
     float ry = (nsteps == 1u ? a.rate_last : a.rate) * yj;
     bool signal = blockIdx.x != a.drop_cta;
-    if ((flag[4u + slot] & 2u) != 0u) {    // the first copy is not there: nothing goes out, the block leaves this step
+    // The first copy is not there: nothing goes out, the block leaves this step.  (The hint is worth 4 % to clusters fed
+    // by TMA, K = 7, n = 1075, d = 1228, batch 100 26.3 -> 25.3 us, and costs the others 2 to 8: K = 3, n = 530,
+    // d = 1611, batch 128 15.8 -> 17.7, gradient of 64 x 24780 5.08 -> 5.26.)
+    const bool missing = (flag[4u + slot] & 2u) != 0u;
+    if (CL && EB == 16 ? __builtin_expect(missing, 0) : missing) {
         signal = false;
         if (!EARLY) next_t = nsteps;       // no refill (EARLY: refused above)
     }
@@ -766,14 +771,17 @@ float modelled_us(const Plan &p, const QesgdTileCall &q, uint32_t nsub, uint32_t
 // Which kernel.  Both times are modelled (the other kernel's by qesgd_lr_epoch.cu, within a quarter of what it takes).
 // Measured, whole epochs back to back, other kernel -> this one:
 //   K = 4, n = 128, d = 4096, batch 32 (cluster of 16, two blocks): 14.4 -> 7.0 us
-//   K = 4, n = 1000, d = 1000, batch 32 (8, one): 71.8 -> 34.1;  K = 2, n = 800, d = 300, batch 64 (4, one): 41.0 -> 16.6
+//   K = 4, n = 1000, d = 1000, batch 32 (8, one): 71.8 -> 34.1
+//   K = 2, n = 800, d = 300, batch 64 (4, one): 41.0 -> 16.6
 //   K = 8, n = 500, d = 2000, batch 100 (8, two, sixteen warps): 28.7 -> 12.4
 //   K = 8, n = 2000, d = 128, batch 16 (one CTA): 271 -> 126;  one gradient of 64 x 4096 (16, two): 6.7 -> 3.5
 //   gradients of 64 x 65536 (128 CTAs, four): 8.2 -> 6.2
-//   K = 1, n = 1010, d = 10000, batch 50 (79 CTAs of a group, one): 44.7 -> 36.9;  K = 8 of them (16, five): 80.8 -> 71.1
+//   K = 1, n = 1010, d = 10000, batch 50 (79 CTAs of a group, one): 44.7 -> 36.9
+//   K = 8 of them (16, five): 80.8 -> 71.1
 //   K = 4, n = 1000, d = 16384, batch 32 (32 CTAs, four): 89.5 -> 72.3
-// Where it loses and is not taken: more clusters than the device holds at once (K = 16, n = 200, d = 8000, batch 64: 32.5
-// in three turns against 28.7); element-wise copies of many columns (K = 6, n = 700, d = 8003, batch 50: 57 against 49).
+// Where it loses and is not taken: more clusters than the device holds at once (K = 16, n = 200, d = 8000, batch 64:
+// 32.5 in three turns against 28.7); element-wise copies of many columns (K = 6, n = 700, d = 8003, batch 50: 57
+// against 49).
 // A cluster starts when one GPC has its SMs free: one of 16 beside up to 48 held SMs at once, beside 64 after them (one
 // of 8 beside 100, not beside 130).
 int qesgd_launch_lr_tile(const QesgdTileCall &q, uint32_t smem_limit, float other_us, int *launched,
