@@ -152,7 +152,7 @@ __device__ __forceinline__ uint32_t kept(uint32_t v)
 // late.  So a CTA never waits for one that has not started: each claims its slice when it starts, a wait longer than
 // 20 us claims one that is still free and does its margins here, by the same operations in the same order, and after
 // its own update the CTA does theirs.  A CTA that finds its slice claimed has nothing left to do.  64 x 65536 beside
-// 24, 64, 100 and 130 held SMs: 96, 133, 147 and 180 us; a cooperative launch waits for those SMs.
+// 24, 64, 100 and 130 held SMs: 95, 131, 156 and 194 us; a cooperative launch waits for those SMs.
 //
 // The wait limit is about CTAs that run and do not answer.  Time in which slices have not been begun, because other
 // streams' kernels hold the SMs, or are being made up for, does not count: a limit of 100 us is no reason to give up
@@ -179,17 +179,30 @@ __device__ __noinline__ bool take_over(const TileArgs &a, uint32_t *list, bool d
     if (lane == 0) list[1u + atomicAdd(list, 1u)] = slice;
     const uint32_t m = a.m_last, nsub = a.nsub_last;
     const float *const X = a.X, *const u = a.u;
-    const uint64_t d = a.d;
+    const uint64_t d = a.d, c0 = (uint64_t)slice * (U * 128u) + lane * 4u;
     for (uint32_t s = 0; s < nsub; ++s) {
         float acc[SUB];
-        for (int r = 0; r < SUB; ++r) acc[r] = 0.0f;
-        for (uint32_t it = 0; it < (uint32_t)U; ++it)
-            for (int r = 0; r < SUB; ++r)
+        // Two rows at a time: what this needs of registers the kernel saves around the call, and for sixteen warps of two
+        // blocks all eight at once cost the way without it too (gradient of 100 x 30001 8.4 us, so 7.5).
+#pragma unroll 1
+        for (uint32_t g = 0; g < 4u; ++g) {
+            const float *line = X + (uint64_t)(s * SUB + g * 2u) * d + c0;
+            float p[2];
+#pragma unroll
+            for (int r = 0; r < 2; ++r) p[r] = 0.0f;
+#pragma unroll 1
+            for (uint32_t c = 0; c < U * 128u; c += 128u)
+#pragma unroll
                 for (uint32_t e = 0; e < 4u; ++e) {
-                    const uint64_t c = (uint64_t)slice * (U * 128u) + it * 128u + lane * 4u + e;
-                    const bool in = s * SUB + r < m && c < d;
-                    acc[r] = fmaf(in ? X[(uint64_t)(s * SUB + r) * d + c] : 0.0f, c < d ? u[c] : 0.0f, acc[r]);
+                    const float w = c0 + c + e < d ? u[c0 + c + e] : 0.0f;
+#pragma unroll
+                    for (uint32_t r = 0; r < 2u; ++r)
+                        p[r] = fmaf(s * SUB + g * 2u + r < m && c0 + c + e < d ? line[r * d + c + e] : 0.0f, w, p[r]);
                 }
+#pragma unroll
+            for (uint32_t r = 0; r < (uint32_t)SUB; ++r)
+                if (r / 2u == g) acc[r] = p[r % 2u];
+        }
         const float tot = reduce8(acc, lane);
         const uint32_t row = s * SUB + (lane >> 2);
         if ((lane & 3u) == 0u && row < m)
